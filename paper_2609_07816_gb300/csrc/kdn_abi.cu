@@ -297,7 +297,8 @@ size_t workspace_layout(Args *a, char *base, bool bwd) {
     a->fpin = take(BH * NC64 * dk);
     return off;
   }
-  a->phat = take(BH * Tp * P);
+  a->comp = take(BH * NC * P * 4);
+  a->pin = take(BH * NC * P);
   a->isotok = a->variant == 1 ? take(BH * Tp * 2) : nullptr;
   a->W = take(BH * NC * C * dk);
   a->U = take(BH * NC * C * dv);
@@ -306,6 +307,11 @@ size_t workspace_layout(Args *a, char *base, bool bwd) {
   a->Kt = take(BH * NC * C * dk);
   a->gC = take(BH * NC * dk);
   if (bwd) {
+    a->phat = take(BH * Tp * P);
+    a->gam = take(BH * Tp * dk);
+    a->Ainv = take(BH * NC * C * C);
+    a->stok = take(BH * Tp);
+    a->R = take(BH * NC * C * dv);
     a->Sin = take(BH * NC * dk * dv);
     a->dSout = take(BH * NC * dk * dv);
     a->dR = take(BH * NC * C * dv);
@@ -313,8 +319,8 @@ size_t workspace_layout(Args *a, char *base, bool bwd) {
     a->dgpart = take(BH * Tp * dk);
     a->dphloc = take(BH * Tp * P);
     a->drpart = take(BH * Tp);
-    a->drw = take(BH * Tp * 4);
-    a->isoadj = a->variant == 1 ? take(BH * Tp * 2) : nullptr;
+    a->aff = take(BH * NC * P * 2);
+    a->dpout = take(BH * NC * P);
   }
   return off;
 }

@@ -108,22 +108,29 @@ struct Args {
   float *dmu;  // [B,H] gradient with respect to mu (nullable)
   // workspace regions (float32 unless noted)
   unsigned *status;
-  float *phat;    // [BH][Tp][P]   predictive variance phat_t (pre-write)
+  float *comp;    // [BH][NC][P][4] Moebius summaries of the chunks
+  float *pin;     // [BH][NC][P]    uncertainty entering every chunk
   float *isotok;  // [BH][Tp][2]   isotropic: a_t, |k_t|^2
   float *W, *U;   // [BH][NC][C][dk], [BH][NC][C][dv]
   float *Qb;      // [BH][NC][C][dk]
   float *Aqk;     // [BH][NC][C][C]
   float *Kt;      // [BH][NC][C][dk]
   float *gC;      // [BH][NC][dk]   gamma_C
-  float *Sin;     // [BH][NC][dk][dv] chunk-entry memory (backward)
+  // backward only
+  float *phat;    // [BH][Tp][P]   predictive variance phat_t (pre-write)
+  float *gam;     // [BH][Tp][dk]  cumulative decay inside the chunk
+  float *Ainv;    // [BH][NC][C][C] A = (I + T)^-1
+  float *stok;    // [BH][Tp]      s_t (diag) or beta_t (iso)
+  float *R;       // [BH][NC][C][dv]
+  float *Sin;     // [BH][NC][dk][dv] chunk-entry memory
   float *dSout;   // [BH][NC][dk][dv] cotangent of the chunk-exit memory
   float *dR;      // [BH][NC][C][dv]
   float *dkpart;  // [BH][Tp][dk]
   float *dgpart;  // [BH][Tp][dk]
   float *dphloc;  // [BH][Tp][P]
   float *drpart;  // [BH][Tp]
-  float *drw;     // [BH][Tp][4]
-  float *isoadj;  // [BH][Tp][2]
+  float *aff;     // [BH][NC][P][2] chunk summaries of the uncertainty adjoint
+  float *dpout;   // [BH][NC][P]    cotangent of the uncertainty leaving every chunk
   unsigned char *fSin;  // fused backward: [BH][NC] context records (S_in, R, -W, A_qk, A)
   float *fpin;          // fused backward: [BH][NC][dk] uncertainty entering each chunk
 };
@@ -185,7 +192,8 @@ size_t seg_workspace_bytes(const Args &a, int P);
 kdn_status_t launch_seg_fwd(const Args &a, int P, char *ws, cudaStream_t s);
 
 // Launchers (each returns KDN_OK or KDN_ERR_CUDA).
-kdn_status_t launch_chunked_fwd(const Args &a, cudaStream_t s, bool save_states);
+// save: also keep what the chunked backward reads (the backward part of the workspace)
+kdn_status_t launch_chunked_fwd(const Args &a, cudaStream_t s, bool save);
 kdn_status_t launch_chunked_bwd(const Args &a, cudaStream_t s);
 kdn_status_t launch_decode(const Args &a, float *S, float *p, cudaStream_t s);
 
