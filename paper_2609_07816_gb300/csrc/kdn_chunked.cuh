@@ -27,6 +27,14 @@ template <> __device__ __forceinline__ void ld4<__nv_bfloat16>(const void *p, si
   v[2] = __uint_as_float(u.y << 16);
   v[3] = __uint_as_float(u.y & 0xffff0000u);
 }
+// n / d for a normal d: the approximate reciprocal and one Newton (residual) correction
+// of the quotient, which leaves the last bit's rounding at most.
+__device__ __forceinline__ float div_nr(float n, float d) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
+  const float q = n * r;
+  return fmaf(fmaf(-d, q, n), r, q);
+}
 __device__ __forceinline__ float4 f4(const float *v) { return make_float4(v[0], v[1], v[2], v[3]); }
 __device__ __forceinline__ void st4(float *p, const float *v) { *reinterpret_cast<float4 *>(p) = f4(v); }
 // four adjacent outputs in the caller's output dtype
@@ -45,9 +53,9 @@ __device__ __forceinline__ void sto4(int odt, void *p, size_t i, const float *v)
 // acc[m][n] += sum_k A[row m][k] B[k][n].  The thread's rows of A start at A and lie
 // `sa` floats apart, k contiguous.  BK: its four columns are rows of a tile with k
 // contiguous (ldb apart); else four adjacent columns of a [k][n] tile.
-template <int K, int TM, bool BK>
-__device__ __forceinline__ void tile_mm(float (*acc)[4], const float *A, int sa, const float *B, int ldb) {
-#pragma unroll 2
+template <int K, int TM, bool BK, typename TB = float>
+__device__ __forceinline__ void tile_mm(float (*acc)[4], const float *A, int sa, const TB *B, int ldb) {
+#pragma unroll(TM > 2 ? 2 : 4)
   for (int k = 0; k < K; k += 4) {
     float a[TM][4], b[4][4];
 #pragma unroll
@@ -55,7 +63,7 @@ __device__ __forceinline__ void tile_mm(float (*acc)[4], const float *A, int sa,
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       float x[4];
-      ld4<float>(BK ? B + q * ldb + k : B + (k + q) * ldb, 0, x);
+      ld4<TB>(BK ? B + q * ldb + k : B + (k + q) * ldb, 0, x);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         if (BK) b[u][q] = x[u];
@@ -121,7 +129,7 @@ __device__ __forceinline__ void cp_wait() {
 }
 
 // CW value columns per CTA.  [W; Qbar] S_in is a 64 x CW product; TM of its rows and
-// four columns a thread: 16 / TM * CW threads.  The 32 rows of R and of O are split evenly over
+// four columns a thread: 16 CW / TM threads.  The 32 rows of R and of O are split evenly over
 // the threads (rows ga + GA m: the first half of a thread's rows are R's).
 template <int DK, int CW, int TM>
 struct StateCfg {

@@ -326,7 +326,9 @@ __global__ void __launch_bounds__(BwdCfg<DK>::NTH) k_chunk_bwd(Args a) {
   // Back through the scaling by gamma = exp(G): dq, the key/gain cotangents, and dG (into sdQ).
   for (int e = tid; e < CC * (DK / 4); e += NTH) {
     const int t = e / (DK / 4), i4 = 4 * (e % (DK / 4)), o = t * LD + i4;
-    float gam[4], dKb[4], dKx[4], dQb[4], kb[4], kk[4], qb[4], dq[4];
+    float gam[4], dKb[4], dKx[4], dQb[4], kb[4], kk[4], qb[4], dq[4], kx[4] = {0.f, 0.f, 0.f, 0.f}, px[4];
+    if (t < tn) ld4<DT>(a.k, tok_index(a, b, c * CC + t, h) * DK + i4, kx);
+    if (V == 0) ld4<float>(a.phat + (row0 + t) * DK, i4, px);
     ld4<float>(sGa, o, gam);
     ld4<float>(sdW, o, dKb);
     ld4<float>(sdKk, o, dKx);
@@ -349,6 +351,14 @@ __global__ void __launch_bounds__(BwdCfg<DK>::NTH) k_chunk_bwd(Args a) {
     st4(sdW + o, dKb);
     st4(sdKk + o, dKx);
     st4(sKk + o, kk);
+    st4(sGa + o, kx);  // k and phat for the gain adjoint, over tiles that are dead now
+    if (V == 0) st4(sQ + o, px);
+  }
+  float gvv[CC];  // the decay inputs of this thread's channel, loaded ahead of the chunk's summary
+  if (V == 0 && tid < DK) {
+#pragma unroll
+    for (int t = 0; t < CC; ++t)
+      gvv[t] = t < tn ? ld<DT>(a.g, tok_index(a, b, c * CC + t, h) * DK + tid) : 0.f;
   }
   __syncthreads();
   // reverse cumulative sum over the chunk: dg_j = sum_{r >= j} dG_r
@@ -367,7 +377,7 @@ __global__ void __launch_bounds__(BwdCfg<DK>::NTH) k_chunk_bwd(Args a) {
     float kv[DK / 32];
 #pragma unroll
     for (int m = 0; m < DK / 32; ++m)
-      kv[m] = t < tn ? ld<DT>(a.k, tok_index(a, b, c * CC + t, h) * DK + lane + 32 * m) : 0.f;
+      kv[m] = sGa[t * LD + lane + 32 * m];
     float part = 0.f;
 #pragma unroll
     for (int m = 0; m < DK / 32; ++m) {
@@ -379,7 +389,7 @@ __global__ void __launch_bounds__(BwdCfg<DK>::NTH) k_chunk_bwd(Args a) {
 #pragma unroll
       for (int m = 0; m < DK / 32; ++m) {
         const int i = lane + 32 * m;
-        const float dkap = sdKk[t * LD + i], ph = a.phat[row * DK + i];
+        const float dkap = sdKk[t * LD + i], ph = sQ[t * LD + i];
         const float dphl = dkap * kv[m] / s + ds * kv[m] * kv[m];
         a.dphloc[row * DK + i] = dphl;
         a.dkpart[row * DK + i] = sdW[t * LD + i] + dkap * ph / s + 2.f * ds * ph * kv[m];
@@ -408,9 +418,9 @@ __global__ void __launch_bounds__(BwdCfg<DK>::NTH) k_chunk_bwd(Args a) {
   if (V == 0) {
     if (tid < DK) {
       float A = 1.f, Bv = 0.f;
-#pragma unroll 8
+#pragma unroll
       for (int t = CC - 1; t >= 0; --t) {
-        const float lg = t < tn ? gate_logalpha(a.gates, ld<DT>(a.g, tok_index(a, b, c * CC + t, h) * DK + tid)) : 0.f;
+        const float lg = t < tn ? gate_logalpha(a.gates, gvv[t]) : 0.f;
         const float al2 = expf(2.f * lg), rd = sKk[t * LD + tid], f = al2 * rd * rd;
         Bv = fmaf(f, Bv, al2 * sdKk[t * LD + tid]);
         A *= f;

@@ -165,10 +165,12 @@ __global__ void __launch_bounds__(128) k_gain_scan(Args a) {
 // Chunk-local factors.
 // Tokens past T are identity tokens: k = q = v = 0, g = 0, omega = 0, r = 1, kappa = 0.
 
-template <int DK>
+// row stride (elements) of the V tile, kept in the activations' dtype: 16-byte rows
+template <typename DT> __host__ __device__ constexpr int v_stride(int dv) { return dv + 16 / (int)sizeof(DT); }
+template <typename DT, int DK>
 constexpr size_t prep_smem_bytes(int dv) {
-  return sizeof(float) * (3 * CC * (DK + 4) + CC * (dv + 4) + 2 * CC * LC + 16 * 20 + 4 * CC + DK +
-                          PT * 5);
+  return sizeof(float) * (3 * CC * (DK + 4) + 2 * CC * LC + 16 * 20 + 4 * CC + DK + PT * 5) +
+         sizeof(DT) * CC * v_stride<DT>(dv);
 }
 
 // A = (I + T)^-1 (32 x 32, T strictly lower in sT; zero above the diagonal of A):
@@ -241,13 +243,14 @@ __device__ __forceinline__ void inverse32(const float *sT, float *sA, float *sX)
 
 // SAVE: also keep phat, gamma, A and s_t (iso: beta_t) for the backward.
 template <int V, typename DT, int DK, int SAVE>
-__global__ void __launch_bounds__(PT) k_chunk_prep(Args a) {
+__global__ void __launch_bounds__(PT, DK < 128 ? 5 : 3) k_chunk_prep(Args a) {
   constexpr int LD = DK + 4, NSEG = PT / DK, SL = CC / NSEG;  // token segments per channel
   extern __shared__ __align__(16) float sm[];
-  const int dv = a.dv, lv = dv + 4;
+  const int dv = a.dv, lv = v_stride<DT>(dv);
   float *sK = sm, *sQ = sK + CC * LD, *sKk = sQ + CC * LD, *sT = sKk + CC * LD, *sA = sT + CC * LC;
-  float *sV = sA + CC * LC, *sX = sV + CC * lv, *s_r = sX + 16 * 20, *s_mr = s_r + CC;
+  float *sX = sA + CC * LC, *s_r = sX + 16 * 20, *s_mr = s_r + CC;
   float *s_is = s_mr + CC, *s_be = s_is + CC, *s_gC = s_be + CC, *s_seg = s_gC + DK;
+  DT *sV = reinterpret_cast<DT *>(s_seg + PT * 5);
   const int tid = KDN_TID;
   const int bh = (int)(blockIdx.x / (unsigned)a.NC), c = (int)(blockIdx.x % (unsigned)a.NC);
   const int b = bh / a.H, h = bh % a.H, tn = min(CC, a.T - c * CC);
@@ -256,22 +259,46 @@ __global__ void __launch_bounds__(PT) k_chunk_prep(Args a) {
   // this thread's channel and tokens; all loads issued ahead of their uses
   const int i = tid % DK, t0 = (tid / DK) * SL;
   constexpr int LB = SL > 16 ? 16 : SL;  // tokens held in registers at a time
-  float kv[LB], qv[LB], gv[LB], wv[LB];
+  float kv[LB], qv[LB], gv[LB], wv[LB], a2[LB];
+  const size_t tok0 = tok_index(a, b, c * CC, h), row_e = (size_t)a.H * DK;
   auto load = [&](int tb) {
+    const size_t o = (tok0 + (size_t)tb * a.H) * DK + i;
 #pragma unroll
     for (int j = 0; j < LB; ++j) {
-      const int t = tb + j;
       kv[j] = qv[j] = gv[j] = wv[j] = 0.f;
-      if (t < tn) {
-        const size_t th = tok_index(a, b, c * CC + t, h);
-        kv[j] = ld<DT>(a.k, th * DK + i);
-        qv[j] = ld<DT>(a.q, th * DK + i);
-        gv[j] = ld<DT>(a.g, a.pcd ? th * DK + i : th);
-        if (V == 0) wv[j] = ld<DT>(a.omega, th * DK + i);
+      if (tb + j < tn) {
+        kv[j] = ld<DT>(a.k, o + j * row_e);
+        qv[j] = ld<DT>(a.q, o + j * row_e);
+        gv[j] = ld<DT>(a.g, a.pcd ? o + j * row_e : tok0 + (size_t)(tb + j) * a.H);
+        if (V == 0) wv[j] = ld<DT>(a.omega, o + j * row_e);
       }
     }
   };
+  auto gates = [&](int tb) {  // log alpha (gv), alpha^2, omega; identity tokens past T
+    if (a.gates) {
+#pragma unroll
+      for (int j = 0; j < LB; ++j) {
+        gv[j] = tb + j < tn ? gate_logalpha(1, gv[j]) : 0.f;
+        if (V == 0) wv[j] = tb + j < tn ? gate_omega(1, wv[j]) : 0.f;
+      }
+    }
+    if (V == 0) {
+#pragma unroll
+      for (int j = 0; j < LB; ++j) a2[j] = expf(2.f * gv[j]);
+    }
+  };
   load(t0);
+  float p = 1.f;
+  if (V == 0) p = a.pin[base * DK + i];
+  {  // V by asynchronous copies, waited for ahead of U = A V
+    constexpr int EP = 16 / (int)sizeof(DT);  // elements per 16-byte piece
+    const int pieces = dv / EP;
+    for (int e = tid; e < CC * pieces; e += PT) {
+      const int t = e / pieces, j = EP * (e % pieces);
+      cp16(sV + t * lv + j, static_cast<const DT *>(a.v) + (tok0 + (size_t)(t < tn ? t : 0) * a.H) * dv + j, t < tn);
+    }
+    cp_commit();
+  }
   if (tid < CC) {
     const float rr =
         tid < tn ? gate_r(a.gates, a.rmin, ld<DT>(a.r, tok_index(a, b, c * CC + tid, h))) : 1.f;
@@ -312,28 +339,18 @@ __global__ void __launch_bounds__(PT) k_chunk_prep(Args a) {
       if (a.pT && c == a.NC - 1 && tid == tn - 1) a.pT[bh] = bt;
     }
   }
-  for (int e = tid; e < CC * (dv / 4); e += PT) {
-    const int t = e / (dv / 4), j = 4 * (e % (dv / 4));
-    float x[4] = {0.f, 0.f, 0.f, 0.f};
-    if (t < tn) ld4<DT>(a.v, tok_index(a, b, c * CC + t, h) * dv + j, x);
-    st4(sV + t * lv + j, x);
-  }
   __syncthreads();
 
   // gains and decay of the segment's tokens
-  float p = 1.f, G = 0.f;
-  if (V == 0) p = a.pin[base * DK + i];
+  float G = 0.f;
+  gates(t0);
   if (NSEG > 1) {  // the segments before this one: their decay sums and Moebius products
     float m[4] = {1.f, 0.f, 0.f, 1.f}, gs = 0.f;
 #pragma unroll
     for (int j = 0; j < LB; ++j) {
-      if (t0 + j < tn) {
-        const float lg = gate_logalpha(a.gates, gv[j]);
-        gs += lg;
-        if (V == 0)
-          moebius_step(m, expf(2.f * lg), gate_omega(a.gates, wv[j]), s_mr[t0 + j] * kv[j] * kv[j]);
-      }
-      if ((j & 3) == 3) renorm_pow2(m);
+      gs += gv[j];
+      if (V == 0) moebius_step(m, a2[j], wv[j], s_mr[t0 + j] * kv[j] * kv[j]);
+      if (V == 0 && (j & 3) == 3) renorm_pow2(m);
     }
     float *mine = s_seg + tid * 5;
 #pragma unroll
@@ -349,26 +366,27 @@ __global__ void __launch_bounds__(PT) k_chunk_prep(Args a) {
   float gam = expf(G);
   const size_t grow = ((size_t)bh * a.Tp + c * CC) * DK + i;
   for (int tb = t0; tb < t0 + SL; tb += LB) {
-    if (tb > t0) load(tb);
+    if (tb > t0) {
+      load(tb);
+      gates(tb);
+    }
 #pragma unroll
     for (int j = 0; j < LB; ++j) {
       const int t = tb + j;
-      float kk = 0.f, ph = 0.f;
-      if (t < tn) {
-        const float lg = gate_logalpha(a.gates, gv[j]);
-        G += lg;
-        gam = expf(G);
-        if (V == 0) {
-          ph = fmaf(expf(2.f * lg), p, gate_omega(a.gates, wv[j]));  // eq. diag-covariance-prediction
-          p = ph / (1.f + s_mr[t] * kv[j] * kv[j] * ph);             // eq. diag-cov-update
-          kk = ph * kv[j] / gam;
-        } else {
-          kk = s_be[t] * kv[j] / gam;
-        }
+      float ph = 0.f, kk;
+      G += gv[j];
+      gam = expf(G);
+      if (V == 0) {
+        ph = fmaf(a2[j], p, wv[j]);                             // eq. diag-covariance-prediction
+        p = div_nr(ph, fmaf(s_mr[t] * kv[j] * kv[j], ph, 1.f));  // eq. diag-cov-update
+        kk = ph * kv[j];
+      } else {
+        kk = s_be[t] * kv[j];
       }
       sK[t * LD + i] = kv[j] * gam;
       sQ[t * LD + i] = a.tau * qv[j] * gam;
-      sKk[t * LD + i] = kk;  // diag: still without 1 / s_t
+      // (diag: still without 1 / s_t; a subnormal gamma's reciprocal may overflow where the quotient does not)
+      sKk[t * LD + i] = gam > 1e-37f ? div_nr(kk, gam) : kk / gam;
       if (SAVE) {
         if (V == 0) a.phat[grow + (size_t)t * DK] = ph;
         a.gam[grow + (size_t)t * DK] = gam;
@@ -415,6 +433,7 @@ __global__ void __launch_bounds__(PT) k_chunk_prep(Args a) {
     else st4(a.Aqk + (base * CC + r) * CC + 4 * gb, x);
   }
   __syncthreads();
+  cp_wait<0>();  // V (the barriers of the solve make every thread's copies visible)
   inverse32(sT, sA, sX);
 
   // W = A Kbar and U = A V (32 x dk, 32 x dv; 16 columns a warp), then Qbar, K_tail
@@ -423,7 +442,7 @@ __global__ void __launch_bounds__(PT) k_chunk_prep(Args a) {
     const bool isW = col < DK;
     zero<4>(acc);
     if (isW) tile_mm<CC, 4, false>(acc, sA + ga * LC, 8 * LC, sK + col, LD);
-    else tile_mm<CC, 4, false>(acc, sA + ga * LC, 8 * LC, sV + col - DK, lv);
+    else tile_mm<CC, 4, false, DT>(acc, sA + ga * LC, 8 * LC, sV + col - DK, lv);
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       const int r = ga + 8 * m;
@@ -542,9 +561,9 @@ kdn_status_t fwd_impl(const Args &a, cudaStream_t s) {
   bool ok = V == 0 ? launch(k_gain_comp_diag<DT, DK>, (n + per - 1) / per, 128, 0, s, a)
                    : launch(k_gain_comp_iso<DT, DK>, (n + 3) / 4, 128, 0, s, a);
   ok = ok && launch(k_gain_scan, (BH * a.P + 127) / 128, 128, 0, s, a);
-  ok = ok && launch(k_chunk_prep<V, DT, DK, SAVE>, n, PT, prep_smem_bytes<DK>(a.dv), s, a);
+  ok = ok && launch(k_chunk_prep<V, DT, DK, SAVE>, n, PT, prep_smem_bytes<DT, DK>(a.dv), s, a);
   switch (state_cols(a)) {
-    case 64: ok = ok && state_fwd<DK, 64, 4, SAVE>(a, s); break;
+    case 64: ok = ok && state_fwd<DK, 64, 8, SAVE>(a, s); break;
     case 32: ok = ok && state_fwd<DK, 32, 4, SAVE>(a, s); break;
     default: ok = ok && state_fwd<DK, 16, 2, SAVE>(a, s);
   }
