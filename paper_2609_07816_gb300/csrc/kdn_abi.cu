@@ -169,7 +169,7 @@ kdn_status_t bwd_entry(int variant, const kdn_desc_t *d, const void *q, const vo
   a.dq = dq; a.dk_ = dk; a.dv_ = dv; a.dg = dg; a.domega = domega; a.dr = dr;
   a.dS0 = dS0; a.dp0 = dp0; a.dmu = dmu;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(a.status, 0, sizeof(unsigned), s) != cudaSuccess) return KDN_ERR_CUDA;
+  if (cudaMemsetAsync(a.status, 0, 2 * sizeof(unsigned), s) != cudaSuccess) return KDN_ERR_CUDA;
   if ((size_t)a.B * a.H == 0) return KDN_OK;
   if (a.T == 0) return empty_bwd(a, s);
   if (use_fused_bwd(a)) return launch_fused_bwd(a, s);
@@ -205,7 +205,7 @@ kdn_status_t fwd_save_entry(int variant, const kdn_desc_t *d, const void *q, con
   if (cudaMemsetAsync(a.status, 0, sizeof(unsigned), s) != cudaSuccess) return KDN_ERR_CUDA;
   if ((size_t)a.B * a.H == 0) return KDN_OK;
   if (a.T == 0) return empty_fwd(a, s);
-  const size_t nsv = (size_t)a.B * a.H * ((a.T + 63) / 64) * fused_ctx_record_bytes();
+  const size_t nsv = (size_t)a.B * a.H * ((a.T + 63) / 64) * fused_ctx_record_bytes(a);
   if (wy_fwd_supported(a, true))
     return launch_wy_fwd(a, s, static_cast<unsigned char *>(saved),
                          reinterpret_cast<float *>(static_cast<char *>(saved) + nsv));
@@ -238,12 +238,14 @@ kdn_status_t bwd_saved_entry(int variant, const kdn_desc_t *d, const void *q, co
   a.dq = dq; a.dk_ = dk; a.dv_ = dv; a.dg = dg; a.domega = domega; a.dr = dr;
   a.dS0 = dS0; a.dp0 = dp0; a.dmu = dmu;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(a.status, 0, sizeof(unsigned), s) != cudaSuccess) return KDN_ERR_CUDA;
+  if (cudaMemsetAsync(a.status, 0, 2 * sizeof(unsigned), s) != cudaSuccess) return KDN_ERR_CUDA;
   if ((size_t)a.B * a.H == 0) return KDN_OK;
   if (a.T == 0) return empty_bwd(a, s);
-  const size_t nsv = (size_t)a.B * a.H * ((a.T + 63) / 64) * fused_ctx_record_bytes();
+  const size_t nsv = (size_t)a.B * a.H * ((a.T + 63) / 64) * fused_ctx_record_bytes(a);
   a.fSin = static_cast<unsigned char *>(const_cast<void *>(saved));
   a.fpin = reinterpret_cast<float *>(static_cast<char *>(const_cast<void *>(saved)) + nsv);
+  const size_t split = split_bwd_workspace_bytes(a);
+  if (split && ws_bytes >= need + split) a.split_ws = static_cast<char *>(ws) + need;
   return launch_fused_bwd_sweep(a, s);
 }
 
@@ -293,8 +295,10 @@ size_t workspace_layout(Args *a, char *base, bool bwd) {
   if (!bwd && use_fused(*a)) return off;
   if (bwd && a->T > 0 && use_fused_bwd(*a)) {
     const size_t NC64 = (a->T + 63) / 64;  // the fused kernels use 64-token chunks
-    a->fSin = reinterpret_cast<unsigned char *>(take(BH * NC64 * fused_ctx_record_bytes() / sizeof(float)));
+    a->fSin = reinterpret_cast<unsigned char *>(take(BH * NC64 * fused_ctx_record_bytes(*a) / sizeof(float)));
     a->fpin = take(BH * NC64 * dk);
+    const size_t split = split_bwd_workspace_bytes(*a);
+    if (split) a->split_ws = reinterpret_cast<char *>(take(split / sizeof(float)));
     return off;
   }
   a->comp = take(BH * NC * P * 4);
@@ -350,7 +354,9 @@ size_t kdn_fwd_workspace_bytes(const kdn_desc_t *desc, int variant) {
   Args a;
   if (fill_sizes(desc, variant, false, &a) != KDN_OK) return 0;
   const int nseg = seg_count(a);
-  return workspace_layout(&a, nullptr, false) + (nseg > 1 ? seg_workspace_bytes(a, nseg) : 0);
+  // (the training backward of ragged lengths takes its scratch from the same workspace)
+  return workspace_layout(&a, nullptr, false) +
+         (nseg > 1 ? seg_workspace_bytes(a, nseg) : split_bwd_workspace_bytes(a));
 }
 
 size_t kdn_bwd_workspace_bytes(const kdn_desc_t *desc, int variant) {
@@ -458,10 +464,10 @@ int kdn_kernel_launches(const kdn_desc_t *desc, int variant, int op) {
   if (fill_sizes(desc, variant, op == 2, &a) != KDN_OK) return -1;
   switch (op) {
     case 0: return seg_count(a) > 1 ? 5 : use_fused(a) ? 1 : chunked_fwd_launches(a);
-    case 1: return (a.T > 0 && use_fused_bwd(a)) ? 2 : chunked_bwd_launches(a);
+    case 1: return (a.T > 0 && use_fused_bwd(a)) ? (split_bwd_context(a) ? 3 : 2) : chunked_bwd_launches(a);
     case 2: return 1;
+    case 4: return fused_saved_bytes(a) > 0 ? (split_bwd_context(a) ? 2 : 1) : -1;
     case 3:
-    case 4:
     case 5: return fused_saved_bytes(a) > 0 ? 1 : -1;
   }
   return -1;

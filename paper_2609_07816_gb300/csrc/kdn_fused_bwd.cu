@@ -51,7 +51,7 @@
 // KDN_ERR_TIMEOUT in the workspace status word and returns.
 #include "kdn_internal.cuh"
 #include "kdn_sm103.cuh"
-#include "kdn_fused_common.cuh"
+#include "kdn_bwd_common.cuh"
 
 namespace kdn {
 namespace {
@@ -104,77 +104,8 @@ static_assert(O_AQ + 8 * KB <= O_WN && O_XT + 8 * KB <= O_RH, "map");
 
 struct BwdParams {
   Args a;
+  size_t rec;  // bytes of a context record
 };
-
-__device__ __forceinline__ uint64_t kdesc(const unsigned char *p) {
-  return sw128_desc(smem_u32(p), 16, 1024);
-}
-__device__ __forceinline__ uint64_t mdesc(const unsigned char *p, uint32_t lbo) {
-  return sw128_desc(smem_u32(p), lbo, 1024);
-}
-// x ~ hi + lo, both fp16: returns hi, writes the lo chunk
-__device__ __forceinline__ uint4 split_h8(const float *x, uint4 *lo) {
-  float h[8], l[8];
-  const uint4 hi = pack_h8(x);
-  unpack_h8(hi, h);
-#pragma unroll
-  for (int j = 0; j < 8; ++j) l[j] = x[j] - h[j];
-  *lo = pack_h8(l);
-  return hi;
-}
-
-// Row `row` of a [128][64] 16-bit tile (one 128-byte-swizzled slab), tokens
-// 16 q .. 16 q + 15: two 16-byte chunks.
-__device__ __forceinline__ void st_row16_bf(unsigned char *tile, int row, int q, const float *v) {
-  sm16(tile, chunk_off(row, 2 * q)) = pack_bf8(v);
-  sm16(tile, chunk_off(row, 2 * q + 1)) = pack_bf8(v + 8);
-}
-__device__ __forceinline__ void st_row16_h(unsigned char *tile, int row, int q, const float *v) {
-  sm16(tile, chunk_off(row, 2 * q)) = pack_h8(v);
-  sm16(tile, chunk_off(row, 2 * q + 1)) = pack_h8(v + 8);
-}
-__device__ __forceinline__ void st_row16_split(unsigned char *hi, unsigned char *lo, int row, int q,
-                                               const float *v) {
-  uint4 l0, l1;
-  sm16(hi, chunk_off(row, 2 * q)) = split_bf8(v, &l0);
-  sm16(hi, chunk_off(row, 2 * q + 1)) = split_bf8(v + 8, &l1);
-  sm16(lo, chunk_off(row, 2 * q)) = l0;
-  sm16(lo, chunk_off(row, 2 * q + 1)) = l1;
-}
-
-// Reduce-scatter of 16 per-lane values over a warp: returns, in lanes 2j and
-// 2j + 1, the warp-wide sum of v[j].
-__device__ __forceinline__ float rs16(const float *v, int lane) {
-  float w8[8], w4[4], w2[2];
-  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const float keep = b4 ? v[8 + j] : v[j], send = b4 ? v[j] : v[8 + j];
-    w8[j] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-  }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float keep = b3 ? w8[4 + j] : w8[j], send = b3 ? w8[j] : w8[4 + j];
-    w4[j] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-  }
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const float keep = b2 ? w4[2 + j] : w4[j], send = b2 ? w4[j] : w4[2 + j];
-    w2[j] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-  }
-  const float keep = b1 ? w2[1] : w2[0], send = b1 ? w2[0] : w2[1];
-  const float w1 = keep + __shfl_xor_sync(0xffffffffu, send, 2);
-  return w1 + __shfl_xor_sync(0xffffffffu, w1, 1);
-}
-
-// Output store in the gradient dtype (OBF: bfloat16, else float32).  float32
-// gradients are written with the streaming hint: they are not read again by this
-// kernel, and evicting them first keeps L2 for the context records it prefetches.
-template <int OBF>
-__device__ __forceinline__ void st_grad(void *p, size_t i, float x) {
-  if (OBF) static_cast<__nv_bfloat16 *>(p)[i] = __float2bfloat16_rn(x);
-  else __stcs(static_cast<float *>(p) + i, x);
-}
 
 // G: the gate inputs are logits (KDN_GATES_LOGITS), a compile-time choice so
 // that the post-activation path carries none of the chain-rule code.
@@ -233,6 +164,7 @@ __global__ void __launch_bounds__(BT, 1)
   uint64_t *bar_g = bars + 5;  // diagonal KDN: phat and gamma of the chunk
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int warp_u = __shfl_sync(0xffffffffu, warp, 0);  // warp-uniform: the MMA issue stays uniform
   const int wq = warp & 3, wg = warp >> 2;  // TMEM lane quarter, column group
   const int ci = tid & (D - 1), qq = tid >> 7, t0 = 16 * qq;  // channel view: channel, token quarter
   const int bh = blockIdx.x, b = bh / a.H, h = bh % a.H;
@@ -272,7 +204,7 @@ __global__ void __launch_bounds__(BT, 1)
   // (diagonal KDN: the context's Y in place of v)
   const uint32_t kBytesA = 81920u + 16384u * 2 + (V == 0 ? 16384u : 0u);
   auto issue_a_ctx = [&](int c) {
-    const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * kCtxBytes;
+    const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * P.rec;
     mbar_expect_tx(bar_a, kBytesA);
     bulk_g2s(sin, rec + kCtxS, 32768, bar_a);
     bulk_g2s(sm + O_RH, rec + kCtxR, 16384, bar_a);
@@ -295,7 +227,7 @@ __global__ void __launch_bounds__(BT, 1)
     for (int s = 0; s < 2; ++s) tma_load_4d(rv + s * 8192, &mv, bar_b, 64 * s, h, c * CM, b);
   };
   auto issue_g = [&](int c) {
-    const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * kCtxBytes;
+    const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * P.rec;
     mbar_expect_tx(bar_g, 65536);
     bulk_g2s(sm + O_PHB, rec + kCtxPh, 32768, bar_g);
     bulk_g2s(sm + O_GA0, rec + kCtxGa, 16384, bar_g);
@@ -448,7 +380,7 @@ __global__ void __launch_bounds__(BT, 1)
       s_fr[tid] = nfr;
       s_fw[tid] = nfw;
     }
-    const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * kCtxBytes;
+    const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * P.rec;
     float e16[16], ph16[16], tk[5];
     {
       // gamma [64][128] (SD: one value per token, [64]) of the isotropic KDN
@@ -561,20 +493,24 @@ __global__ void __launch_bounds__(BT, 1)
     tc_fence_before();
     __syncthreads();
     // ---- [10] B1: X2 = dR^T;  B3: X3 = dA_qk^T (before masking);  B4: X0 = dK_tail^T
-    if (tid == 0) {
+    if (warp_u == 0) {
       tc_fence_after();
+      const uint32_t lead = elect_one();
       const uint32_t id11 = idesc_f16(128, 64, 1, 1), id00 = idesc_f16(128, 64, 0, 0);
+#pragma unroll
       for (int kk = 0; kk < 4; ++kk)
-        umma_bf16(X2, mdesc(rdo + kk * 2048, 8192), mdesc(sm + O_AQ + kk * 2048, 8192), id11, kk > 0);
+        umma_if(lead, X2, step(mdesc(rdo, 8192), kk * 2048), step(mdesc(sm + O_AQ, 8192), kk * 2048), id11, kk > 0);
+#pragma unroll
       for (int kk = 0; kk < 8; ++kk)
-        umma_bf16(X2, mdesc(sm + O_DSH + kk * 2048, 16384), mdesc(sm + O_KT + kk * 2048, 8192), id11, 1);
+        umma_if(lead, X2, step(mdesc(sm + O_DSH, 16384), kk * 2048), step(mdesc(sm + O_KT, 8192), kk * 2048), id11, 1);
+#pragma unroll
       for (int kk = 0; kk < 8; ++kk) {
         const uint32_t o8 = (kk >> 2) * 8192 + (kk & 3) * 32;
-        umma_bf16(X3, kdesc(sm + O_RH + o8), kdesc(rdo + o8), id00, kk > 0);
-        umma_bf16(X0, kdesc(sm + O_DSH + (kk >> 2) * 16384 + (kk & 3) * 32), kdesc(sm + O_RH + o8),
+        umma_if(lead, X3, step(kdesc(sm + O_RH), o8), step(kdesc(rdo), o8), id00, kk > 0);
+        umma_if(lead, X0, step(kdesc(sm + O_DSH), (kk >> 2) * 16384 + (kk & 3) * 32), step(kdesc(sm + O_RH), o8),
                   id00, kk > 0);
       }
-      umma_commit(bar_mma);
+      commit_if(lead, bar_mma);
     }
     bool mm_ok = true;
     if constexpr (V == 0) {
@@ -659,22 +595,25 @@ __global__ void __launch_bounds__(BT, 1)
       // other products, and X = A^T dA one round later.
       // ---- [12] B2: TS += Qbar^T dO - W^T dR;  B5: X1 = -dW^T;  B6: X2 = dA^T = (dR Y^T)^T;
       //           B8a: X3 = (dO S_in^T)^T
-      if (tid == 0) {
+      if (warp_u == 0) {
         tc_fence_after();
+        const uint32_t lead = elect_one();
         const uint32_t idS01 = idesc_f16(128, 128, 0, 1), idS10 = idesc_f16(128, 128, 1, 0);
         const uint32_t id01 = idesc_f16(128, 64, 0, 1), id00 = idesc_f16(128, 64, 0, 0);
+#pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-          umma_bf16(TS, kdesc(sm + O_QH + kk * 32), mdesc(rdo + kk * 2048, 8192), idS01, 1);
-          umma_bf16(TS, mdesc(sm + O_WN + kk * 2048, 8192), kdesc(sm + O_DRT + kk * 32), idS10, 1);
+          umma_if(lead, TS, step(kdesc(sm + O_QH), kk * 32), step(mdesc(rdo, 8192), kk * 2048), idS01, 1);
+          umma_if(lead, TS, step(mdesc(sm + O_WN, 8192), kk * 2048), step(kdesc(sm + O_DRT), kk * 32), idS10, 1);
         }
+#pragma unroll
         for (int kk = 0; kk < 8; ++kk) {
-          const uint64_t as = kdesc(sin + (kk >> 2) * 16384 + (kk & 3) * 32);
-          const uint64_t drt = mdesc(sm + O_DRT + kk * 2048, 8192);
-          umma_bf16(X1, as, drt, id01, kk > 0);
-          umma_bf16(X3, as, kdesc(rdo + (kk >> 2) * 8192 + (kk & 3) * 32), id00, kk > 0);
-          umma_bf16(X2, kdesc(rv + (kk >> 2) * 8192 + (kk & 3) * 32), drt, id01, kk > 0);
+          const uint64_t as = step(kdesc(sin), (kk >> 2) * 16384 + (kk & 3) * 32);
+          const uint64_t drt = step(mdesc(sm + O_DRT, 8192), kk * 2048);
+          umma_if(lead, X1, as, drt, id01, kk > 0);
+          umma_if(lead, X3, as, step(kdesc(rdo), (kk >> 2) * 8192 + (kk & 3) * 32), id00, kk > 0);
+          umma_if(lead, X2, step(kdesc(rv), (kk >> 2) * 8192 + (kk & 3) * 32), drt, id01, kk > 0);
         }
-        umma_commit(bar_mma);
+        commit_if(lead, bar_mma);
       }
       mm_ok = mma_poll();
       tc_fence_after();
@@ -719,27 +658,29 @@ __global__ void __launch_bounds__(BT, 1)
       }
       // ---- [14] B8b: X3 += (dA_qk Kk)^T;  B9a: X0 += (dA_qk^T Qbar)^T (hi/lo bf16 pairs);
       //           B7: X2 = dV^T = (A^T dR)^T (dR as hi + lo fp16);  X1 = A^T dA (fp16)
-      if (tid == 0) {
+      if (warp_u == 0) {
         tc_fence_after();
+        const uint32_t lead = elect_one();
         const uint32_t id01 = idesc_bf16(128, 64, 0, 1), id00 = idesc_bf16(128, 64, 0, 0);
         const uint32_t ih01 = idesc_f16(128, 64, 0, 1), ih10 = idesc_f16(128, 64, 1, 0);
+#pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-          const uint64_t kh = kdesc(sm + O_KKH2 + kk * 32), kl = kdesc(sm + O_KKL2 + kk * 32);
-          const uint64_t dh = mdesc(sm + O_DAQ + kk * 2048, 8192), dl = mdesc(sm + O_DAQ + 8192 + kk * 2048, 8192);
-          umma_bf16(X3, kh, dh, id01, 1);
-          umma_bf16(X3, kl, dh, id01, 1);
-          umma_bf16(X3, kh, dl, id01, 1);
-          const uint64_t qh = kdesc(sm + O_KQH2 + 16384 + kk * 32), ql = kdesc(sm + O_QL2 + kk * 32);
-          const uint64_t eh = kdesc(sm + O_DAQ + kk * 32), el = kdesc(sm + O_DAQ + 8192 + kk * 32);
-          umma_bf16(X0, qh, eh, id00, 1);
-          umma_bf16(X0, ql, eh, id00, 1);
-          umma_bf16(X0, qh, el, id00, 1);
-          const uint64_t ah = mdesc(sm + O_AH + kk * 2048, 8192);
-          umma_bf16(X2, kdesc(sm + O_DRT + kk * 32), ah, ih01, kk > 0);
-          umma_bf16(X2, kdesc(sm + O_DRTL + kk * 32), ah, ih01, 1);
-          umma_bf16(X1, ah, kdesc(sm + O_DAY + kk * 32), ih10, kk > 0);
+          const uint64_t kh = step(kdesc(sm + O_KKH2), kk * 32), kl = step(kdesc(sm + O_KKL2), kk * 32);
+          const uint64_t dh = step(mdesc(sm + O_DAQ, 8192), kk * 2048), dl = step(mdesc(sm + O_DAQ + 8192, 8192), kk * 2048);
+          umma_if(lead, X3, kh, dh, id01, 1);
+          umma_if(lead, X3, kl, dh, id01, 1);
+          umma_if(lead, X3, kh, dl, id01, 1);
+          const uint64_t qh = step(kdesc(sm + O_KQH2 + 16384), kk * 32), ql = step(kdesc(sm + O_QL2), kk * 32);
+          const uint64_t eh = step(kdesc(sm + O_DAQ), kk * 32), el = step(kdesc(sm + O_DAQ + 8192), kk * 32);
+          umma_if(lead, X0, qh, eh, id00, 1);
+          umma_if(lead, X0, ql, eh, id00, 1);
+          umma_if(lead, X0, qh, el, id00, 1);
+          const uint64_t ah = step(mdesc(sm + O_AH, 8192), kk * 2048);
+          umma_if(lead, X2, step(kdesc(sm + O_DRT), kk * 32), ah, ih01, kk > 0);
+          umma_if(lead, X2, step(kdesc(sm + O_DRTL), kk * 32), ah, ih01, 1);
+          umma_if(lead, X1, ah, step(kdesc(sm + O_DAY), kk * 32), ih10, kk > 0);
         }
-        umma_commit(bar_mma);
+        commit_if(lead, bar_mma);
       }
       mm_ok = mma_poll();
       tc_fence_after();
@@ -786,14 +727,16 @@ __global__ void __launch_bounds__(BT, 1)
         bulk_commit();
       }
       // ---- [16] X1 = X A^T (fp16), so that dT = strict_lower(-A^T dA A^T);  B10a: X2 = (A^T dW)^T
-      if (tid == 0) {
+      if (warp_u == 0) {
         tc_fence_after();
+        const uint32_t lead = elect_one();
         const uint32_t ih00 = idesc_f16(128, 64, 0, 0), ib01 = idesc_bf16(128, 64, 0, 1);
+#pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-          umma_bf16(X1, kdesc(sm + O_XT + kk * 32), kdesc(sm + O_AH + kk * 32), ih00, kk > 0);
-          umma_bf16(X2, kdesc(sm + O_DWY + kk * 32), mdesc(sm + O_AB + kk * 2048, 8192), ib01, kk > 0);
+          umma_if(lead, X1, step(kdesc(sm + O_XT), kk * 32), step(kdesc(sm + O_AH), kk * 32), ih00, kk > 0);
+          umma_if(lead, X2, step(kdesc(sm + O_DWY), kk * 32), step(mdesc(sm + O_AB, 8192), kk * 2048), ib01, kk > 0);
         }
-        umma_commit(bar_mma);
+        commit_if(lead, bar_mma);
       }
       mm_ok = mma_poll();
       tc_fence_after();
@@ -813,36 +756,41 @@ __global__ void __launch_bounds__(BT, 1)
         break;
       }
       // ---- [17] B9b: X0 += (dT^T Kbar)^T;  B10b: X2 += (dT Kk)^T
-      if (tid == 0) {
+      if (warp_u == 0) {
         tc_fence_after();
+        const uint32_t lead = elect_one();
         const uint32_t id01 = idesc_bf16(128, 64, 0, 1), id00 = idesc_bf16(128, 64, 0, 0);
+#pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-          umma_bf16(X0, kdesc(sm + O_KQH2 + kk * 32), mdesc(sm + O_DT + kk * 2048, 8192), id01, 1);
-          umma_bf16(X2, kdesc(sm + O_KKH2 + kk * 32), kdesc(sm + O_DT + kk * 32), id00, 1);
+          umma_if(lead, X0, step(kdesc(sm + O_KQH2), kk * 32), step(mdesc(sm + O_DT, 8192), kk * 2048), id01, 1);
+          umma_if(lead, X2, step(kdesc(sm + O_KKH2), kk * 32), step(kdesc(sm + O_DT), kk * 32), id00, 1);
         }
-        umma_commit(bar_mma);
+        commit_if(lead, bar_mma);
       }
     } else {
       // Isotropic KDN: seven rounds (its context keeps no Y; B6 forms dA from V and dW)
       // ---- [12] B2: TS += Qbar^T dO - W^T dR;  B5: X1 = -dW^T;  B7: X2 = dV^T (dR as hi + lo fp16);
       //           B8a: X3 = (dO S_in^T)^T
-      if (tid == 0) {
+      if (warp_u == 0) {
         tc_fence_after();
+        const uint32_t lead = elect_one();
         const uint32_t idS01 = idesc_f16(128, 128, 0, 1), idS10 = idesc_f16(128, 128, 1, 0);
         const uint32_t id01 = idesc_f16(128, 64, 0, 1), id00 = idesc_f16(128, 64, 0, 0);
+#pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-          umma_bf16(TS, kdesc(sm + O_QH + kk * 32), mdesc(rdo + kk * 2048, 8192), idS01, 1);
-          umma_bf16(TS, mdesc(sm + O_WN + kk * 2048, 8192), kdesc(sm + O_DRT + kk * 32), idS10, 1);
-          const uint64_t ah = mdesc(sm + O_AH + kk * 2048, 8192);
-          umma_bf16(X2, kdesc(sm + O_DRT + kk * 32), ah, id01, kk > 0);
-          umma_bf16(X2, kdesc(sm + O_DRTL + kk * 32), ah, id01, 1);
+          umma_if(lead, TS, step(kdesc(sm + O_QH), kk * 32), step(mdesc(rdo, 8192), kk * 2048), idS01, 1);
+          umma_if(lead, TS, step(mdesc(sm + O_WN, 8192), kk * 2048), step(kdesc(sm + O_DRT), kk * 32), idS10, 1);
+          const uint64_t ah = step(mdesc(sm + O_AH, 8192), kk * 2048);
+          umma_if(lead, X2, step(kdesc(sm + O_DRT), kk * 32), ah, id01, kk > 0);
+          umma_if(lead, X2, step(kdesc(sm + O_DRTL), kk * 32), ah, id01, 1);
         }
+#pragma unroll
         for (int kk = 0; kk < 8; ++kk) {
-          const uint64_t as = kdesc(sin + (kk >> 2) * 16384 + (kk & 3) * 32);
-          umma_bf16(X1, as, mdesc(sm + O_DRT + kk * 2048, 8192), id01, kk > 0);
-          umma_bf16(X3, as, kdesc(rdo + (kk >> 2) * 8192 + (kk & 3) * 32), id00, kk > 0);
+          const uint64_t as = step(kdesc(sin), (kk >> 2) * 16384 + (kk & 3) * 32);
+          umma_if(lead, X1, as, step(mdesc(sm + O_DRT, 8192), kk * 2048), id01, kk > 0);
+          umma_if(lead, X3, as, step(kdesc(rdo), (kk >> 2) * 8192 + (kk & 3) * 32), id00, kk > 0);
         }
-        umma_commit(bar_mma);
+        commit_if(lead, bar_mma);
       }
       if (!(ok = mma_wait())) break;
       tc_fence_after();
@@ -868,34 +816,38 @@ __global__ void __launch_bounds__(BT, 1)
       fence_proxy_async();
       tc_fence_before();
       __syncthreads();
-      if (SD && tid == 0) {  // raw K^T, Q^T (channel-major) against the scaled 64 x 64 partners
+      if (SD && warp_u == 0) {  // raw K^T, Q^T (channel-major) against the scaled 64 x 64 partners
         tc_fence_after();
+        const uint32_t lead = elect_one();
         const uint32_t id11 = idesc_bf16(128, 64, 1, 1), id10 = idesc_bf16(128, 64, 1, 0);
+#pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-          const uint64_t kt = mdesc(rkq + kk * 2048, 16384), qt = mdesc(rkq + 8192 + kk * 2048, 16384);
-          umma_bf16(X3, kt, mdesc(sm + O_DAQ + kk * 2048, 8192), id11, 1);
-          umma_bf16(X3, kt, mdesc(sm + O_DAQ + 8192 + kk * 2048, 8192), id11, 1);
-          umma_bf16(X0, qt, kdesc(sm + O_AQ + kk * 32), id10, 1);
-          umma_bf16(X0, qt, kdesc(sm + O_DT + kk * 32), id10, 1);
+          const uint64_t kt = step(mdesc(rkq, 16384), kk * 2048), qt = step(mdesc(rkq + 8192, 16384), kk * 2048);
+          umma_if(lead, X3, kt, step(mdesc(sm + O_DAQ, 8192), kk * 2048), id11, 1);
+          umma_if(lead, X3, kt, step(mdesc(sm + O_DAQ + 8192, 8192), kk * 2048), id11, 1);
+          umma_if(lead, X0, qt, step(kdesc(sm + O_AQ), kk * 32), id10, 1);
+          umma_if(lead, X0, qt, step(kdesc(sm + O_DT), kk * 32), id10, 1);
         }
-        umma_commit(bar_mma);
+        commit_if(lead, bar_mma);
       }
-      if (!SD && tid == 0) {
+      if (!SD && warp_u == 0) {
         tc_fence_after();
+        const uint32_t lead = elect_one();
         const uint32_t id01 = idesc_bf16(128, 64, 0, 1), id00 = idesc_bf16(128, 64, 0, 0);
+#pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-          const uint64_t kh = kdesc(sm + O_KKH2 + kk * 32), kl = kdesc(sm + O_KKL2 + kk * 32);
-          const uint64_t dh = mdesc(sm + O_DAQ + kk * 2048, 8192), dl = mdesc(sm + O_DAQ + 8192 + kk * 2048, 8192);
-          umma_bf16(X3, kh, dh, id01, 1);
-          umma_bf16(X3, kl, dh, id01, 1);
-          umma_bf16(X3, kh, dl, id01, 1);
-          const uint64_t qh = kdesc(sm + O_KQH2 + 16384 + kk * 32), ql = kdesc(sm + O_QL2 + kk * 32);
-          const uint64_t eh = kdesc(sm + O_DAQ + kk * 32), el = kdesc(sm + O_DAQ + 8192 + kk * 32);
-          umma_bf16(X0, qh, eh, id00, 1);
-          umma_bf16(X0, ql, eh, id00, 1);
-          umma_bf16(X0, qh, el, id00, 1);
+          const uint64_t kh = step(kdesc(sm + O_KKH2), kk * 32), kl = step(kdesc(sm + O_KKL2), kk * 32);
+          const uint64_t dh = step(mdesc(sm + O_DAQ, 8192), kk * 2048), dl = step(mdesc(sm + O_DAQ + 8192, 8192), kk * 2048);
+          umma_if(lead, X3, kh, dh, id01, 1);
+          umma_if(lead, X3, kl, dh, id01, 1);
+          umma_if(lead, X3, kh, dl, id01, 1);
+          const uint64_t qh = step(kdesc(sm + O_KQH2 + 16384), kk * 32), ql = step(kdesc(sm + O_QL2), kk * 32);
+          const uint64_t eh = step(kdesc(sm + O_DAQ), kk * 32), el = step(kdesc(sm + O_DAQ + 8192), kk * 32);
+          umma_if(lead, X0, qh, eh, id00, 1);
+          umma_if(lead, X0, ql, eh, id00, 1);
+          umma_if(lead, X0, qh, el, id00, 1);
         }
-        umma_commit(bar_mma);
+        commit_if(lead, bar_mma);
       }
       if (!(ok = mma_wait())) break;
       tc_fence_after();
@@ -933,19 +885,22 @@ __global__ void __launch_bounds__(BT, 1)
         bulk_commit();
       }
       // ---- [15] B6: X1 = dA^T = (dR V^T + dW Kbar^T)^T;  B10a: X2 = (A^T dW)^T
-      if (tid == 0) {
+      if (warp_u == 0) {
         tc_fence_after();
+        const uint32_t lead = elect_one();
         const uint32_t ih01 = idesc_f16(128, 64, 0, 1), ib01 = idesc_bf16(128, 64, 0, 1);
         const uint32_t ib11 = idesc_bf16(128, 64, 1, 1);
+#pragma unroll
         for (int kk = 0; kk < 8; ++kk) {
-          umma_bf16(X1, kdesc(rv + (kk >> 2) * 8192 + (kk & 3) * 32), mdesc(sm + O_DRT + kk * 2048, 8192),
+          umma_if(lead, X1, step(kdesc(rv), (kk >> 2) * 8192 + (kk & 3) * 32), step(mdesc(sm + O_DRT, 8192), kk * 2048),
                     ih01, kk > 0);
-          umma_bf16(X1, mdesc(sm + O_KQH2 + kk * 2048, 16384), mdesc(sm + O_DWT + kk * 2048, 8192), ib11,
+          umma_if(lead, X1, step(mdesc(sm + O_KQH2, 16384), kk * 2048), step(mdesc(sm + O_DWT, 8192), kk * 2048), ib11,
                     1);
         }
+#pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          umma_bf16(X2, kdesc(sm + O_DWT + kk * 32), mdesc(sm + O_AB + kk * 2048, 8192), ib01, kk > 0);
-        umma_commit(bar_mma);
+          umma_if(lead, X2, step(kdesc(sm + O_DWT), kk * 32), step(mdesc(sm + O_AB, 8192), kk * 2048), ib01, kk > 0);
+        commit_if(lead, bar_mma);
       }
       if (!(ok = mma_wait())) break;
       tc_fence_after();
@@ -965,12 +920,14 @@ __global__ void __launch_bounds__(BT, 1)
       fence_proxy_async();
       tc_fence_before();
       __syncthreads();
-      if (tid == 0) {
+      if (warp_u == 0) {
         tc_fence_after();
+        const uint32_t lead = elect_one();
         const uint32_t id = idesc_f16(128, 64, 1, 0);
+#pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          umma_bf16(X1, mdesc(sm + O_AH + kk * 2048, 8192), kdesc(sm + O_DAT + kk * 32), id, kk > 0);
-        umma_commit(bar_mma);
+          umma_if(lead, X1, step(mdesc(sm + O_AH, 8192), kk * 2048), step(kdesc(sm + O_DAT), kk * 32), id, kk > 0);
+        commit_if(lead, bar_mma);
       }
       if (!(ok = mma_wait())) break;
       tc_fence_after();
@@ -984,12 +941,14 @@ __global__ void __launch_bounds__(BT, 1)
       fence_proxy_async();
       tc_fence_before();
       __syncthreads();
-      if (tid == 0) {
+      if (warp_u == 0) {
         tc_fence_after();
+        const uint32_t lead = elect_one();
         const uint32_t id = idesc_f16(128, 64, 0, 0);
+#pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          umma_bf16(X1, kdesc(sm + O_XT + kk * 32), kdesc(sm + O_AH + kk * 32), id, kk > 0);
-        umma_commit(bar_mma);
+          umma_if(lead, X1, step(kdesc(sm + O_XT), kk * 32), step(kdesc(sm + O_AH), kk * 32), id, kk > 0);
+        commit_if(lead, bar_mma);
       }
       if (!(ok = mma_wait())) break;
       tc_fence_after();
@@ -1016,21 +975,23 @@ __global__ void __launch_bounds__(BT, 1)
       tc_fence_before();
       __syncthreads();
       // ---- [17] B9b: X0 += (dT^T Kbar)^T;  B10b: X2 += (dT Kk)^T
-      if (tid == 0) {
+      if (warp_u == 0) {
         tc_fence_after();
+        const uint32_t lead = elect_one();
         const uint32_t id01 = idesc_bf16(128, 64, 0, 1), id00 = idesc_bf16(128, 64, 0, 0);
         const uint32_t id11 = idesc_bf16(128, 64, 1, 1), id10 = idesc_bf16(128, 64, 1, 0);
+#pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
           if (SD) {
-            const uint64_t kt = mdesc(rkq + kk * 2048, 16384);
-            umma_bf16(X0, kt, mdesc(sm + O_DT + kk * 2048, 8192), id11, 1);
-            umma_bf16(X2, kt, kdesc(sm + O_AQ + kk * 32), id10, 1);
+            const uint64_t kt = step(mdesc(rkq, 16384), kk * 2048);
+            umma_if(lead, X0, kt, step(mdesc(sm + O_DT, 8192), kk * 2048), id11, 1);
+            umma_if(lead, X2, kt, step(kdesc(sm + O_AQ), kk * 32), id10, 1);
           } else {
-            umma_bf16(X0, kdesc(sm + O_KQH2 + kk * 32), mdesc(sm + O_DT + kk * 2048, 8192), id01, 1);
-            umma_bf16(X2, kdesc(sm + O_KKH2 + kk * 32), kdesc(sm + O_DT + kk * 32), id00, 1);
+            umma_if(lead, X0, step(kdesc(sm + O_KQH2), kk * 32), step(mdesc(sm + O_DT, 8192), kk * 2048), id01, 1);
+            umma_if(lead, X2, step(kdesc(sm + O_KKH2), kk * 32), step(kdesc(sm + O_DT), kk * 32), id00, 1);
           }
         }
-        umma_commit(bar_mma);
+        commit_if(lead, bar_mma);
       }
     }
     if constexpr (V == 0) {
@@ -1044,7 +1005,7 @@ __global__ void __launch_bounds__(BT, 1)
       issue_a_ctx(c - 1);  // the context buffers are free
       // phat, gamma and the token scalars of chunk c - 1 are read with plain loads at the
       // top of its iteration: bring them into L2 now
-      bulk_prefetch_l2(rec - kCtxBytes + kCtxPh, kCtxBytes - kCtxPh);
+      bulk_prefetch_l2(rec - P.rec + kCtxPh, kCtxBytes - kCtxPh);
     }
     // ---- [18] per channel (lane ci, tokens t0..t0+15): back through Gamma and the
     //           gain emission, then the uncertainty recursion backwards in time.
@@ -1439,14 +1400,17 @@ bool fused_bwd_supported(const Args &a) { return a.chunk != 32 && fused_fwd_supp
 size_t fused_saved_bytes(const Args &a) {
   if (!fused_bwd_supported(a)) return 0;
   const size_t nc = (a.T + CM - 1) / CM;
-  return (size_t)a.B * a.H * nc * (kCtxBytes + D * sizeof(float));
+  return (size_t)a.B * a.H * nc * (fused_ctx_record_bytes(a) + D * sizeof(float));
 }
 
-size_t fused_ctx_record_bytes() { return kCtxBytes; }
+size_t fused_ctx_record_bytes(const Args &a) { return split_bwd_context(a) ? kCtxSplitBytes : kCtxBytes; }
 
 kdn_status_t launch_fused_bwd_sweep(const Args &a, cudaStream_t s) {
+  // (a ragged length needs scratch in the workspace; without it the one-kernel sweep runs)
+  if (split_bwd_context(a) && (a.T % CM == 0 || a.split_ws)) return launch_split_bwd(a, a.T % CM == 0 ? nullptr : a.split_ws, s);
   BwdParams P;
   P.a = a;
+  P.rec = fused_ctx_record_bytes(a);
   CUtensorMap mq, mk, mv, mdo;
   if (!make_map(&mq, a.q, a) || !make_map(&mk, a.k, a) || !make_map(&mv, a.v, a) ||
       !make_map(&mdo, a.dO, a))

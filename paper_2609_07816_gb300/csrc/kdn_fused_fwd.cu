@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(FT, 1)
   uint32_t *s_tbase = reinterpret_cast<uint32_t *>(bars + 4);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int warp_u = __shfl_sync(0xffffffffu, warp, 0);  // warp-uniform: the MMA issue stays uniform
   const int wq = warp & 3, wg = warp >> 2;  // TMEM lane quarter, column group
   const int bh = blockIdx.x, b = bh / a.H, h = bh % a.H;
   const int NC = (a.T + CM - 1) / CM;
@@ -546,21 +547,24 @@ __global__ void __launch_bounds__(FT, 1)
       bulk_commit();
     }
     // ---- [4] MMA-T: D1 = [Kbar; Qbar] Kk^T, hi.hi + lo.hi + hi.lo
-    if (tid == 0) {
+    if (warp_u == 0) {
       tc_fence_after();
+      const uint32_t lead = elect_one();
       const uint32_t AH = smem_u32(kq), AL = smem_u32(a1l), BH = smem_u32(rw), BL = smem_u32(b1l);
+#pragma unroll
       for (int kk = 0; SD && kk < 8; ++kk) {  // [K; Q] K^T on the raw tiles (B: rows 0..63)
-        const uint64_t ad = sw128_desc(AH + (kk >> 2) * 16384 + (kk & 3) * 32, 16, 1024);
-        umma_bf16(TD1, ad, ad, id_T, kk > 0);
+        const uint64_t ad = step(sw128_desc(AH, 16, 1024), (kk >> 2) * 16384 + (kk & 3) * 32);
+        umma_if(lead, TD1, ad, ad, id_T, kk > 0);
       }
+#pragma unroll
       for (int kk = 0; !SD && kk < 8; ++kk) {
         const uint32_t ao = (kk >> 2) * 16384 + (kk & 3) * 32, bo = (kk >> 2) * 8192 + (kk & 3) * 32;
-        const uint64_t ah = sw128_desc(AH + ao, 16, 1024), bh_ = sw128_desc(BH + bo, 16, 1024);
-        umma_bf16(TD1, ah, bh_, id_T, kk > 0);
-        umma_bf16(TD1, sw128_desc(AL + ao, 16, 1024), bh_, id_T, 1);
-        umma_bf16(TD1, ah, sw128_desc(BL + bo, 16, 1024), id_T, 1);
+        const uint64_t ah = step(sw128_desc(AH, 16, 1024), ao), bh_ = step(sw128_desc(BH, 16, 1024), bo);
+        umma_if(lead, TD1, ah, bh_, id_T, kk > 0);
+        umma_if(lead, TD1, step(sw128_desc(AL, 16, 1024), ao), bh_, id_T, 1);
+        umma_if(lead, TD1, ah, step(sw128_desc(BL, 16, 1024), bo), id_T, 1);
       }
-      umma_commit(bar_mma);
+      commit_if(lead, bar_mma);
     }
     // V -> fp16 in place while MMA-T runs (the tile arrived during the previous chunk);
     // on a timeout the MMA is still waited for before leaving
@@ -638,16 +642,18 @@ __global__ void __launch_bounds__(FT, 1)
     tc_fence_before();
     __syncthreads();
     // ---- [6] MMA-W (bf16; Kbar enters as its hi part), MMA-U (fp16)
-    if (tid == 0) {
+    if (warp_u == 0) {
       tc_fence_after();
+      const uint32_t lead = elect_one();
       const uint32_t A2 = smem_u32(a2), AF = smem_u32(af), KQ = smem_u32(kq), VR = smem_u32(vr);
+#pragma unroll
       for (int kk = 0; kk < 4; ++kk) {
-        umma_bf16(TW, sw128_desc(A2 + kk * 32, 16, 1024), sw128_desc(KQ + kk * 2048, 16384, 1024), id_WU,
+        umma_if(lead, TW, step(sw128_desc(A2, 16, 1024), kk * 32), step(sw128_desc(KQ, 16384, 1024), kk * 2048), id_WU,
                   kk > 0);
-        umma_bf16(TU, sw128_desc(AF + kk * 32, 16, 1024), sw128_desc(VR + kk * 2048, 8192, 1024), id_U,
+        umma_if(lead, TU, step(sw128_desc(AF, 16, 1024), kk * 32), step(sw128_desc(VR, 8192, 1024), kk * 2048), id_U,
                   kk > 0);
       }
-      umma_commit(bar_mma);
+      commit_if(lead, bar_mma);
     }
     tc_fence_after();
     // While MMA-W/U run, the state operands that depend on neither W nor U
@@ -759,19 +765,22 @@ __global__ void __launch_bounds__(FT, 1)
       bulk_commit();
     }
     // ---- [8] MMA-S1 (fp16): [U; 0] += [-W; Qbar] S_in
-    if (tid == 0) {
+    if (warp_u == 0) {
       tc_fence_after();
+      const uint32_t lead = elect_one();
       const uint32_t A1 = smem_u32(a1l), B3 = smem_u32(b3);
+#pragma unroll
       for (int kk = 0; kk < 8; ++kk)
-        umma_bf16(TU, sw128_desc(A1 + (kk >> 2) * 16384 + (kk & 3) * 32, 16, 1024),
-                  sw128_desc(B3 + kk * 2048, 16384, 1024), ih_S1, 1);
+        umma_if(lead, TU, step(sw128_desc(A1, 16, 1024), (kk >> 2) * 16384 + (kk & 3) * 32),
+                  step(sw128_desc(B3, 16384, 1024), kk * 2048), ih_S1, 1);
       if (PH) {  // [R_Phi; .] = [-W; Qbar] Phi_in  (U = 0: v = 0 for Phi)
         const uint32_t B4 = smem_u32(fs);
+#pragma unroll
         for (int kk = 0; kk < 8; ++kk)
-          umma_bf16(TW, sw128_desc(A1 + (kk >> 2) * 16384 + (kk & 3) * 32, 16, 1024),
-                    sw128_desc(B4 + kk * 2048, 16384, 1024), ih_S1, kk > 0);
+          umma_if(lead, TW, step(sw128_desc(A1, 16, 1024), (kk >> 2) * 16384 + (kk & 3) * 32),
+                    step(sw128_desc(B4, 16384, 1024), kk * 2048), ih_S1, kk > 0);
       }
-      umma_commit(bar_mma);
+      commit_if(lead, bar_mma);
     }
     if (!(ok = mma_wait())) break;
     tc_fence_after();
@@ -800,20 +809,22 @@ __global__ void __launch_bounds__(FT, 1)
       bulk_commit();
     }
     // ---- [10] MMA-O and MMA-S2 (fp16)
-    if (tid == 0) {
+    if (warp_u == 0) {
       tc_fence_after();
+      const uint32_t lead = elect_one();
       const uint32_t A2 = smem_u32(a2), B1 = smem_u32(b1l), VR = smem_u32(vr);
+#pragma unroll
       for (int kk = 0; kk < 4; ++kk) {
-        const uint64_t bd = sw128_desc(VR + kk * 2048, 8192, 1024);
-        umma_bf16(TU, sw128_desc(A2 + kk * 32, 16, 1024), bd, ih_S1, 1);
-        umma_bf16(TS, sw128_desc(B1 + kk * 2048, 8192, 1024), bd, ih_S2, 1);
+        const uint64_t bd = step(sw128_desc(VR, 8192, 1024), kk * 2048);
+        umma_if(lead, TU, step(sw128_desc(A2, 16, 1024), kk * 32), bd, ih_S1, 1);
+        umma_if(lead, TS, step(sw128_desc(B1, 8192, 1024), kk * 2048), bd, ih_S2, 1);
         if (PH) {  // O_Phi += A_qk R_Phi;  Phi += K_tail^T R_Phi
-          const uint64_t bp = sw128_desc(smem_u32(fs) + kk * 2048, 8192, 1024);
-          umma_bf16(TW, sw128_desc(A2 + kk * 32, 16, 1024), bp, ih_S1, 1);
-          umma_bf16(TPH, sw128_desc(B1 + kk * 2048, 8192, 1024), bp, ih_S2, 1);
+          const uint64_t bp = step(sw128_desc(smem_u32(fs), 8192, 1024), kk * 2048);
+          umma_if(lead, TW, step(sw128_desc(A2, 16, 1024), kk * 32), bp, ih_S1, 1);
+          umma_if(lead, TPH, step(sw128_desc(B1, 8192, 1024), kk * 2048), bp, ih_S2, 1);
         }
       }
-      umma_commit(bar_mma);
+      commit_if(lead, bar_mma);
     }
     if (io && P.save_S) bulk_wait_read();  // the saved R and A have left vr and fs
     if (!(ok = mma_wait())) break;
@@ -915,11 +926,11 @@ __global__ void __launch_bounds__(FT, 1)
 // kappa = phat k / s_t, so k^T kappa = (s_t - r_t) / s_t = 1 - r_t / s_t;
 // Isotropic KDN kappa = beta_t k, so k^T kappa = beta_t |k_t|^2.  One thread per
 // token, one CTA per (chunk, batch * head).
-__global__ void __launch_bounds__(CM) k_beta_eff(const Args a, const unsigned char *saved, float *out) {
+__global__ void __launch_bounds__(CM) k_beta_eff(const Args a, size_t rec, const unsigned char *saved, float *out) {
   const int c = blockIdx.x, bh = blockIdx.y, t = threadIdx.x;
   const int b = bh / a.H, h = bh % a.H, NC = (a.T + CM - 1) / CM, tt = c * CM + t;
   if (tt >= a.T) return;
-  const float *tok = reinterpret_cast<const float *>(saved + ((size_t)bh * NC + c) * kCtxBytes + kCtxTok);
+  const float *tok = reinterpret_cast<const float *>(saved + ((size_t)bh * NC + c) * rec + kCtxTok);
   const size_t th = tok_index(a, b, tt, h);
   if (a.variant == 0) {
     const float rr = gate_r(a.gates, a.rmin, ld<__nv_bfloat16>(a.r, th));
@@ -957,7 +968,7 @@ kdn_status_t launch_wait_selftest(unsigned *status, cudaStream_t s) {
 kdn_status_t launch_beta_eff(const Args &a, const void *saved, float *out, cudaStream_t s) {
   const int NC = (a.T + CM - 1) / CM;
   k_beta_eff<<<dim3((unsigned)NC, (unsigned)(a.B * a.H)), CM, 0, s>>>(
-      a, static_cast<const unsigned char *>(saved), out);
+      a, fused_ctx_record_bytes(a), static_cast<const unsigned char *>(saved), out);
   return cudaGetLastError() == cudaSuccess ? KDN_OK : KDN_ERR_CUDA;
 }
 

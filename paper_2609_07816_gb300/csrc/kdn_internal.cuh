@@ -132,6 +132,7 @@ struct Args {
   float *aff;     // [BH][NC][P][2] chunk summaries of the uncertainty adjoint
   float *dpout;   // [BH][NC][P]    cotangent of the uncertainty leaving every chunk
   unsigned char *fSin;  // fused backward: [BH][NC] context records (S_in, R, -W, A_qk, A)
+  char *split_ws;       // two-kernel backward: scratch in the workspace (null: none)
   float *fpin;          // fused backward: [BH][NC][dk] uncertainty entering each chunk
 };
 
@@ -178,7 +179,13 @@ kdn_status_t launch_fused_bwd_sweep(const Args &a, cudaStream_t s);
 // (batch, head) and 64-token chunk one record of fused_ctx_record_bytes(), then
 // per chunk the 128 float32 uncertainties entering it.
 size_t fused_saved_bytes(const Args &a);
-size_t fused_ctx_record_bytes();
+size_t fused_ctx_record_bytes(const Args &a);
+// Two-kernel backward of the Diagonal KDN (kdn_split_bwd.cu): whether the context of this
+// problem feeds it, the scratch it needs in the workspace (ragged lengths; otherwise its
+// scratch lies in the gradient buffers) and its launcher.
+bool split_bwd_context(const Args &a);
+size_t split_bwd_workspace_bytes(const Args &a);
+kdn_status_t launch_split_bwd(const Args &a, char *ws, cudaStream_t s);
 
 // Sequence-parallel forward (kdn_segmented.cu): the number of segments P each
 // sequence is cut into (1: not used), the workspace it needs after the common

@@ -248,6 +248,34 @@ __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint6
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// MMA issue by a whole warp with one elected lane.  In a branch on a warp-uniform warp index
+// the descriptors and addresses stay in uniform registers, which the instruction takes;
+// inside `if (tid == 0)` every operand is moved there first, ~100 cycles an MMA (eight
+// M = N = 128 products and their completion: 1.9 K cycles, 0.55 K this way).
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p;
+}
+__device__ __forceinline__ void umma_if(uint32_t lead, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
+                                        uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(lead)
+      : "memory");
+}
+__device__ __forceinline__ void commit_if(uint32_t lead, uint64_t *bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(
+          smem_u32(bar)),
+      "r"(lead)
+      : "memory");
+}
+// A shared-memory descriptor moved on by `bytes` (a multiple of 16): the address field is its
+// low part, so one addition replaces building the descriptor again.
+__device__ __forceinline__ uint64_t step(uint64_t desc, uint32_t bytes) { return desc + (bytes >> 4); }
 // Arrive on `bar` once all previously issued MMAs of this thread complete.
 __device__ __forceinline__ void umma_commit(uint64_t *bar) {
   asm volatile(

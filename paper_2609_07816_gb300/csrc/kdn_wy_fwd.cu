@@ -166,22 +166,22 @@ __device__ __forceinline__ bool bar_or(int id, int n, bool p) {
 __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N) {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-__device__ __forceinline__ void umma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc,
-                                          uint32_t acc) {
+__device__ __forceinline__ void umma_tf32(uint32_t lead, uint32_t d, uint64_t a, uint64_t b,
+                                          uint32_t idesc, uint32_t acc) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(lead)
       : "memory");
 }
 // A operand in tensor memory: lane = row, 32-bit column c holds the 16-bit
 // elements 2c (low half) and 2c + 1 of that row
-__device__ __forceinline__ void umma_f16_tA(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t idesc,
-                                            uint32_t acc) {
+__device__ __forceinline__ void umma_f16_tA(uint32_t lead, uint32_t d, uint32_t a_tmem, uint64_t b,
+                                            uint32_t idesc, uint32_t acc) {
   asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
-      "r"(a_tmem), "l"(b), "r"(idesc), "r"(acc)
+      "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
+      "r"(a_tmem), "l"(b), "r"(idesc), "r"(acc), "r"(lead)
       : "memory");
 }
 __device__ __forceinline__ void tmem_st4u(uint32_t taddr, const uint32_t *v) {
@@ -445,7 +445,8 @@ __device__ __noinline__ void direct_products(int tid, const unsigned char *rk, c
 
 struct WyParams {
   Args a;
-  unsigned char *save_S;  // SV: [BH][NC] context records of the backward (kCtxBytes each)
+  unsigned char *save_S;  // SV: [BH][NC] context records of the backward
+  size_t rec;             // SV: bytes of a record; beyond kCtxBytes it also takes Qbar and K'^T
   float *save_p;          // SV: [BH][NC][128] uncertainty carry entering each chunk
 };
 
@@ -486,7 +487,9 @@ __global__ void __launch_bounds__(WT, 1)
   const int wq = warp & 3, wg = warp >> 2;  // TMEM lane quarter, column group
   const int bh = blockIdx.x, b = bh / a.H, h = bh % a.H;
   const int NC = (a.T + CM - 1) / CM;
-  const bool issuer = tid == 128;
+  const bool issuer = tid == 128;  // copies; the MMAs: its whole warp with an elected lane
+  const int warp_u = __shfl_sync(0xffffffffu, warp, 0);
+  const bool ext = SV && P.rec > (size_t)kCtxBytes;
   const uint32_t lane_base = (uint32_t)(32 * wq) << 16;
 
   if (issuer) {
@@ -577,15 +580,12 @@ __global__ void __launch_bounds__(WT, 1)
   const int wgm = (warp >> 2) - 1;    // main warps: 0, 1, 2 within a lane quarter
   float p = 1.f;                      // gain threads: uncertainty carry of channel tid
   if (gain && a.p0) p = a.p0[(size_t)bh * D + tid];
-  float rnext = 1.f;                  // gain threads tid < 64: r of the next chunk's token tid
+  // gain threads tid < 64: the r input of the next chunk's token tid, converted when it is
+  // used (a conversion here would wait for the load)
+  __nv_bfloat16 znext = __float2bfloat16_rn(0.f);
   auto load_r = [&](int c) {
-    if (tid < CM) {
-      rnext = 1.f;
-      if (c < NC && c * CM + tid < a.T) {
-        const float z = ld<__nv_bfloat16>(a.r, tok_index(a, b, c * CM + tid, h));
-        rnext = LG ? a.rmin + softplus_w(z) : z;  // r = r_min + softplus(z) (Sec. 5)
-      }
-    }
+    if (tid < CM && c < NC)
+      znext = static_cast<const __nv_bfloat16 *>(a.r)[tok_index(a, b, min(c * CM + tid, a.T - 1), h)];
   };
   load_r(0);
 
@@ -606,8 +606,16 @@ __global__ void __launch_bounds__(WT, 1)
     const int i = tid, sb = c & 1;
     float *sr = s_r + 64 * sb, *smur = s_mur + 64 * sb;
     if (tid < CM) {
-      sr[tid] = rnext;
-      smur[tid] = a.mu / rnext;
+      const bool live = c * CM + tid < a.T;
+      const float z = live ? __bfloat162float(znext) : 0.f;
+      const float r = !live ? 1.f : LG ? a.rmin + softplus_w(z) : z;  // r = r_min + softplus(z) (Sec. 5)
+      sr[tid] = r;
+      smur[tid] = a.mu / r;
+      if (ext) {  // r_t and z_t for the backward (tokens past T: 1 and 0)
+        float *tok = reinterpret_cast<float *>(P.save_S + ((size_t)bh * NC + c) * P.rec + kCtxTok);
+        tok[CM + tid] = r;
+        tok[2 * CM + tid] = z;
+      }
     }
     load_r(c + 1);
     bar_sync(kBarGain, 128);
@@ -681,7 +689,7 @@ __global__ void __launch_bounds__(WT, 1)
     const bool oor = !SV && bar_or(kBarGain, 128, cref < kMinHalfG);
     if (tid == 0) s_oor[sb] = oor ? 1 : 0;
     float Gt = 0.f;  // G_t of this channel (range mode)
-    unsigned char *gctx = SV ? P.save_S + ((size_t)bh * NC + c) * kCtxBytes : nullptr;
+    unsigned char *gctx = SV ? P.save_S + ((size_t)bh * NC + c) * P.rec : nullptr;
     if (SV) P.save_p[((size_t)bh * NC + c) * D + i] = p;
     float *cph = SV ? reinterpret_cast<float *>(gctx + kCtxPh) + i : nullptr;
     float f = ex2f(cref * kLog2e);                // exp(c - G_t), G_{-1} = 0
@@ -761,6 +769,7 @@ __global__ void __launch_bounds__(WT, 1)
           else kt[j >> 1] |= hb << 16;
         }
         tmem_st4u(tkt + lane_base + (uint32_t)(4 * blk), kt);
+        if (ext) *reinterpret_cast<uint4 *>(gctx + kCtxKt + chunk_off(i, blk)) = make_uint4(kt[0], kt[1], kt[2], kt[3]);
         if (blk < 7) {
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
@@ -783,7 +792,7 @@ __global__ void __launch_bounds__(WT, 1)
 
   for (int c = 0; c < NC; ++c) {
     const uint32_t tkt = TKT + (uint32_t)((c & 1) * 32);
-    unsigned char *ctx = SV ? P.save_S + ((size_t)bh * NC + c) * kCtxBytes : nullptr;
+    unsigned char *ctx = SV ? P.save_S + ((size_t)bh * NC + c) * P.rec : nullptr;
     if (SV && issuer) bulk_wait_read();  // the previous chunk's context tiles have left shared memory
     // ---- [0] the previous chunk's MMA-O / MMA-S2 must be done before V is brought
     //          into its R' buffer; the gain of this chunk is done (its warps arrive here)
@@ -927,13 +936,15 @@ __global__ void __launch_bounds__(WT, 1)
         }
       }
     };
-    if (issuer && !oor) {
+    if (warp_u == 4 && !oor) {
       tc_fence_after();
-      const uint32_t A0 = smem_u32(ta), B0 = smem_u32(tb);
+      const uint32_t lead = elect_one();
+      const uint64_t A0 = sw128_desc(smem_u32(ta), 16, 1024), B0 = sw128_desc(smem_u32(tb), 16, 1024);
+#pragma unroll
       for (int kk = 0; kk < 16; ++kk)
-        umma_tf32(TD1, sw128_desc(A0 + (kk >> 2) * 16384 + (kk & 3) * 32, 16, 1024),
-                  sw128_desc(B0 + (kk >> 2) * 8192 + (kk & 3) * 32, 16, 1024), id_T, kk > 0);
-      umma_commit(bar_t);
+        umma_tf32(lead, TD1, step(A0, (kk >> 2) * 16384 + (kk & 3) * 32),
+                  step(B0, (kk >> 2) * 8192 + (kk & 3) * 32), id_T, kk > 0);
+      commit_if(lead, bar_t);
     }
     // the next chunk's tiles (the raw tiles are free: the preparing pass is done), from a
     // main thread outside the MMA issuer's warp: its ~20 TMA operations then overlap
@@ -1017,14 +1028,20 @@ __global__ void __launch_bounds__(WT, 1)
     bar_sync(kBarMain, kMain);
     tc_fence_after();
     // MMA-KS: TU = [-Kbar; Qbar] S_in (fp16), while the CUDA cores solve
-    if (issuer) {
-      const uint32_t A1 = smem_u32(as1), B1 = smem_u32(s16);
+    if (warp_u == 4) {
+      const uint32_t lead = elect_one();
+      const uint64_t A1 = sw128_desc(smem_u32(as1), 16, 1024), B1 = sw128_desc(smem_u32(s16), 16384, 1024);
+#pragma unroll
       for (int kk = 0; kk < 8; ++kk)
-        umma_bf16(TU, sw128_desc(A1 + (kk >> 2) * 16384 + (kk & 3) * 32, 16, 1024),
-                  sw128_desc(B1 + kk * 2048, 16384, 1024), id_16, kk > 0);
-      umma_commit(bar_mma);
+        umma_if(lead, TU, step(A1, (kk >> 2) * 16384 + (kk & 3) * 32), step(B1, kk * 2048), id_16, kk > 0);
+      commit_if(lead, bar_mma);
+    }
+    if (issuer) {
       if (SV) {
         bulk_s2g(ctx + kCtxS, s16, 32768);
+        if (ext)
+          for (int s = 0; s < 2; ++s)
+            bulk_s2g(ctx + kCtxKQ + s * 16384 + 8192, as1 + s * 16384 + 8192, 8192);
         bulk_commit();
       }
     }
@@ -1089,12 +1106,15 @@ __global__ void __launch_bounds__(WT, 1)
         bulk_s2g(ctx + kCtxA, awu, 8192);
         bulk_s2g(ctx + kCtxY, vr, 16384);  // Y, before R' is written over it
         bulk_commit();
+      }
+      if (warp_u == 4) {
         tc_fence_after();
-        const uint32_t AW = smem_u32(awu), KN = smem_u32(as1);
+        const uint32_t lead = elect_one();
+        const uint64_t AW = sw128_desc(smem_u32(awu), 16, 1024), KN = sw128_desc(smem_u32(as1), 16384, 1024);
+#pragma unroll
         for (int kk = 0; kk < 4; ++kk)  // B = rows 0..63 of [-Kbar; Qbar], MN-major
-          umma_bf16(TW, sw128_desc(AW + kk * 32, 16, 1024), sw128_desc(KN + kk * 2048, 16384, 1024),
-                    id_16, kk > 0);
-        umma_commit(bar_w);  // its own barrier: MMA-KS may not have been observed yet
+          umma_if(lead, TW, step(AW, kk * 32), step(KN, kk * 2048), id_16, kk > 0);
+        commit_if(lead, bar_w);  // its own barrier: MMA-KS may not have been observed yet
       }
     }
     // ---- [6] (context only) -W out of TMEM
@@ -1121,16 +1141,17 @@ __global__ void __launch_bounds__(WT, 1)
     }
 
     // ---- [7] MMA-R: TW = [A; 0] Y = [R; 0]  (fp16)
-    if (issuer) {
-      // (context: the copy of Y has left shared memory before MMA-R completes, after
-      // which R' is written over Y; the copy of -W, committed after it, may still run)
-      if (SV) bulk_wait_read_but1();
+    // (context: the copy of Y has left shared memory before MMA-R completes, after
+    // which R' is written over Y; the copy of -W, committed after it, may still run)
+    if (SV && issuer) bulk_wait_read_but1();
+    if (warp_u == 4) {
+      __syncwarp();
       tc_fence_after();
-      const uint32_t AW = smem_u32(awu), VR = smem_u32(vr);
-      for (int kk = 0; kk < 4; ++kk)
-        umma_bf16(TW, sw128_desc(AW + kk * 32, 16, 1024), sw128_desc(VR + kk * 2048, 8192, 1024), id_16,
-                  kk > 0);
-      umma_commit(bar_mma);
+      const uint32_t lead = elect_one();
+      const uint64_t AW = sw128_desc(smem_u32(awu), 16, 1024), VR = sw128_desc(smem_u32(vr), 8192, 1024);
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) umma_if(lead, TW, step(AW, kk * 32), step(VR, kk * 2048), id_16, kk > 0);
+      commit_if(lead, bar_mma);
     }
     mine = mma_wait_main() && mine;
     tc_fence_after();
@@ -1159,19 +1180,21 @@ __global__ void __launch_bounds__(WT, 1)
 
     // ---- [9] MMA-O (rows 64..127 of TU += A'_qk R', A'_qk in TMEM) and
     //          MMA-S2 (S += K'^T R', K' in TMEM)
-    if (issuer) {
-      if (SV) {
-        bulk_s2g(ctx + kCtxR, awu, 16384);
-        bulk_commit();
-      }
+    if (SV && issuer) {
+      bulk_s2g(ctx + kCtxR, awu, 16384);
+      bulk_commit();
+    }
+    if (warp_u == 4) {
       tc_fence_after();
-      const uint32_t VR = smem_u32(vr);
+      const uint32_t lead = elect_one();
+      const uint64_t VR = sw128_desc(smem_u32(vr), 8192, 1024);
+#pragma unroll
       for (int kk = 0; kk < 4; ++kk) {
-        const uint64_t bd = sw128_desc(VR + kk * 2048, 8192, 1024);
-        umma_f16_tA(TU, TD1 + (uint32_t)(kk * 8), bd, id_16, 1);
-        umma_f16_tA(TS, tkt + (uint32_t)(kk * 8), bd, id_16, 1);
+        const uint64_t bd = step(VR, kk * 2048);
+        umma_f16_tA(lead, TU, TD1 + (uint32_t)(kk * 8), bd, id_16, 1);
+        umma_f16_tA(lead, TS, tkt + (uint32_t)(kk * 8), bd, id_16, 1);
       }
-      umma_commit(bar_mma);
+      commit_if(lead, bar_mma);
     }
   }
 
@@ -1245,6 +1268,7 @@ kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S,
   WyParams P;
   P.a = a;
   P.save_S = save_S;
+  P.rec = fused_ctx_record_bytes(a);
   P.save_p = save_p;
   CUtensorMap mk, mg, mw, mv, mq;
   if (!make_map(&mk, a.k, a) || !make_map(&mg, a.g, a) || !make_map(&mw, a.omega, a) ||
