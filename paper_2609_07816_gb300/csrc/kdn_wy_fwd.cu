@@ -105,7 +105,7 @@ constexpr int O_S16 = O_TA;                      // fp16 S_in [128 i][128 j], tw
 constexpr int O_SWT = O_TA + 32768;              // fp32 T' [64][LT]
 constexpr int O_SWA = O_SWT + 64 * LT * 4;       // fp32 L^-1 [64][LT]
 static_assert(O_SWA + 64 * LT * 4 <= O_TB, "T and A tiles overlap the Kk' tile");
-constexpr int O_AWU = O_SWT;           // fp16 [A; 0] [128][64] (MMA-R A), over T' after the solve
+constexpr int O_AWU = O_SWT;           // fp16 [A; .] [128][64] (MMA-R A), over T' after the solve
 // small arrays (floats); r and mu / r per token for two chunks (the gain works one chunk ahead)
 constexpr int SM_R = 0, SM_MUR = 128, SM_S = 256, SM_IS = 320, SM_C = 384, SM_GC = 512,
               SM_PART = 640, SM_OOR = 640 + 8 * 128, SM_FLOATS = SM_OOR + 16;
@@ -224,30 +224,39 @@ __device__ __forceinline__ void wy_inverse(int tid, const float *sT, float *sA, 
                                            const float *s_r, float *s_s, float *s_is,
                                            unsigned char *awu, Side side) {
   const int w = tid >> 5;  // main warp 0 .. 11 (lane quarter w & 3)
-  if (tid < 64) {
-    // column c of D_I: x_r = (delta_rc - sum_{m<r} L_rm x_m) / L_rr, rows read 16 bytes at a time
-    const int o = 16 * (tid >> 4), c = tid & 15;
+  if (w == 2 || w == 3) {
+    const int st = tid - 64;
+    // column c of D_I: x_r = (delta_rc - sum_{m<r} L_rm x_m) / L_rr.  Lane c also forms row c's
+    // s_t and its reciprocal, handed round by shuffles; rows are loaded two steps ahead
+    const int o = 16 * (st >> 4), c = st & 15;
     const float *tb = sT + o * (LT + 1);
-    float x[16];
+    const float sc = s_r[o + c] + tb[c * (LT + 1)];  // s_t = r_t + sum_i phat k^2 (eq. kla-box-gain)
+    const float ic = rcpf(sc);
+    s_s[o + c] = sc;
+    s_is[o + c] = ic;
+    float x[16], row[3][16];
+    auto load = [&](int r) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (4 * j < r) {
+          const float4 t4 = *reinterpret_cast<const float4 *>(tb + r * LT + 4 * j);
+          float *d = row[r % 3] + 4 * j;
+          d[0] = t4.x; d[1] = t4.y; d[2] = t4.z; d[3] = t4.w;
+        }
+    };
+    load(1);
+    load(2);
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
-      float lr[16];
-#pragma unroll
-      for (int j = 0; 4 * j <= r; ++j) {
-        const float4 t4 = *reinterpret_cast<const float4 *>(tb + r * LT + 4 * j);
-        lr[4 * j] = t4.x; lr[4 * j + 1] = t4.y; lr[4 * j + 2] = t4.z; lr[4 * j + 3] = t4.w;
-      }
-      const float lrr = s_r[o + r] + lr[r];  // s_t = r_t + sum_i phat k^2 (eq. kla-box-gain)
-      const float inv = rcpf(lrr);
-      if (r == c) {
-        s_s[o + r] = lrr;
-        s_is[o + r] = inv;
-      }
+      if (r + 2 < 16 && r > 0) load(r + 2);
+      const float inv = __shfl_sync(0xffffffffu, ic, r, 16);
       float acc0 = (r == c) ? 1.f : 0.f, acc1 = 0.f;
 #pragma unroll
-      for (int m = 0; m < r; ++m) {
-        if (m & 1) acc1 = fmaf(-lr[m], x[m], acc1);
-        else acc0 = fmaf(-lr[m], x[m], acc0);
+      for (int m = 0; m < 15; ++m) {
+        if (m < r) {
+          if (m & 1) acc1 = fmaf(-row[r % 3][m], x[m], acc1);
+          else acc0 = fmaf(-row[r % 3][m], x[m], acc0);
+        }
       }
       x[r] = (acc0 + acc1) * inv;  // x[r] = 0 for r < c
     }
@@ -255,16 +264,12 @@ __device__ __forceinline__ void wy_inverse(int tid, const float *sT, float *sA, 
 #pragma unroll
     for (int r = 0; r < 16; ++r) ab[r * LT] = x[r];
   } else if ((w & 3) < 2) {
-    side();  // warps 4, 5, 8, 9 of the main group (lane quarters 0, 1)
+    side();  // lane quarters 0, 1
   } else {
-    // zero the strictly upper 16 x 16 blocks (I < J): 6 blocks x 16 rows x 4 float4
-    const int z = 64 * (w >> 2) + 32 * ((w & 3) - 2) + (tid & 31);  // 0 .. 191
-    for (int e = z; e < 384; e += 192) {
-      const int blk = e >> 6, rr = (e >> 2) & 15, q4 = e & 3;
-      const int I = blk < 3 ? 0 : (blk < 5 ? 1 : 2);
-      const int J = blk < 3 ? blk + 1 : (blk < 5 ? blk - 1 : 3);
-      *reinterpret_cast<float4 *>(sA + (16 * I + rr) * LT + 16 * J + 4 * q4) = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    // zero the upper right 16 x 16 blocks of X11 and X22: 2 blocks x 16 rows x 4 float4
+    const int z = 32 * (w == 6 ? 0 : w == 7 ? 1 : w == 10 ? 2 : 3) + (tid & 31);
+    const int o = 32 * (z >> 6), rr = (z >> 2) & 15, q4 = z & 3;
+    *reinterpret_cast<float4 *>(sA + (o + rr) * LT + o + 16 + 4 * q4) = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   bar_sync(kBarMain, kMain);
   // X_10, X_32: one thread per (block, row, 4 columns)
@@ -329,7 +334,7 @@ __device__ __forceinline__ void wy_inverse(int tid, const float *sT, float *sA, 
     *reinterpret_cast<float4 *>(sY + r3 * 32 + cq3) = acc;
   }
   bar_sync(kBarMain, kMain);
-  // T' is dead from here on: [A; 0] fp16 [128 t][64 s] (A = diag(s) L^-1) is written over it.
+  // T' is dead from here on: [A; .] fp16 [128 t][64 s] (A = diag(s) L^-1) is written over it.
   // X_21 = -X22 Y by threads 0..255, straight to fp16; threads 256..383 convert the rest.
   if (tid < 256) {
     const float *dp = sA + (32 + r3) * LT + 32;
@@ -352,31 +357,17 @@ __device__ __forceinline__ void wy_inverse(int tid, const float *sT, float *sA, 
     *reinterpret_cast<uint2 *>(awu + chunk_off(r, cq3 >> 3) + 2 * (cq3 & 4)) =
         pack_h4(sr * acc.x, sr * acc.y, sr * acc.z, sr * acc.w);
   } else {
-    // rows 0..31 (8 column chunks), rows 32..63 columns 32..63 (4 chunks), rows 64..127 zero
-    for (int e = tid - 256; e < 896; e += 128) {
-      int r, cc;
-      if (e < 256) {
-        r = e >> 3;
-        cc = e & 7;
-      } else if (e < 384) {
-        r = 32 + ((e - 256) >> 2);
-        cc = 4 + (e & 3);
-      } else {
-        r = 64 + ((e - 384) >> 3);
-        cc = e & 7;
-      }
+    // rows 0..31 (8 column chunks), rows 32..63 columns 32..63 (4 chunks).  (Rows 64..127 of
+    // [A; .] keep what is there: they only reach accumulator rows that nobody reads.)
+    for (int e = tid - 256; e < 384; e += 128) {
+      const int r = e < 256 ? e >> 3 : 32 + ((e - 256) >> 2), cc = e < 256 ? e & 7 : 4 + (e & 3);
       float v[8];
-      if (r < 64) {
-        const float sr = s_s[r];
-        const float4 a0 = *reinterpret_cast<const float4 *>(sA + r * LT + 8 * cc);
-        const float4 a1 = *reinterpret_cast<const float4 *>(sA + r * LT + 8 * cc + 4);
-        const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+      const float sr = s_s[r];
+      const float4 a0 = *reinterpret_cast<const float4 *>(sA + r * LT + 8 * cc);
+      const float4 a1 = *reinterpret_cast<const float4 *>(sA + r * LT + 8 * cc + 4);
+      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
 #pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = (8 * cc + j <= r) ? sr * av[j] : 0.f;
-      } else {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = 0.f;
-      }
+      for (int j = 0; j < 8; ++j) v[j] = (8 * cc + j <= r) ? sr * av[j] : 0.f;
       sm16(awu, chunk_off(r, cc)) = pack_h8(v);
     }
   }
@@ -1047,9 +1038,9 @@ __global__ void __launch_bounds__(WT, 1)
     }
 
     // ---- [4] A = (I + T)^-1 = diag(s) L^-1 with L = diag(s) + strict_lower(T')
-    //          (T = strict_lower(T') diag(1/s)), then [A; 0] fp16 over T';
+    //          (T = strict_lower(T') diag(1/s)), then [A; .] fp16 over T';
     //          Y = V - Kbar S_in (rows 0..63 of TU plus V) -> fp16 in place over V, by warps
-    //          8, 9, 12, 13 while warps 4, 5 solve the diagonal blocks
+    //          4, 5, 8, 9, 12, 13 while warps 6, 7 solve the diagonal blocks
     {
       auto y_side = [&]() {
         const bool ks_ok = mma_wait_main();  // MMA-KS
@@ -1057,7 +1048,7 @@ __global__ void __launch_bounds__(WT, 1)
         mine = ks_ok && v_ok && mine;
         tc_fence_after();
         const int t = 32 * wq + lane;
-        for (int g = wgm - 1; g < 8; g += 2) {
+        for (int g = wgm; g < 8; g += 3) {
           float v[16], vv[16];
           const int j0 = 16 * g, sl = j0 >> 6, cc0 = (j0 & 63) >> 3;
           tmem_ld16(TU + lane_base + j0, v);
@@ -1071,7 +1062,7 @@ __global__ void __launch_bounds__(WT, 1)
         }
       };
       wy_inverse(mt, sT, sA, sX, sY, s_r + 64 * (c & 1), s_s, s_is, awu, y_side);
-      if (!(wq < 2 && wgm >= 1)) ++mph;  // MMA-KS, observed by the Y warps
+      if (wq >= 2) ++mph;  // MMA-KS, observed by the Y warps
     }
     if (SV) {
       if (wq >= 2 && wgm == 0) {  // A_qk = lower(A'_qk) diag(1/s) into the context
@@ -1140,7 +1131,7 @@ __global__ void __launch_bounds__(WT, 1)
       }
     }
 
-    // ---- [7] MMA-R: TW = [A; 0] Y = [R; 0]  (fp16)
+    // ---- [7] MMA-R: TW = [A; .] Y = [R; 0]  (fp16)
     // (context: the copy of Y has left shared memory before MMA-R completes, after
     // which R' is written over Y; the copy of -W, committed after it, may still run)
     if (SV && issuer) bulk_wait_read_but1();
@@ -1164,7 +1155,7 @@ __global__ void __launch_bounds__(WT, 1)
         float v[16];
         const int j0 = 16 * g, sl = j0 >> 6, cc0 = (j0 & 63) >> 3;
         tmem_ld16(TW + lane_base + j0, v);
-        if (SV) {  // R for the context, staged over [A; 0] (MMA-R has read it) for one bulk copy
+        if (SV) {  // R for the context, staged over [A; .] (MMA-R has read it) for one bulk copy
           sm16(awu, sl * 8192 + chunk_off(t, cc0)) = pack_h8(v);
           sm16(awu, sl * 8192 + chunk_off(t, cc0 + 1)) = pack_h8(v + 8);
         }
