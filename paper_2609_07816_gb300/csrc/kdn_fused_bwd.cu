@@ -306,25 +306,16 @@ __global__ void __launch_bounds__(BT, 1)
     s_dp[tid] = a.dpT ? lam * a.dpT[pi] : 0.f;
   }
 
-  // per-token scalars of the next chunk (r; the scalar decay of the isotropic KDN),
-  // prefetched into registers
-  // (and, with logit gates, the chain factors sigmoid(z_t), sigmoid(y_t) of r and omega)
-  float nr = 1.f, ng = 0.f, nfr = 1.f, nfw = 1.f;
+  // per-token inputs of the next chunk (r; the scalar decay and omega of the isotropic KDN),
+  // prefetched into registers and converted when they are used (a conversion here would
+  // wait for the loads)
+  __nv_bfloat16 nz = __float2bfloat16_rn(0.f), nx = nz, ny = nz;
   auto load_r = [&](int c) {
-    nr = 1.f;
-    ng = 0.f;
-    nfr = 1.f;
-    nfw = 1.f;
     if (tid < CM && c >= 0) {
-      const int t = c * CM + tid;
-      if (t < a.T) {
-        const size_t th = tok_index(a, b, t, h);
-        const float z = ld<__nv_bfloat16>(a.r, th);
-        nr = gate_r(G, a.rmin, z);
-        nfr = dgate_sig(G, z);
-        if (V == 1 && !a.pcd) ng = gate_logalpha(G, ld<__nv_bfloat16>(a.g, th));
-        if (V == 1 && G) nfw = sigmoid_f(ld<__nv_bfloat16>(a.omega, th));
-      }
+      const size_t th = tok_index(a, b, min(c * CM + tid, a.T - 1), h);
+      nz = static_cast<const __nv_bfloat16 *>(a.r)[th];
+      if (V == 1 && !a.pcd) nx = static_cast<const __nv_bfloat16 *>(a.g)[th];
+      if (V == 1 && G) ny = static_cast<const __nv_bfloat16 *>(a.omega)[th];
     }
   };
   load_r(NC - 1);
@@ -374,11 +365,14 @@ __global__ void __launch_bounds__(BT, 1)
     //          (diagonal KDN: bulk copies issued at the end of the previous chunk, on
     //          bar_g; isotropic: global loads issued before the wait for the tiles); raw tiles
     if (tid < CM) {
+      // (with logit gates: and the chain factors sigmoid(z_t), sigmoid(y_t) of r and omega)
+      const bool live = c * CM + tid < a.T;
+      const float z = __bfloat162float(nz), nr = live ? gate_r(G, a.rmin, z) : 1.f;
       s_r[tid] = nr;
       s_ri[tid] = 1.f / nr;
-      s_gs[tid] = ng;
-      s_fr[tid] = nfr;
-      s_fw[tid] = nfw;
+      s_gs[tid] = V == 1 && !a.pcd && live ? gate_logalpha(G, __bfloat162float(nx)) : 0.f;
+      s_fr[tid] = live ? dgate_sig(G, z) : 1.f;
+      s_fw[tid] = V == 1 && G && live ? sigmoid_f(__bfloat162float(ny)) : 1.f;
     }
     const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * P.rec;
     float e16[16], ph16[16], tk[5];

@@ -107,65 +107,32 @@ __device__ __forceinline__ void check_gamma_range(float gC, unsigned *status) {
 // Row stride (floats) of the fp32 T and A tiles: 16-byte rows, conflict-free.
 constexpr int LT = 68;
 
-// Level L (= I - J) of the blocked inverse below: one thread per (block J, row,
-// 4 columns), float4 operands; X_IJ = sum_{K=J}^{I-1} T_IK A_KJ, then A_IJ = -D_I X_IJ.
-template <int L>
-__device__ __forceinline__ void tri_inverse_level(const float *sT, float *sA, float *sX) {
-  constexpr int nb = 4 - L;
-  const int tid = threadIdx.x;
-  const int J = tid >> 6, rr = (tid >> 2) & 15, cg = tid & 3, I = J + L;
-  if (J < nb) {
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+// acc += P Q over 16 values of k: one row of P (stride-LT tile), four adjacent columns of Q
+// (row stride ldq).
+__device__ __forceinline__ void tri_term(float4 &acc, const float *P, const float *Q, int ldq) {
 #pragma unroll
-    for (int k = 0; k < L; ++k) {
-      const int K = J + k;
-      const float *tr = sT + (16 * I + rr) * LT + 16 * K;
-      const float *ac = sA + (16 * K) * LT + 16 * J + 4 * cg;
+  for (int m4 = 0; m4 < 4; ++m4) {
+    const float4 t4 = *reinterpret_cast<const float4 *>(P + 4 * m4);
+    const float tv[4] = {t4.x, t4.y, t4.z, t4.w};
 #pragma unroll
-      for (int m4 = 0; m4 < 4; ++m4) {
-        const float4 t4 = *reinterpret_cast<const float4 *>(tr + 4 * m4);
-        const float tv[4] = {t4.x, t4.y, t4.z, t4.w};
-#pragma unroll
-        for (int mm = 0; mm < 4; ++mm) {
-          const float4 a4 = *reinterpret_cast<const float4 *>(ac + (4 * m4 + mm) * LT);
-          acc.x += tv[mm] * a4.x;
-          acc.y += tv[mm] * a4.y;
-          acc.z += tv[mm] * a4.z;
-          acc.w += tv[mm] * a4.w;
-        }
-      }
+    for (int mm = 0; mm < 4; ++mm) {
+      const float4 a4 = *reinterpret_cast<const float4 *>(Q + (4 * m4 + mm) * ldq);
+      acc.x += tv[mm] * a4.x;
+      acc.y += tv[mm] * a4.y;
+      acc.z += tv[mm] * a4.z;
+      acc.w += tv[mm] * a4.w;
     }
-    *reinterpret_cast<float4 *>(sX + J * 256 + rr * 16 + 4 * cg) = acc;
   }
-  __syncthreads();
-  if (J < nb) {
-    const float *dr = sA + (16 * I + rr) * LT + 16 * I;
-    const float *xc = sX + J * 256 + 4 * cg;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int m4 = 0; m4 < 4; ++m4) {
-      const float4 d4 = *reinterpret_cast<const float4 *>(dr + 4 * m4);
-      const float dv[4] = {d4.x, d4.y, d4.z, d4.w};
-#pragma unroll
-      for (int mm = 0; mm < 4; ++mm) {
-        const float4 x4 = *reinterpret_cast<const float4 *>(xc + (4 * m4 + mm) * 16);
-        acc.x += dv[mm] * x4.x;
-        acc.y += dv[mm] * x4.y;
-        acc.z += dv[mm] * x4.z;
-        acc.w += dv[mm] * x4.w;
-      }
-    }
-    *reinterpret_cast<float4 *>(sA + (16 * I + rr) * LT + 16 * J + 4 * cg) =
-        make_float4(-acc.x, -acc.y, -acc.z, -acc.w);
-  }
-  __syncthreads();
 }
 
 // A = (I + T)^-1 for a strictly lower triangular 64 x 64 fp32 T (row stride
 // LT, zero on and above the diagonal), by 16 x 16 blocks, with 512 threads:
 // diagonal blocks D_I = (I + T_II)^-1 by column substitution (rows across a
-// half-warp), then A_IJ = -D_I sum_{K=J}^{I-1} T_IK A_KJ level by level
-// (I - J = 1, 2, 3).  sX holds 3 x 256 floats of scratch.  Entries of A above
+// half-warp), then A_IJ = -D_I sum_{K=J}^{I-1} T_IK A_KJ level by level (I - J = 1, 2, 3):
+// 64 threads per off-diagonal block, one per (row, 4 columns), which add each term
+// as soon as its A_KJ exists, so that only the last term of a level waits for the
+// level before (B1 H12 T32768 isotropic forward, this and the barriers around the output store:
+// see k_fused_fwd).  sX holds 3 x 256 floats of scratch.  Entries of A above
 // the diagonal are left unwritten except inside the diagonal blocks (zero).
 // Contains block-wide barriers; every thread of the CTA must call it.
 __device__ __forceinline__ void tri_inverse64(const float *sT, float *sA, float *sX) {
@@ -193,10 +160,26 @@ __device__ __forceinline__ void tri_inverse64(const float *sT, float *sA, float 
     sA[(o0 + rr) * LT + o0 + cl + 1] = x1;
   }
   __syncthreads();
-  // off-diagonal levels, each with its K sum fully unrolled
-  tri_inverse_level<1>(sT, sA, sX);
-  tri_inverse_level<2>(sT, sA, sX);
-  tri_inverse_level<3>(sT, sA, sX);
+  // blocks in the order of their levels: (1,0) (2,1) (3,2) | (2,0) (3,1) | (3,0)
+  const int blk = tid >> 6, lvl = blk < 3 ? 1 : blk < 5 ? 2 : 3;
+  const int J = blk < 3 ? blk : blk < 5 ? blk - 3 : 0, I = J + lvl;
+  const int rr = (tid >> 2) & 15, c4 = 4 * (tid & 3);
+  const float *tr = sT + (16 * I + rr) * LT + 16 * J, *ac = sA + 16 * J * LT + 16 * J + c4;
+  float *xb = sX + J * 256 + c4;
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (blk < 6) tri_term(acc, tr, ac, LT);
+#pragma unroll
+  for (int l = 1; l <= 3; ++l) {
+    if (blk < 6 && lvl == l) *reinterpret_cast<float4 *>(xb + rr * 16) = acc;
+    __syncthreads();
+    if (blk < 6 && lvl == l) {
+      float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+      tri_term(d, sA + (16 * I + rr) * LT + 16 * I, xb, 16);
+      *reinterpret_cast<float4 *>(sA + (16 * I + rr) * LT + 16 * J + c4) = make_float4(-d.x, -d.y, -d.z, -d.w);
+    }
+    __syncthreads();
+    if (l < 3 && blk < 6 && lvl > l) tri_term(acc, tr + 16 * l, ac + 16 * l * LT, LT);
+  }
 }
 
 inline PFN_cuTensorMapEncodeTiled_v12000 encoder() {

@@ -235,19 +235,16 @@ __global__ void __launch_bounds__(FT, 1)
   }
   // uncertainty carry (diag: one value per channel)
   if (V == 0 && tid < D) s_p[tid] = a.p0 ? a.p0[(size_t)bh * D + tid] : 1.f;
-  // per-token scalars of the next chunk, prefetched into registers
-  float nr = 1.f, nom = 0.f, ng = 0.f;
+  // per-token inputs of the next chunk, prefetched into registers and converted when they are
+  // used (a conversion here would wait for the loads)
+  __nv_bfloat16 nz = __float2bfloat16_rn(0.f), ny = nz, nx = nz;
   auto load_scalars = [&](int c) {
-    if (tid < CM) {
-      const int t = c * CM + tid;
-      nr = 1.f; nom = 0.f; ng = 0.f;
-      if (c < NC && t < a.T) {
-        const size_t th = tok_index(a, b, t, h);
-        nr = gate_r(G, a.rmin, ld<__nv_bfloat16>(a.r, th));
-        if (V == 1) {
-          nom = gate_omega(G, ld<__nv_bfloat16>(a.omega, th));
-          if (!a.pcd) ng = gate_logalpha(G, ld<__nv_bfloat16>(a.g, th));
-        }
+    if (tid < CM && c < NC) {
+      const size_t th = tok_index(a, b, min(c * CM + tid, a.T - 1), h);
+      nz = static_cast<const __nv_bfloat16 *>(a.r)[th];
+      if (V == 1) {
+        ny = static_cast<const __nv_bfloat16 *>(a.omega)[th];
+        if (!a.pcd) nx = static_cast<const __nv_bfloat16 *>(a.g)[th];
       }
     }
   };
@@ -271,12 +268,16 @@ __global__ void __launch_bounds__(FT, 1)
   for (int c = 0; c < NC && ok; ++c) {
     // ---- [1] raw tiles and per-token scalars of this chunk
     if (tid < CM) {
+      const bool live = c * CM + tid < a.T;
+      const float nr = live ? gate_r(G, a.rmin, __bfloat162float(nz)) : 1.f;
       s_r[tid] = nr;
       s_ri[tid] = 1.f / nr;
-      s_om[tid] = nom;
-      s_gs[tid] = ng;
+      s_om[tid] = V == 1 && live ? gate_omega(G, __bfloat162float(ny)) : 0.f;
+      s_gs[tid] = V == 1 && !a.pcd && live ? gate_logalpha(G, __bfloat162float(nx)) : 0.f;
     }
-    if (io) bulk_wait_read();  // O staging and the saved S image have been read
+    // the O staging tiles (fs, a2) and the saved S image are written again from [2] on, by the
+    // isotropic KDN with one decay per head only from [5] on: that one waits later
+    if (io && !SD && V == 1) bulk_wait_read();
     if (P.save_p && tid < D)
       P.save_p[((size_t)bh * NC + c) * D + tid] = (V == 0) ? s_p[tid] : s_b[0];
     unsigned char *ctx = P.save_S ? P.save_S + ((size_t)bh * NC + c) * kCtxBytes : nullptr;
@@ -316,8 +317,8 @@ __global__ void __launch_bounds__(FT, 1)
           uk[j] = a.mu * kk * kk * s_ri[t0 + j];
         }
         // a quarter's summary is read by the later quarters only: the last one skips it
+        float m00 = 1.f, m01 = 0.f, m10 = 0.f, m11 = 1.f, eq = 1.f;
         if (qq < 3) {
-          float m00 = 1.f, m01 = 0.f, m10 = 0.f, m11 = 1.f, eq = 1.f;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const float a2_ = al[j] * al[j], ua2 = uk[j] * a2_, d1 = 1.f + uk[j] * w[j];
@@ -330,6 +331,10 @@ __global__ void __launch_bounds__(FT, 1)
               m00 *= sc; m01 *= sc; m10 *= sc; m11 *= sc;
             }
           }
+        }
+        if (io) bulk_wait_read();  // the previous chunk's stores, beside the products above
+        __syncthreads();
+        if (qq < 3) {
           float *mine = sQ + (qq * D + i) * 5;
           mine[0] = m00; mine[1] = m01; mine[2] = m10; mine[3] = m11; mine[4] = eq;
         }
@@ -566,6 +571,7 @@ __global__ void __launch_bounds__(FT, 1)
       }
       commit_if(lead, bar_mma);
     }
+    if (SD && io) bulk_wait_read();  // the previous chunk's stores, and this chunk's per-token values
     // V -> fp16 in place while MMA-T runs (the tile arrived during the previous chunk);
     // on a timeout the MMA is still waited for before leaving
     const bool v_ok = __syncthreads_and(mbar_wait(bar_v, c & 1, kWaitIters));
@@ -862,7 +868,9 @@ __global__ void __launch_bounds__(FT, 1)
       }
     }
     fence_proxy_async();
+    tc_fence_before();
     __syncthreads();
+    tc_fence_after();
     if (io && P.write_o) {
       const unsigned char *stg = reinterpret_cast<const unsigned char *>(fs);
       const int nbox = a.odt == KDN_BF16 ? 2 : 4, bw = a.odt == KDN_BF16 ? 64 : 32;
@@ -871,9 +879,6 @@ __global__ void __launch_bounds__(FT, 1)
         for (int bx = 0; bx < 2; ++bx) tma_store_4d(&mo2, a2 + bx * 8192, bx * 64, h, c * CM, b);
       bulk_commit();
     }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
   }
 
   if (ok) {
