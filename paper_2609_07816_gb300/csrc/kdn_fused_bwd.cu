@@ -98,7 +98,8 @@ static_assert(O_AB + 8 * KB == O_DT, "gamma's first half spans the A bf16 and dT
 constexpr int OFF_SM = BUF_END;
 constexpr int SMALL_FLOATS = 64 * 18 + 256 * 2 + 128 * 2 + 16;
 constexpr int OFF_BAR = OFF_SM + SMALL_FLOATS * 4;
-constexpr int SMEM_BYTES = OFF_BAR + 64 + 1024;  // + alignment slack
+constexpr int OFF_NX = OFF_BAR + 64;  // next chunk's per-token values: [5][64], then gamma [64] (SD)
+constexpr int SMEM_BYTES = OFF_NX + 1536 + 1024;  // + alignment slack
 static_assert(SMEM_BYTES <= 232448, "shared memory");
 static_assert(O_AQ + 8 * KB <= O_WN && O_XT + 8 * KB <= O_RH, "map");
 
@@ -172,12 +173,12 @@ __global__ void __launch_bounds__(BT, 1)
   const float tau = a.tau, mu = a.mu;
   const bool pcd = (V == 0) || a.pcd;
 
-  if (tid == 0) {
-    mbar_init(bar_a, 1);
-    mbar_init(bar_b, 1);
+  if (tid == 0) {  // arrivals: one per issuing thread
+    mbar_init(bar_a, V == 0 ? 11 : SD ? 11 : 10);
+    mbar_init(bar_b, V == 0 ? 2 : 4);
     mbar_init(bar_mma, 1);
-    if (WT) mbar_init(bar_w, 1);
-    if (V == 0) mbar_init(bar_g, 1);
+    if (WT) mbar_init(bar_w, 2);
+    if (V == 0) mbar_init(bar_g, 3);
     fence_mbar_init();
     prefetch_tmap(&mq);
     prefetch_tmap(&mk);
@@ -198,48 +199,86 @@ __global__ void __launch_bounds__(BT, 1)
   const uint32_t X0 = tb + 256, X1 = tb + 320, X2 = tb + 384, X3 = tb + 448;
   const uint32_t lane_base = (uint32_t)(32 * wq) << 16;
 
-  // loads of chunk c on bar_a: the context record (S_in, R, -W, A_qk, A; issued as
-  // soon as their buffers free up) and the raw k, q, g, omega tiles (issued once the
-  // previous chunk is done; the one expect_tx covers both groups); bar_b <- dO (isotropic: and v)
-  // (diagonal KDN: the context's Y in place of v)
-  const uint32_t kBytesA = 81920u + 16384u * 2 + (V == 0 ? 16384u : 0u);
+  // loads of chunk c on bar_a: the context record (S_in, R, -W, A_qk, A, the per-token values;
+  // issued as soon as their buffers free up) and the raw k, q tiles (issued once the
+  // previous chunk is done); bar_b <- dO (isotropic: and v; diagonal KDN: the context's Y in
+  // place of v).  The copies are spread over lane 0 of the warps, each arriving with its own
+  // bytes: one thread issuing them all holds the whole CTA up.
+  float *n_tok = reinterpret_cast<float *>(sm + OFF_NX), *n_gm = n_tok + 5 * CM;
   auto issue_a_ctx = [&](int c) {
     const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * P.rec;
-    mbar_expect_tx(bar_a, kBytesA);
-    bulk_g2s(sin, rec + kCtxS, 32768, bar_a);
-    bulk_g2s(sm + O_RH, rec + kCtxR, 16384, bar_a);
-    bulk_g2s(sm + O_WN, rec + kCtxW, 16384, bar_a);
-    bulk_g2s(sm + O_AQ, rec + kCtxAqk, 8192, bar_a);
-    bulk_g2s(sm + O_AH, rec + kCtxA, 8192, bar_a);
-    if (V == 0) bulk_g2s(rv, rec + kCtxY, 16384, bar_a);
+    switch (lane == 0 ? warp : -1) {
+      case 0: mbar_expect_tx(bar_a, 32768); bulk_g2s(sin, rec + kCtxS, 32768, bar_a); break;
+      case 1:
+        if (DVT) bulk_wait_read();  // the dv tile has left the R buffer (this thread stored it)
+        mbar_expect_tx(bar_a, 16384);
+        bulk_g2s(sm + O_RH, rec + kCtxR, 16384, bar_a);
+        break;
+      case 2: mbar_expect_tx(bar_a, 16384); bulk_g2s(sm + O_WN, rec + kCtxW, 16384, bar_a); break;
+      case 3: mbar_expect_tx(bar_a, 8192); bulk_g2s(sm + O_AQ, rec + kCtxAqk, 8192, bar_a); break;
+      case 4: mbar_expect_tx(bar_a, 8192); bulk_g2s(sm + O_AH, rec + kCtxA, 8192, bar_a); break;
+      case 5: mbar_expect_tx(bar_a, 1280); bulk_g2s(n_tok, rec + kCtxTok, 1280, bar_a); break;
+      case 6:
+        if (V == 0) {
+          mbar_expect_tx(bar_a, 16384);
+          bulk_g2s(rv, rec + kCtxY, 16384, bar_a);
+        } else if (SD) {
+          mbar_expect_tx(bar_a, 256);
+          bulk_g2s(n_gm, rec + kCtxGa, 256, bar_a);
+        }
+        break;
+    }
   };
   auto issue_a_raw = [&](int c) {
-    for (int s = 0; s < 2; ++s) {
-      tma_load_4d(rkq + s * 16384, &mk, bar_a, 64 * s, h, c * CM, b);
-      tma_load_4d(rkq + s * 16384 + 8192, &mq, bar_a, 64 * s, h, c * CM, b);
+    switch (lane == 0 ? warp : -1) {
+      case 7: mbar_expect_tx(bar_a, 8192); tma_load_4d(rkq, &mk, bar_a, 0, h, c * CM, b); break;
+      case 8: mbar_expect_tx(bar_a, 8192); tma_load_4d(rkq + 8192, &mq, bar_a, 0, h, c * CM, b); break;
+      case 9: mbar_expect_tx(bar_a, 8192); tma_load_4d(rkq + 16384, &mk, bar_a, 64, h, c * CM, b); break;
+      case 10: mbar_expect_tx(bar_a, 8192); tma_load_4d(rkq + 24576, &mq, bar_a, 64, h, c * CM, b); break;
     }
   };
   auto issue_b_do = [&](int c) {
-    mbar_expect_tx(bar_b, V == 0 ? 16384 : 32768);  // (isotropic: and v)
-    for (int s = 0; s < 2; ++s) tma_load_4d(rdo + s * 8192, &mdo, bar_b, 64 * s, h, c * CM, b);
+    if (lane == 0 && (warp == 11 || warp == 12)) {
+      const int s = warp - 11;
+      mbar_expect_tx(bar_b, 8192);
+      tma_load_4d(rdo + s * 8192, &mdo, bar_b, 64 * s, h, c * CM, b);
+    }
   };
   auto issue_b_v = [&](int c) {
-    for (int s = 0; s < 2; ++s) tma_load_4d(rv + s * 8192, &mv, bar_b, 64 * s, h, c * CM, b);
+    if (lane == 0 && (warp == 13 || warp == 14)) {
+      const int s = warp - 13;
+      mbar_expect_tx(bar_b, 8192);
+      tma_load_4d(rv + s * 8192, &mv, bar_b, 64 * s, h, c * CM, b);
+    }
   };
   auto issue_g = [&](int c) {
     const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * P.rec;
-    mbar_expect_tx(bar_g, 65536);
-    bulk_g2s(sm + O_PHB, rec + kCtxPh, 32768, bar_g);
-    bulk_g2s(sm + O_GA0, rec + kCtxGa, 16384, bar_g);
-    bulk_g2s(sm + O_GA1, rec + kCtxGa + 16384, 16384, bar_g);
+    switch (lane == 0 ? warp : -1) {
+      case 2: mbar_expect_tx(bar_g, 32768); bulk_g2s(sm + O_PHB, rec + kCtxPh, 32768, bar_g); break;
+      case 3: mbar_expect_tx(bar_g, 16384); bulk_g2s(sm + O_GA0, rec + kCtxGa, 16384, bar_g); break;
+      case 4: mbar_expect_tx(bar_g, 16384); bulk_g2s(sm + O_GA1, rec + kCtxGa + 16384, 16384, bar_g); break;
+    }
   };
-  if (tid == 0) {
-    issue_a_ctx(NC - 1);
-    issue_a_raw(NC - 1);
-    issue_b_do(NC - 1);
-    if (V != 0) issue_b_v(NC - 1);
-    if (V == 0) issue_g(NC - 1);
-  }
+  // this chunk's omega logits for pass C (diagonal KDN with logit gates)
+  auto issue_w = [&](int c) {
+    if (WT && lane == 0 && (warp == 13 || warp == 14)) {
+      const int s = warp - 13;
+      mbar_expect_tx(bar_w, 8192);
+      tma_load_4d(sm + O_KT + s * 8192, &mw, bar_w, 64 * s, h, c * CM, b);
+    }
+  };
+  auto store_dv = [&](int c) {
+    if (DVT && tid == 32) {
+      tma_store_4d(&mdv, sm + O_DVS, 0, h, c * CM, b);
+      tma_store_4d(&mdv, sm + O_DVS + 8192, 64, h, c * CM, b);
+      bulk_commit();
+    }
+  };
+  issue_a_ctx(NC - 1);
+  issue_a_raw(NC - 1);
+  issue_b_do(NC - 1);
+  if (V != 0) issue_b_v(NC - 1);
+  if (V == 0) issue_g(NC - 1);
 
   // ---- cotangent scale lambda = 2^-e with max(|dO|, |dS_T|) * lambda in [1, 2)
   {
@@ -322,17 +361,9 @@ __global__ void __launch_bounds__(BT, 1)
 
   uint32_t mma_phase = 0;
   bool ok = true;
-  // One thread polls the MMA-completion barrier; the CTA barrier then orders every
-  // thread's TMEM reads after it (each caller issues tcgen05.fence::after_thread_sync).
-  auto mma_wait = [&]() -> bool {
-    bool r = true;
-    if (tid == 0) r = mbar_wait(bar_mma, mma_phase & 1, kWaitIters);
-    ++mma_phase;
-    return __syncthreads_and(r);
-  };
-  // Diagonal KDN: every thread polls the MMA-completion barrier itself (no CTA barrier
-  // between the completion and the TMEM reads); the outcome is combined at the stage's
-  // closing barrier, so that every thread leaves the loop at the same point
+  // Every thread polls the MMA-completion barrier itself (no CTA barrier between the
+  // completion and the TMEM reads); the outcome is combined at the stage's closing barrier,
+  // so that every thread leaves the loop at the same point
   auto mma_poll = [&]() -> bool {
     const bool r = mbar_wait(bar_mma, mma_phase & 1, kWaitIters);
     ++mma_phase;
@@ -361,9 +392,8 @@ __global__ void __launch_bounds__(BT, 1)
   if (tid < CM) s_dmu[tid] = 0.f;  // ordered before use by the loop's barriers
   for (int it = 0; it < NC && ok; ++it) {
     const int c = NC - 1 - it;
-    // ---- [1] per-token scalars; the chunk's gains from the context the forward saved
-    //          (diagonal KDN: bulk copies issued at the end of the previous chunk, on
-    //          bar_g; isotropic: global loads issued before the wait for the tiles); raw tiles
+    // ---- [1] per-token scalars; the chunk's gains from the context the forward saved (bulk
+    //          copies; isotropic KDN with per-channel decay: global loads); raw tiles
     if (tid < CM) {
       // (with logit gates: and the chain factors sigmoid(z_t), sigmoid(y_t) of r and omega)
       const bool live = c * CM + tid < a.T;
@@ -375,19 +405,11 @@ __global__ void __launch_bounds__(BT, 1)
       s_fw[tid] = V == 1 && G && live ? sigmoid_f(__bfloat162float(ny)) : 1.f;
     }
     const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * P.rec;
-    float e16[16], ph16[16], tk[5];
-    {
-      // gamma [64][128] (SD: one value per token, [64]) of the isotropic KDN
-      const float *cga = reinterpret_cast<const float *>(rec + kCtxGa) + (SD ? t0 : t0 * D + ci);
-      const float *tok = reinterpret_cast<const float *>(rec + kCtxTok);
-      if (V != 0) {  // (the diagonal KDN's arrive in shared memory on bar_g)
+    float e16[16], ph16[16];
+    if (V != 0 && !SD) {  // gamma [64][128] of the isotropic KDN with per-channel decay
+      const float *cga = reinterpret_cast<const float *>(rec + kCtxGa) + t0 * D + ci;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) e16[j] = cga[SD ? j : j * D];
-      }
-      if (tid < CM) {
-#pragma unroll
-        for (int m = 0; m < (V == 0 ? 1 : 5); ++m) tk[m] = tok[64 * m + tid];
-      }
+      for (int j = 0; j < 16; ++j) e16[j] = cga[j * D];
     }
     ok = __syncthreads_and(mbar_wait(bar_a, it & 1, kWaitIters) &&
                            (V != 0 || mbar_wait(bar_g, it & 1, kWaitIters)));
@@ -409,6 +431,10 @@ __global__ void __launch_bounds__(BT, 1)
         }
         tmem_st16(TPH + lane_base + t0, ph16);
       }
+      if (SD) {  // one gamma per token
+#pragma unroll
+        for (int j = 0; j < 16; ++j) e16[j] = n_gm[t0 + j];
+      }
       tmem_st16(TGM + lane_base + t0, e16);
       if (qq == 3) {
         s_gC[ci] = e16[15];
@@ -420,14 +446,14 @@ __global__ void __launch_bounds__(BT, 1)
       }
       if (tid < CM) {
         if (V == 0) {
-          s_s[tid] = tk[0];
-          s_si[tid] = 1.f / tk[0];
+          s_s[tid] = n_tok[tid];
+          s_si[tid] = 1.f / n_tok[tid];
         } else {
-          s_x[tid] = tk[0];
-          s_n2[tid] = tk[1];
-          s_a[tid] = tk[2];
-          s_bh[tid] = tk[3];
-          s_bp[tid] = tk[4];
+          s_x[tid] = n_tok[tid];
+          s_n2[tid] = n_tok[CM + tid];
+          s_a[tid] = n_tok[2 * CM + tid];
+          s_bh[tid] = n_tok[3 * CM + tid];
+          s_bp[tid] = n_tok[4 * CM + tid];
         }
       }
       tmem_st_wait();
@@ -506,12 +532,7 @@ __global__ void __launch_bounds__(BT, 1)
       }
       commit_if(lead, bar_mma);
     }
-    bool mm_ok = true;
-    if constexpr (V == 0) {
-      mm_ok = mma_poll();
-    } else {
-      if (!(ok = mma_wait())) break;
-    }
+    bool mm_ok = mma_poll();
     tc_fence_after();
     // ---- [11] dR^T -> fp16 [j][t] (and its fp16 remainder); dA_qk^T (masked to s <= t) -> hi/lo bf16 [s][t];
     //           X0 <- gamma_C dK_tail^T (start of dKk^T) and its dgamma_C part; Qbar fp16
@@ -678,11 +699,8 @@ __global__ void __launch_bounds__(BT, 1)
       }
       mm_ok = mma_poll();
       tc_fence_after();
-      if (tid == 0 && c > 0) issue_b_do(c - 1);  // the dO / Qbar lo buffer is free
-      if (WT && tid == 0) {  // this chunk's omega logits for pass C, into the dR^T buffer (free
-        mbar_expect_tx(bar_w, 16384);  // until [3] of the next chunk)
-        for (int s = 0; s < 2; ++s) tma_load_4d(sm + O_KT + s * 8192, &mw, bar_w, 64 * s, h, c * CM, b);
-      }
+      if (c > 0) issue_b_do(c - 1);  // the dO / Qbar lo buffer is free
+      issue_w(c);  // into the dR^T buffer (free until [3] of the next chunk)
       // ---- [15] dV^T -> dv (bf16: into the dR^T lo tile, free since B7, in the layout of
       //           the TMA box, then two TMA stores; rows past T are clipped by the map);
       //           X = A^T dA -> fp16 [r][s]
@@ -715,11 +733,7 @@ __global__ void __launch_bounds__(BT, 1)
         ok = false;
         break;
       }
-      if (DVT && tid == 0) {
-        tma_store_4d(&mdv, sm + O_DVS, 0, h, c * CM, b);
-        tma_store_4d(&mdv, sm + O_DVS + 8192, 64, h, c * CM, b);
-        bulk_commit();
-      }
+      store_dv(c);
       // ---- [16] X1 = X A^T (fp16), so that dT = strict_lower(-A^T dA A^T);  B10a: X2 = (A^T dW)^T
       if (warp_u == 0) {
         tc_fence_after();
@@ -786,7 +800,7 @@ __global__ void __launch_bounds__(BT, 1)
         }
         commit_if(lead, bar_mma);
       }
-      if (!(ok = mma_wait())) break;
+      mm_ok = mma_poll();
       tc_fence_after();
       // ---- [13] second operand set: [Kbar; Qbar] hi (interleaved), Qbar lo, Kk hi / lo;
       //           B8b: X3 += (dA_qk Kk)^T;  B9a: X0 += (dA_qk^T Qbar)^T
@@ -809,7 +823,10 @@ __global__ void __launch_bounds__(BT, 1)
       }
       fence_proxy_async();
       tc_fence_before();
-      __syncthreads();
+      if (!__syncthreads_and(mm_ok)) {
+        ok = false;
+        break;
+      }
       if (SD && warp_u == 0) {  // raw K^T, Q^T (channel-major) against the scaled 64 x 64 partners
         tc_fence_after();
         const uint32_t lead = elect_one();
@@ -843,9 +860,9 @@ __global__ void __launch_bounds__(BT, 1)
         }
         commit_if(lead, bar_mma);
       }
-      if (!(ok = mma_wait())) break;
+      mm_ok = mma_poll();
       tc_fence_after();
-      if (tid == 0 && c > 0) issue_b_do(c - 1);  // dO / Qbar lo buffer is free
+      if (c > 0) issue_b_do(c - 1);  // dO / Qbar lo buffer is free
       // ---- [14] dW^T -> bf16 [i][t];  dV^T -> dv
       {
         const int j = 32 * wq + lane, tc0 = 16 * wg;
@@ -872,12 +889,11 @@ __global__ void __launch_bounds__(BT, 1)
       }
       fence_proxy_async();
       tc_fence_before();
-      __syncthreads();
-      if (DVT && tid == 0) {
-        tma_store_4d(&mdv, sm + O_DVS, 0, h, c * CM, b);
-        tma_store_4d(&mdv, sm + O_DVS + 8192, 64, h, c * CM, b);
-        bulk_commit();
+      if (!__syncthreads_and(mm_ok)) {
+        ok = false;
+        break;
       }
+      store_dv(c);
       // ---- [15] B6: X1 = dA^T = (dR V^T + dW Kbar^T)^T;  B10a: X2 = (A^T dW)^T
       if (warp_u == 0) {
         tc_fence_after();
@@ -896,13 +912,9 @@ __global__ void __launch_bounds__(BT, 1)
           umma_if(lead, X2, step(kdesc(sm + O_DWT), kk * 32), step(mdesc(sm + O_AB, 8192), kk * 2048), ib01, kk > 0);
         commit_if(lead, bar_mma);
       }
-      if (!(ok = mma_wait())) break;
+      mm_ok = mma_poll();
       tc_fence_after();
-      if (tid == 0 && c > 0) issue_b_v(c - 1);  // v buffer is free
-      if (WT && tid == 0) {  // this chunk's omega logits for pass C (B6 has read dR^T in O_KT,
-        mbar_expect_tx(bar_w, 16384);  // which is free until [3] of the next chunk)
-        for (int s = 0; s < 2; ++s) tma_load_4d(sm + O_KT + s * 8192, &mw, bar_w, 64 * s, h, c * CM, b);
-      }
+      if (c > 0) issue_b_v(c - 1);  // v buffer is free
       // ---- [16] dT = strict_lower(-A^T dA A^T): X = A^T dA, Y = X A^T (fp16)
       if (wq < 2) {
         const int s = 32 * wq + lane, tc0 = 16 * wg;
@@ -913,7 +925,10 @@ __global__ void __launch_bounds__(BT, 1)
       }
       fence_proxy_async();
       tc_fence_before();
-      __syncthreads();
+      if (!__syncthreads_and(mm_ok)) {
+        ok = false;
+        break;
+      }
       if (warp_u == 0) {
         tc_fence_after();
         const uint32_t lead = elect_one();
@@ -923,7 +938,7 @@ __global__ void __launch_bounds__(BT, 1)
           umma_if(lead, X1, step(mdesc(sm + O_AH, 8192), kk * 2048), step(kdesc(sm + O_DAT), kk * 32), id, kk > 0);
         commit_if(lead, bar_mma);
       }
-      if (!(ok = mma_wait())) break;
+      mm_ok = mma_poll();
       tc_fence_after();
       if (wq < 2) {
         const int r = 32 * wq + lane, tc0 = 16 * wg;
@@ -934,7 +949,10 @@ __global__ void __launch_bounds__(BT, 1)
       }
       fence_proxy_async();
       tc_fence_before();
-      __syncthreads();
+      if (!__syncthreads_and(mm_ok)) {
+        ok = false;
+        break;
+      }
       if (warp_u == 0) {
         tc_fence_after();
         const uint32_t lead = elect_one();
@@ -944,7 +962,7 @@ __global__ void __launch_bounds__(BT, 1)
           umma_if(lead, X1, step(kdesc(sm + O_XT), kk * 32), step(kdesc(sm + O_AH), kk * 32), id, kk > 0);
         commit_if(lead, bar_mma);
       }
-      if (!(ok = mma_wait())) break;
+      mm_ok = mma_poll();
       tc_fence_after();
       if (wq < 2) {
         const int r = 32 * wq + lane, tc0 = 16 * wg;
@@ -967,7 +985,10 @@ __global__ void __launch_bounds__(BT, 1)
       }
       fence_proxy_async();
       tc_fence_before();
-      __syncthreads();
+      if (!__syncthreads_and(mm_ok)) {
+        ok = false;
+        break;
+      }
       // ---- [17] B9b: X0 += (dT^T Kbar)^T;  B10b: X2 += (dT Kk)^T
       if (warp_u == 0) {
         tc_fence_after();
@@ -988,18 +1009,12 @@ __global__ void __launch_bounds__(BT, 1)
         commit_if(lead, bar_mma);
       }
     }
-    if constexpr (V == 0) {
-      mm_ok = mma_poll();
-    } else {
-      if (!(ok = mma_wait())) break;
-    }
+    mm_ok = mma_poll();
     tc_fence_after();
-    if (tid == 0 && c > 0) {
-      if (DVT) bulk_wait_read();  // the dv tile has left the R buffer
+    if (c > 0) {
       issue_a_ctx(c - 1);  // the context buffers are free
-      // phat, gamma and the token scalars of chunk c - 1 are read with plain loads at the
-      // top of its iteration: bring them into L2 now
-      bulk_prefetch_l2(rec - P.rec + kCtxPh, kCtxBytes - kCtxPh);
+      // phat and gamma of chunk c - 1, which are read later, into L2 now
+      if (tid == 480) bulk_prefetch_l2(rec - P.rec + kCtxPh, SD ? 256 : 65536);
     }
     // ---- [18] per channel (lane ci, tokens t0..t0+15): back through Gamma and the
     //           gain emission, then the uncertainty recursion backwards in time.
@@ -1026,7 +1041,7 @@ __global__ void __launch_bounds__(BT, 1)
         ok = false;
         break;
       }
-      if (tid == 0 && c > 0) issue_a_raw(c - 1);
+      if (c > 0) issue_a_raw(c - 1);
       // outputs of token t0 + j live at obase + j * ostride; nval tokens of the quarter are real
       const size_t ostride = (size_t)a.H * D;
       const size_t obase = tok_index(a, b, c * CM + t0, h) * D + ci;
@@ -1167,7 +1182,7 @@ __global__ void __launch_bounds__(BT, 1)
         __syncthreads();
         // every read of the dG scratch, the pass summaries and the omega logits is done:
         // the next chunk's phat and gamma may land over them
-        if (tid == 0 && c > 0) issue_g(c - 1);
+        if (c > 0) issue_g(c - 1);
         if (qq == 0) s_dp[ci] = dp;
         if (tid < CM) {
           const int tt = c * CM + tid;
@@ -1195,8 +1210,12 @@ __global__ void __launch_bounds__(BT, 1)
         q16[j] = raw_q(t0 + j);
       }
       fence_proxy_async();
-      __syncthreads();  // raw k, q are in registers: the next chunk's tiles may land
-      if (tid == 0 && c > 0) issue_a_raw(c - 1);
+      // raw k, q are in registers: the next chunk's tiles may land
+      if (!__syncthreads_and(mm_ok)) {
+        ok = false;
+        break;
+      }
+      if (c > 0) issue_a_raw(c - 1);
       const size_t ostride = (size_t)a.H * D;
       const size_t obase = tok_index(a, b, c * CM + t0, h) * D + ci;
       const int nval = min(16, a.T - (c * CM + t0));
@@ -1362,10 +1381,10 @@ __global__ void __launch_bounds__(BT, 1)
       for (int w = 0; w < CM; ++w) tot += s_dmu[w];
       a.dmu[bh] = tot * invl;
     }
-    if (DVT && tid == 0) bulk_wait_all();  // the last chunk's dv stores
+    if (DVT && tid == 32) bulk_wait_all();  // the last chunk's dv stores
   } else {
     if (tid == 0) atomicExch(a.status, (unsigned)KDN_ERR_TIMEOUT);
-    if (DVT && tid == 0) bulk_wait_all();
+    if (DVT && tid == 32) bulk_wait_all();
     // let copies already in flight land before the CTA's shared memory goes away
     if (tid == 0) {
       mbar_wait(bar_a, 0, kWaitIters);
