@@ -313,7 +313,8 @@ kdn_status_t kdn_noalloc_device_status(void *stream);
    descriptor when T > 0 (op 0 = kdn_*_fwd, 1 = kdn_*_bwd, 2 = kdn_*_decode_step,
    3 = kdn_*_fwd_save, 4 = kdn_*_bwd_saved, 5 = kdn_*_beta_eff; variant 0 = diagonal,
    1 = isotropic).  -1 for an invalid descriptor or op, or an op the descriptor
-   does not serve.
+   does not serve.  A backward is counted with every gradient asked for; the diagonal
+   backward with bf16 gradients and no state gradients may take one launch more.
    Calls with T = 0 launch at most one small fill kernel. */
 int kdn_kernel_launches(const kdn_desc_t *desc, int variant, int op);
 

@@ -1419,8 +1419,7 @@ size_t fused_saved_bytes(const Args &a) {
 size_t fused_ctx_record_bytes(const Args &a) { return split_bwd_context(a) ? kCtxSplitBytes : kCtxBytes; }
 
 kdn_status_t launch_fused_bwd_sweep(const Args &a, cudaStream_t s) {
-  // (a ragged length needs scratch in the workspace; without it the one-kernel sweep runs)
-  if (split_bwd_context(a) && (a.T % CM == 0 || a.split_ws)) return launch_split_bwd(a, a.T % CM == 0 ? nullptr : a.split_ws, s);
+  if (split_bwd_supported(a)) return launch_split_bwd(a, a.T % CM == 0 ? nullptr : a.split_ws, s);
   BwdParams P;
   P.a = a;
   P.rec = fused_ctx_record_bytes(a);

@@ -180,10 +180,11 @@ kdn_status_t launch_fused_bwd_sweep(const Args &a, cudaStream_t s);
 // per chunk the 128 float32 uncertainties entering it.
 size_t fused_saved_bytes(const Args &a);
 size_t fused_ctx_record_bytes(const Args &a);
-// Two-kernel backward of the Diagonal KDN (kdn_split_bwd.cu): whether the context of this
-// problem feeds it, the scratch it needs in the workspace (ragged lengths; otherwise its
-// scratch lies in the gradient buffers) and its launcher.
+// Two-kernel backward of the Diagonal KDN (kdn_split_bwd.cu): whether the context of these
+// sizes feeds it, whether it serves this call, the scratch it needs in the workspace (ragged
+// lengths; otherwise its scratch lies in the gradient buffers) and its launcher.
 bool split_bwd_context(const Args &a);
+bool split_bwd_supported(const Args &a);
 size_t split_bwd_workspace_bytes(const Args &a);
 kdn_status_t launch_split_bwd(const Args &a, char *ws, cudaStream_t s);
 

@@ -22,7 +22,8 @@
 // chunk's gradients there.  Ragged lengths use the workspace (a tile's rows are not
 // tokens, and rows past T do not exist in the gradients).
 //
-// Numerics are those of the one-kernel sweep: the same operand types (fp16 tiles, hi/lo
+// It serves bf16 gradients without state gradients (see split_bwd_supported).  Numerics are
+// those of the one-kernel sweep up to rounding: the same operand types (fp16 tiles, hi/lo
 // bf16 pairs where Gamma-scaled operands meet, fp16 pairs for dR in A^T dR), fp32
 // accumulators, dS fp32 across chunks, cotangents scaled by the same power of two.
 //
@@ -43,25 +44,23 @@ constexpr uint32_t kDpWait = 1u << 22;  // polls for the uncertainty cotangent o
 constexpr int kSms = 152;
 
 // Where a chunk's small values lie: rows of 256 bytes, one per token of the chunk.
-// Rows 0, 1: dgamma_C's dS part [128]; 2..5: dp [128] as (value, tag) pairs;
-// 6..9: dmu [128] as (value, tag) pairs; 10: lambda.
+// Rows 0, 1: dgamma_C's dS part [128]; 2..5: dp [128] as (value, tag) pairs; 6: lambda.
 struct Scratch {
   unsigned char *small;
-  size_t row;  // bytes from a head's row to the next head's
   int T;       // tokens of the scratch layout (a multiple of 64)
 };
 __device__ __forceinline__ unsigned char *small_row(const Scratch &s, const Args &a, int b, int h, int c, int n) {
-  return s.small + (((size_t)b * s.T + c * CM + n) * a.H + h) * s.row;
+  return s.small + (((size_t)b * s.T + c * CM + n) * a.H + h) * (2 * D);
 }
 __device__ __forceinline__ float *small_dgc(const Scratch &s, const Args &a, int b, int h, int c, int i) {
   return reinterpret_cast<float *>(small_row(s, a, b, h, c, i >> 6)) + (i & 63);
 }
-// (value, tag) slot of channel i; m: 0 dp, 1 dmu
-__device__ __forceinline__ uint2 *small_slot(const Scratch &s, const Args &a, int b, int h, int c, int m, int i) {
-  return reinterpret_cast<uint2 *>(small_row(s, a, b, h, c, 2 + 4 * m + (i >> 5))) + (i & 31);
+// (value, tag) slot of channel i's dp
+__device__ __forceinline__ uint2 *small_slot(const Scratch &s, const Args &a, int b, int h, int c, int i) {
+  return reinterpret_cast<uint2 *>(small_row(s, a, b, h, c, 2 + (i >> 5))) + (i & 31);
 }
 __device__ __forceinline__ float *small_lam(const Scratch &s, const Args &a, int b, int h, int c) {
-  return reinterpret_cast<float *>(small_row(s, a, b, h, c, 10));
+  return reinterpret_cast<float *>(small_row(s, a, b, h, c, 6));
 }
 // A slot is one 8-byte store and one 8-byte load: the value needs no other ordering.
 __device__ __forceinline__ void slot_put(uint2 *p, float v) {
@@ -238,7 +237,7 @@ __global__ void __launch_bounds__(BT, 1)
     }
     __syncthreads();
   }
-  const float lam = s_misc[0], invl = 1.f / lam;
+  const float lam = s_misc[0];
 
   const int i = 32 * wq + lane, j0 = 32 * wg;  // this thread's row and first column of dS
   for (int c0 = 0; c0 < 32; c0 += 16) {
@@ -334,8 +333,7 @@ __global__ void __launch_bounds__(BT, 1)
       const int ii = tid - 128;
       const float *sp = s_part + (it & 1) * 512 + ii;
       *small_dgc(P.s, a, b, h, c, ii) = (sp[0] + sp[D]) + (sp[2 * D] + sp[3 * D]);
-      *small_slot(P.s, a, b, h, c, 0, ii) = make_uint2(0u, 0u);
-      *small_slot(P.s, a, b, h, c, 1, ii) = make_uint2(0u, 0u);
+      *small_slot(P.s, a, b, h, c, ii) = make_uint2(0u, 0u);
       if (ii == 0) *small_lam(P.s, a, b, h, c) = lam;
     }
     // ---- [3] dR^T = XA + XB diag(1/s) -> fp16 hi + lo, [j][t]
@@ -380,20 +378,7 @@ __global__ void __launch_bounds__(BT, 1)
       bulk_commit();
     }
   }
-  if (ok) {
-    ok = mbar_wait(bar_s, (NC - 1) & 1, kWaitIters);
-    tc_fence_after();
-    if (a.dS0) {
-      for (int c0 = 0; c0 < 32; c0 += 16) {
-        float v[16];
-        tmem_ld16(TS + lane_base + j0 + c0, v);
-        float4 *dst = reinterpret_cast<float4 *>(a.dS0 + ((size_t)bh * D + i) * D + j0 + c0);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          dst[u] = make_float4(v[4 * u] * invl, v[4 * u + 1] * invl, v[4 * u + 2] * invl, v[4 * u + 3] * invl);
-      }
-    }
-  }
+  if (ok) ok = mbar_wait(bar_s, (NC - 1) & 1, kWaitIters);
   if (!__syncthreads_and(ok)) {
     if (tid == 0) {
       atomicExch(a.status, (unsigned)KDN_ERR_TIMEOUT);
@@ -434,8 +419,7 @@ constexpr int OFF_BAR = OFF_SM + SMALL_FLOATS * 4;
 constexpr int CHUNK_SMEM = OFF_BAR + 80 + 1024;
 static_assert(CHUNK_SMEM <= 232448, "shared memory");
 
-// OBF: bf16 gradients; G: logit gates; DM: dmu is wanted
-template <int OBF, int G, int DM>
+template <int G>  // G: logit gates
 __global__ void __launch_bounds__(BT, 1)
     k_bwd_chunk(const __grid_constant__ CUtensorMap mq, const __grid_constant__ CUtensorMap mk,
                 const __grid_constant__ CUtensorMap mdo, const __grid_constant__ CUtensorMap mw,
@@ -540,7 +524,7 @@ __global__ void __launch_bounds__(BT, 1)
       case 5: mbar_expect_tx(bar_a, 8192); tma_load_4d(sm + O_KT, &m3, bar_a, 0, o.h, t, o.b); break;
       case 6: mbar_expect_tx(bar_a, 8192); tma_load_4d(sm + O_KT + 8192, &m3, bar_a, 64, o.h, t, o.b); break;
       case 7:
-        if (OBF) bulk_wait_read();  // the dv tile has left the R buffer
+        bulk_wait_read();  // the dv tile has left the R buffer
         mbar_expect_tx(bar_a, 16384);
         bulk_g2s(sm + O_RH, o.rec + kCtxR, 16384, bar_a);
         break;
@@ -717,18 +701,12 @@ __global__ void __launch_bounds__(BT, 1)
       sm16(sm + O_RV, chunk_off(j, tc0 >> 3)) = pack_bf8(v);
       sm16(sm + O_RV, chunk_off(j, (tc0 >> 3) + 1)) = pack_bf8(v + 8);
       tmem_ld16(X5 + lane_base + tc0, v);
-      if constexpr (OBF) {  // into the R tile, in the layout of the TMA box
+      {  // into the R tile, in the layout of the TMA box
         unsigned char *slab = sm + O_RH + (j >> 6) * 8192;
 #pragma unroll
         for (int u = 0; u < 16; ++u)
           *reinterpret_cast<__nv_bfloat16 *>(slab + chunk_off(tc0 + u, (j & 63) >> 3) + 2 * (j & 7)) =
               __float2bfloat16_rn(v[u] * invl);
-      } else {
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-          const int t = c * CM + tc0 + u;
-          if (t < a.T) st_grad<OBF>(a.dv_, tok_index(a, b, t, h) * D + j, v[u] * invl);
-        }
       }
       if (wq < 2) {
         tmem_ld16(X4 + lane_base + tc0, v);
@@ -808,7 +786,7 @@ __global__ void __launch_bounds__(BT, 1)
         umma_if(lead, X2, step(w0, kk * 32), step(ab, kk * 2048), id01, kk > 0);
       }
       commit_if(lead, bar_mma);
-    } else if (OBF && tid == 224) {
+    } else if (tid == 224) {
       tma_store_4d(&mdv, sm + O_RH, 0, h, c * CM, b);
       tma_store_4d(&mdv, sm + O_RH + 8192, 64, h, c * CM, b);
       bulk_commit();
@@ -887,7 +865,7 @@ __global__ void __launch_bounds__(BT, 1)
     // every tile but k, q has been read: the next chunk's may land
     if (on.j < njobs) issue_a(on);
     if (tid < 64 && c < NC - 1)  // dp leaving this chunk, if the next chunk's job has handed it on already
-      cp16(s_red2 + 4 * tid, small_slot(P.s, a, b, h, c, 0, 2 * tid));
+      cp16(s_red2 + 4 * tid, small_slot(P.s, a, b, h, c, 2 * tid));
     if (on.j < njobs) load_small(on);
     cp_commit();
     // ---- per channel (lane ci, tokens t0..t0+15): back through Gamma and the gain emission,
@@ -898,11 +876,11 @@ __global__ void __launch_bounds__(BT, 1)
     //      gamma are read again from TMEM, eight tokens at a time: few live registers
     {
       const uint32_t XE = X5 + lane_base;  // columns qq: sum of dG; 4 + qq: dgamma_C part;
-                                           // 8 + 4 qq ..: A, B (and dmu's) of the quarter
+                                           // 8 + 2 qq ..: A, B of the quarter
       const size_t ostride = (size_t)a.H * D;
       const size_t obase = tok_index(a, b, c * CM + t0, h) * D + ci;
       const int nval = min(16, a.T - (c * CM + t0));
-      auto out = [&](void *p, int j, float x) { st_grad<OBF>(p, obase + (size_t)j * ostride, x); };
+      auto out = [&](void *p, int j, float x) { st_grad<1>(p, obase + (size_t)j * ostride, x); };
       float k16[16];
       // pass A: dq, dG, the ds_t partial sums and the ds-free parts of dphat and dk
       {
@@ -952,9 +930,9 @@ __global__ void __launch_bounds__(BT, 1)
         p_prev = __fdividef(pp, 1.f + mu * kprev * kprev * s_ri[t0 - 1] * pp);
       }
       // pass B: per-token coefficients of dp_{t-1} = a_t dp_t + b_t and the quarter's
-      //         composition dp_before = A dp_after + B (and dmu = dmA dp_after + dmB)
+      //         composition dp_before = A dp_after + B
       {
-        float A = 1.f, Bv = 0.f, dmA = 0.f, dmB = 0.f;
+        float A = 1.f, Bv = 0.f;
 #pragma unroll
         for (int h8 = 1; h8 >= 0; --h8) {
           float c1[8], p8[8], g8[8], a2v[8], rdv[8], gp = ga_prev;
@@ -969,11 +947,6 @@ __global__ void __launch_bounds__(BT, 1)
             const float al = __fdividef(g8[u], u > 0 ? g8[u - 1] : gp), al2 = al * al;
             const float rd = __fdividef(1.f, 1.f + mu * kk * kk * s_ri[t] * p8[u]);
             const float dphl = c1[u] + s_ds[t] * kk * kk;
-            if (DM) {  // dmu gains du k^2 / r with du = -dp_t p_t^2
-              const float pt = p8[u] * rd, w = -pt * pt * kk * kk * s_ri[t];
-              dmA = fmaf(w, A, dmA);
-              dmB = fmaf(w, Bv, dmB);
-            }
             const float aj = al2 * rd * rd;
             Bv = aj * Bv + al2 * dphl;
             A = aj * A;
@@ -985,12 +958,8 @@ __global__ void __launch_bounds__(BT, 1)
           tmem_st8(X3 + lane_base + t0 + 8 * h8, rdv);
           tmem_st8(X2 + lane_base + t0 + 8 * h8, c1);
         }
-        tmem_st1(XE + 8 + 4 * qq, A);
-        tmem_st1(XE + 9 + 4 * qq, Bv);
-        if (DM) {
-          tmem_st1(XE + 10 + 4 * qq, dmA);
-          tmem_st1(XE + 11 + 4 * qq, dmB);
-        }
+        tmem_st1(XE + 8 + 2 * qq, A);
+        tmem_st1(XE + 9 + 2 * qq, Bv);
       }
       tmem_st_wait();
       tc_fence_before();
@@ -999,47 +968,35 @@ __global__ void __launch_bounds__(BT, 1)
       if (G) mm_ok = mbar_wait(bar_w, it & 1, kWaitIters);  // the omega-logit tile has landed
       __syncthreads();
       tc_fence_after();
-      float ex[16];  // the quarters' maps of this channel
-      tmem_ld16(XE + 8, ex);
+      float ex[8];  // the quarters' maps of this channel
+      tmem_ld8(XE + 8, ex);
       // dp leaving the chunk: from the next chunk's job (thread i: channel i), handed on at once
       if (tid < D) {
-        float dp = 0.f, dm = 0.f;
+        float dp = 0.f;
         if (c == NC - 1) {
           if (a.dpT) dp = lam * a.dpT[((size_t)b * a.H + h) * D + tid];
         } else {
           const uint2 early = reinterpret_cast<const uint2 *>(s_red2)[tid];
           if (early.y == 1u) dp = __uint_as_float(early.x);
-          else mm_ok = slot_get(small_slot(P.s, a, b, h, c, 0, tid), &dp) && mm_ok;
-          if (DM) mm_ok = slot_get(small_slot(P.s, a, b, h, c, 1, tid), &dm) && mm_ok;
+          else mm_ok = slot_get(small_slot(P.s, a, b, h, c, tid), &dp) && mm_ok;
         }
         s_dp[tid] = dp;
-#pragma unroll
-        for (int q2 = 3; q2 >= 0; --q2) {
-          if (DM) dm += fmaf(ex[4 * q2 + 2], dp, ex[4 * q2 + 3]);
-          dp = fmaf(ex[4 * q2], dp, ex[4 * q2 + 1]);
-        }
         if (c > 0) {
-          slot_put(small_slot(P.s, a, b, h, c - 1, 0, tid), dp);
-          if (DM) slot_put(small_slot(P.s, a, b, h, c - 1, 1, tid), dm);
-        } else {
-          if (a.dp0) a.dp0[((size_t)b * a.H + h) * D + tid] = dp * invl;
-          if (DM) s_red[tid] = dm;
+#pragma unroll
+          for (int q2 = 3; q2 >= 0; --q2) dp = fmaf(ex[2 * q2], dp, ex[2 * q2 + 1]);
+          slot_put(small_slot(P.s, a, b, h, c - 1, tid), dp);
         }
       }
       if (!__syncthreads_and(mm_ok)) {
         ok = false;
         break;
       }
-      if (DM && c == 0 && warp == 0) {  // dL/dmu of this sequence
-        const float tot = warp_sum((s_red[lane] + s_red[32 + lane]) + (s_red[64 + lane] + s_red[96 + lane]));
-        if (lane == 0) a.dmu[(size_t)b * a.H + h] = tot * invl;
-      }
       // pass C: the recursion backwards through this quarter's tokens
       {
         float dp = s_dp[ci];
 #pragma unroll
         for (int q2 = 3; q2 > 0; --q2)
-          if (q2 > qq) dp = fmaf(ex[4 * q2], dp, ex[4 * q2 + 1]);
+          if (q2 > qq) dp = fmaf(ex[2 * q2], dp, ex[2 * q2 + 1]);
         float es[8];  // the quarters' sums of dG, then of dgamma_C
         tmem_ld8(XE, es);
         // dG_63 gains dgamma_C gamma_C; it lies in every suffix
@@ -1095,7 +1052,7 @@ __global__ void __launch_bounds__(BT, 1)
         if (tt < a.T) {
           // the part of dr_t through u = mu k^2 / r: -sum_i du mu k^2 / r^2
           const float dru = (s_red2[tid] + s_red2[64 + tid]) + (s_red2[128 + tid] + s_red2[192 + tid]);
-          st_grad<OBF>(a.dr, tok_index(a, b, tt, h), (s_ds[tid] + dru) * (G ? s_fr[tid] : 1.f) * invl);
+          st_grad<1>(a.dr, tok_index(a, b, tt, h), (s_ds[tid] + dru) * (G ? s_fr[tid] : 1.f) * invl);
         }
       }
     }
@@ -1110,42 +1067,38 @@ __global__ void __launch_bounds__(BT, 1)
       }
     }
   }
-  if (OBF && tid == 224) bulk_wait_all();  // the last chunk's dv stores
+  if (tid == 224) bulk_wait_all();  // the last chunk's dv stores
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tb, 512);
 }
 
-// A [B, T, H, 128] tensor of 16-bit elements whose (b, t, h) rows lie `row` bytes apart; the
-// box and swizzle of make_map.
-bool make_scratch_map(CUtensorMap *m, void *ptr, const Args &a, int T, size_t row) {
-  auto enc = encoder();
-  if (!enc) return false;
-  cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)a.H, (cuuint64_t)T, (cuuint64_t)a.B};
-  cuuint64_t strides[3] = {(cuuint64_t)row, (cuuint64_t)a.H * row, (cuuint64_t)T * a.H * row};
-  cuuint32_t box[4] = {64, 1, 64, 1}, es[4] = {1, 1, 1, 1};
-  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, ptr, dims, strides, box, es,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-template <int OBF, int G>
-auto chunk_kernel(bool dm) {
-  return dm ? k_bwd_chunk<OBF, G, 1> : k_bwd_chunk<OBF, G, 0>;
-}
-
 }  // namespace
 
-// Diagonal KDN with enough chunks in all to give every SM one: below that the two
-// launches and the hand-over of dp cost more than the idle SMs of the one-kernel sweep.
-constexpr long long kSplitMinChunks = 96;
+// Where the two kernels finish sooner than the one-kernel sweep, in thousands of cycles as
+// measured: the sweep takes 40 a chunk with one CTA per sequence; k_bwd_state 6 a chunk with
+// one CTA per sequence, k_bwd_chunk 32 a chunk on any SM, and the second launch with its first
+// tiles 12.  B8 H16 T4096: 2.1 M cycles against 2.5 M (1120 us, 1326 us); B2 H16 T1999 with
+// logit gates: 0.49 M against 1.28 M (255 us, 668 us); with as many sequences as SMs and one
+// or two chunks each the sweep is ahead.  Fewer than 96 chunks in all are left to the sweep (a
+// few tens of us either way).  The rule reads sizes only: a context is saved before it is
+// known which gradients will be asked for.
 bool split_bwd_context(const Args &a) {
-  return a.variant == 0 && a.chunk != 32 && fused_fwd_supported(a) &&
-         (long long)a.B * a.H * ((a.T + CM - 1) / CM) >= kSplitMinChunks;
+  if (a.variant != 0 || a.chunk == 32 || !fused_fwd_supported(a)) return false;
+  const long long bh = (long long)a.B * a.H, nc = (a.T + CM - 1) / CM, waves = (bh + kSms - 1) / kSms;
+  if (bh * nc < 96) return false;
+  return waves * nc * 6 + (bh * nc + kSms - 1) / kSms * 32 + 12 < waves * nc * 40;
+}
+
+// The calls served: bf16 gradients and none of the initial state or mu.  Float32 results stay
+// with the sweep: K' unnormalised rounds otherwise in fp16 than K_tail, and a slow decay
+// carries the difference on (up to 1e-4 of a gradient's norm; bf16 stores round by 2e-3).
+bool split_bwd_supported(const Args &a) {
+  return split_bwd_context(a) && a.odt == KDN_BF16 && !a.dS0 && !a.dp0 && !a.dmu && (a.T % CM == 0 || a.split_ws);
 }
 
 size_t split_bwd_workspace_bytes(const Args &a) {
-  if (!split_bwd_context(a) || a.T % CM == 0) return 0;
+  if (!split_bwd_context(a) || a.odt != KDN_BF16 || a.T % CM == 0) return 0;
   const size_t n = (size_t)a.B * a.H * ((a.T + CM - 1) / CM);
   return n * 5 * 16384;
 }
@@ -1156,31 +1109,28 @@ kdn_status_t launch_split_bwd(const Args &a, char *ws, cudaStream_t s) {
   P.rec = fused_ctx_record_bytes(a);
   P.ticket = a.status + 1;
   const int NC = (a.T + CM - 1) / CM;
-  const bool obf = a.odt == KDN_BF16;
   void *buf[4] = {a.dq, a.dk_, a.dv_, a.dg};
   P.s.T = NC * CM;
-  P.s.row = obf ? 2 * D : 4 * D;
   P.s.small = static_cast<unsigned char *>(a.domega);
   if (ws) {
     const size_t n = (size_t)a.B * a.H * NC * 16384;
     for (int k = 0; k < 4; ++k) buf[k] = ws + k * n;
     P.s.small = reinterpret_cast<unsigned char *>(ws + 4 * n);
-    P.s.row = 2 * D;
   }
-  CUtensorMap m[4], mq, mk, mdo;
+  Args t = a;  // the scratch tiles: bf16 tensors of whole chunks
+  t.T = P.s.T;
+  CUtensorMap m[4], mq, mk, mdo, mdv;
   for (int k = 0; k < 4; ++k)
-    if (!make_scratch_map(&m[k], buf[k], a, P.s.T, P.s.row)) return KDN_ERR_CUDA;
-  if (!make_map(&mq, a.q, a) || !make_map(&mk, a.k, a) || !make_map(&mdo, a.dO, a)) return KDN_ERR_CUDA;
-  CUtensorMap mw = mq, mdv = mq;
+    if (!make_map(&m[k], buf[k], t)) return KDN_ERR_CUDA;
+  if (!make_map(&mq, a.q, a) || !make_map(&mk, a.k, a) || !make_map(&mdo, a.dO, a) || !make_map(&mdv, a.dv_, a))
+    return KDN_ERR_CUDA;
+  CUtensorMap mw = mq;  // the omega logits
   if (a.gates && !make_map(&mw, a.omega, a)) return KDN_ERR_CUDA;
-  if (obf && !make_map(&mdv, a.dv_, a)) return KDN_ERR_CUDA;
   if (cudaFuncSetAttribute(k_bwd_state, cudaFuncAttributeMaxDynamicSharedMemorySize, STATE_SMEM) != cudaSuccess)
     return KDN_ERR_CUDA;
   k_bwd_state<<<a.B * a.H, BT, STATE_SMEM, s>>>(mdo, m[0], m[1], m[2], m[3], P);
   if (cudaGetLastError() != cudaSuccess) return KDN_ERR_CUDA;
-  const bool dm = a.dmu != nullptr;
-  const auto kern = a.gates ? (obf ? chunk_kernel<1, 1>(dm) : chunk_kernel<0, 1>(dm))
-                            : (obf ? chunk_kernel<1, 0>(dm) : chunk_kernel<0, 0>(dm));
+  const auto kern = a.gates ? k_bwd_chunk<1> : k_bwd_chunk<0>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, CHUNK_SMEM) != cudaSuccess)
     return KDN_ERR_CUDA;
   const long long njobs = (long long)a.B * a.H * NC;
