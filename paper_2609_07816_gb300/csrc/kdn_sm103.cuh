@@ -100,12 +100,6 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 __device__ __forceinline__ void bulk_wait_read() {
   asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
-// Wait until every committed bulk store but the most recent group has finished
-// reading shared memory.
-__device__ __forceinline__ void bulk_wait_read_but1() {
-  asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-}
-// Wait until every committed bulk store has completed.
 __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // Prefetch `bytes` (a multiple of 16) of global memory at `src` (16-byte aligned) into L2.
 __device__ __forceinline__ void bulk_prefetch_l2(const void *src, uint32_t bytes) {

@@ -784,7 +784,7 @@ __global__ void __launch_bounds__(WT, 1)
   for (int c = 0; c < NC; ++c) {
     const uint32_t tkt = TKT + (uint32_t)((c & 1) * 32);
     unsigned char *ctx = SV ? P.save_S + ((size_t)bh * NC + c) * P.rec : nullptr;
-    if (SV && issuer) bulk_wait_read();  // the previous chunk's context tiles have left shared memory
+    if (SV && lane == 0) bulk_wait_read();  // the previous chunk's context tiles have left shared memory
     // ---- [0] the previous chunk's MMA-O / MMA-S2 must be done before V is brought
     //          into its R' buffer; the gain of this chunk is done (its warps arrive here)
     if (!gain) mine = mbar_wait(bar_raw, c & 1, kWait) && mine;
@@ -1027,14 +1027,13 @@ __global__ void __launch_bounds__(WT, 1)
         umma_if(lead, TU, step(A1, (kk >> 2) * 16384 + (kk & 3) * 32), step(B1, kk * 2048), id_16, kk > 0);
       commit_if(lead, bar_mma);
     }
-    if (issuer) {
-      if (SV) {
-        bulk_s2g(ctx + kCtxS, s16, 32768);
-        if (ext)
-          for (int s = 0; s < 2; ++s)
-            bulk_s2g(ctx + kCtxKQ + s * 16384 + 8192, as1 + s * 16384 + 8192, 8192);
-        bulk_commit();
-      }
+    // (the copies of the context tiles are issued one per warp, by warps with nothing else to
+    // do at that point: each costs its warp a few hundred cycles)
+    if (SV && lane == 0) {
+      if (warp == 10) bulk_s2g(ctx + kCtxS, s16, 32768);
+      else if (ext && (warp == 11 || warp == 14))
+        bulk_s2g(ctx + kCtxKQ + (warp == 14) * 16384 + 8192, as1 + (warp == 14) * 16384 + 8192, 8192);
+      bulk_commit();
     }
 
     // ---- [4] A = (I + T)^-1 = diag(s) L^-1 with L = diag(s) + strict_lower(T')
@@ -1064,38 +1063,15 @@ __global__ void __launch_bounds__(WT, 1)
       wy_inverse(mt, sT, sA, sX, sY, s_r + 64 * (c & 1), s_s, s_is, awu, y_side);
       if (wq >= 2) ++mph;  // MMA-KS, observed by the Y warps
     }
-    if (SV) {
-      if (wq >= 2 && wgm == 0) {  // A_qk = lower(A'_qk) diag(1/s) into the context
-        const int t = 32 * (wq - 2) + lane;
-        for (int h2 = 0; h2 < 2; ++h2) {
-          float pv[16];
-          tmem_ld16(TD1 + lane_base + 16 * h2, pv);  // 32 fp16 of columns 32 h2 ..
-#pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4) {
-            const int cc = 4 * h2 + q4;
-            float v8[8];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const uint32_t bits = __float_as_uint(pv[4 * q4 + j]);
-              const float2 f2 = __half22float2(*reinterpret_cast<const __half2 *>(&bits));
-              v8[2 * j] = f2.x * s_is[8 * cc + 2 * j];
-              v8[2 * j + 1] = f2.y * s_is[8 * cc + 2 * j + 1];
-            }
-            *reinterpret_cast<uint4 *>(ctx + kCtxAqk + chunk_off(t, cc)) = pack_h8(v8);
-          }
-        }
-      }
-      if (mt < CM) reinterpret_cast<float *>(ctx + kCtxTok)[mt] = s_s[mt];
-    }
     fence_proxy_async();
     tc_fence_before();
     bar_sync(kBarMain, kMain);
 
     // ---- [5] (context only) -W = A (-Kbar) into TW, then to the context
     if (SV) {
-      if (issuer) {
-        bulk_s2g(ctx + kCtxA, awu, 8192);
-        bulk_s2g(ctx + kCtxY, vr, 16384);  // Y, before R' is written over it
+      if (lane == 0 && warp >= 14) {
+        if (warp == 14) bulk_s2g(ctx + kCtxA, awu, 8192);
+        else bulk_s2g(ctx + kCtxY, vr, 16384);  // Y, before R' is written over it
         bulk_commit();
       }
       if (warp_u == 4) {
@@ -1108,8 +1084,29 @@ __global__ void __launch_bounds__(WT, 1)
         commit_if(lead, bar_w);  // its own barrier: MMA-KS may not have been observed yet
       }
     }
-    // ---- [6] (context only) -W out of TMEM
+    // ---- [6] (context only) -W out of TMEM; A_qk and s_t
     if (SV) {  // -W of the context (rows 0..63 of TW), once MMA-W has completed
+      if (wq >= 2 && wgm < 2) {  // A_qk = lower(A'_qk) diag(1/s) into the context, columns 32 wgm ..
+        const int t = 32 * (wq - 2) + lane;
+        float pv[16];
+        tmem_ld16(TD1 + lane_base + 16 * wgm, pv);
+#pragma unroll
+        for (int q4 = 0; q4 < 4; ++q4) {
+          const int cc = 4 * wgm + q4;
+          float v8[8];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint32_t bits = __float_as_uint(pv[4 * q4 + j]);
+            const float2 f2 = __half22float2(*reinterpret_cast<const __half2 *>(&bits));
+            v8[2 * j] = f2.x * s_is[8 * cc + 2 * j];
+            v8[2 * j + 1] = f2.y * s_is[8 * cc + 2 * j + 1];
+          }
+          *reinterpret_cast<uint4 *>(ctx + kCtxAqk + chunk_off(t, cc)) = pack_h8(v8);
+        }
+      } else if (wq >= 2) {
+        const int t = 32 * (wq - 2) + lane;
+        reinterpret_cast<float *>(ctx + kCtxTok)[t] = s_s[t];
+      }
       mine = mbar_wait(bar_w, c & 1, kWait) && mine;
       tc_fence_after();
       if (wq < 2) {  // into the fp32 L^-1 tile, dead since the solve, for one bulk copy
@@ -1122,21 +1119,18 @@ __global__ void __launch_bounds__(WT, 1)
           sm16(wst, sl * 8192 + chunk_off(t, cc0 + 1)) = pack_h8(v + 8);
         }
       }
+      if (lane == 0 && warp >= 14) bulk_wait_read();  // [A; .] and Y may be written over in [8]
       fence_proxy_async();
       tc_fence_before();
       bar_sync(kBarMain, kMain);  // TW is free for MMA-R
-      if (issuer) {
+      if (tid == 32 * 10) {
         bulk_s2g(ctx + kCtxW, wst, 16384);
         bulk_commit();
       }
     }
 
     // ---- [7] MMA-R: TW = [A; .] Y = [R; 0]  (fp16)
-    // (context: the copy of Y has left shared memory before MMA-R completes, after
-    // which R' is written over Y; the copy of -W, committed after it, may still run)
-    if (SV && issuer) bulk_wait_read_but1();
     if (warp_u == 4) {
-      __syncwarp();
       tc_fence_after();
       const uint32_t lead = elect_one();
       const uint64_t AW = sw128_desc(smem_u32(awu), 16, 1024), VR = sw128_desc(smem_u32(vr), 8192, 1024);
@@ -1171,7 +1165,7 @@ __global__ void __launch_bounds__(WT, 1)
 
     // ---- [9] MMA-O (rows 64..127 of TU += A'_qk R', A'_qk in TMEM) and
     //          MMA-S2 (S += K'^T R', K' in TMEM)
-    if (SV && issuer) {
+    if (SV && tid == 32 * 11) {
       bulk_s2g(ctx + kCtxR, awu, 16384);
       bulk_commit();
     }
@@ -1240,7 +1234,7 @@ __global__ void __launch_bounds__(WT, 1)
       }
     }
   }
-  if (SV && issuer) bulk_wait_all();
+  if (SV && lane == 0) bulk_wait_all();
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tbase, 512);
