@@ -107,20 +107,24 @@ __device__ __forceinline__ void check_gamma_range(float gC, unsigned *status) {
 // Row stride (floats) of the fp32 T and A tiles: 16-byte rows, conflict-free.
 constexpr int LT = 68;
 
-// acc += P Q over 16 values of k: one row of P (stride-LT tile), four adjacent columns of Q
-// (row stride ldq).
-__device__ __forceinline__ void tri_term(float4 &acc, const float *P, const float *Q, int ldq) {
+// a0, a1 += P0 Q, P1 Q over 4 K4 values of k: one row each of P (stride-LT tile), four
+// adjacent columns of Q.  The solves are bound by shared-memory reads (a 16-byte load takes
+// four cycles of the SM whatever its lanes share), so a thread forms two rows from each load of Q.
+template <int K4>
+__device__ __forceinline__ void tri_term2(float4 &a0, float4 &a1, const float *P0, const float *P1, const float *Q,
+                                          int ldq) {
 #pragma unroll
-  for (int m4 = 0; m4 < 4; ++m4) {
-    const float4 t4 = *reinterpret_cast<const float4 *>(P + 4 * m4);
-    const float tv[4] = {t4.x, t4.y, t4.z, t4.w};
+  for (int m4 = 0; m4 < K4; ++m4) {
+    const float4 s4 = *reinterpret_cast<const float4 *>(P0 + 4 * m4);
+    const float4 t4 = *reinterpret_cast<const float4 *>(P1 + 4 * m4);
+    const float sv[4] = {s4.x, s4.y, s4.z, s4.w}, tv[4] = {t4.x, t4.y, t4.z, t4.w};
 #pragma unroll
     for (int mm = 0; mm < 4; ++mm) {
-      const float4 a4 = *reinterpret_cast<const float4 *>(Q + (4 * m4 + mm) * ldq);
-      acc.x += tv[mm] * a4.x;
-      acc.y += tv[mm] * a4.y;
-      acc.z += tv[mm] * a4.z;
-      acc.w += tv[mm] * a4.w;
+      const float4 q = *reinterpret_cast<const float4 *>(Q + (4 * m4 + mm) * ldq);
+      a0.x = fmaf(sv[mm], q.x, a0.x); a0.y = fmaf(sv[mm], q.y, a0.y);
+      a0.z = fmaf(sv[mm], q.z, a0.z); a0.w = fmaf(sv[mm], q.w, a0.w);
+      a1.x = fmaf(tv[mm], q.x, a1.x); a1.y = fmaf(tv[mm], q.y, a1.y);
+      a1.z = fmaf(tv[mm], q.z, a1.z); a1.w = fmaf(tv[mm], q.w, a1.w);
     }
   }
 }
@@ -128,11 +132,12 @@ __device__ __forceinline__ void tri_term(float4 &acc, const float *P, const floa
 // A = (I + T)^-1 for a strictly lower triangular 64 x 64 fp32 T (row stride
 // LT, zero on and above the diagonal), by 16 x 16 blocks, with 512 threads:
 // diagonal blocks D_I = (I + T_II)^-1 by column substitution (rows across a
-// half-warp), then A_IJ = -D_I sum_{K=J}^{I-1} T_IK A_KJ level by level (I - J = 1, 2, 3):
-// 64 threads per off-diagonal block, one per (row, 4 columns), which add each term
+// half-warp), then A_IJ = -D_I sum_{K=J}^{I-1} T_IK A_KJ level by level (I - J = 1, 2, 3),
+// one warp per off-diagonal block, two rows x four columns a lane, which adds each term
 // as soon as its A_KJ exists, so that only the last term of a level waits for the
-// level before (B1 H12 T32768 isotropic forward, this and the barriers around the output store:
-// see k_fused_fwd).  sX holds 3 x 256 floats of scratch.  Entries of A above
+// level before, and a block's own products need no barrier (before: 64 threads a block, one
+// row each, two CTA barriers a level; 4350 -> 3700 cycles a chunk with the transition,
+// 4070 -> 3090 in the isotropic training forward).  sX holds 3 x 256 floats of scratch.  Entries of A above
 // the diagonal are left unwritten except inside the diagonal blocks (zero).
 // Contains block-wide barriers; every thread of the CTA must call it.
 __device__ __forceinline__ void tri_inverse64(const float *sT, float *sA, float *sX) {
@@ -161,25 +166,33 @@ __device__ __forceinline__ void tri_inverse64(const float *sT, float *sA, float 
   }
   __syncthreads();
   // blocks in the order of their levels: (1,0) (2,1) (3,2) | (2,0) (3,1) | (3,0)
-  const int blk = tid >> 6, lvl = blk < 3 ? 1 : blk < 5 ? 2 : 3;
-  const int J = blk < 3 ? blk : blk < 5 ? blk - 3 : 0, I = J + lvl;
-  const int rr = (tid >> 2) & 15, c4 = 4 * (tid & 3);
-  const float *tr = sT + (16 * I + rr) * LT + 16 * J, *ac = sA + 16 * J * LT + 16 * J + c4;
-  float *xb = sX + J * 256 + c4;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (blk < 6) tri_term(acc, tr, ac, LT);
+  if (warp < 6) {
+    const int lvl = warp < 3 ? 1 : warp < 5 ? 2 : 3;
+    const int J = warp < 3 ? warp : warp < 5 ? warp - 3 : 0, I = J + lvl;
+    const int rr = lane >> 2, c4 = 4 * (lane & 3);  // rows rr, rr + 8
+    const float *tr = sT + (16 * I + rr) * LT + 16 * J, *ac = sA + 16 * J * LT + 16 * J + c4;
+    const float *dr = sA + (16 * I + rr) * LT + 16 * I;
+    float *xb = sX + J * 256 + c4, *out = sA + (16 * I + rr) * LT + 16 * J + c4;
+    float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
+    tri_term2<4>(a0, a1, tr, tr + 8 * LT, ac, LT);
 #pragma unroll
-  for (int l = 1; l <= 3; ++l) {
-    if (blk < 6 && lvl == l) *reinterpret_cast<float4 *>(xb + rr * 16) = acc;
-    __syncthreads();
-    if (blk < 6 && lvl == l) {
-      float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-      tri_term(d, sA + (16 * I + rr) * LT + 16 * I, xb, 16);
-      *reinterpret_cast<float4 *>(sA + (16 * I + rr) * LT + 16 * J + c4) = make_float4(-d.x, -d.y, -d.z, -d.w);
+    for (int l = 1; l <= 3; ++l) {
+      if (lvl == l) {
+        *reinterpret_cast<float4 *>(xb + rr * 16) = a0;
+        *reinterpret_cast<float4 *>(xb + (rr + 8) * 16) = a1;
+        __syncwarp();
+        float4 d0 = make_float4(0.f, 0.f, 0.f, 0.f), d1 = d0;
+        tri_term2<4>(d0, d1, dr, dr + 8 * LT, xb, 16);
+        *reinterpret_cast<float4 *>(out) = make_float4(-d0.x, -d0.y, -d0.z, -d0.w);
+        *reinterpret_cast<float4 *>(out + 8 * LT) = make_float4(-d1.x, -d1.y, -d1.z, -d1.w);
+      }
+      if (l < 3) {
+        asm volatile("bar.sync 1, 192;" ::: "memory");
+        if (lvl > l) tri_term2<4>(a0, a1, tr + 16 * l, tr + 16 * l + 8 * LT, ac + 16 * l * LT, LT);
+      }
     }
-    __syncthreads();
-    if (l < 3 && blk < 6 && lvl > l) tri_term(acc, tr + 16 * l, ac + 16 * l * LT, LT);
   }
+  __syncthreads();
 }
 
 inline PFN_cuTensorMapEncodeTiled_v12000 encoder() {

@@ -313,13 +313,15 @@ __device__ __forceinline__ void wy_inverse(int tid, const float *sT, float *sA, 
     *reinterpret_cast<float4 *>(sA + (R0 + r2) * LT + C0 + cq2) = make_float4(-acc.x, -acc.y, -acc.z, -acc.w);
   }
   bar_sync(kBarMain, kMain);
-  // Y = L21 X11 (32 x 32 x 32): one thread per (row, 4 columns)
-  const int r3 = tid >> 3, cq3 = 4 * (tid & 7);
+  // Y = L21 X11 (32 x 32 x 32): one thread per (row, 4 columns), warps 0..3 the left columns,
+  // 4..7 the right ones, which need k >= 16 only (X11's upper right quarter is zero)
   if (tid < 256) {
+    const int r3 = 8 * (w & 3) + ((tid & 31) >> 2), cq3 = 16 * (w >> 2) + 4 * (tid & 3);
     const float *tp = sT + (32 + r3) * LT;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
+      if (j < 4 && w >= 4) continue;
       const float4 t4 = *reinterpret_cast<const float4 *>(tp + 4 * j);
       const float tv[4] = {t4.x, t4.y, t4.z, t4.w};
 #pragma unroll
@@ -335,12 +337,15 @@ __device__ __forceinline__ void wy_inverse(int tid, const float *sT, float *sA, 
   }
   bar_sync(kBarMain, kMain);
   // T' is dead from here on: [A; .] fp16 [128 t][64 s] (A = diag(s) L^-1) is written over it.
-  // X_21 = -X22 Y by threads 0..255, straight to fp16; threads 256..383 convert the rest.
+  // X_21 = -X22 Y by threads 0..255 (rows 0..15 of X22 end at k = 15), straight to fp16;
+  // threads 256..383 convert the rest.
   if (tid < 256) {
+    const int r3 = tid >> 3, cq3 = 4 * (tid & 7);
     const float *dp = sA + (32 + r3) * LT + 32;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
+      if (j >= 4 && w < 4) continue;
       const float4 d4 = *reinterpret_cast<const float4 *>(dp + 4 * j);
       const float dv[4] = {d4.x, d4.y, d4.z, d4.w};
 #pragma unroll
