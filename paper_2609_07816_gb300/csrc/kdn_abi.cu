@@ -4,6 +4,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "kdn_internal.cuh"
 
 namespace kdn {
@@ -142,7 +144,11 @@ kdn_status_t fwd_entry(int variant, const kdn_desc_t *d, const void *q, const vo
   if ((size_t)a.B * a.H == 0) return KDN_OK;
   if (a.T == 0) return empty_fwd(a, s);
   if (nseg > 1) return launch_seg_fwd(a, nseg, static_cast<char *>(ws) + base, s);
-  if (use_fused(a) && wy_fwd_supported(a, false)) return launch_wy_fwd(a, s);
+  if (use_fused(a) && wy_fwd_supported(a, false)) {
+    const size_t split = wy_split_workspace_bytes(a);
+    return launch_wy_fwd(a, s, nullptr, nullptr,
+                         split && ws_bytes >= base + split ? static_cast<char *>(ws) + base : nullptr);
+  }
   if (use_fused(a)) return launch_fused_fwd(a, s);
   return launch_chunked_fwd(a, s, false);
 }
@@ -282,6 +288,12 @@ size_t fwd_min_workspace_bytes(const kdn_desc_t *desc, int variant) {
   return workspace_layout(&a, nullptr, false);
 }
 
+size_t fwd_noalloc_bytes(const kdn_desc_t *desc, size_t have) {
+  Args a;
+  if (fill_sizes(desc, 0, false, &a) != KDN_OK) return 0;
+  return seg_count(a) == 1 && wy_split_sizes(a) ? workspace_layout(&a, nullptr, false) : have;
+}
+
 size_t workspace_layout(Args *a, char *base, bool bwd) {
   const size_t BH = (size_t)a->B * a->H, Tp = a->Tp, NC = a->NC, C = a->C;
   const size_t dk = a->dk, dv = a->dv, P = a->P;
@@ -356,7 +368,8 @@ size_t kdn_fwd_workspace_bytes(const kdn_desc_t *desc, int variant) {
   const int nseg = seg_count(a);
   // (the training backward of ragged lengths takes its scratch from the same workspace)
   return workspace_layout(&a, nullptr, false) +
-         (nseg > 1 ? seg_workspace_bytes(a, nseg) : split_bwd_workspace_bytes(a));
+         (nseg > 1 ? seg_workspace_bytes(a, nseg)
+                   : std::max(split_bwd_workspace_bytes(a), wy_split_workspace_bytes(a)));
 }
 
 size_t kdn_bwd_workspace_bytes(const kdn_desc_t *desc, int variant) {
@@ -463,11 +476,11 @@ int kdn_kernel_launches(const kdn_desc_t *desc, int variant, int op) {
   Args a;
   if (fill_sizes(desc, variant, op == 2, &a) != KDN_OK) return -1;
   switch (op) {
-    case 0: return seg_count(a) > 1 ? 5 : use_fused(a) ? 1 : chunked_fwd_launches(a);
-    case 1: return (a.T > 0 && use_fused_bwd(a)) ? 2 : chunked_bwd_launches(a);
+    case 0: return seg_count(a) > 1 ? 5 : use_fused(a) ? (wy_split_sizes(a) ? 3 : 1) : chunked_fwd_launches(a);
+    case 1: return (a.T > 0 && use_fused_bwd(a)) ? (wy_split_save(a) ? 4 : 2) : chunked_bwd_launches(a);
     case 2: return 1;
-    case 4: return fused_saved_bytes(a) > 0 ? 1 : -1;
-    case 3:
+    case 3: return fused_saved_bytes(a) > 0 ? (wy_split_save(a) ? 3 : 1) : -1;
+    case 4:
     case 5: return fused_saved_bytes(a) > 0 ? 1 : -1;
   }
   return -1;

@@ -163,7 +163,12 @@ kdn_status_t launch_fused_fwd(const Args &a, cudaStream_t s, unsigned char *save
 // launch_fused_fwd's saving mode).
 bool wy_fwd_supported(const Args &a, bool save);  // save: the context-saving instantiation
 kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S = nullptr,
-                           float *save_p = nullptr);
+                           float *save_p = nullptr, char *ws = nullptr);
+// The same in three kernels (gain, chunks in parallel, memory) where these sizes gain from it:
+// with the extended context, or with this much scratch in the workspace.
+bool wy_split_sizes(const Args &a);
+bool wy_split_save(const Args &a);  // the context-saving forward
+size_t wy_split_workspace_bytes(const Args &a);
 // beta_eff [B,T,H] (float32) from the per-token gain scalars of a context saved by
 // the fused training forward (one launch).
 kdn_status_t launch_beta_eff(const Args &a, const void *saved, float *out, cudaStream_t s);
@@ -196,6 +201,9 @@ int seg_count(const Args &a);
 // Smallest forward workspace for a descriptor (the single-pass layout; 0 for an
 // invalid descriptor); kdn_fwd_workspace_bytes adds the segment buffers.
 size_t fwd_min_workspace_bytes(const kdn_desc_t *desc, int variant);
+// What the forward that cannot allocate lets its diagonal call use of `have` bytes: only the
+// status word where the one fused kernel serves, so that such calls may overlap.
+size_t fwd_noalloc_bytes(const kdn_desc_t *desc, size_t have);
 size_t seg_workspace_bytes(const Args &a, int P);
 kdn_status_t launch_seg_fwd(const Args &a, int P, char *ws, cudaStream_t s);
 

@@ -97,7 +97,8 @@ kdn_status_t kdn_diag_fwd_noalloc(const kdn_desc_t *desc, const void *q, const v
   void *ws = nullptr;
   kdn_status_t st = scratch_address(&ws);
   if (st != KDN_OK) return st;
-  return kdn_diag_fwd(desc, q, k, v, g, omega, r, S0, p0, o, ST, pT, ws, kScratchBytes, stream);
+  return kdn_diag_fwd(desc, q, k, v, g, omega, r, S0, p0, o, ST, pT, ws,
+                      kdn::fwd_noalloc_bytes(desc, kScratchBytes), stream);
 }
 
 kdn_status_t kdn_noalloc_device_status(void *stream) {

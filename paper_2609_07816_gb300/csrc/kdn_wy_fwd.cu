@@ -80,6 +80,7 @@ constexpr int WT = 512;  // threads
 constexpr int CM = 64;   // chunk length
 constexpr int D = 128;   // d_k = d_v
 constexpr uint32_t kWait = 1u << 25;
+constexpr int kSms = 152;
 constexpr uint32_t kDrain = 1u << 14;  // bounded waits of the failure path
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
@@ -151,6 +152,9 @@ __device__ __forceinline__ uint32_t sw32_off(uint32_t row, uint32_t col) {
 }
 __device__ __forceinline__ void bar_sync(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int n) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 // named barrier that also returns the OR of a predicate over its n threads
 __device__ __forceinline__ bool bar_or(int id, int n, bool p) {
@@ -444,6 +448,20 @@ struct WyParams {
   unsigned char *save_S;  // SV: [BH][NC] context records of the backward
   size_t rec;             // SV: bytes of a record; beyond kCtxBytes it also takes Qbar and K'^T
   float *save_p;          // SV: [BH][NC][128] uncertainty carry entering each chunk
+  // CH: records of the per-chunk operands (SV: the context records), what enters every chunk
+  unsigned char *pre;
+  size_t prec;
+  const float *pin;       // [BH][NC][128]
+};
+
+// Per-chunk operands of the three-kernel forward, in a context record (SV) or in a record of
+// their own: [-Kbar; Qbar] fp16 32 KB, K'^T fp16 [128 i][64 s] 16 KB, A fp16 8 KB, A'_qk fp16
+// 8 KB (context: in R's place until R is there), gamma_C [128], s_t [64].
+constexpr size_t kPreBytes = 66560;
+template <int SV>
+struct Pre {
+  static constexpr int KQ = SV ? kCtxKQ : 0, Kt = SV ? kCtxKt : 32768, A = SV ? kCtxA : 49152;
+  static constexpr int Aq = SV ? kCtxR : 57344, gC = SV ? kCtxGa + 63 * D * 4 : 65536, s = SV ? kCtxTok : 66048;
 };
 
 // SV: besides o, S_T and p_T (each written when its pointer is non-null), keep
@@ -453,7 +471,10 @@ struct WyParams {
 // phat and gamma in float32 [64 t][128 i], s_t per token, and the uncertainty
 // entering the chunk.  The arithmetic is the same with and without it.
 
-template <int SV, int LG>  // LG: g, omega, r hold the logits x, y, z of the gates
+// CH: the part of this work that needs no memory S, for the chunks blockIdx.x, + gridDim.x, ..
+// of all sequences, its results left in records for k_wy_state; the uncertainty entering
+// each chunk is known (k_wy_gain).  The same instructions, so the same bits.
+template <int SV, int LG, int CH>  // LG: g, omega, r hold the logits x, y, z of the gates
 __global__ void __launch_bounds__(WT, 1)
     k_wy_fwd(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mg,
              const __grid_constant__ CUtensorMap mw, const __grid_constant__ CUtensorMap mv,
@@ -481,8 +502,20 @@ __global__ void __launch_bounds__(WT, 1)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int wq = warp & 3, wg = warp >> 2;  // TMEM lane quarter, column group
-  const int bh = blockIdx.x, b = bh / a.H, h = bh % a.H;
-  const int NC = (a.T + CM - 1) / CM;
+  const int bh = blockIdx.x;  // (not CH)
+  const int NCs = (a.T + CM - 1) / CM, BH = a.B * a.H;
+  // chunks of this CTA, counted by `c` below; ct, b, h: a chunk's place in its sequence
+  const int NC = CH ? (NCs * BH - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : NCs;
+  struct Job { int ct, b, h; size_t rc; };
+  auto job = [&](int c) {
+    Job o;
+    const int j = CH ? (int)(blockIdx.x + c * gridDim.x) : 0, q = CH ? j % BH : bh;
+    o.ct = CH ? j / BH : c;
+    o.b = q / a.H;
+    o.h = q % a.H;
+    o.rc = (size_t)q * NCs + o.ct;
+    return o;
+  };
   const bool issuer = tid == 128;  // copies; the MMAs: its whole warp with an elected lane
   const int warp_u = __shfl_sync(0xffffffffu, warp, 0);
   const bool ext = SV && P.rec > (size_t)kCtxBytes;
@@ -515,38 +548,39 @@ __global__ void __launch_bounds__(WT, 1)
 
   // k, g, omega of chunk c (the gain and the preparing pass), q of chunk c (the
   // preparing pass), V of chunk c (once MMA-O / MMA-S2 of chunk c - 1 has read R')
-  auto issue_raw = [&](int c) {
+  auto issue_raw = [&](const Job &o) {
     mbar_expect_tx(bar_raw, 49152);
     for (int s = 0; s < 2; ++s) {
-      tma_load_4d(rk + s * 8192, &mk, bar_raw, 64 * s, h, c * CM, b);
-      tma_load_4d(rg + s * 8192, &mg, bar_raw, 64 * s, h, c * CM, b);
-      tma_load_4d(rw + s * 8192, &mw, bar_raw, 64 * s, h, c * CM, b);
+      tma_load_4d(rk + s * 8192, &mk, bar_raw, 64 * s, o.h, o.ct * CM, o.b);
+      tma_load_4d(rg + s * 8192, &mg, bar_raw, 64 * s, o.h, o.ct * CM, o.b);
+      tma_load_4d(rw + s * 8192, &mw, bar_raw, 64 * s, o.h, o.ct * CM, o.b);
     }
   };
-  auto issue_q = [&](int c) {
+  auto issue_q = [&](const Job &o) {
     mbar_expect_tx(bar_q, 16384);
-    for (int s = 0; s < 2; ++s) tma_load_4d(rq + s * 8192, &mq, bar_q, 64 * s, h, c * CM, b);
+    for (int s = 0; s < 2; ++s) tma_load_4d(rq + s * 8192, &mq, bar_q, 64 * s, o.h, o.ct * CM, o.b);
   };
-  auto issue_v = [&](int c) {
+  auto issue_v = [&](const Job &o) {
     mbar_expect_tx(bar_v, 16384);
-    for (int s = 0; s < 2; ++s) tma_load_4d(vr + s * 8192, &mv, bar_v, 64 * s, h, c * CM, b);
+    for (int s = 0; s < 2; ++s) tma_load_4d(vr + s * 8192, &mv, bar_v, 64 * s, o.h, o.ct * CM, o.b);
+  };
+  auto prefetch = [&](const Job &o) {  // k, g, omega, q into L2
+    for (int s = 0; s < 2; ++s) {
+      tma_prefetch_4d(&mk, 64 * s, o.h, o.ct * CM, o.b);
+      tma_prefetch_4d(&mg, 64 * s, o.h, o.ct * CM, o.b);
+      tma_prefetch_4d(&mw, 64 * s, o.h, o.ct * CM, o.b);
+      tma_prefetch_4d(&mq, 64 * s, o.h, o.ct * CM, o.b);
+    }
   };
   if (issuer && NC > 0) {
-    issue_raw(0);
-    issue_q(0);
-    issue_v(0);
-    if (NC > 1) {
-      for (int s = 0; s < 2; ++s) {
-        tma_prefetch_4d(&mk, 64 * s, h, CM, b);
-        tma_prefetch_4d(&mg, 64 * s, h, CM, b);
-        tma_prefetch_4d(&mw, 64 * s, h, CM, b);
-        tma_prefetch_4d(&mq, 64 * s, h, CM, b);
-      }
-    }
+    issue_raw(job(0));
+    issue_q(job(0));
+    if (!CH) issue_v(job(0));
+    if (NC > 1) prefetch(job(1));
   }
 
   // initial memory S_0 -> TMEM (row = key channel i, column = value j)
-  {
+  if constexpr (!CH) {
     const int i = 32 * wq + lane;
     for (int c0 = 0; c0 < 32; c0 += 16) {
       float v[16];
@@ -575,13 +609,16 @@ __global__ void __launch_bounds__(WT, 1)
   const int mt = tid - 128;           // main thread 0 .. kMain - 1
   const int wgm = (warp >> 2) - 1;    // main warps: 0, 1, 2 within a lane quarter
   float p = 1.f;                      // gain threads: uncertainty carry of channel tid
-  if (gain && a.p0) p = a.p0[(size_t)bh * D + tid];
+  if (!CH && gain && a.p0) p = a.p0[(size_t)bh * D + tid];
   // gain threads tid < 64: the r input of the next chunk's token tid, converted when it is
   // used (a conversion here would wait for the load)
   __nv_bfloat16 znext = __float2bfloat16_rn(0.f);
+  float pnext = 1.f;  // CH: the uncertainty entering the next chunk
   auto load_r = [&](int c) {
-    if (tid < CM && c < NC)
-      znext = static_cast<const __nv_bfloat16 *>(a.r)[tok_index(a, b, min(c * CM + tid, a.T - 1), h)];
+    if (c >= NC) return;
+    const Job o = job(c);
+    if (tid < CM) znext = static_cast<const __nv_bfloat16 *>(a.r)[tok_index(a, o.b, min(o.ct * CM + tid, a.T - 1), o.h)];
+    if (CH && gain) pnext = P.pin[o.rc * D + tid];
   };
   load_r(0);
 
@@ -600,15 +637,18 @@ __global__ void __launch_bounds__(WT, 1)
   //      once MMA-T of chunk c - 1 has read the previous one.
   auto gain_chunk = [&](int c) -> bool {
     const int i = tid, sb = c & 1;
+    const Job o = job(c);
+    const int left = a.T - o.ct * CM;  // tokens of the sequence from this chunk on
+    if (CH) p = pnext;
     float *sr = s_r + 64 * sb, *smur = s_mur + 64 * sb;
     if (tid < CM) {
-      const bool live = c * CM + tid < a.T;
+      const bool live = tid < left;
       const float z = live ? __bfloat162float(znext) : 0.f;
       const float r = !live ? 1.f : LG ? a.rmin + softplus_w(z) : z;  // r = r_min + softplus(z) (Sec. 5)
       sr[tid] = r;
       smur[tid] = a.mu / r;
       if (ext) {  // r_t and z_t for the backward (tokens past T: 1 and 0)
-        float *tok = reinterpret_cast<float *>(P.save_S + ((size_t)bh * NC + c) * P.rec + kCtxTok);
+        float *tok = reinterpret_cast<float *>(P.save_S + o.rc * P.rec + kCtxTok);
         tok[CM + tid] = r;
         tok[2 * CM + tid] = z;
       }
@@ -629,9 +669,9 @@ __global__ void __launch_bounds__(WT, 1)
     // Their rows of the g and omega tiles, zero-filled by TMA, get the logits +-1e30,
     // whose activations are exactly those (softplus(-1e30) = 0), so that no pass
     // masks its elements; the preparing pass reads the same rows
-    if (LG && a.T - c * CM < CM) {
+    if (LG && left < CM) {
       const __nv_bfloat16 big = __float2bfloat16_rn(1e30f), nbig = __float2bfloat16_rn(-1e30f);
-      for (int t = a.T - c * CM; t < CM; ++t) {
+      for (int t = left; t < CM; ++t) {
         *reinterpret_cast<__nv_bfloat16 *>(rg + (i >> 6) * 8192 + sw128_off(t, cl)) = big;
         *reinterpret_cast<__nv_bfloat16 *>(rw + (i >> 6) * 8192 + sw128_off(t, cl)) = nbig;
       }
@@ -685,8 +725,9 @@ __global__ void __launch_bounds__(WT, 1)
     const bool oor = !SV && bar_or(kBarGain, 128, cref < kMinHalfG);
     if (tid == 0) s_oor[sb] = oor ? 1 : 0;
     float Gt = 0.f;  // G_t of this channel (range mode)
-    unsigned char *gctx = SV ? P.save_S + ((size_t)bh * NC + c) * P.rec : nullptr;
-    if (SV) P.save_p[((size_t)bh * NC + c) * D + i] = p;
+    unsigned char *gctx = SV ? P.save_S + o.rc * P.rec : nullptr;
+    unsigned char *gpre = CH ? P.pre + o.rc * P.prec : gctx;
+    if (SV && !CH) P.save_p[o.rc * D + i] = p;
     float *cph = SV ? reinterpret_cast<float *>(gctx + kCtxPh) + i : nullptr;
     float f = ex2f(cref * kLog2e);                // exp(c - G_t), G_{-1} = 0
     const float E2 = ex2f((GC - cref) * kLog2e);  // exp(G_C - c)
@@ -728,7 +769,8 @@ __global__ void __launch_bounds__(WT, 1)
           if ((j & 1) == 0) kt[j >> 1] = hb;
           else kt[j >> 1] |= hb << 16;
         }
-        tmem_st4u(tkt + lane_base + (uint32_t)(4 * blk), kt);
+        if (CH) *reinterpret_cast<uint4 *>(gpre + Pre<SV>::Kt + chunk_off(i, blk)) = make_uint4(kt[0], kt[1], kt[2], kt[3]);
+        else tmem_st4u(tkt + lane_base + (uint32_t)(4 * blk), kt);
       }
     } else {
 #pragma unroll
@@ -764,8 +806,9 @@ __global__ void __launch_bounds__(WT, 1)
           if ((j & 1) == 0) kt[j >> 1] = hb;
           else kt[j >> 1] |= hb << 16;
         }
-        tmem_st4u(tkt + lane_base + (uint32_t)(4 * blk), kt);
-        if (ext) *reinterpret_cast<uint4 *>(gctx + kCtxKt + chunk_off(i, blk)) = make_uint4(kt[0], kt[1], kt[2], kt[3]);
+        if (!CH) tmem_st4u(tkt + lane_base + (uint32_t)(4 * blk), kt);
+        if (CH || ext)
+          *reinterpret_cast<uint4 *>(gpre + Pre<SV>::Kt + chunk_off(i, blk)) = make_uint4(kt[0], kt[1], kt[2], kt[3]);
         if (blk < 7) {
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
@@ -788,14 +831,16 @@ __global__ void __launch_bounds__(WT, 1)
 
   for (int c = 0; c < NC; ++c) {
     const uint32_t tkt = TKT + (uint32_t)((c & 1) * 32);
-    unsigned char *ctx = SV ? P.save_S + ((size_t)bh * NC + c) * P.rec : nullptr;
-    if (SV && lane == 0) bulk_wait_read();  // the previous chunk's context tiles have left shared memory
+    const Job o = job(c);
+    unsigned char *ctx = SV ? P.save_S + o.rc * P.rec : nullptr;
+    unsigned char *pre = CH ? P.pre + o.rc * P.prec : ctx;
+    if ((SV || CH) && lane == 0) bulk_wait_read();  // the previous chunk's context tiles have left shared memory
     // ---- [0] the previous chunk's MMA-O / MMA-S2 must be done before V is brought
     //          into its R' buffer; the gain of this chunk is done (its warps arrive here)
     if (!gain) mine = mbar_wait(bar_raw, c & 1, kWait) && mine;
-    if (issuer && c > 0) {
+    if (!CH && issuer && c > 0) {
       mine = mma_wait_main() && mine;  // MMA-O / MMA-S2 of chunk c - 1
-      if (mine) issue_v(c);
+      if (mine) issue_v(o);
     } else if (!gain && c > 0) {
       ++mph;
     }
@@ -887,13 +932,13 @@ __global__ void __launch_bounds__(WT, 1)
         if (SV)
           for (int u = 0; u < 4; ++u) check_gamma_range(gm[u], a.status);
       }
-    } else if (!gain && wq >= 2 && wgm == 2 && c > 0 && a.o) {  // warps 14, 15: O of chunk c - 1
+    } else if (!CH && !gain && wq >= 2 && wgm == 2 && c > 0 && a.o) {  // warps 14, 15: O of chunk c - 1
       const int t = 32 * (wq - 2) + lane, tt = (c - 1) * CM + t;
       for (int j0 = 0; j0 < D; j0 += 16) {
         float v[16];
         tmem_ld16(TU + lane_base + j0, v);
         if (tt < a.T) {
-          const size_t base = tok_index(a, b, tt, h) * D + j0;
+          const size_t base = tok_index(a, o.b, tt, o.h) * D + j0;
           if (a.odt == KDN_BF16) {
             uint4 *dst = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(a.o) + base);
             dst[0] = pack_bf8(v);
@@ -919,18 +964,13 @@ __global__ void __launch_bounds__(WT, 1)
     const bool oor = !SV && s_oor[c & 1] != 0;
     auto issue_next = [&]() {
       if (c + 1 < NC) {
-        issue_raw(c + 1);
-        issue_q(c + 1);
-        for (int s = 0; s < 2; ++s) tma_prefetch_4d(&mv, 64 * s, h, (c + 1) * CM, b);
+        const Job n = job(c + 1);
+        issue_raw(n);
+        issue_q(n);
+        if (!CH)
+          for (int s = 0; s < 2; ++s) tma_prefetch_4d(&mv, 64 * s, n.h, n.ct * CM, n.b);
       }
-      if (c + 2 < NC) {  // chunk c + 2 into L2: its tiles are loaded during chunk c + 1
-        for (int s = 0; s < 2; ++s) {
-          tma_prefetch_4d(&mk, 64 * s, h, (c + 2) * CM, b);
-          tma_prefetch_4d(&mg, 64 * s, h, (c + 2) * CM, b);
-          tma_prefetch_4d(&mw, 64 * s, h, (c + 2) * CM, b);
-          tma_prefetch_4d(&mq, 64 * s, h, (c + 2) * CM, b);
-        }
-      }
+      if (c + 2 < NC) prefetch(job(c + 2));  // into L2: its tiles are loaded during chunk c + 1
     };
     if (warp_u == 4 && !oor) {
       tc_fence_after();
@@ -980,7 +1020,7 @@ __global__ void __launch_bounds__(WT, 1)
           *reinterpret_cast<float4 *>(sT + t * LT + s0 + 4 * u) = o;
         }
       }
-    } else if (wgm == 0) {
+    } else if (wgm == 0 && wq >= 2) {
       // A'_qk rows 64..127, lower triangle: columns 16g .. 16g + 15 -> fp16 pairs in
       // columns 8g .. 8g + 7 (each column is read before it is overwritten)
       const int t = 32 * (wq - 2) + lane;
@@ -1001,10 +1041,17 @@ __global__ void __launch_bounds__(WT, 1)
                                                (16 * g + 2 * j + 1 <= t) ? v[2 * j + 1] : 0.f);
           hv[j] = __uint_as_float(*reinterpret_cast<const uint32_t *>(&h2));
         }
-        tmem_st8(TD1 + lane_base + 8 * g, hv);
+        if (CH) {
+#pragma unroll
+          for (int w = 0; w < 2; ++w)
+            *reinterpret_cast<float4 *>(pre + Pre<SV>::Aq + chunk_off(t, 2 * g + w)) =
+                make_float4(hv[4 * w], hv[4 * w + 1], hv[4 * w + 2], hv[4 * w + 3]);
+        }
+        if (!CH || SV) tmem_st8(TD1 + lane_base + 8 * g, hv);
       }
     }
-    {  // S_in -> fp16 (MN-major B of MMA-KS); diag(gamma_C) S_in back to TMEM
+    if (CH && !SV && mt < D) reinterpret_cast<float *>(pre + Pre<SV>::gC)[mt] = s_gC[mt];
+    if constexpr (!CH) {  // S_in -> fp16 (MN-major B of MMA-KS); diag(gamma_C) S_in back to TMEM
       const int i = 32 * wq + lane;
       const float gC = s_gC[i];
       for (int g = wgm; g < 8; g += 3) {
@@ -1024,7 +1071,7 @@ __global__ void __launch_bounds__(WT, 1)
     bar_sync(kBarMain, kMain);
     tc_fence_after();
     // MMA-KS: TU = [-Kbar; Qbar] S_in (fp16), while the CUDA cores solve
-    if (warp_u == 4) {
+    if (!CH && warp_u == 4) {
       const uint32_t lead = elect_one();
       const uint64_t A1 = sw128_desc(smem_u32(as1), 16, 1024), B1 = sw128_desc(smem_u32(s16), 16384, 1024);
 #pragma unroll
@@ -1034,7 +1081,10 @@ __global__ void __launch_bounds__(WT, 1)
     }
     // (the copies of the context tiles are issued one per warp, by warps with nothing else to
     // do at that point: each costs its warp a few hundred cycles)
-    if (SV && lane == 0) {
+    if (CH && lane == 0 && (warp == 11 || warp == 14)) {
+      bulk_s2g(pre + Pre<SV>::KQ + (warp == 14) * 16384, as1 + (warp == 14) * 16384, 16384);
+      bulk_commit();
+    } else if (!CH && SV && lane == 0) {
       if (warp == 10) bulk_s2g(ctx + kCtxS, s16, 32768);
       else if (ext && (warp == 11 || warp == 14))
         bulk_s2g(ctx + kCtxKQ + (warp == 14) * 16384 + 8192, as1 + (warp == 14) * 16384 + 8192, 8192);
@@ -1047,6 +1097,7 @@ __global__ void __launch_bounds__(WT, 1)
     //          4, 5, 8, 9, 12, 13 while warps 6, 7 solve the diagonal blocks
     {
       auto y_side = [&]() {
+        if (CH) return;
         const bool ks_ok = mma_wait_main();  // MMA-KS
         const bool v_ok = mbar_wait(bar_v, c & 1, kWait);
         mine = ks_ok && v_ok && mine;
@@ -1066,17 +1117,24 @@ __global__ void __launch_bounds__(WT, 1)
         }
       };
       wy_inverse(mt, sT, sA, sX, sY, s_r + 64 * (c & 1), s_s, s_is, awu, y_side);
-      if (wq >= 2) ++mph;  // MMA-KS, observed by the Y warps
+      if (!CH && wq >= 2) ++mph;  // MMA-KS, observed by the Y warps
     }
     fence_proxy_async();
     tc_fence_before();
     bar_sync(kBarMain, kMain);
 
     // ---- [5] (context only) -W = A (-Kbar) into TW, then to the context
+    if (CH && !SV) {
+      if (lane == 0 && warp == 14) {
+        bulk_s2g(pre + Pre<SV>::A, awu, 8192);
+        bulk_commit();
+      }
+      if (mt < CM) reinterpret_cast<float *>(pre + Pre<SV>::s)[mt] = s_s[mt];
+    }
     if (SV) {
       if (lane == 0 && warp >= 14) {
         if (warp == 14) bulk_s2g(ctx + kCtxA, awu, 8192);
-        else bulk_s2g(ctx + kCtxY, vr, 16384);  // Y, before R' is written over it
+        else if (!CH) bulk_s2g(ctx + kCtxY, vr, 16384);  // Y, before R' is written over it
         bulk_commit();
       }
       if (warp_u == 4) {
@@ -1134,6 +1192,7 @@ __global__ void __launch_bounds__(WT, 1)
       }
     }
 
+    if (CH) continue;  // the rest needs the memory
     // ---- [7] MMA-R: TW = [A; .] Y = [R; 0]  (fp16)
     if (warp_u == 4) {
       tc_fence_after();
@@ -1188,13 +1247,16 @@ __global__ void __launch_bounds__(WT, 1)
     }
   }
 
-  if (!failed && NC > 0) {
+  if (!CH && !failed && NC > 0) {
     if (!gain) mine = mma_wait_main() && mine;  // MMA-O / MMA-S2 of the last chunk
     tc_fence_before();
     failed = !__syncthreads_and(mine);
     tc_fence_after();
   }
-  if (!failed) {
+  if (CH && !failed) {
+    // (nothing is in flight but the copies of the records, awaited below)
+  } else if (!failed) {
+    const Job o = job(NC - 1);
     if (!gain && wq >= 2 && NC > 0 && a.o) {  // O of the last chunk
       const int t = 32 * (wq - 2) + lane, tt = (NC - 1) * CM + t;
       for (int g = wgm; g < 8; g += 3) {
@@ -1202,7 +1264,7 @@ __global__ void __launch_bounds__(WT, 1)
         const int j0 = 16 * g;
         tmem_ld16(TU + lane_base + j0, v);
         if (tt < a.T) {
-          const size_t base = tok_index(a, b, tt, h) * D + j0;
+          const size_t base = tok_index(a, o.b, tt, o.h) * D + j0;
           if (a.odt == KDN_BF16) {
             uint4 *dst = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(a.o) + base);
             dst[0] = pack_bf8(v);
@@ -1239,10 +1301,416 @@ __global__ void __launch_bounds__(WT, 1)
       }
     }
   }
-  if (SV && lane == 0) bulk_wait_all();
+  if ((SV || CH) && lane == 0) bulk_wait_all();
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tbase, 512);
+}
+
+// ---------------------------------------------------------------------------
+// k_wy_gain: the uncertainty entering every chunk, one CTA per sequence: nothing but the serial
+// chain of p, with the operations of gain_chunk.  Warps 4..15 form alpha, omega and mu k^2 / r
+// half a chunk ahead of warps 0..3, whose loop is the chain alone (~45 cycles a token).  With
+// the inputs loaded by the chain's own threads 16 tokens ahead it took 13 K cycles a chunk.
+constexpr int kBarFull = 1, kBarEmpty = 3, kBarProd = 5;  // (full, empty: + half of the chunk)
+constexpr int kProd = WT - 128;
+constexpr int SG_RAW = 49152, SG_X = 2 * SG_RAW, SG_HALF = 3 * 32 * D * 4, SG_SS = SG_X + 2 * SG_HALF;
+constexpr int SG_MR = SG_SS + 16 * D * 4, SG_BAR = SG_MR + 2 * CM * 4, SG_SMEM = SG_BAR + 64 + 1024;
+static_assert(SG_SMEM <= 232448, "shared memory");
+
+template <int SV, int LG>
+__global__ void __launch_bounds__(WT, 1)
+    k_wy_gain(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mg,
+              const __grid_constant__ CUtensorMap mw, const Args a, float *pin) {
+  extern __shared__ unsigned char smraw[];
+  unsigned char *sm =
+      reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
+  float *s_ss = reinterpret_cast<float *>(sm + SG_SS), *s_mr = reinterpret_cast<float *>(sm + SG_MR);
+  uint64_t *bars = reinterpret_cast<uint64_t *>(sm + SG_BAR);
+  int *s_oor = reinterpret_cast<int *>(bars + 2);
+  const int tid = threadIdx.x, bh = blockIdx.x, b = bh / a.H, h = bh % a.H, NC = (a.T + CM - 1) / CM;
+  auto alpha = [&](int half) { return reinterpret_cast<float *>(sm + SG_X + half * SG_HALF); };  // then omega, u
+  if (tid == 0) {
+    mbar_init(bars, 1);
+    mbar_init(bars + 1, 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  if (tid < D) {  // ---- the chain
+    float p = a.p0 ? a.p0[(size_t)bh * D + tid] : 1.f;
+    for (int c = 0; c < NC; ++c) {
+      pin[((size_t)bh * NC + c) * D + tid] = p;
+#pragma unroll 1
+      for (int half = 0; half < 2; ++half) {
+        bar_sync(kBarFull + half, WT);
+        const float *xa = alpha(half) + tid, *xw = xa + 32 * D, *xu = xw + 32 * D;
+        if (!SV && s_oor[c & 1]) {  // range mode (see gain_chunk)
+#pragma unroll 8
+          for (int t = 0; t < 32; ++t) {
+            const float al = xa[t * D], ph = fmaf(al * al, p, xw[t * D]);
+            p = ph * rcpf(fmaf(xu[t * D], ph, 1.f));
+          }
+        } else {
+#pragma unroll
+          for (int t = 0; t < 32; ++t) {
+            const float al = xa[t * D], ph = fmaf(al * al, p, xw[t * D]);
+            const float x = rcpf(al * fmaf(xu[t * D], ph, 1.f));
+            p = ph * (x * al);
+          }
+        }
+        if (c + 1 < NC) bar_arrive(kBarEmpty + half, WT);
+      }
+    }
+    if (a.pT) a.pT[(size_t)bh * D + tid] = p;
+  } else {  // ---- its inputs
+    const int pt = tid - D;
+    auto issue = [&](int c) {
+      unsigned char *d = sm + (c & 1) * SG_RAW;
+      mbar_expect_tx(bars + (c & 1), SG_RAW);
+      for (int s = 0; s < 2; ++s) {
+        tma_load_4d(d + s * 8192, &mk, bars + (c & 1), 64 * s, h, c * CM, b);
+        tma_load_4d(d + 16384 + s * 8192, &mg, bars + (c & 1), 64 * s, h, c * CM, b);
+        tma_load_4d(d + 32768 + s * 8192, &mw, bars + (c & 1), 64 * s, h, c * CM, b);
+      }
+    };
+    __nv_bfloat16 znext = __float2bfloat16_rn(0.f);
+    auto load_r = [&](int c) {
+      if (pt < CM && c < NC)
+        znext = static_cast<const __nv_bfloat16 *>(a.r)[tok_index(a, b, min(c * CM + pt, a.T - 1), h)];
+    };
+    auto lga = [&](float x) { return LG ? -softplus_w(-x) : x; };
+    if (pt == 0) {
+      issue(0);
+      if (NC > 1) issue(1);
+    }
+    load_r(0);
+    bool ok = true;
+    for (int c = 0; c < NC; ++c) {
+      const int left = a.T - c * CM;  // tokens past T: alpha 1, omega 0, u 0
+      float *mr = s_mr + (c & 1) * CM;
+      if (pt < CM) {
+        const float z = __bfloat162float(znext), r = LG ? a.rmin + softplus_w(z) : z;
+        mr[pt] = pt < left ? a.mu / r : 0.f;
+      }
+      load_r(c + 1);
+      ok = mbar_wait(bars + (c & 1), (c >> 1) & 1, kWait) && ok;
+      const unsigned char *d = sm + (c & 1) * SG_RAW;
+      auto raw = [&](int which, int t, int i) {  // channels i, i + 1 of token t
+        return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(d + which * 16384 + (i >> 6) * 8192 +
+                                                                            sw128_off(t, i & 63)));
+      };
+      if (SV) {
+        bar_sync(kBarProd, kProd);
+      } else {  // does a channel leave the referenced range?  G_C summed in gain_chunk's order
+        for (int e = pt; e < 16 * (D / 2); e += kProd) {  // four tokens of two channels
+          const int i = 2 * (e & 63), t = 4 * (e >> 6);
+          float2 x[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float2 y = raw(1, t + j, i);
+            x[j] = t + j < left ? make_float2(lga(y.x), lga(y.y)) : make_float2(0.f, 0.f);
+          }
+          *reinterpret_cast<float2 *>(s_ss + (e >> 6) * D + i) =
+              make_float2((x[0].x + x[1].x) + (x[2].x + x[3].x), (x[0].y + x[1].y) + (x[2].y + x[3].y));
+        }
+        bar_sync(kBarProd, kProd);
+        float GC = 0.f;
+        if (pt < D)
+          for (int sg = 0; sg < 8; ++sg) GC += s_ss[2 * sg * D + pt] + s_ss[(2 * sg + 1) * D + pt];
+        const bool oor = bar_or(kBarProd, kProd, pt < D && 0.5f * GC < kMinHalfG);
+        if (pt == 0) s_oor[c & 1] = oor ? 1 : 0;
+      }
+#pragma unroll 1
+      for (int half = 0; half < 2; ++half) {
+        if (c > 0) bar_sync(kBarEmpty + half, WT);
+        float *xa = alpha(half), *xw = xa + 32 * D, *xu = xw + 32 * D;
+        for (int e = pt; e < 16 * (D / 2); e += kProd) {  // two tokens of two channels
+          const int i = 2 * (e & 63), t0 = 2 * (e >> 6);
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const int t = 32 * half + t0 + j, o = (t0 + j) * D + i;
+            const bool live = t < left;
+            const float2 k = raw(0, t, i), x = raw(1, t, i), y = raw(2, t, i);
+            const float m = mr[t];
+            float2 al = make_float2(ex2f(lga(x.x) * kLog2e), ex2f(lga(x.y) * kLog2e));
+            float2 w = LG ? make_float2(softplus_w(y.x), softplus_w(y.y)) : y;
+            if (!live) {
+              al = make_float2(1.f, 1.f);
+              w = make_float2(0.f, 0.f);
+            }
+            *reinterpret_cast<float2 *>(xa + o) = al;
+            *reinterpret_cast<float2 *>(xw + o) = w;
+            *reinterpret_cast<float2 *>(xu + o) = make_float2(k.x * k.x * m, k.y * k.y * m);
+          }
+        }
+        bar_arrive(kBarFull + half, WT);
+      }
+      bar_sync(kBarProd, kProd);  // the raw tiles have been read
+      if (pt == 0 && c + 2 < NC) issue(c + 2);
+    }
+    if (!ok) atomicExch(a.status, (unsigned)KDN_ERR_TIMEOUT);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// k_wy_state: the memory over the chunks of one sequence, from the records of the chunk part:
+//   TU = [-Kbar; Qbar] S;  Y = V + TU;  R = A Y;  R' = R / s;  O = TU + A'_qk R';
+//   S = gamma_C S + K'^T R'.
+// One CTA per sequence; warp w: TMEM lanes 32 (w % 4) .., columns by w / 4.  A chunk's
+// operands (80 KB) are double-buffered bulk copies; O is stored beside the next chunk's first
+// product (TU has two buffers).
+constexpr int SB_KQ = 0, SB_KT = 32768, SB_AA = 49152, SB_V = 65536, SB_SC = 81920, SB_BUF = 82944;
+constexpr int SO_S16 = 2 * SB_BUF, SO_R = SO_S16 + 32768, SO_BARS = SO_R + 16384, ST_SMEM = SO_BARS + 64 + 1024;
+static_assert(SB_BUF % 1024 == 0 && ST_SMEM <= 232448, "shared memory");
+
+template <int SV>
+__global__ void __launch_bounds__(WT, 1) k_wy_state(const __grid_constant__ CUtensorMap mv, const WyParams P) {
+  using R = Pre<SV>;
+  const Args &a = P.a;
+  extern __shared__ unsigned char smraw[];
+  unsigned char *sm =
+      reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
+  unsigned char *s16 = sm + SO_S16, *rst = sm + SO_R;
+  uint64_t *bars = reinterpret_cast<uint64_t *>(sm + SO_BARS);
+  uint64_t *bar_ld = bars, *bar_mma = bars + 2, *bar_o = bars + 3;
+  uint32_t *s_tbase = reinterpret_cast<uint32_t *>(bars + 4);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wq = warp & 3, wg = warp >> 2;
+  const int bh = blockIdx.x, b = bh / a.H, h = bh % a.H, NC = (a.T + CM - 1) / CM;
+  const int warp_u = __shfl_sync(0xffffffffu, warp, 0);
+  const uint32_t lane_base = (uint32_t)(32 * wq) << 16;
+  if (tid == 0) {
+    mbar_init(bar_ld, 8);
+    mbar_init(bar_ld + 1, 8);
+    mbar_init(bar_mma, 1);
+    mbar_init(bar_o, 1);
+    fence_mbar_init();
+    prefetch_tmap(&mv);
+  }
+  if (warp == 0) {
+    tmem_alloc(s_tbase, 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t TS = *s_tbase, TW = TS + 128, TUb = TS + 256;
+  auto record = [&](int c) { return P.pre + ((size_t)bh * NC + c) * P.prec; };
+  auto issue = [&](int c) {  // lane 0 of warps 8..15
+    const unsigned char *rec = record(c);
+    unsigned char *d = sm + (c & 1) * SB_BUF;
+    uint64_t *bar = bar_ld + (c & 1);
+    switch (lane == 0 ? warp : -1) {
+      case 8: mbar_expect_tx(bar, 16384); bulk_g2s(d + SB_KQ, rec + R::KQ, 16384, bar); break;
+      case 9: mbar_expect_tx(bar, 16384); bulk_g2s(d + SB_KQ + 16384, rec + R::KQ + 16384, 16384, bar); break;
+      case 10: mbar_expect_tx(bar, 16384); bulk_g2s(d + SB_KT, rec + R::Kt, 16384, bar); break;
+      case 11: mbar_expect_tx(bar, 8192); bulk_g2s(d + SB_AA, rec + R::A, 8192, bar); break;
+      case 12: mbar_expect_tx(bar, 8192); bulk_g2s(d + SB_AA + 8192, rec + R::Aq, 8192, bar); break;
+      case 13: mbar_expect_tx(bar, 8192); tma_load_4d(d + SB_V, &mv, bar, 0, h, c * CM, b); break;
+      case 14: mbar_expect_tx(bar, 8192); tma_load_4d(d + SB_V + 8192, &mv, bar, 64, h, c * CM, b); break;
+      case 15:
+        mbar_expect_tx(bar, 768);
+        bulk_g2s(d + SB_SC, rec + R::gC, 512, bar);
+        bulk_g2s(d + SB_SC + 512, rec + R::s, 256, bar);
+        break;
+    }
+  };
+  issue(0);
+  const int i = 32 * wq + lane, j0 = 32 * wg;  // this thread's row and first column of S
+  for (int c0 = 0; c0 < 32; c0 += 16) {
+    float v[16];
+    if (a.S0) {
+      const float4 *src = reinterpret_cast<const float4 *>(a.S0 + ((size_t)bh * D + i) * D + j0 + c0);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float4 x = src[u];
+        v[4 * u] = x.x; v[4 * u + 1] = x.y; v[4 * u + 2] = x.z; v[4 * u + 3] = x.w;
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < 16; ++u) v[u] = 0.f;
+    }
+    tmem_st16(TS + lane_base + j0 + c0, v);
+  }
+  tmem_st_wait();
+  auto store_o = [&](int c) {  // O of chunk c: rows 64..127 of its TU, 32 columns a thread
+    const int t = 32 * (wq - 2) + lane, tt = c * CM + t;
+    for (int c0 = 0; c0 < 32; c0 += 16) {
+      float v[16];
+      tmem_ld16(TUb + (c & 1) * 128 + lane_base + j0 + c0, v);
+      if (tt < a.T) {
+        const size_t base = tok_index(a, b, tt, h) * D + j0 + c0;
+        if (a.odt == KDN_BF16) {
+          uint4 *dst = reinterpret_cast<uint4 *>(static_cast<__nv_bfloat16 *>(a.o) + base);
+          dst[0] = pack_bf8(v);
+          dst[1] = pack_bf8(v + 8);
+        } else {
+          float4 *dst = reinterpret_cast<float4 *>(static_cast<float *>(a.o) + base);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) dst[u] = make_float4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
+        }
+      }
+    }
+  };
+  uint32_t mph = 0;
+  auto mma_wait = [&]() -> bool {
+    const bool r = mbar_wait(bar_mma, mph & 1, kWait);
+    ++mph;
+    tc_fence_after();
+    return r;
+  };
+  const uint32_t id_16 = idesc_f16(128, 128, 0, 1);  // A K-major, B MN-major
+  bool ok = true;
+  for (int c = 0; c < NC; ++c) {
+    unsigned char *d = sm + (c & 1) * SB_BUF, *vr = d + SB_V;
+    unsigned char *ctx = SV ? P.save_S + ((size_t)bh * NC + c) * P.rec : nullptr;
+    const float *sc = reinterpret_cast<const float *>(d + SB_SC);
+    const uint32_t TU = TUb + (c & 1) * 128;
+    // ---- [1] S -> fp16; diag(gamma_C) S back
+    ok = mbar_wait(bar_ld + (c & 1), (c >> 1) & 1, kWait) && ok;
+    if (c > 0) ok = mma_wait() && ok;  // MMA-S2 of chunk c - 1
+    if (SV && lane == 0) bulk_wait_read();  // its S, Y and R tiles have left shared memory
+    if (SV) __syncthreads();
+    {
+      const float gC = sc[i];
+#pragma unroll
+      for (int c0 = 0; c0 < 32; c0 += 16) {
+        float v[16];
+        tmem_ld16(TS + lane_base + j0 + c0, v);
+        const int sl = j0 >> 6, cc0 = ((j0 & 63) + c0) >> 3;
+        sm16(s16, sl * 16384 + chunk_off(i, cc0)) = pack_h8(v);
+        sm16(s16, sl * 16384 + chunk_off(i, cc0 + 1)) = pack_h8(v + 8);
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] *= gC;
+        tmem_st16(TS + lane_base + j0 + c0, v);
+      }
+    }
+    tmem_st_wait();
+    fence_proxy_async();
+    tc_fence_before();
+    if (!__syncthreads_and(ok)) {
+      ok = false;
+      break;
+    }
+    // ---- [2] MMA-KS; the next chunk's operands; O of chunk c - 1
+    if (warp_u == 0) {
+      tc_fence_after();
+      const uint32_t lead = elect_one();
+      const uint64_t A1 = sw128_desc(smem_u32(d + SB_KQ), 16, 1024), B1 = sw128_desc(smem_u32(s16), 16384, 1024);
+#pragma unroll
+      for (int kk = 0; kk < 8; ++kk)
+        umma_if(lead, TU, step(A1, (kk >> 2) * 16384 + (kk & 3) * 32), step(B1, kk * 2048), id_16, kk > 0);
+      commit_if(lead, bar_mma);
+    }
+    if (c > 0) ok = mbar_wait(bar_o, (c - 1) & 1, kWait) && ok;  // MMA-O of chunk c - 1: its buffer is free
+    if (c + 1 < NC) issue(c + 1);
+    if (SV && tid == 32) {
+      bulk_s2g(ctx + kCtxS, s16, 32768);
+      bulk_commit();
+    }
+    if (wq >= 2 && c > 0 && a.o) {
+      tc_fence_after();
+      store_o(c - 1);
+      tc_fence_before();
+    }
+    ok = mma_wait() && ok;
+    // ---- [3] Y = V - Kbar S_in -> fp16 over V
+    if (wq < 2) {
+      for (int c0 = 0; c0 < 32; c0 += 16) {
+        float v[16], vv[16];
+        const int jj = j0 + c0, sl = jj >> 6, cc0 = (jj & 63) >> 3;
+        tmem_ld16(TU + lane_base + jj, v);
+        const uint32_t o0 = sl * 8192 + chunk_off(i, cc0), o1 = sl * 8192 + chunk_off(i, cc0 + 1);
+        unpack_bf8(sm16(vr, o0), vv);
+        unpack_bf8(sm16(vr, o1), vv + 8);
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] += vv[u];
+        sm16(vr, o0) = pack_h8(v);
+        sm16(vr, o1) = pack_h8(v + 8);
+      }
+    }
+    fence_proxy_async();
+    tc_fence_before();
+    __syncthreads();
+    // ---- [4] MMA-R: TW = [A; A'_qk] Y (rows 0..63: R)
+    const uint64_t AA = sw128_desc(smem_u32(d + SB_AA), 16, 1024), VR = sw128_desc(smem_u32(vr), 8192, 1024);
+    if (warp_u == 0) {
+      tc_fence_after();
+      const uint32_t lead = elect_one();
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) umma_if(lead, TW, step(AA, kk * 32), step(VR, kk * 2048), id_16, kk > 0);
+      commit_if(lead, bar_mma);
+    }
+    if (SV && tid == 64) {
+      bulk_s2g(ctx + kCtxY, vr, 16384);
+      bulk_commit();
+      bulk_wait_read();  // R' is written over it
+    }
+    ok = mma_wait() && ok;
+    if (SV) __syncthreads();
+    // ---- [5] R' = diag(1/s) R -> fp16 over Y
+    if (wq < 2) {
+      const float ist = rcpf(sc[D + i]);
+      for (int c0 = 0; c0 < 32; c0 += 16) {
+        float v[16];
+        const int jj = j0 + c0, sl = jj >> 6, cc0 = (jj & 63) >> 3;
+        const uint32_t o0 = sl * 8192 + chunk_off(i, cc0), o1 = sl * 8192 + chunk_off(i, cc0 + 1);
+        tmem_ld16(TW + lane_base + jj, v);
+        if (SV) {
+          sm16(rst, o0) = pack_h8(v);
+          sm16(rst, o1) = pack_h8(v + 8);
+        }
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] *= ist;
+        sm16(vr, o0) = pack_h8(v);
+        sm16(vr, o1) = pack_h8(v + 8);
+      }
+    }
+    fence_proxy_async();
+    tc_fence_before();
+    __syncthreads();
+    // ---- [6] MMA-S2 (S += K'^T R'), which the next chunk waits for, then MMA-O (rows 64..127
+    //          of TU += A'_qk R')
+    if (warp_u == 0) {
+      tc_fence_after();
+      const uint32_t lead = elect_one();
+      const uint64_t KT = sw128_desc(smem_u32(d + SB_KT), 16, 1024);
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) umma_if(lead, TS, step(KT, kk * 32), step(VR, kk * 2048), id_16, 1);
+      commit_if(lead, bar_mma);
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) umma_if(lead, TU, step(AA, kk * 32), step(VR, kk * 2048), id_16, 1);
+      commit_if(lead, bar_o);
+    }
+    if (SV && tid == 96) {
+      bulk_s2g(ctx + kCtxR, rst, 16384);
+      bulk_commit();
+    }
+  }
+  if (ok && NC > 0) ok = mma_wait() && mbar_wait(bar_o, (NC - 1) & 1, kWait);
+  if (__syncthreads_and(ok)) {
+    tc_fence_after();
+    if (wq >= 2 && a.o) store_o(NC - 1);
+    if (a.ST) {
+      for (int c0 = 0; c0 < 32; c0 += 16) {
+        float v[16];
+        tmem_ld16(TS + lane_base + j0 + c0, v);
+        float4 *dst = reinterpret_cast<float4 *>(a.ST + ((size_t)bh * D + i) * D + j0 + c0);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) dst[u] = make_float4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
+      }
+    }
+  } else if (tid == 0) {
+    atomicExch(a.status, (unsigned)KDN_ERR_TIMEOUT);
+    // copies and MMAs in flight land before the CTA's memory goes away
+    for (int k = 0; k < 4; ++k) {
+      mbar_wait(bars + k, 0, kDrain);
+      mbar_wait(bars + k, 1, kDrain);
+    }
+  }
+  if (SV && lane == 0) bulk_wait_all();
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(TS, 512);
 }
 
 }  // namespace
@@ -1253,24 +1721,79 @@ bool wy_fwd_supported(const Args &a, bool save) {
          a.dtype == KDN_BF16 && a.dk == D && a.dv == D && a.T > 0 && a.chunk != 32;
 }
 
-kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S, float *save_p) {
+// Where the three kernels finish sooner than the one, in thousands of cycles as measured: the
+// one takes 17 a chunk with one CTA per sequence; k_wy_gain and k_wy_state together 10 a chunk
+// with one CTA per sequence, the chunk part 18 a chunk on any SM, and the two more launches with
+// their first tiles 50.  Post-activation gates, the three and the one in us: B1 H16 T824 120 and
+// 131, T2047 238 and 282, T8191 799 and 1062, B2 H16 T2047 269 and 290, but B3 H16 T640 126 and
+// 107, B4 H16 T2047 328 and 297.  Fewer than 96 chunks in all are left to the one kernel.
+bool wy_split_sizes(const Args &a) {
+  if (!wy_fwd_supported(a, false)) return false;
+  const long long bh = (long long)a.B * a.H, nc = (a.T + CM - 1) / CM, waves = (bh + kSms - 1) / kSms;
+  if (bh * nc < 96) return false;
+  return waves * nc * 10 + (bh * nc + kSms - 1) / kSms * 18 + 50 < waves * nc * 17;
+}
+
+bool wy_split_save(const Args &a) {
+  return wy_split_sizes(a) && fused_ctx_record_bytes(a) > (size_t)kCtxBytes;
+}
+
+size_t wy_split_workspace_bytes(const Args &a) {
+  if (!wy_split_sizes(a)) return 0;
+  return (size_t)a.B * a.H * ((a.T + CM - 1) / CM) * (kPreBytes + D * sizeof(float));
+}
+
+namespace {
+template <int SV, int LG>
+kdn_status_t launch_wy(const WyParams &W, bool split, cudaStream_t s) {
+  const Args &a = W.a;
+  CUtensorMap mk, mg, mw, mv, mq;
+  if (!make_map(&mk, a.k, a) || !make_map(&mg, a.g, a) || !make_map(&mw, a.omega, a) ||
+      !make_map(&mv, a.v, a) || !make_map(&mq, a.q, a))
+    return KDN_ERR_CUDA;
+  const int bh = a.B * a.H;
+  const long long njobs = (long long)bh * ((a.T + CM - 1) / CM);
+  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  if (!split) {
+    if (cudaFuncSetAttribute(k_wy_fwd<SV, LG, 0>, attr, SMEM_BYTES) != cudaSuccess) return KDN_ERR_CUDA;
+    k_wy_fwd<SV, LG, 0><<<bh, WT, SMEM_BYTES, s>>>(mk, mg, mw, mv, mq, W);
+    return cudaGetLastError() == cudaSuccess ? KDN_OK : KDN_ERR_CUDA;
+  }
+  if (cudaFuncSetAttribute(k_wy_fwd<SV, LG, 1>, attr, SMEM_BYTES) != cudaSuccess ||
+      cudaFuncSetAttribute(k_wy_gain<SV, LG>, attr, SG_SMEM) != cudaSuccess ||
+      cudaFuncSetAttribute(k_wy_state<SV>, attr, ST_SMEM) != cudaSuccess)
+    return KDN_ERR_CUDA;
+  k_wy_gain<SV, LG><<<bh, WT, SG_SMEM, s>>>(mk, mg, mw, a, const_cast<float *>(W.pin));
+  if (cudaGetLastError() != cudaSuccess) return KDN_ERR_CUDA;
+  k_wy_fwd<SV, LG, 1><<<(unsigned)(njobs < kSms ? njobs : kSms), WT, SMEM_BYTES, s>>>(mk, mg, mw, mv, mq, W);
+  if (cudaGetLastError() != cudaSuccess) return KDN_ERR_CUDA;
+  k_wy_state<SV><<<bh, WT, ST_SMEM, s>>>(mv, W);
+  return cudaGetLastError() == cudaSuccess ? KDN_OK : KDN_ERR_CUDA;
+}
+}  // namespace
+
+// ws: room for wy_split_workspace_bytes() (null: the one kernel, unless the context has the room)
+kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S, float *save_p, char *ws) {
   if (!wy_fwd_supported(a, save_S != nullptr) || (!save_S) != (!save_p)) return KDN_ERR_UNSUPPORTED;
   WyParams P;
   P.a = a;
   P.save_S = save_S;
   P.rec = fused_ctx_record_bytes(a);
   P.save_p = save_p;
-  CUtensorMap mk, mg, mw, mv, mq;
-  if (!make_map(&mk, a.k, a) || !make_map(&mg, a.g, a) || !make_map(&mw, a.omega, a) ||
-      !make_map(&mv, a.v, a) || !make_map(&mq, a.q, a))
-    return KDN_ERR_CUDA;
-  const bool lg = a.gates == KDN_GATES_LOGITS;
-  const auto kern = save_S ? (lg ? k_wy_fwd<1, 1> : k_wy_fwd<1, 0>) : (lg ? k_wy_fwd<0, 1> : k_wy_fwd<0, 0>);
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES) !=
-      cudaSuccess)
-    return KDN_ERR_CUDA;
-  kern<<<a.B * a.H, WT, SMEM_BYTES, s>>>(mk, mg, mw, mv, mq, P);
-  return cudaGetLastError() == cudaSuccess ? KDN_OK : KDN_ERR_CUDA;
+  bool split = wy_split_sizes(a);
+  if (save_S) {
+    split = wy_split_save(a);
+    P.pre = save_S;
+    P.prec = P.rec;
+    P.pin = save_p;
+  } else {
+    split = split && ws;
+    P.pre = reinterpret_cast<unsigned char *>(ws);
+    P.prec = kPreBytes;
+    P.pin = split ? reinterpret_cast<float *>(ws + (size_t)a.B * a.H * ((a.T + CM - 1) / CM) * kPreBytes) : nullptr;
+  }
+  if (a.gates == KDN_GATES_LOGITS) return save_S ? launch_wy<1, 1>(P, split, s) : launch_wy<0, 1>(P, split, s);
+  return save_S ? launch_wy<1, 0>(P, split, s) : launch_wy<0, 0>(P, split, s);
 }
 
 }  // namespace kdn

@@ -98,6 +98,36 @@ def test_context_serves_either_gradient_type(kdn, first, then):
         check(n, gr[n], rg[n], then == "bf16")
 
 
+@pytest.mark.parametrize("out", ["f32", "bf16"])
+@pytest.mark.parametrize("B,T,H,gates,slow,fast", [
+    (1, 824, 16, "post", False, 0), (2, 1985, 14, "logits", True, 0), (1, 1537, 5, "post", False, 9.0),
+    (2, 1100, 12, "logits", False, 9.0), (1, 700, 10, "post", True, 0)])
+def test_three_kernel_forward_equals_the_one(kdn, B, T, H, gates, slow, fast, out):
+    """The chunk part and the memory part in kernels of their own run the same arithmetic: the
+    outputs are those of the one-kernel forward (a workspace without room) bit for bit, also
+    where a chunk's decay leaves the referenced range (fast: log alpha of -9)."""
+    ins, _, _ = _case(B, T, H, T + B, gates, slow)
+    if fast:  # some channels decay by e^-9 a token (logits: log sigmoid(-9))
+        ins["g"][:, T // 2:, :, ::5] = -fast
+    d = to_dev(ins)
+    x = [d[n] for n in NAMES]
+    dt = torch.float32 if out == "f32" else torch.bfloat16
+    G = kdn.KDN_GATES_LOGITS if gates == "logits" else kdn.KDN_GATES_POST
+    desc = kdn.make_desc(B, T, H, 128, 128, torch.bfloat16, out_dtype=dt, gates=G)
+    assert kdn.kdn_kernel_launches(desc, 0, 0) == 3
+    kw = dict(out_dtype=dt, gates=G)
+    for state in ((d["S0"], d["p0"]), (None, None)):
+        ws = kdn.alloc_workspace(desc, 0)
+        three = kdn.kdn_diag_fwd(*x, *state, workspace=ws, **kw)
+        one = kdn.kdn_diag_fwd(*x, *state, workspace=torch.empty(256, dtype=torch.uint8, device="cuda"), **kw)
+        saving = kdn.kdn_diag_fwd_save(*x, *state, **kw)
+        torch.cuda.synchronize()
+        assert kdn.kdn_get_device_status(ws) == 0
+        for u, v, w in zip(three, one, saving):
+            assert torch.equal(u, v)
+            assert fast or torch.equal(v, w)  # (the context keeps the referenced form)
+
+
 def test_ragged_without_scratch_runs_the_sweep(kdn):
     """A workspace that holds only the status word: the one-kernel sweep reads the same context."""
     ins, dST, dpT = _case(2, 449, 6, 3, "post", True)
