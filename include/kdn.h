@@ -136,6 +136,10 @@ const char *kdn_status_string(kdn_status_t status);
    (S_in, v)), and kdn_fwd_workspace_bytes includes its segment buffers
    (160 KB per (batch, head, segment), 2 KB per (batch, head, chunk), and
    2 bytes per element of o, 6 when out_dtype is KDN_BF16).
+   For sequences too few to fill the GPU but not served so, the diagonal
+   forward uses 65.5 KB per (batch, head, chunk) to run all chunks' work that
+   needs no memory in parallel (same results), and the backward of the training
+   pair with bfloat16 gradients 80 KB per chunk when T is no multiple of 64.
    A smaller workspace that still holds the single-pass layout (256 bytes)
    runs the single pass. */
 size_t kdn_fwd_workspace_bytes(const kdn_desc_t *desc, int variant);
@@ -187,9 +191,13 @@ kdn_status_t kdn_iso_bwd(const kdn_desc_t *desc, const void *q, const void *k,
    chunk the memory S entering it, its R = U - W S_in, -W, A_qk,
    A = (I + T)^-1 and (Diagonal KDN) Y = V - Kbar S_in as fp16 tiles (96 KB),
    the pre-write variance phat and the cumulative decay gamma of every
-   (token, channel) in float32 (64 KB), per-token scalars (2 KB), and the
+   (token, channel) in float32 (64 KB), per-token scalars (2 KB), for most
+   diagonal problems of 96 chunks and more also [-Kbar; Qbar] and
+   K'^T (48 KB), and the
    float32 uncertainty p entering it.  kdn_diag_bwd_saved is kdn_diag_bwd that starts from that
-   context instead of recomputing the forward (same gradients, one kernel).
+   context instead of recomputing the forward (same gradients).  The diagonal
+   backward may use dq, dk, dv, dg and domega as scratch before it writes them:
+   they overlap no input.
    kdn_iso_fwd_save / kdn_iso_bwd_saved are the same for the Isotropic KDN.
    Served for bfloat16 activations, dk = dv = 128 and the default chunk; for
    every other descriptor kdn_saved_bytes() returns 0 and the calls return
@@ -287,7 +295,8 @@ kdn_status_t kdn_iso_decode_step(const kdn_desc_t *desc, const void *q,
    single-pass workspace (kdn_fwd_workspace_bytes without the segment buffers
    of the sequence-parallel forward) exceeds it is rejected with
    KDN_ERR_WORKSPACE before anything runs.  The sequence-parallel forward is
-   used when its larger workspace fits the array, else the single pass.  The
+   used when its larger workspace fits the array, else the single pass (in one
+   kernel, which uses the array for its status word only).  The
    first call on a device looks up the array's device address
    (cudaGetSymbolAddress, with that device current) and caches it with the
    device's CUDA context; a later call under another context (after a device

@@ -110,7 +110,9 @@ struct SplitParams {
 };
 
 // ---------------------------------------------------------------------------
-// k_bwd_state.  16 warps; warp w holds TMEM lanes 32 (w % 4) .. + 31 and value columns
+// k_bwd_state.  Bound by HBM: 104 KB read and 64 KB written per chunk, 255 us at B8 H16 T4096
+// (5.4 TB/s); with few sequences by its chain, ~6 K cycles a chunk (94 us at B2 H16 T1999).
+// 16 warps; warp w holds TMEM lanes 32 (w % 4) .. + 31 and value columns
 // 32 (w / 4) .. + 31 of dS.  Per chunk: dS -> fp16 tile; MMA dR; dR -> fp16 hi + lo;
 // MMA dS.  A_qk, K' and dO are double-buffered bulk copies; Qbar, W (needed
 // last) and S_in (for dgamma_C, needed first) are loaded again as soon as they have been read.
@@ -396,7 +398,12 @@ __global__ void __launch_bounds__(BT, 1)
 }
 
 // ---------------------------------------------------------------------------
-// k_bwd_chunk.  Shared-memory map (bytes from the 1024-aligned base), with the sequence
+// k_bwd_chunk.  Bound by the chain of a chunk's stages (ncu, B2 H16 T4096: 40 % of the issue
+// slots, tensor pipe 8 %; the waits are on tensor-memory reads, barriers and instruction
+// fetches): ~32 K cycles a chunk, of which the four tensor-core rounds with their read-outs 13 K
+// and the per-channel passes 14 K.  865 us at B8 H16 T4096 (with k_bwd_state 1120; the one-kernel
+// sweep 1326), 161 us at B2 H16 T1999 logits (255; 668).
+// Shared-memory map (bytes from the 1024-aligned base), with the sequence
 // of tenants within a chunk; the next chunk's tiles arrive as their buffers fall free.
 constexpr int O_RKQ = 0;         // raw k | q, interleaved per 64-channel slab
 constexpr int O_SIN = 32 * KB;   // S_in fp16 [i][j] -> Kbar^T hi | Qbar^T hi

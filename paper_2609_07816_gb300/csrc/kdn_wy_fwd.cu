@@ -27,7 +27,9 @@
 //   MMA-KS   [-Kbar; Qbar] S_in = [-Kbar S_in; Qbar S_in]  (fp16), on the tensor
 //            cores while the CUDA cores solve
 //   solve    with L = diag(s) + strict_lower(T'), A = (I + T)^-1 = diag(s) L^-1
-//            (T = strict_lower(T') diag(1/s)) on CUDA cores in fp32.
+//            (T = strict_lower(T') diag(1/s)) on CUDA cores in fp32: diagonal blocks on two
+//            warps beside Y = V - Kbar S_in on six, the 32 x 32 products without the zero
+//            quarter of their triangular factor.
 //   MMA-R    R = U - W S_in = A (V - Kbar S_in)  (fp16; W = A Kbar, U = A V of
 //            eq. chunk-memory-wy are only formed for the backward's context)
 //   MMA-O    O = Qbar S_in + A'_qk R'          with R' = diag(1/s) R
@@ -36,9 +38,13 @@
 // chunk-memory-output-state, with A_qk = lower(A'_qk) diag(1/s).  Every MMA
 // accumulates in float32 in tensor memory.
 //
-// The chunk is a chain of dependent stages inside one CTA, and the gain (run one
-// chunk ahead on its own warps) is as long as the rest: the kernel is bound by
-// that latency, not by HBM or shared-memory throughput.  Every per-element pass
+// The chunk is a chain of dependent stages inside one CTA, and with logit gates the gain (run
+// one chunk ahead on its own warps) is as long as the rest: the kernel is bound by
+// that latency, not by HBM or shared-memory throughput.  B8 H16 T4096: 540 us (646 with the
+// solve's diagonal blocks and Y on the same warps, and MMAs issued under a divergent branch),
+// with the context 687 us (730; its copies go out one per warp, and A_qk is written
+// beside the -W product).  Few sequences: three kernels (below).
+// Every per-element pass
 // still reads and writes 8 or 16 bytes per shared-memory instruction wherever the
 // layout allows (the gain's per-channel recursion is the exception), and the
 // next chunk's TMA operations are issued from a thread outside the MMA issuer's
