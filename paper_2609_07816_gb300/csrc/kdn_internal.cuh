@@ -164,7 +164,7 @@ kdn_status_t launch_fused_fwd(const Args &a, cudaStream_t s, unsigned char *save
 bool wy_fwd_supported(const Args &a, bool save);  // save: the context-saving instantiation
 kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S = nullptr,
                            float *save_p = nullptr, char *ws = nullptr);
-// The same in three kernels (gain, chunks in parallel, memory) where these sizes gain from it:
+// The same with the gain, the chunks and the memory on CTAs of their own where these sizes gain from it:
 // with the extended context, or with this much scratch in the workspace.
 bool wy_split_sizes(const Args &a);
 bool wy_split_save(const Args &a);  // the context-saving forward

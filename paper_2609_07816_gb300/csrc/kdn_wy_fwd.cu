@@ -43,7 +43,7 @@
 // that latency, not by HBM or shared-memory throughput.  B8 H16 T4096: 540 us (646 with the
 // solve's diagonal blocks and Y on the same warps, and MMAs issued under a divergent branch),
 // with the context 687 us (730; its copies go out one per warp, and A_qk is written
-// beside the -W product).  Few sequences: three kernels (below).
+// beside the -W product).  Few sequences: k_wy_flow (below).
 // Every per-element pass
 // still reads and writes 8 or 16 bytes per shared-memory instruction wherever the
 // layout allows (the gain's per-channel recursion is the exception), and the
@@ -70,6 +70,7 @@
 // Every wait on an mbarrier is bounded; on timeout the kernel records
 // KDN_ERR_TIMEOUT in the status word, waits (bounded) for its copies in flight,
 // frees its tensor memory and returns.
+#include <algorithm>
 #include <type_traits>
 
 #include "kdn_internal.cuh"
@@ -159,6 +160,8 @@ __device__ __forceinline__ uint32_t sw32_off(uint32_t row, uint32_t col) {
 __device__ __forceinline__ void bar_sync(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
+// generic-proxy accesses before, async-proxy (bulk copy) accesses after, for every state space
+__device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
 __device__ __forceinline__ void bar_arrive(int id, int n) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
@@ -457,10 +460,51 @@ struct WyParams {
   // CH: records of the per-chunk operands (SV: the context records), what enters every chunk
   unsigned char *pre;
   size_t prec;
-  const float *pin;       // [BH][NC][128]
+  float *pin;             // [BH][NC][128], preset to kUnset
+  unsigned *flag;         // per chunk, fstride apart, zeroed: warps that have written their part of its record
+  size_t fstride;
 };
 
-// Per-chunk operands of the three-kernel forward, in a context record (SV) or in a record of
+// The uncertainty entering a chunk is handed over as the 4-byte value itself, in place of a
+// pattern no result has (a NaN other than the one that arithmetic gives).
+constexpr unsigned kUnset = 0xffffffffu;
+constexpr uint32_t kFlowWait = 1u << 22;  // polls
+__device__ __forceinline__ bool is_unset(float p) { return __float_as_uint(p) == kUnset; }
+__device__ __forceinline__ float pin_peek(const float *q) {
+  unsigned v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(q) : "memory");
+  return __uint_as_float(v);
+}
+__device__ __forceinline__ bool pin_get(const float *q, float *p) {
+  for (uint32_t n = 0; n < kFlowWait; ++n) {
+    *p = pin_peek(q);
+    if (!is_unset(*p)) return true;
+    if (n > 64) __nanosleep(32);
+  }
+  return false;
+}
+__device__ __forceinline__ void pin_put(float *q, float p) {
+  const unsigned v = is_unset(p) ? 0x7fffffffu : __float_as_uint(p);
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(q), "r"(v) : "memory");
+}
+// One count per warp once its stores to a record are visible; a reader waits for all of them.
+constexpr unsigned kFlowWarps = WT / 32;
+__device__ __forceinline__ void publish(unsigned *flag) {
+  __threadfence();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(flag) : "memory");
+}
+__device__ __forceinline__ bool flow_wait(const unsigned *flag) {
+  for (uint32_t n = 0; n < kFlowWait; ++n) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
+    if (v >= kFlowWarps) return true;
+    if (n > 64) __nanosleep(32);
+  }
+  return false;
+}
+
+// Per-chunk operands that k_wy_flow's chunk part leaves for its memory part, in a context record (SV) or in a record of
 // their own: [-Kbar; Qbar] fp16 32 KB, K'^T fp16 [128 i][64 s] 16 KB, A fp16 8 KB, A'_qk fp16
 // 8 KB (context: in R's place until R is there), gamma_C [128], s_t [64].
 constexpr size_t kPreBytes = 66560;
@@ -477,14 +521,13 @@ struct Pre {
 // phat and gamma in float32 [64 t][128 i], s_t per token, and the uncertainty
 // entering the chunk.  The arithmetic is the same with and without it.
 
-// CH: the part of this work that needs no memory S, for the chunks blockIdx.x, + gridDim.x, ..
-// of all sequences, its results left in records for k_wy_state; the uncertainty entering
-// each chunk is known (k_wy_gain).  The same instructions, so the same bits.
+// CH: the part of this work that needs no memory S, for the chunks block, block + nblocks, ..
+// of all sequences, its results left in records for wy_state; the uncertainty entering
+// each chunk comes from wy_gain.  The same instructions, so the same bits.
 template <int SV, int LG, int CH>  // LG: g, omega, r hold the logits x, y, z of the gates
-__global__ void __launch_bounds__(WT, 1)
-    k_wy_fwd(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mg,
-             const __grid_constant__ CUtensorMap mw, const __grid_constant__ CUtensorMap mv,
-             const __grid_constant__ CUtensorMap mq, const WyParams P) {
+__device__ __forceinline__ void wy_body(const CUtensorMap &mk, const CUtensorMap &mg, const CUtensorMap &mw,
+                                        const CUtensorMap &mv, const CUtensorMap &mq, const WyParams &P,
+                                        const int block, const int nblocks) {
   const Args &a = P.a;
   extern __shared__ unsigned char smraw[];
   unsigned char *sm =
@@ -508,14 +551,14 @@ __global__ void __launch_bounds__(WT, 1)
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int wq = warp & 3, wg = warp >> 2;  // TMEM lane quarter, column group
-  const int bh = blockIdx.x;  // (not CH)
+  const int bh = block;  // (not CH)
   const int NCs = (a.T + CM - 1) / CM, BH = a.B * a.H;
   // chunks of this CTA, counted by `c` below; ct, b, h: a chunk's place in its sequence
-  const int NC = CH ? (NCs * BH - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : NCs;
+  const int NC = CH ? (NCs * BH - block + nblocks - 1) / nblocks : NCs;
   struct Job { int ct, b, h; size_t rc; };
   auto job = [&](int c) {
     Job o;
-    const int j = CH ? (int)(blockIdx.x + c * gridDim.x) : 0, q = CH ? j % BH : bh;
+    const int j = CH ? block + c * nblocks : 0, q = CH ? j % BH : bh;
     o.ct = CH ? j / BH : c;
     o.b = q / a.H;
     o.h = q % a.H;
@@ -624,7 +667,7 @@ __global__ void __launch_bounds__(WT, 1)
     if (c >= NC) return;
     const Job o = job(c);
     if (tid < CM) znext = static_cast<const __nv_bfloat16 *>(a.r)[tok_index(a, o.b, min(o.ct * CM + tid, a.T - 1), o.h)];
-    if (CH && gain) pnext = P.pin[o.rc * D + tid];
+    if (CH && gain) pnext = pin_peek(P.pin + o.rc * D + tid);
   };
   load_r(0);
 
@@ -645,7 +688,11 @@ __global__ void __launch_bounds__(WT, 1)
     const int i = tid, sb = c & 1;
     const Job o = job(c);
     const int left = a.T - o.ct * CM;  // tokens of the sequence from this chunk on
-    if (CH) p = pnext;
+    bool g_in = true;
+    if (CH) {
+      if (is_unset(pnext)) g_in = pin_get(P.pin + o.rc * D + i, &pnext);
+      p = pnext;
+    }
     float *sr = s_r + 64 * sb, *smur = s_mur + 64 * sb;
     if (tid < CM) {
       const bool live = tid < left;
@@ -661,7 +708,7 @@ __global__ void __launch_bounds__(WT, 1)
     }
     load_r(c + 1);
     bar_sync(kBarGain, 128);
-    bool g_ok = mbar_wait(bar_raw, c & 1, kWait);
+    bool g_ok = mbar_wait(bar_raw, c & 1, kWait) && g_in;
     const unsigned char *pg = rg + (i >> 6) * 8192, *pw = rw + (i >> 6) * 8192, *pk = rk + (i >> 6) * 8192;
     const int cl = i & 63;
     // element (t, i) of a raw slab: row t, 128-byte swizzle
@@ -828,6 +875,7 @@ __global__ void __launch_bounds__(WT, 1)
     }
     tmem_st_wait();
     fence_proxy_async();
+    if (CH) publish(P.flag + o.rc * P.fstride);  // K'^T
     return g_ok;
   };
 
@@ -1198,7 +1246,11 @@ __global__ void __launch_bounds__(WT, 1)
       }
     }
 
-    if (CH) continue;  // the rest needs the memory
+    if (CH) {  // the rest needs the memory
+      if (lane == 0) bulk_wait_all();  // (the records' bulk copies have been written)
+      publish(P.flag + o.rc * P.fstride);
+      continue;
+    }
     // ---- [7] MMA-R: TW = [A; .] Y = [R; 0]  (fp16)
     if (warp_u == 4) {
       tc_fence_after();
@@ -1313,11 +1365,20 @@ __global__ void __launch_bounds__(WT, 1)
   if (warp == 0) tmem_dealloc(tbase, 512);
 }
 
+template <int SV, int LG>
+__global__ void __launch_bounds__(WT, 1)
+    k_wy_fwd(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mg,
+             const __grid_constant__ CUtensorMap mw, const __grid_constant__ CUtensorMap mv,
+             const __grid_constant__ CUtensorMap mq, const WyParams P) {
+  wy_body<SV, LG, 0>(mk, mg, mw, mv, mq, P, (int)blockIdx.x, (int)gridDim.x);
+}
+
 // ---------------------------------------------------------------------------
-// k_wy_gain: the uncertainty entering every chunk, one CTA per sequence: nothing but the serial
+// wy_gain: the uncertainty entering every chunk, one CTA per sequence: nothing but the serial
 // chain of p, with the operations of gain_chunk.  Warps 4..15 form alpha, omega and mu k^2 / r
 // half a chunk ahead of warps 0..3, whose loop is the chain alone (~45 cycles a token).  With
-// the inputs loaded by the chain's own threads 16 tokens ahead it took 13 K cycles a chunk.
+// the inputs loaded by the chain's own threads 16 tokens ahead it took 13 K cycles a chunk,
+// this way 5 K (with the range test 6.5 K).
 constexpr int kBarFull = 1, kBarEmpty = 3, kBarProd = 5;  // (full, empty: + half of the chunk)
 constexpr int kProd = WT - 128;
 constexpr int SG_RAW = 49152, SG_X = 2 * SG_RAW, SG_HALF = 3 * 32 * D * 4, SG_SS = SG_X + 2 * SG_HALF;
@@ -1325,16 +1386,15 @@ constexpr int SG_MR = SG_SS + 16 * D * 4, SG_BAR = SG_MR + 2 * CM * 4, SG_SMEM =
 static_assert(SG_SMEM <= 232448, "shared memory");
 
 template <int SV, int LG>
-__global__ void __launch_bounds__(WT, 1)
-    k_wy_gain(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mg,
-              const __grid_constant__ CUtensorMap mw, const Args a, float *pin) {
+__device__ __forceinline__ void wy_gain(const CUtensorMap &mk, const CUtensorMap &mg, const CUtensorMap &mw,
+                                        const Args &a, float *pin, const int bh) {
   extern __shared__ unsigned char smraw[];
   unsigned char *sm =
       reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   float *s_ss = reinterpret_cast<float *>(sm + SG_SS), *s_mr = reinterpret_cast<float *>(sm + SG_MR);
   uint64_t *bars = reinterpret_cast<uint64_t *>(sm + SG_BAR);
   int *s_oor = reinterpret_cast<int *>(bars + 2);
-  const int tid = threadIdx.x, bh = blockIdx.x, b = bh / a.H, h = bh % a.H, NC = (a.T + CM - 1) / CM;
+  const int tid = threadIdx.x, b = bh / a.H, h = bh % a.H, NC = (a.T + CM - 1) / CM;
   auto alpha = [&](int half) { return reinterpret_cast<float *>(sm + SG_X + half * SG_HALF); };  // then omega, u
   if (tid == 0) {
     mbar_init(bars, 1);
@@ -1345,7 +1405,7 @@ __global__ void __launch_bounds__(WT, 1)
   if (tid < D) {  // ---- the chain
     float p = a.p0 ? a.p0[(size_t)bh * D + tid] : 1.f;
     for (int c = 0; c < NC; ++c) {
-      pin[((size_t)bh * NC + c) * D + tid] = p;
+      pin_put(pin + ((size_t)bh * NC + c) * D + tid, p);
 #pragma unroll 1
       for (int half = 0; half < 2; ++half) {
         bar_sync(kBarFull + half, WT);
@@ -1459,18 +1519,19 @@ __global__ void __launch_bounds__(WT, 1)
 }
 
 // ---------------------------------------------------------------------------
-// k_wy_state: the memory over the chunks of one sequence, from the records of the chunk part:
+// wy_state: the memory over the chunks of one sequence, from the records of the chunk part:
 //   TU = [-Kbar; Qbar] S;  Y = V + TU;  R = A Y;  R' = R / s;  O = TU + A'_qk R';
 //   S = gamma_C S + K'^T R'.
 // One CTA per sequence; warp w: TMEM lanes 32 (w % 4) .., columns by w / 4.  A chunk's
 // operands (80 KB) are double-buffered bulk copies; O is stored beside the next chunk's first
-// product (TU has two buffers).
+// product (TU has two buffers).  Bound by the chain of its three products and their
+// conversions, ~6 K cycles a chunk.
 constexpr int SB_KQ = 0, SB_KT = 32768, SB_AA = 49152, SB_V = 65536, SB_SC = 81920, SB_BUF = 82944;
 constexpr int SO_S16 = 2 * SB_BUF, SO_R = SO_S16 + 32768, SO_BARS = SO_R + 16384, ST_SMEM = SO_BARS + 64 + 1024;
 static_assert(SB_BUF % 1024 == 0 && ST_SMEM <= 232448, "shared memory");
 
 template <int SV>
-__global__ void __launch_bounds__(WT, 1) k_wy_state(const __grid_constant__ CUtensorMap mv, const WyParams P) {
+__device__ __forceinline__ void wy_state(const CUtensorMap &mv, const WyParams &P, const int bh) {
   using R = Pre<SV>;
   const Args &a = P.a;
   extern __shared__ unsigned char smraw[];
@@ -1481,9 +1542,10 @@ __global__ void __launch_bounds__(WT, 1) k_wy_state(const __grid_constant__ CUte
   uint64_t *bar_ld = bars, *bar_mma = bars + 2, *bar_o = bars + 3;
   uint32_t *s_tbase = reinterpret_cast<uint32_t *>(bars + 4);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wq = warp & 3, wg = warp >> 2;
-  const int bh = blockIdx.x, b = bh / a.H, h = bh % a.H, NC = (a.T + CM - 1) / CM;
+  const int b = bh / a.H, h = bh % a.H, NC = (a.T + CM - 1) / CM;
   const int warp_u = __shfl_sync(0xffffffffu, warp, 0);
   const uint32_t lane_base = (uint32_t)(32 * wq) << 16;
+  bool ok = true;
   if (tid == 0) {
     mbar_init(bar_ld, 8);
     mbar_init(bar_ld + 1, 8);
@@ -1505,6 +1567,10 @@ __global__ void __launch_bounds__(WT, 1) k_wy_state(const __grid_constant__ CUte
     const unsigned char *rec = record(c);
     unsigned char *d = sm + (c & 1) * SB_BUF;
     uint64_t *bar = bar_ld + (c & 1);
+    if (lane == 0 && warp >= 8) {  // (a record that never comes is read as it is: the call fails)
+      ok = flow_wait(P.flag + ((size_t)bh * NC + c) * P.fstride) && ok;
+      fence_proxy_async_all();
+    }
     switch (lane == 0 ? warp : -1) {
       case 8: mbar_expect_tx(bar, 16384); bulk_g2s(d + SB_KQ, rec + R::KQ, 16384, bar); break;
       case 9: mbar_expect_tx(bar, 16384); bulk_g2s(d + SB_KQ + 16384, rec + R::KQ + 16384, 16384, bar); break;
@@ -1565,7 +1631,6 @@ __global__ void __launch_bounds__(WT, 1) k_wy_state(const __grid_constant__ CUte
     return r;
   };
   const uint32_t id_16 = idesc_f16(128, 128, 0, 1);  // A K-major, B MN-major
-  bool ok = true;
   for (int c = 0; c < NC; ++c) {
     unsigned char *d = sm + (c & 1) * SB_BUF, *vr = d + SB_V;
     unsigned char *ctx = SV ? P.save_S + ((size_t)bh * NC + c) * P.rec : nullptr;
@@ -1719,6 +1784,25 @@ __global__ void __launch_bounds__(WT, 1) k_wy_state(const __grid_constant__ CUte
   if (warp == 0) tmem_dealloc(TS, 512);
 }
 
+// ---------------------------------------------------------------------------
+// k_wy_flow: the three parts at once, one CTA per SM: first the gain's CTAs (one per sequence),
+// then the chunk part's, then the memory's (one per sequence).  A part waits only for CTAs of
+// lower index (bounded), so whatever of the grid is resident makes progress.  B1 H16 T824 with
+// logit gates 119 us as three launches, 78 us as one (one CTA per sequence: 143 us); training
+// forward B2 H16 T1999 302 and ~200 us (430).
+constexpr int FLOW_SMEM = SMEM_BYTES > SG_SMEM ? (SMEM_BYTES > ST_SMEM ? SMEM_BYTES : ST_SMEM)
+                                               : (SG_SMEM > ST_SMEM ? SG_SMEM : ST_SMEM);
+template <int SV, int LG>
+__global__ void __launch_bounds__(WT, 1)
+    k_wy_flow(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mg,
+              const __grid_constant__ CUtensorMap mw, const __grid_constant__ CUtensorMap mv,
+              const __grid_constant__ CUtensorMap mq, const WyParams P) {
+  const int BH = P.a.B * P.a.H, block = (int)blockIdx.x, workers = (int)gridDim.x - 2 * BH;
+  if (block < BH) wy_gain<SV, LG>(mk, mg, mw, P.a, P.pin, block);
+  else if (block < BH + workers) wy_body<SV, LG, 1>(mk, mg, mw, mv, mq, P, block - BH, workers);
+  else wy_state<SV>(mv, P, block - BH - workers);
+}
+
 }  // namespace
 
 bool wy_fwd_supported(const Args &a, bool save) {
@@ -1727,17 +1811,20 @@ bool wy_fwd_supported(const Args &a, bool save) {
          a.dtype == KDN_BF16 && a.dk == D && a.dv == D && a.T > 0 && a.chunk != 32;
 }
 
-// Where the three kernels finish sooner than the one, in thousands of cycles as measured: the
-// one takes 17 a chunk with one CTA per sequence; k_wy_gain and k_wy_state together 10 a chunk
-// with one CTA per sequence, the chunk part 18 a chunk on any SM, and the two more launches with
-// their first tiles 50.  Post-activation gates, the three and the one in us: B1 H16 T824 120 and
-// 131, T2047 238 and 282, T8191 799 and 1062, B2 H16 T2047 269 and 290, but B3 H16 T640 126 and
-// 107, B4 H16 T2047 328 and 297.  Fewer than 96 chunks in all are left to the one kernel.
+// Where k_wy_flow finishes sooner than k_wy_fwd, in thousands of cycles as measured: the one
+// takes 17 a chunk with one CTA per sequence; k_wy_flow 7 a chunk of a sequence (its memory part)
+// or 19 a chunk of all sequences over its workers, whichever is longer, and 45 until the first
+// records are there.  Post-activation gates, k_wy_flow and k_wy_fwd in us: B1 H16 T824 87 and
+// 131, T2047 161 and 282, T8191 488 and 1060, B2 H16 T2047 175 and 287, B24 H1 T257 59 and 66;
+// logit gates: 95 and 158, 182 and 347, 503 and 1353, 201 and 359, 66 and 80.  With 48 sequences
+// the one is ahead (B3 H16 T1300 216 and 198, T2047 301 and 298); more sequences than 56 leave too few workers.  Fewer than 96
+// chunks in all are left to the one kernel (tens of us either way).
 bool wy_split_sizes(const Args &a) {
   if (!wy_fwd_supported(a, false)) return false;
-  const long long bh = (long long)a.B * a.H, nc = (a.T + CM - 1) / CM, waves = (bh + kSms - 1) / kSms;
-  if (bh * nc < 96) return false;
-  return waves * nc * 10 + (bh * nc + kSms - 1) / kSms * 18 + 50 < waves * nc * 17;
+  const long long bh = (long long)a.B * a.H, nc = (a.T + CM - 1) / CM;
+  if (bh * nc < 96 || bh > 56) return false;
+  const long long workers = kSms - 2 * bh;
+  return std::max(nc * 7, (bh * nc + workers - 1) / workers * 19) + 45 < nc * 17;
 }
 
 bool wy_split_save(const Args &a) {
@@ -1746,7 +1833,7 @@ bool wy_split_save(const Args &a) {
 
 size_t wy_split_workspace_bytes(const Args &a) {
   if (!wy_split_sizes(a)) return 0;
-  return (size_t)a.B * a.H * ((a.T + CM - 1) / CM) * (kPreBytes + D * sizeof(float));
+  return (size_t)a.B * a.H * ((a.T + CM - 1) / CM) * (kPreBytes + D * sizeof(float) + sizeof(unsigned));
 }
 
 namespace {
@@ -1758,22 +1845,19 @@ kdn_status_t launch_wy(const WyParams &W, bool split, cudaStream_t s) {
       !make_map(&mv, a.v, a) || !make_map(&mq, a.q, a))
     return KDN_ERR_CUDA;
   const int bh = a.B * a.H;
-  const long long njobs = (long long)bh * ((a.T + CM - 1) / CM);
+  const size_t n = (size_t)bh * ((a.T + CM - 1) / CM);
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
   if (!split) {
-    if (cudaFuncSetAttribute(k_wy_fwd<SV, LG, 0>, attr, SMEM_BYTES) != cudaSuccess) return KDN_ERR_CUDA;
-    k_wy_fwd<SV, LG, 0><<<bh, WT, SMEM_BYTES, s>>>(mk, mg, mw, mv, mq, W);
+    if (cudaFuncSetAttribute(k_wy_fwd<SV, LG>, attr, SMEM_BYTES) != cudaSuccess) return KDN_ERR_CUDA;
+    k_wy_fwd<SV, LG><<<bh, WT, SMEM_BYTES, s>>>(mk, mg, mw, mv, mq, W);
     return cudaGetLastError() == cudaSuccess ? KDN_OK : KDN_ERR_CUDA;
   }
-  if (cudaFuncSetAttribute(k_wy_fwd<SV, LG, 1>, attr, SMEM_BYTES) != cudaSuccess ||
-      cudaFuncSetAttribute(k_wy_gain<SV, LG>, attr, SG_SMEM) != cudaSuccess ||
-      cudaFuncSetAttribute(k_wy_state<SV>, attr, ST_SMEM) != cudaSuccess)
+  if (cudaFuncSetAttribute(k_wy_flow<SV, LG>, attr, FLOW_SMEM) != cudaSuccess ||
+      cudaMemsetAsync(W.pin, 0xff, n * D * sizeof(float), s) != cudaSuccess ||
+      (SV ? cudaMemset2DAsync(W.flag, W.rec, 0, sizeof(unsigned), n, s)
+          : cudaMemsetAsync(W.flag, 0, n * sizeof(unsigned), s)) != cudaSuccess)
     return KDN_ERR_CUDA;
-  k_wy_gain<SV, LG><<<bh, WT, SG_SMEM, s>>>(mk, mg, mw, a, const_cast<float *>(W.pin));
-  if (cudaGetLastError() != cudaSuccess) return KDN_ERR_CUDA;
-  k_wy_fwd<SV, LG, 1><<<(unsigned)(njobs < kSms ? njobs : kSms), WT, SMEM_BYTES, s>>>(mk, mg, mw, mv, mq, W);
-  if (cudaGetLastError() != cudaSuccess) return KDN_ERR_CUDA;
-  k_wy_state<SV><<<bh, WT, ST_SMEM, s>>>(mv, W);
+  k_wy_flow<SV, LG><<<kSms, WT, FLOW_SMEM, s>>>(mk, mg, mw, mv, mq, W);
   return cudaGetLastError() == cudaSuccess ? KDN_OK : KDN_ERR_CUDA;
 }
 }  // namespace
@@ -1786,17 +1870,25 @@ kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S,
   P.save_S = save_S;
   P.rec = fused_ctx_record_bytes(a);
   P.save_p = save_p;
-  bool split = wy_split_sizes(a);
-  if (save_S) {
-    split = wy_split_save(a);
+  P.pre = nullptr;
+  P.prec = 0;
+  P.pin = nullptr;
+  P.flag = nullptr;
+  P.fstride = 0;
+  const bool split = save_S ? wy_split_save(a) : wy_split_sizes(a) && ws;
+  if (split && save_S) {
     P.pre = save_S;
     P.prec = P.rec;
     P.pin = save_p;
-  } else {
-    split = split && ws;
+    P.flag = reinterpret_cast<unsigned *>(save_S + kCtxTok + 3 * CM * sizeof(float));  // (no value there)
+    P.fstride = P.rec / sizeof(unsigned);
+  } else if (split) {
+    const size_t n = (size_t)a.B * a.H * ((a.T + CM - 1) / CM);
     P.pre = reinterpret_cast<unsigned char *>(ws);
     P.prec = kPreBytes;
-    P.pin = split ? reinterpret_cast<float *>(ws + (size_t)a.B * a.H * ((a.T + CM - 1) / CM) * kPreBytes) : nullptr;
+    P.pin = reinterpret_cast<float *>(ws + n * kPreBytes);
+    P.flag = reinterpret_cast<unsigned *>(P.pin + n * D);
+    P.fstride = 1;
   }
   if (a.gates == KDN_GATES_LOGITS) return save_S ? launch_wy<1, 1>(P, split, s) : launch_wy<0, 1>(P, split, s);
   return save_S ? launch_wy<1, 0>(P, split, s) : launch_wy<0, 0>(P, split, s);

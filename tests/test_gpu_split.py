@@ -101,9 +101,9 @@ def test_context_serves_either_gradient_type(kdn, first, then):
 @pytest.mark.parametrize("out", ["f32", "bf16"])
 @pytest.mark.parametrize("B,T,H,gates,slow,fast", [
     (1, 824, 16, "post", False, 0), (2, 1985, 14, "logits", True, 0), (1, 1537, 5, "post", False, 9.0),
-    (2, 1100, 12, "logits", False, 9.0), (1, 700, 10, "post", True, 0)])
-def test_three_kernel_forward_equals_the_one(kdn, B, T, H, gates, slow, fast, out):
-    """The chunk part and the memory part in kernels of their own run the same arithmetic: the
+    (2, 1100, 12, "logits", False, 9.0), (1, 700, 10, "post", True, 0), (2, 1000, 16, "post", False, 0)])
+def test_flow_forward_equals_the_one(kdn, B, T, H, gates, slow, fast, out):
+    """The gain, the chunk part and the memory part on CTAs of their own run the same arithmetic: the
     outputs are those of the one-kernel forward (a workspace without room) bit for bit, also
     where a chunk's decay leaves the referenced range (fast: log alpha of -9)."""
     ins, _, _ = _case(B, T, H, T + B, gates, slow)
@@ -114,7 +114,7 @@ def test_three_kernel_forward_equals_the_one(kdn, B, T, H, gates, slow, fast, ou
     dt = torch.float32 if out == "f32" else torch.bfloat16
     G = kdn.KDN_GATES_LOGITS if gates == "logits" else kdn.KDN_GATES_POST
     desc = kdn.make_desc(B, T, H, 128, 128, torch.bfloat16, out_dtype=dt, gates=G)
-    assert kdn.kdn_kernel_launches(desc, 0, 0) == 3
+    assert kdn.workspace_bytes(desc, 0) >= B * H * ((T + 63) // 64) * 66560  # its records
     kw = dict(out_dtype=dt, gates=G)
     for state in ((d["S0"], d["p0"]), (None, None)):
         ws = kdn.alloc_workspace(desc, 0)
