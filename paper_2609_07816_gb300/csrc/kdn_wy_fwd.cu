@@ -1787,7 +1787,7 @@ __device__ __forceinline__ void wy_state(const CUtensorMap &mv, const WyParams &
 // ---------------------------------------------------------------------------
 // k_wy_flow: the three parts at once, one CTA per SM: first the gain's CTAs (one per sequence),
 // then the chunk part's, then the memory's (one per sequence).  A part waits only for CTAs of
-// lower index (bounded), so whatever of the grid is resident makes progress.  B1 H16 T824 with
+// lower index (bounded), so whatever of the grid is resident makes progress.  B1 H16 T777 with
 // logit gates 119 us as three launches, 78 us as one (one CTA per sequence: 143 us); training
 // forward B2 H16 T1999 302 and ~200 us (430).
 constexpr int FLOW_SMEM = SMEM_BYTES > SG_SMEM ? (SMEM_BYTES > ST_SMEM ? SMEM_BYTES : ST_SMEM)
