@@ -291,7 +291,10 @@ size_t fwd_min_workspace_bytes(const kdn_desc_t *desc, int variant) {
 size_t fwd_noalloc_bytes(const kdn_desc_t *desc, size_t have) {
   Args a;
   if (fill_sizes(desc, 0, false, &a) != KDN_OK) return 0;
-  return seg_count(a) == 1 && wy_split_sizes(a) ? workspace_layout(&a, nullptr, false) : have;
+  const size_t base = workspace_layout(&a, nullptr, false);
+  const int P = seg_count(a);
+  const bool seg = P > 1 && base + seg_workspace_bytes(a, P) <= have;
+  return !seg && wy_split_sizes(a) ? base : have;
 }
 
 size_t workspace_layout(Args *a, char *base, bool bwd) {

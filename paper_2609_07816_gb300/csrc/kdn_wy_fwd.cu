@@ -40,7 +40,7 @@
 //
 // The chunk is a chain of dependent stages inside one CTA, and with logit gates the gain (run
 // one chunk ahead on its own warps) is as long as the rest: the kernel is bound by
-// that latency, not by HBM or shared-memory throughput.  B8 H16 T4096: 540 us (646 with the
+// that latency, not by HBM or shared-memory throughput.  B8 H16 T4096: 545 us (646 with the
 // solve's diagonal blocks and Y on the same warps, and MMAs issued under a divergent branch),
 // with the context 687 us (730; its copies go out one per warp, and A_qk is written
 // beside the -W product).  Few sequences: k_wy_flow (below).
