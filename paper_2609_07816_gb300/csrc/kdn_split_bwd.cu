@@ -1,31 +1,32 @@
 // kdn_split_bwd.cu -- backward of the Diagonal KDN (bfloat16 activations, d_k = d_v =
-// 128, 64-token chunks) in two kernels, so that only what is sequential over chunks
+// 128, 64-token chunks) in two steps, so that only what is sequential over chunks
 // runs sequentially:
 //   k_bwd_state   one CTA per (batch, head) carries the memory cotangent dS (128 x 128
 //                 fp32 in tensor memory) backwards over the chunks:
 //                   dR   = A_qk^T dO + K_tail dS
 //                   dS_in = diag(gamma_C) dS + Qbar^T dO - W^T dR
-//                 and leaves dS and dR of every chunk in 16 bits;
+//                 and leaves dS and dR of every chunk in 16 bits (its operands K_tail and
+//                 Qbar are formed before, in parallel over chunks, by k_bwd_tiles);
 //   k_bwd_chunk   every other adjoint of a chunk, in parallel over (chunk, batch, head):
 //                 persistent CTAs take chunks in reverse time order.  The uncertainty
-//                 cotangent dp is the one value that still runs backwards: a chunk's map
-//                 dp_in = A dp_out + B is formed first, dp_out is then awaited, and dp_in
-//                 handed on before the chunk's last pass.
+//                 cotangent dp is the one value that still runs backwards: a chunk awaits dp_out
+//                 ahead of its last pass and hands on at once the dp_in that the pass will end with.
 // The one-kernel sweep (kdn_fused_bwd.cu) spends ~40 K cycles on a chunk, nearly all of it
 // on work that needs no other chunk, with one CTA per (batch, head): 128 CTAs at most
-// busy on 152 SMs, 32 at B2 H16.  Here the serial part is ~2-3 K cycles a chunk.
+// busy on 152 SMs, 32 at B2 H16.  Here the serial part is ~6 K cycles a chunk.
 //
-// Scratch per chunk and head: dS fp16 (32 KB), dR as an fp16 pair (32 KB), and ~3 KB of
-// small values.  With whole chunks (T a multiple of 64) it lies in the gradient buffers
-// themselves: a chunk's rows of dq, dk, dv, dg hold its tiles and its rows of domega the
-// small values until k_bwd_chunk, which is the only one to read them, writes the
+// Scratch per chunk and head: dS fp16 (32 KB), dR as an fp16 pair (32 KB; K_tail and Qbar
+// before), and ~4 KB of small values.  With whole chunks (T a multiple of 64) it lies in the
+// gradient buffers themselves: a chunk's rows of dq, dk, dv, dg hold its tiles and its rows of
+// domega the small values until k_bwd_chunk, which is the only one to read them, writes the
 // chunk's gradients there.  Ragged lengths use the workspace (a tile's rows are not
 // tokens, and rows past T do not exist in the gradients).
 //
-// It serves bf16 gradients without state gradients (see split_bwd_supported).  Numerics are
-// those of the one-kernel sweep up to rounding: the same operand types (fp16 tiles, hi/lo
-// bf16 pairs where Gamma-scaled operands meet, fp16 pairs for dR in A^T dR), fp32
-// accumulators, dS fp32 across chunks, cotangents scaled by the same power of two.
+// It serves bf16 gradients without state gradients (see split_bwd_supported).  The gradients are
+// those of the one-kernel sweep bit for bit: the same operand tiles (fp16 tiles, hi/lo
+// bf16 pairs where Gamma-scaled operands meet, fp16 pairs for dR in A^T dR), products and sums
+// in the same order, fp32 accumulators, dS fp32 across chunks, cotangents scaled by the same
+// power of two.
 //
 // Every wait is bounded; on timeout KDN_ERR_TIMEOUT goes to the status word.
 #include "kdn_internal.cuh"
@@ -44,7 +45,8 @@ constexpr uint32_t kDpWait = 1u << 22;  // polls for the uncertainty cotangent o
 constexpr int kSms = 152;
 
 // Where a chunk's small values lie: rows of 256 bytes, one per token of the chunk.
-// Rows 0, 1: dgamma_C's dS part [128]; 2..5: dp [128] as (value, tag) pairs; 6: lambda.
+// Rows 0..7: dgamma_C's dS part [4][128]; 8..11: dp [128] as (value, tag) pairs; 12: lambda;
+// 13: the r inputs z_t [64].
 struct Scratch {
   unsigned char *small;
   int T;       // tokens of the scratch layout (a multiple of 64)
@@ -57,10 +59,13 @@ __device__ __forceinline__ float *small_dgc(const Scratch &s, const Args &a, int
 }
 // (value, tag) slot of channel i's dp
 __device__ __forceinline__ uint2 *small_slot(const Scratch &s, const Args &a, int b, int h, int c, int i) {
-  return reinterpret_cast<uint2 *>(small_row(s, a, b, h, c, 2 + (i >> 5))) + (i & 31);
+  return reinterpret_cast<uint2 *>(small_row(s, a, b, h, c, 8 + (i >> 5))) + (i & 31);
 }
 __device__ __forceinline__ float *small_lam(const Scratch &s, const Args &a, int b, int h, int c) {
-  return reinterpret_cast<float *>(small_row(s, a, b, h, c, 6));
+  return reinterpret_cast<float *>(small_row(s, a, b, h, c, 12));
+}
+__device__ __forceinline__ float *small_z(const Scratch &s, const Args &a, int b, int h, int c) {
+  return reinterpret_cast<float *>(small_row(s, a, b, h, c, 13));
 }
 // A slot is one 8-byte store and one 8-byte load: the value needs no other ordering.
 __device__ __forceinline__ void slot_put(uint2 *p, float v) {
@@ -110,17 +115,85 @@ struct SplitParams {
 };
 
 // ---------------------------------------------------------------------------
+// k_bwd_tiles.  One CTA per 64 channels of a chunk: K_tail^T [i][s] and Qbar^T [i][t] in fp16 from
+// the context's phat, gamma and s_t, in the operations of the one-kernel sweep (the context does not
+// hold them: K_tail needs s_t, which the forward knows only after the gain has moved on).  Left where
+// the chunk's dR goes, which k_bwd_state writes once it has read them.  Bound by HBM: 96 KB read and
+// 32 KB written per chunk.  A thread takes two channels of eight tokens, all loads ahead.
+constexpr int TT = 256, TILE_SMEM = 16 * KB + 1024;
+
+__global__ void __launch_bounds__(TT, 4)
+    k_bwd_tiles(const __grid_constant__ CUtensorMap m2, const __grid_constant__ CUtensorMap m3,
+                const SplitParams P) {
+  const Args &a = P.a;
+  extern __shared__ unsigned char smraw[];
+  __shared__ float s_si[CM];
+  unsigned char *sm =
+      reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
+  const int tid = threadIdx.x, half = (int)(blockIdx.x & 1u), r0 = 2 * (tid & 31), ci = 64 * half + r0;
+  const int t0 = 8 * (tid >> 5), job = (int)(blockIdx.x >> 1);
+  const int NC = (a.T + CM - 1) / CM, c = job % NC, bh = job / NC, b = bh / a.H, h = bh % a.H;
+  const unsigned char *rec = a.fSin + (size_t)job * P.rec;
+  const float *cph = reinterpret_cast<const float *>(rec + kCtxPh) + t0 * D + ci;
+  const float *cga = reinterpret_cast<const float *>(rec + kCtxGa) + ci;
+  float2 ph[8], ga[8];
+  __nv_bfloat162 kk[8], qv[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    ph[j] = *reinterpret_cast<const float2 *>(cph + j * D);
+    ga[j] = *reinterpret_cast<const float2 *>(cga + (t0 + j) * D);
+    const size_t e = tok_index(a, b, min(c * CM + t0 + j, a.T - 1), h) * D + ci;
+    kk[j] = *reinterpret_cast<const __nv_bfloat162 *>(static_cast<const __nv_bfloat16 *>(a.k) + e);
+    qv[j] = *reinterpret_cast<const __nv_bfloat162 *>(static_cast<const __nv_bfloat16 *>(a.q) + e);
+  }
+  const float2 gC = *reinterpret_cast<const float2 *>(cga + (CM - 1) * D);
+  if (tid < CM) {
+    s_si[tid] = 1.f / reinterpret_cast<const float *>(rec + kCtxTok)[tid];
+    const int t = c * CM + tid;
+    if (half == 0)
+      small_z(P.s, a, b, h, c)[tid] =
+          t < a.T ? __bfloat162float(static_cast<const __nv_bfloat16 *>(a.r)[tok_index(a, b, t, h)]) : 0.f;
+  }
+  __syncthreads();
+  float kt[2][8], qb[2][8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const bool live = c * CM + t0 + j < a.T;
+    const float si = s_si[t0 + j];
+    const float2 k = live ? __bfloat1622float2(kk[j]) : make_float2(0.f, 0.f);
+    const float2 q = live ? __bfloat1622float2(qv[j]) : make_float2(0.f, 0.f);
+    kt[0][j] = gC.x * __fdividef(ph[j].x * si * k.x, ga[j].x);
+    kt[1][j] = gC.y * __fdividef(ph[j].y * si * k.y, ga[j].y);
+    qb[0][j] = a.tau * ga[j].x * q.x;
+    qb[1][j] = a.tau * ga[j].y * q.y;
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const uint32_t off = chunk_off(r0 + r, t0 >> 3);
+    sm16(sm, off) = pack_h8(kt[r]);
+    sm16(sm + 8 * KB, off) = pack_h8(qb[r]);
+  }
+  fence_proxy_async();
+  __syncthreads();
+  if (tid == 0 || tid == 32) {  // 64 rows of each: one box, at channel 64 half of the scratch tile
+    tma_store_4d(tid == 0 ? &m2 : &m3, sm + (tid >> 5) * 8 * KB, 64 * half, h, c * CM, b);
+    bulk_commit();
+    bulk_wait_all();
+  }
+}
+
+// ---------------------------------------------------------------------------
 // k_bwd_state.  Bound by HBM: 104 KB read and 64 KB written per chunk, 255 us at B8 H16 T4096
 // (5.4 TB/s); with few sequences by its chain, ~6 K cycles a chunk (94 us at B2 H16 T1999).
 // 16 warps; warp w holds TMEM lanes 32 (w % 4) .. + 31 and value columns
 // 32 (w / 4) .. + 31 of dS.  Per chunk: dS -> fp16 tile; MMA dR; dR -> fp16 hi + lo;
-// MMA dS.  A_qk, K' and dO are double-buffered bulk copies; Qbar, W (needed
+// MMA dS.  A_qk, K_tail and dO are double-buffered bulk copies; Qbar, W (needed
 // last) and S_in (for dgamma_C, needed first) are loaded again as soon as they have been read.
 constexpr int SB_AQ = 0, SB_KT = 8 * KB, SB_DO = 24 * KB, SB_BUF = 40 * KB;
 constexpr int SO_QB = 2 * SB_BUF, SO_WN = SO_QB + 16 * KB, SO_SIN = SO_WN + 16 * KB;
 constexpr int SO_DSH = SO_SIN + 32 * KB, SO_DRH = SO_DSH + 32 * KB, SO_DRL = SO_DRH + 16 * KB;
-constexpr int SO_PART = SO_DRL + 16 * KB, SO_SC = SO_PART + 4096 + 512;
-constexpr int SO_BAR = SO_SC + 2 * 768, STATE_SMEM = SO_BAR + 64 + 1024;  // SC: gamma_C [128], s_t [64], two buffers
+constexpr int SO_PART = SO_DRL + 16 * KB, SO_SC = SO_PART + 256;
+constexpr int SO_BAR = SO_SC + 2 * 512, STATE_SMEM = SO_BAR + 64 + 1024;  // SC: gamma_C [128], two buffers
 static_assert(STATE_SMEM <= 232448, "shared memory");
 
 __global__ void __launch_bounds__(BT, 1)
@@ -132,7 +205,7 @@ __global__ void __launch_bounds__(BT, 1)
   unsigned char *sm =
       reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   unsigned char *dsh = sm + SO_DSH, *drh = sm + SO_DRH, *drl = sm + SO_DRL;
-  float *s_part = reinterpret_cast<float *>(sm + SO_PART), *s_is = s_part + 1024, *s_misc = s_is + 64;
+  float *s_part = reinterpret_cast<float *>(sm + SO_PART), *s_misc = s_part + 32;
   uint64_t *bars = reinterpret_cast<uint64_t *>(sm + SO_BAR);
   uint64_t *bar_full = bars, *bar_r = bars + 2, *bar_s = bars + 3, *bar_w = bars + 4, *bar_i = bars + 5;
   uint32_t *s_tbase = reinterpret_cast<uint32_t *>(bars + 6);
@@ -143,7 +216,7 @@ __global__ void __launch_bounds__(BT, 1)
   if (tid == 0) {
     mbar_init(bar_full, 5);  // arrivals: one per issuing thread
     mbar_init(bar_full + 1, 5);
-    mbar_init(bar_w, 3);
+    mbar_init(bar_w, 2);
     mbar_init(bar_i, 1);
     mbar_init(bar_r, 1);
     mbar_init(bar_s, 1);
@@ -157,25 +230,25 @@ __global__ void __launch_bounds__(BT, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t TS = *s_tbase, TXA = TS + 128, TXB = TS + 192;
+  const uint32_t TS = *s_tbase, TX = TS + 128;
   const uint32_t lane_base = (uint32_t)(32 * wq) << 16;
   auto record = [&](int c) { return a.fSin + ((size_t)bh * NC + c) * P.rec; };
   // The copies are issued one per warp (lane 0): a single thread's run of them would hold
   // up the chain of products.  Warps 1..7 load, 8..11 store dS, 12..15 store dR.
-  auto issue = [&](int c, int buf) {  // A_qk, K', dO, gamma_C, s_t
+  auto issue = [&](int c, int buf) {  // A_qk, K_tail, dO, gamma_C
     const unsigned char *rec = record(c);
-    unsigned char *d = sm + buf * SB_BUF, *sc = sm + SO_SC + buf * 768;
+    unsigned char *d = sm + buf * SB_BUF, *sc = sm + SO_SC + buf * 512;
     uint64_t *bar = bar_full + buf;
     switch (lane == 0 ? warp : -1) {
       case 1: mbar_expect_tx(bar, 8192); bulk_g2s(d + SB_AQ, rec + kCtxAqk, 8192, bar); break;
-      case 2: mbar_expect_tx(bar, 16384); bulk_g2s(d + SB_KT, rec + kCtxKt, 16384, bar); break;
+      case 2:
+        mbar_expect_tx(bar, 16384);
+        tma_load_4d(d + SB_KT, &m2, bar, 0, h, c * CM, b);
+        tma_load_4d(d + SB_KT + 8192, &m2, bar, 64, h, c * CM, b);
+        break;
       case 3: mbar_expect_tx(bar, 8192); tma_load_4d(d + SB_DO, &mdo, bar, 0, h, c * CM, b); break;
       case 4: mbar_expect_tx(bar, 8192); tma_load_4d(d + SB_DO + 8192, &mdo, bar, 64, h, c * CM, b); break;
-      case 5:
-        mbar_expect_tx(bar, 768);
-        bulk_g2s(sc, rec + kCtxGa + 63 * D * 4, 512, bar);
-        bulk_g2s(sc + 512, rec + kCtxTok, 256, bar);
-        break;
+      case 5: mbar_expect_tx(bar, 512); bulk_g2s(sc, rec + kCtxGa + 63 * D * 4, 512, bar); break;
     }
   };
   auto issue_sin = [&](int c) {
@@ -184,17 +257,23 @@ __global__ void __launch_bounds__(BT, 1)
       bulk_g2s(sm + SO_SIN, record(c) + kCtxS, 32768, bar_i);
     }
   };
-  auto issue_w = [&](int c) {  // Qbar (rows 64..127 of the two slabs of [-Kbar; Qbar]), -W
+  auto issue_w = [&](int c) {  // Qbar, -W
     const unsigned char *rec = record(c);
     switch (lane == 0 ? warp : -1) {
-      case 5: mbar_expect_tx(bar_w, 8192); bulk_g2s(sm + SO_QB, rec + kCtxKQ + 8192, 8192, bar_w); break;
-      case 6: mbar_expect_tx(bar_w, 8192); bulk_g2s(sm + SO_QB + 8192, rec + kCtxKQ + 24576, 8192, bar_w); break;
+      case 6:
+        mbar_expect_tx(bar_w, 16384);
+        tma_load_4d(sm + SO_QB, &m3, bar_w, 0, h, c * CM, b);
+        tma_load_4d(sm + SO_QB + 8192, &m3, bar_w, 64, h, c * CM, b);
+        break;
       case 7: mbar_expect_tx(bar_w, 16384); bulk_g2s(sm + SO_WN, rec + kCtxW, 16384, bar_w); break;
       case 8:  // the next chunk's, into L2
         if (c > 0) {
           bulk_prefetch_l2(rec - P.rec + kCtxS, 32768);
           bulk_prefetch_l2(rec - P.rec + kCtxW, 16384);
-          bulk_prefetch_l2(rec - P.rec + kCtxKQ, 32768);
+          for (int s = 0; s < 2; ++s) {
+            tma_prefetch_4d(&m2, 64 * s, h, (c - 1) * CM, b);
+            tma_prefetch_4d(&m3, 64 * s, h, (c - 1) * CM, b);
+          }
         }
         break;
     }
@@ -269,9 +348,7 @@ __global__ void __launch_bounds__(BT, 1)
     issue_w(c);  // (MMA dS of the previous chunk has read the last ones)
     tc_fence_after();
     {
-      const float *sc = reinterpret_cast<const float *>(sm + SO_SC + buf * 768);
-      const float gC = sc[i];
-      if (tid < CM) s_is[tid] = 1.f / sc[D + tid];
+      const float gC = reinterpret_cast<const float *>(sm + SO_SC + buf * 512)[i];
       float dgc = 0.f;
 #pragma unroll
       for (int c0 = 0; c0 < 32; c0 += 16) {
@@ -289,7 +366,7 @@ __global__ void __launch_bounds__(BT, 1)
         }
         tmem_st16(TS + lane_base + j0 + c0, v);
       }
-      s_part[(it & 1) * 512 + wg * D + i] = dgc;  // (read after the barrier: two buffers)
+      *small_dgc(P.s, a, b, h, c, wg * D + i) = dgc;
 #pragma unroll
       for (int e = tid; e < 64 * 16; e += BT) {
         const uint32_t off = SB_DO + ((e & 15) >> 3) * 8192 + chunk_off(e >> 4, e & 7);
@@ -308,7 +385,7 @@ __global__ void __launch_bounds__(BT, 1)
       ok = false;
       break;
     }
-    // ---- [2] MMA: XA = (A_qk^T dO)^T, XB = (K' dS)^T, [j][t] (K_tail = diag(1/s) K')
+    // ---- [2] MMA: X = (A_qk^T dO + K_tail dS)^T = dR^T, [j][t]
     if (warp_u == 0) {
       tc_fence_after();
       const uint32_t lead = elect_one();
@@ -316,9 +393,9 @@ __global__ void __launch_bounds__(BT, 1)
       const uint64_t aq = mdesc(d + SB_AQ, 8192), dov = mdesc(d + SB_DO, 8192), kt = mdesc(d + SB_KT, 8192),
                      ds = mdesc(dsh, 16384);
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) umma_if(lead, TXA, step(dov, kk * 2048), step(aq, kk * 2048), id11, kk > 0);
+      for (int kk = 0; kk < 4; ++kk) umma_if(lead, TX, step(dov, kk * 2048), step(aq, kk * 2048), id11, kk > 0);
 #pragma unroll
-      for (int kk = 0; kk < 8; ++kk) umma_if(lead, TXB, step(ds, kk * 2048), step(kt, kk * 2048), id11, kk > 0);
+      for (int kk = 0; kk < 8; ++kk) umma_if(lead, TX, step(ds, kk * 2048), step(kt, kk * 2048), id11, 1);
       commit_if(lead, bar_r);
     }
     if (c > 0) {
@@ -333,21 +410,15 @@ __global__ void __launch_bounds__(BT, 1)
     }
     if (warp >= 4 && warp < 8) {  // the small values of this chunk
       const int ii = tid - 128;
-      const float *sp = s_part + (it & 1) * 512 + ii;
-      *small_dgc(P.s, a, b, h, c, ii) = (sp[0] + sp[D]) + (sp[2 * D] + sp[3 * D]);
       *small_slot(P.s, a, b, h, c, ii) = make_uint2(0u, 0u);
       if (ii == 0) *small_lam(P.s, a, b, h, c) = lam;
     }
-    // ---- [3] dR^T = XA + XB diag(1/s) -> fp16 hi + lo, [j][t]
+    // ---- [3] dR^T -> fp16 hi + lo, [j][t]
     ok = mbar_wait(bar_r, it & 1, kWaitIters) && ok;
     tc_fence_after();
     {
-      float x[16], y[16];
-      const int tc0 = 16 * wg;
-      tmem_ld16(TXA + lane_base + tc0, x);
-      tmem_ld16(TXB + lane_base + tc0, y);
-#pragma unroll
-      for (int u = 0; u < 16; ++u) x[u] = fmaf(s_is[tc0 + u], y[u], x[u]);
+      float x[16];
+      tmem_ld16(TX + lane_base + 16 * wg, x);
       uint4 l0, l1;
       sm16(drh, chunk_off(i, 2 * wg)) = split_h8(x, &l0);
       sm16(drh, chunk_off(i, 2 * wg + 1)) = split_h8(x + 8, &l1);
@@ -363,18 +434,19 @@ __global__ void __launch_bounds__(BT, 1)
       ok = mbar_wait(bar_w, it & 1, kWaitIters) && ok;
       tc_fence_after();
       const uint32_t lead = elect_one();
-      const uint32_t id11 = idesc_f16(128, 128, 1, 1), id10 = idesc_f16(128, 128, 1, 0);
-      const uint64_t qb = mdesc(sm + SO_QB, 8192), dov = mdesc(d + SB_DO, 8192), wn = mdesc(sm + SO_WN, 8192),
+      const uint32_t id01 = idesc_f16(128, 128, 0, 1), id10 = idesc_f16(128, 128, 1, 0);
+      const uint64_t qb = kdesc(sm + SO_QB), dov = mdesc(d + SB_DO, 8192), wn = mdesc(sm + SO_WN, 8192),
                      dr = kdesc(drh);
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk) {
-        umma_if(lead, TS, step(qb, kk * 2048), step(dov, kk * 2048), id11, 1);
+        umma_if(lead, TS, step(qb, kk * 32), step(dov, kk * 2048), id01, 1);
         umma_if(lead, TS, step(wn, kk * 2048), step(dr, kk * 32), id10, 1);
       }
       commit_if(lead, bar_s);
     }
-    if (lane == 0 && warp >= 12) {  // dR^T rows j 0..63, 64..127
+    if (lane == 0 && warp >= 12) {  // dR^T rows j 0..63, 64..127, over K_tail and Qbar, which have been read
       const int s = warp & 1;
+      ok = mbar_wait(bar_w, it & 1, kWaitIters) && ok;
       if (warp < 14) tma_store_4d(&m2, drh + s * 8192, 64 * s, h, c * CM, b);
       else tma_store_4d(&m3, drl + s * 8192, 64 * s, h, c * CM, b);
       bulk_commit();
@@ -421,7 +493,7 @@ constexpr int O_GA3 = 208 * KB;  // gamma, tokens 48..63
 constexpr int BUF_END = 216 * KB;
 constexpr int O_DAQ = O_G, O_KKL = O_G + 16 * KB, O_XT = O_G + 24 * KB;
 constexpr int OFF_SM = BUF_END;
-constexpr int SMALL_FLOATS = 64 * 8 + 512 + 128 * 2 + 32 + 128 + 452;
+constexpr int SMALL_FLOATS = 64 * 8 + 512 + 128 * 2 + 32 + 128 + 772;
 constexpr int OFF_BAR = OFF_SM + SMALL_FLOATS * 4;
 constexpr int CHUNK_SMEM = OFF_BAR + 80 + 1024;
 static_assert(CHUNK_SMEM <= 232448, "shared memory");
@@ -450,8 +522,8 @@ __global__ void __launch_bounds__(BT, 1)
   float *s_misc = s_dp + 128;   // [0] lambda
   int *s_next = reinterpret_cast<int *>(s_misc + 8);
   float *s_pin = s_misc + 32;   // [128] p entering the chunk
-  float *n_tok = s_pin + 128;   // next chunk: [3][64] s_t, r_t, z_t; [128] p in; [128] dgamma_C; lambda
-  float *n_pin = n_tok + 192, *n_dgc = n_pin + 128, *n_lam = n_dgc + 128;
+  float *n_tok = s_pin + 128;   // next chunk: [2][64] s_t, z_t; [128] p in; [4][128] dgamma_C; lambda
+  float *n_pin = n_tok + 128, *n_dgc = n_pin + 128, *n_lam = n_dgc + 512;
   uint64_t *bars = reinterpret_cast<uint64_t *>(sm + OFF_BAR);
   uint64_t *bar_a = bars, *bar_b = bars + 1, *bar_mma = bars + 2, *bar_g = bars + 3, *bar_d = bars + 4,
            *bar_w = bars + 5;
@@ -560,10 +632,11 @@ __global__ void __launch_bounds__(BT, 1)
   // the next job's small values, by asynchronous copies: loads into registers would hold up
   // the next wait on a barrier, and be spilled across the passes
   auto load_small = [&](const Job &o) {
-    if (tid < 48) cp16(n_tok + 4 * tid, o.rec + kCtxTok + 16 * tid);
-    else if (tid < 80) cp16(n_pin + 4 * (tid - 48), a.fpin + o.rc * D + 4 * (tid - 48));
-    else if (tid < 112) cp16(n_dgc + 4 * (tid - 80), small_dgc(P.s, a, o.b, o.h, o.c, 4 * (tid - 80)));
-    else if (tid == 112) cp16(n_lam, small_lam(P.s, a, o.b, o.h, o.c));
+    if (tid < 16) cp16(n_tok + 4 * tid, o.rec + kCtxTok + 16 * tid);
+    else if (tid < 32) cp16(n_tok + 4 * tid, small_z(P.s, a, o.b, o.h, o.c) + 4 * (tid - 16));
+    else if (tid < 64) cp16(n_pin + 4 * (tid - 32), a.fpin + o.rc * D + 4 * (tid - 32));
+    else if (tid < 192) cp16(n_dgc + 4 * (tid - 64), small_dgc(P.s, a, o.b, o.h, o.c, 4 * (tid - 64)));
+    else if (tid == 192) cp16(n_lam, small_lam(P.s, a, o.b, o.h, o.c));
   };
   if (tid == 0) take();
   __syncthreads();
@@ -594,15 +667,16 @@ __global__ void __launch_bounds__(BT, 1)
     bool mm_ok = mbar_wait(bar_a, it & 1, kWaitIters);
     mm_ok = mbar_wait(bar_g, it & 1, kWaitIters) && mm_ok;
     if (tid < CM) {
-      const float nr = n_tok[CM + tid];
+      const bool live = c * CM + tid < a.T;
+      const float z = n_tok[CM + tid], nr = live ? gate_r(G, a.rmin, z) : 1.f;
       s_r[tid] = nr;
       s_ri[tid] = 1.f / nr;
-      s_fr[tid] = dgate_sig(G, n_tok[2 * CM + tid]);
+      s_fr[tid] = live ? dgate_sig(G, z) : 1.f;
       s_si[tid] = 1.f / n_tok[tid];
     }
     if (qq == 1) s_pin[ci] = n_pin[ci];
     const float lam = n_lam[0], invl = 1.f / lam;
-    float dgc = qq == 0 ? n_dgc[ci] : 0.f;  // this thread's part of dgamma_C for channel ci
+    float dgc = n_dgc[tid];  // this thread's part of dgamma_C for channel ci
     // ---- [2] phat and gamma -> TMEM (lane = channel)
     float ph[16], ga[16];
     {
@@ -977,9 +1051,15 @@ __global__ void __launch_bounds__(BT, 1)
       tc_fence_after();
       float ex[8];  // the quarters' maps of this channel
       tmem_ld8(XE + 8, ex);
-      // dp leaving the chunk: from the next chunk's job (thread i: channel i), handed on at once
+      // dp leaving the chunk: from the next chunk's job (thread i: channel i)
       if (tid < D) {
-        float dp = 0.f;
+        float dp = 0.f, al0[16], rd0[16], dl0[16];
+#pragma unroll
+        for (int h8 = 0; h8 < 2; ++h8) {
+          tmem_ld8(X0 + lane_base + 8 * h8, al0 + 8 * h8);
+          tmem_ld8(X3 + lane_base + 8 * h8, rd0 + 8 * h8);
+          tmem_ld8(X2 + lane_base + 8 * h8, dl0 + 8 * h8);
+        }
         if (c == NC - 1) {
           if (a.dpT) dp = lam * a.dpT[((size_t)b * a.H + h) * D + tid];
         } else {
@@ -988,9 +1068,15 @@ __global__ void __launch_bounds__(BT, 1)
           else mm_ok = slot_get(small_slot(P.s, a, b, h, c, tid), &dp) && mm_ok;
         }
         s_dp[tid] = dp;
+        // hand on the dp entering this chunk: pass C's recursion through the first quarter, ahead of the pass
         if (c > 0) {
 #pragma unroll
-          for (int q2 = 3; q2 >= 0; --q2) dp = fmaf(ex[2 * q2], dp, ex[2 * q2 + 1]);
+          for (int q2 = 3; q2 > 0; --q2) dp = fmaf(ex[2 * q2], dp, ex[2 * q2 + 1]);
+#pragma unroll
+          for (int u = 15; u >= 0; --u) {
+            const float dph = dp * rd0[u] * rd0[u] + dl0[u];
+            dp = al0[u] * al0[u] * dph;
+          }
           slot_put(small_slot(P.s, a, b, h, c - 1, tid), dp);
         }
       }
@@ -1097,9 +1183,8 @@ bool split_bwd_context(const Args &a) {
   return waves * nc * 6 + (bh * nc + kSms - 1) / kSms * 32 + 12 < waves * nc * 40;
 }
 
-// The calls served: bf16 gradients and none of the initial state or mu.  Float32 results stay
-// with the sweep: K' unnormalised rounds otherwise in fp16 than K_tail, and a slow decay
-// carries the difference on (up to 1e-4 of a gradient's norm; bf16 stores round by 2e-3).
+// The calls served: bf16 gradients and none of the initial state or mu, which the two kernels
+// do not form.
 bool split_bwd_supported(const Args &a) {
   return split_bwd_context(a) && a.odt == KDN_BF16 && !a.dS0 && !a.dp0 && !a.dmu && (a.T % CM == 0 || a.split_ws);
 }
@@ -1133,6 +1218,9 @@ kdn_status_t launch_split_bwd(const Args &a, char *ws, cudaStream_t s) {
     return KDN_ERR_CUDA;
   CUtensorMap mw = mq;  // the omega logits
   if (a.gates && !make_map(&mw, a.omega, a)) return KDN_ERR_CUDA;
+  const long long njobs = (long long)a.B * a.H * NC;
+  k_bwd_tiles<<<(unsigned)(2 * njobs), TT, TILE_SMEM, s>>>(m[2], m[3], P);
+  if (cudaGetLastError() != cudaSuccess) return KDN_ERR_CUDA;
   if (cudaFuncSetAttribute(k_bwd_state, cudaFuncAttributeMaxDynamicSharedMemorySize, STATE_SMEM) != cudaSuccess)
     return KDN_ERR_CUDA;
   k_bwd_state<<<a.B * a.H, BT, STATE_SMEM, s>>>(mdo, m[0], m[1], m[2], m[3], P);
@@ -1140,7 +1228,6 @@ kdn_status_t launch_split_bwd(const Args &a, char *ws, cudaStream_t s) {
   const auto kern = a.gates ? k_bwd_chunk<1> : k_bwd_chunk<0>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, CHUNK_SMEM) != cudaSuccess)
     return KDN_ERR_CUDA;
-  const long long njobs = (long long)a.B * a.H * NC;
   kern<<<(unsigned)(njobs < kSms ? njobs : kSms), BT, CHUNK_SMEM, s>>>(mq, mk, mdo, mw, mdv, m[0], m[1], m[2],
                                                                        m[3], P);
   return cudaGetLastError() == cudaSuccess ? KDN_OK : KDN_ERR_CUDA;
