@@ -58,8 +58,8 @@ __device__ __forceinline__ float *small_dgc(const Scratch &s, const Args &a, int
   return reinterpret_cast<float *>(small_row(s, a, b, h, c, i >> 6)) + (i & 63);
 }
 // (value, tag) slot of channel i's dp
-__device__ __forceinline__ uint2 *small_slot(const Scratch &s, const Args &a, int b, int h, int c, int i) {
-  return reinterpret_cast<uint2 *>(small_row(s, a, b, h, c, 8 + (i >> 5))) + (i & 31);
+__device__ __forceinline__ uint64_t *small_slot(const Scratch &s, const Args &a, int b, int h, int c, int i) {
+  return reinterpret_cast<uint64_t *>(small_row(s, a, b, h, c, 8 + (i >> 5))) + (i & 31);
 }
 __device__ __forceinline__ float *small_lam(const Scratch &s, const Args &a, int b, int h, int c) {
   return reinterpret_cast<float *>(small_row(s, a, b, h, c, 12));
@@ -67,23 +67,25 @@ __device__ __forceinline__ float *small_lam(const Scratch &s, const Args &a, int
 __device__ __forceinline__ float *small_z(const Scratch &s, const Args &a, int b, int h, int c) {
   return reinterpret_cast<float *>(small_row(s, a, b, h, c, 13));
 }
-// A slot is one 8-byte store and one 8-byte load: the value needs no other ordering.
-__device__ __forceinline__ void slot_put(uint2 *p, float v) {
-  asm volatile("st.relaxed.gpu.global.v2.u32 [%0], {%1, %2};" ::"l"(p), "r"(__float_as_uint(v)), "r"(1u) : "memory");
+// A slot is one 64-bit number, tag above value, stored and loaded by one scalar relaxed access
+// (a vector access is two in no set order): value and tag come together and need no other ordering.
+__device__ __forceinline__ void slot_put(uint64_t *p, float v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(((uint64_t)1 << 32) | __float_as_uint(v)) : "memory");
 }
-__device__ __forceinline__ uint2 slot_peek(const uint2 *p) {
-  uint2 v;
-  asm volatile("ld.relaxed.gpu.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+__device__ __forceinline__ uint64_t slot_peek(const uint64_t *p) {
+  uint64_t v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ bool slot_get(const uint2 *p, float *v) {
+// x: what an earlier look at the slot found
+__device__ __forceinline__ bool slot_get(const uint64_t *p, uint64_t x, float *v) {
   for (uint32_t i = 0; i < kDpWait; ++i) {
-    const uint2 x = slot_peek(p);
-    if (x.y == 1u) {
-      *v = __uint_as_float(x.x);
+    if (x >> 32) {
+      *v = __uint_as_float((uint32_t)x);
       return true;
     }
     if (i > 64) __nanosleep(32);
+    x = slot_peek(p);
   }
   return false;
 }
@@ -410,7 +412,7 @@ __global__ void __launch_bounds__(BT, 1)
     }
     if (warp >= 4 && warp < 8) {  // the small values of this chunk
       const int ii = tid - 128;
-      *small_slot(P.s, a, b, h, c, ii) = make_uint2(0u, 0u);
+      *small_slot(P.s, a, b, h, c, ii) = 0;
       if (ii == 0) *small_lam(P.s, a, b, h, c) = lam;
     }
     // ---- [3] dR^T -> fp16 hi + lo, [j][t]
@@ -945,8 +947,6 @@ __global__ void __launch_bounds__(BT, 1)
     }
     // every tile but k, q has been read: the next chunk's may land
     if (on.j < njobs) issue_a(on);
-    if (tid < 64 && c < NC - 1)  // dp leaving this chunk, if the next chunk's job has handed it on already
-      cp16(s_red2 + 4 * tid, small_slot(P.s, a, b, h, c, 2 * tid));
     if (on.j < njobs) load_small(on);
     cp_commit();
     // ---- per channel (lane ci, tokens t0..t0+15): back through Gamma and the gain emission,
@@ -1042,6 +1042,9 @@ __global__ void __launch_bounds__(BT, 1)
         tmem_st1(XE + 8 + 2 * qq, A);
         tmem_st1(XE + 9 + 2 * qq, Bv);
       }
+      // dp leaving this chunk, if the next chunk's job has handed it on already
+      uint64_t early = 0;
+      if (tid < D && c < NC - 1) early = slot_peek(small_slot(P.s, a, b, h, c, tid));
       tmem_st_wait();
       tc_fence_before();
       cp_wait<0>();
@@ -1063,9 +1066,7 @@ __global__ void __launch_bounds__(BT, 1)
         if (c == NC - 1) {
           if (a.dpT) dp = lam * a.dpT[((size_t)b * a.H + h) * D + tid];
         } else {
-          const uint2 early = reinterpret_cast<const uint2 *>(s_red2)[tid];
-          if (early.y == 1u) dp = __uint_as_float(early.x);
-          else mm_ok = slot_get(small_slot(P.s, a, b, h, c, tid), &dp) && mm_ok;
+          mm_ok = slot_get(small_slot(P.s, a, b, h, c, tid), early, &dp) && mm_ok;
         }
         s_dp[tid] = dp;
         // hand on the dp entering this chunk: pass C's recursion through the first quarter, ahead of the pass
