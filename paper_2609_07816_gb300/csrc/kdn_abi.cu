@@ -15,6 +15,8 @@ int chunked_chunk_len();
 namespace {
 
 constexpr size_t kAlign = 256;
+// the status word and the tickets of the two-kernel backward and of k_wy_flow
+constexpr size_t kStatusBytes = 3 * sizeof(unsigned);
 
 size_t round_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
@@ -140,7 +142,7 @@ kdn_status_t fwd_entry(int variant, const kdn_desc_t *d, const void *q, const vo
   a.q = q; a.k = k; a.v = v; a.g = g; a.omega = omega; a.r = r;
   a.S0 = S0; a.p0 = p0; a.o = o; a.ST = ST; a.pT = pT;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(a.status, 0, sizeof(unsigned), s) != cudaSuccess) return KDN_ERR_CUDA;
+  if (cudaMemsetAsync(a.status, 0, kStatusBytes, s) != cudaSuccess) return KDN_ERR_CUDA;
   if ((size_t)a.B * a.H == 0) return KDN_OK;
   if (a.T == 0) return empty_fwd(a, s);
   if (nseg > 1) return launch_seg_fwd(a, nseg, static_cast<char *>(ws) + base, s);
@@ -175,7 +177,7 @@ kdn_status_t bwd_entry(int variant, const kdn_desc_t *d, const void *q, const vo
   a.dq = dq; a.dk_ = dk; a.dv_ = dv; a.dg = dg; a.domega = domega; a.dr = dr;
   a.dS0 = dS0; a.dp0 = dp0; a.dmu = dmu;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(a.status, 0, 2 * sizeof(unsigned), s) != cudaSuccess) return KDN_ERR_CUDA;
+  if (cudaMemsetAsync(a.status, 0, kStatusBytes, s) != cudaSuccess) return KDN_ERR_CUDA;
   if ((size_t)a.B * a.H == 0) return KDN_OK;
   if (a.T == 0) return empty_bwd(a, s);
   if (use_fused_bwd(a)) return launch_fused_bwd(a, s);
@@ -208,7 +210,7 @@ kdn_status_t fwd_save_entry(int variant, const kdn_desc_t *d, const void *q, con
   a.q = q; a.k = k; a.v = v; a.g = g; a.omega = omega; a.r = r;
   a.S0 = S0; a.p0 = p0; a.o = o; a.ST = ST; a.pT = pT;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(a.status, 0, sizeof(unsigned), s) != cudaSuccess) return KDN_ERR_CUDA;
+  if (cudaMemsetAsync(a.status, 0, kStatusBytes, s) != cudaSuccess) return KDN_ERR_CUDA;
   if ((size_t)a.B * a.H == 0) return KDN_OK;
   if (a.T == 0) return empty_fwd(a, s);
   const size_t nsv = (size_t)a.B * a.H * ((a.T + 63) / 64) * fused_ctx_record_bytes(a);
@@ -244,7 +246,7 @@ kdn_status_t bwd_saved_entry(int variant, const kdn_desc_t *d, const void *q, co
   a.dq = dq; a.dk_ = dk; a.dv_ = dv; a.dg = dg; a.domega = domega; a.dr = dr;
   a.dS0 = dS0; a.dp0 = dp0; a.dmu = dmu;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(a.status, 0, 2 * sizeof(unsigned), s) != cudaSuccess) return KDN_ERR_CUDA;
+  if (cudaMemsetAsync(a.status, 0, kStatusBytes, s) != cudaSuccess) return KDN_ERR_CUDA;
   if ((size_t)a.B * a.H == 0) return KDN_OK;
   if (a.T == 0) return empty_bwd(a, s);
   const size_t nsv = (size_t)a.B * a.H * ((a.T + 63) / 64) * fused_ctx_record_bytes(a);

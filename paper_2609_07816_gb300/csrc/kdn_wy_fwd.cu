@@ -463,6 +463,7 @@ struct WyParams {
   float *pin;             // [BH][NC][128], preset to kUnset
   unsigned *flag;         // per chunk, fstride apart, zeroed: warps that have written their part of its record
   size_t fstride;
+  unsigned *ticket;       // zeroed: CTAs of k_wy_flow that have started
 };
 
 // The uncertainty entering a chunk is handed over as the 4-byte value itself, in place of a
@@ -1786,8 +1787,9 @@ __device__ __forceinline__ void wy_state(const CUtensorMap &mv, const WyParams &
 
 // ---------------------------------------------------------------------------
 // k_wy_flow: the three parts at once, one CTA per SM: first the gain's CTAs (one per sequence),
-// then the chunk part's, then the memory's (one per sequence).  A part waits only for CTAs of
-// lower index (bounded), so whatever of the grid is resident makes progress.  B1 H16 T777 with
+// then the chunk part's, then the memory's (one per sequence).  A CTA takes its place by the order
+// in which the CTAs start, and a part waits only for earlier places (bounded), so whatever of
+// the grid is resident makes progress.  B1 H16 T777 with
 // logit gates 119 us as three launches, 78 us as one (one CTA per sequence: 143 us); training
 // forward B2 H16 T1999 302 and ~200 us (430).
 constexpr int FLOW_SMEM = SMEM_BYTES > SG_SMEM ? (SMEM_BYTES > ST_SMEM ? SMEM_BYTES : ST_SMEM)
@@ -1797,7 +1799,10 @@ __global__ void __launch_bounds__(WT, 1)
     k_wy_flow(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mg,
               const __grid_constant__ CUtensorMap mw, const __grid_constant__ CUtensorMap mv,
               const __grid_constant__ CUtensorMap mq, const WyParams P) {
-  const int BH = P.a.B * P.a.H, block = (int)blockIdx.x, workers = (int)gridDim.x - 2 * BH;
+  __shared__ int s_place;
+  if (threadIdx.x == 0) s_place = (int)atomicAdd(P.ticket, 1u);
+  __syncthreads();
+  const int BH = P.a.B * P.a.H, block = s_place, workers = (int)gridDim.x - 2 * BH;
   if (block < BH) wy_gain<SV, LG>(mk, mg, mw, P.a, P.pin, block);
   else if (block < BH + workers) wy_body<SV, LG, 1>(mk, mg, mw, mv, mq, P, block - BH, workers);
   else wy_state<SV>(mv, P, block - BH - workers);
@@ -1875,6 +1880,7 @@ kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S,
   P.pin = nullptr;
   P.flag = nullptr;
   P.fstride = 0;
+  P.ticket = a.status + 2;
   const bool split = save_S ? wy_split_save(a) : wy_split_sizes(a) && ws;
   if (split && save_S) {
     P.pre = save_S;
