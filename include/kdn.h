@@ -196,8 +196,8 @@ kdn_status_t kdn_iso_bwd(const kdn_desc_t *desc, const void *q, const void *k,
    K'^T (48 KB), and the
    float32 uncertainty p entering it.  kdn_diag_bwd_saved is kdn_diag_bwd that starts from that
    context instead of recomputing the forward (same gradients).  The diagonal
-   backward may use dq, dk, dv, dg and domega as scratch before it writes them:
-   they overlap no input.
+   backward may use dq, dk, dv, dg and domega as scratch before it writes them,
+   but not where one of them overlaps an input or another gradient.
    kdn_iso_fwd_save / kdn_iso_bwd_saved are the same for the Isotropic KDN.
    Served for bfloat16 activations, dk = dv = 128 and the default chunk; for
    every other descriptor kdn_saved_bytes() returns 0 and the calls return

@@ -1184,10 +1184,28 @@ bool split_bwd_context(const Args &a) {
   return waves * nc * 6 + (bh * nc + kSms - 1) / kSms * 32 + 12 < waves * nc * 40;
 }
 
+// The gradient buffers serve as scratch only where they overlap neither each other nor anything the
+// backward reads: the sweep reads each chunk's rows before it writes them, so that a gradient may
+// take the place of its input there.
+static bool scratch_is_apart(const Args &a) {
+  struct Range { uintptr_t p; size_t n; };
+  const size_t th = (size_t)a.B * a.T * a.H, bh = (size_t)a.B * a.H, act = th * D * 2;
+  auto at = [](const void *p, size_t n) { return Range{reinterpret_cast<uintptr_t>(p), p ? n : 0}; };
+  const Range r[] = {at(a.dq, act), at(a.dk_, act), at(a.dv_, act), at(a.dg, act), at(a.domega, act),  // scratch
+                     at(a.dr, th * 2), at(a.q, act), at(a.k, act), at(a.v, act), at(a.g, act), at(a.omega, act),
+                     at(a.r, th * 2), at(a.dO, act), at(a.dST, bh * D * D * 4), at(a.dpT, bh * D * 4),
+                     at(a.fSin, fused_saved_bytes(a)), at(a.status, 256)};
+  for (int i = 0; i < 5; ++i)
+    for (size_t j = i + 1; j < sizeof r / sizeof *r; ++j)
+      if (r[i].p < r[j].p + r[j].n && r[j].p < r[i].p + r[i].n) return false;
+  return true;
+}
+
 // The calls served: bf16 gradients and none of the initial state or mu, which the two kernels
 // do not form.
 bool split_bwd_supported(const Args &a) {
-  return split_bwd_context(a) && a.odt == KDN_BF16 && !a.dS0 && !a.dp0 && !a.dmu && (a.T % CM == 0 || a.split_ws);
+  return split_bwd_context(a) && a.odt == KDN_BF16 && !a.dS0 && !a.dp0 && !a.dmu && (a.T % CM == 0 || a.split_ws) &&
+         scratch_is_apart(a);
 }
 
 size_t split_bwd_workspace_bytes(const Args &a) {
