@@ -128,6 +128,23 @@ def _stream(stream):
     return stream.cuda_stream
 
 
+def _keep(stream, *made):
+    """Tensors made in this call for ``stream``: they come from the current stream's pool, which may
+    hand their memory on as soon as the last reference goes, also while ``stream`` still works there
+    (the workspace's goes with this call).  Recorded, they wait for it."""
+    if stream is None:
+        return
+    if not isinstance(stream, torch.cuda.Stream):
+        stream = torch.cuda.ExternalStream(stream.cuda_stream)
+    for t in made:
+        if t is not None:
+            t.record_stream(stream)
+
+
+def _made(given, have):
+    return [t for g, t in zip(given, have) if g is None]
+
+
 def _code(dtype):
     return _DTYPES[dtype] if isinstance(dtype, torch.dtype) else int(dtype)
 
@@ -255,6 +272,7 @@ def _fwd(name, variant, q, k, v, g, omega, r, S0, p0, *, chunk, mu, scale, o, ST
     ns, np_ = _state_sizes(variant, q, v)
     _arg(S0, "S0", torch.float32, ns, required=False)
     _arg(p0, "p0", torch.float32, np_, required=False)
+    given = (o, ST, pT, workspace)
     if o is None:
         o = torch.empty(B, T, H, dv, dtype=out_dtype, device=dev)
     if want_state and ST is None:
@@ -263,6 +281,7 @@ def _fwd(name, variant, q, k, v, g, omega, r, S0, p0, *, chunk, mu, scale, o, ST
         pT = torch.empty((B, H, dk) if variant == 0 else (B, H), dtype=torch.float32, device=dev)
     if workspace is None:
         workspace = alloc_workspace(desc, variant, False, dev)
+    _keep(stream, *_made(given, (o, ST, pT, workspace)))
     _arg(o, "o", _torch_dtype(out_dtype), B * T * H * dv)
     _arg(ST, "ST", torch.float32, ns, required=False)
     _arg(pT, "pT", torch.float32, np_, required=False)
@@ -308,6 +327,7 @@ def _bwd(name, variant, q, k, v, g, omega, r, S0, p0, dO, dST, dpT, *, chunk, mu
     ns, np_ = _state_sizes(variant, q, v)
     for t, n, m in ((S0, "S0", ns), (p0, "p0", np_), (dST, "dST", ns), (dpT, "dpT", np_)):
         _arg(t, n, torch.float32, m, required=False)
+    given = (grads, workspace)
     if grads is None:
         grads = {n: torch.empty(x.shape, dtype=out_dtype, device=dev) for n, x in
                  (("dq", q), ("dk", k), ("dv", v), ("dg", g), ("domega", omega), ("dr", r))}
@@ -318,6 +338,7 @@ def _bwd(name, variant, q, k, v, g, omega, r, S0, p0, dO, dST, dpT, *, chunk, mu
             grads["dmu"] = torch.empty(B, H, dtype=torch.float32, device=dev)
     if workspace is None:
         workspace = alloc_workspace(desc, variant, True, dev)
+    _keep(stream, *(grads.values() if given[0] is None else ()), *_made(given[1:], (workspace,)))
     G = grads
     _check_grads(G, q, k, v, g, omega, r, out_dtype, ns, np_)
     _arg(workspace, "workspace", torch.uint8)
@@ -372,6 +393,7 @@ def _fwd_save(name, variant, q, k, v, g, omega, r, S0, p0, *, mu, scale, o, ST, 
     ns, np_ = _state_sizes(variant, q, v)
     _arg(S0, "S0", torch.float32, ns, required=False)
     _arg(p0, "p0", torch.float32, np_, required=False)
+    given = (o, ST, pT, saved, workspace)
     if o is None:
         o = torch.empty(B, T, H, dv, dtype=out_dtype, device=dev)
     if want_state and ST is None:
@@ -382,6 +404,7 @@ def _fwd_save(name, variant, q, k, v, g, omega, r, S0, p0, *, mu, scale, o, ST, 
         saved = torch.empty(max(saved_bytes(desc, variant), 256), dtype=torch.uint8, device=dev)
     if workspace is None:
         workspace = alloc_workspace(desc, variant, False, dev)
+    _keep(stream, *_made(given, (o, ST, pT, saved, workspace)))
     _arg(o, "o", _torch_dtype(out_dtype), B * T * H * dv)
     _arg(ST, "ST", torch.float32, ns, required=False)
     _arg(pT, "pT", torch.float32, np_, required=False)
@@ -431,6 +454,7 @@ def _bwd_saved(name, variant, q, k, v, g, omega, r, saved, dO, dST, dpT, *, mu, 
     _arg(saved, "saved", torch.uint8)
     _arg(dST, "dST", torch.float32, ns, required=False)
     _arg(dpT, "dpT", torch.float32, np_, required=False)
+    given = (grads, workspace)
     if grads is None:
         grads = {n: torch.empty(x.shape, dtype=out_dtype, device=dev) for n, x in
                  (("dq", q), ("dk", k), ("dv", v), ("dg", g), ("domega", omega), ("dr", r))}
@@ -441,6 +465,7 @@ def _bwd_saved(name, variant, q, k, v, g, omega, r, saved, dO, dST, dpT, *, mu, 
             grads["dmu"] = torch.empty(B, H, dtype=torch.float32, device=dev)
     if workspace is None:
         workspace = alloc_workspace(desc, variant, False, dev)
+    _keep(stream, *(grads.values() if given[0] is None else ()), *_made(given[1:], (workspace,)))
     G = grads
     _check_grads(G, q, k, v, g, omega, r, out_dtype, ns, np_)
     _arg(workspace, "workspace", torch.uint8)
@@ -486,6 +511,7 @@ def _beta_eff(name, variant, k, v, g, r, saved, *, out, stream, gates, r_min):
     _arg(r, "r", k.dtype, B * T * H)
     if out is None:
         out = torch.empty(B, T, H, dtype=torch.float32, device=k.device)
+        _keep(stream, out)
     _arg(out, "out", torch.float32, B * T * H)
     st = getattr(lib(), name)(ctypes.byref(desc), _ptr(saved), ctypes.c_size_t(saved.numel()),
                               _ptr(r), _ptr(out), _stream(stream))
@@ -521,6 +547,7 @@ def _decode(name, variant, q, k, v, g, omega, r, S, p, *, mu, scale, o, stream, 
     _arg(p, "p", torch.float32, np_)
     if o is None:
         o = torch.empty(B, H, dv, dtype=out_dtype, device=q.device)
+        _keep(stream, o)
     _arg(o, "o", _torch_dtype(out_dtype), B * H * dv)
     st = getattr(lib(), name)(ctypes.byref(desc), _ptr(q), _ptr(k), _ptr(v), _ptr(g),
                               _ptr(omega), _ptr(r), _ptr(S), _ptr(p), _ptr(o), _stream(stream))
