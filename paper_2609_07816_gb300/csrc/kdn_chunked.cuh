@@ -27,14 +27,6 @@ template <> __device__ __forceinline__ void ld4<__nv_bfloat16>(const void *p, si
   v[2] = __uint_as_float(u.y << 16);
   v[3] = __uint_as_float(u.y & 0xffff0000u);
 }
-// n / d for a normal d: the approximate reciprocal and one Newton (residual) correction
-// of the quotient, which leaves the last bit's rounding at most.
-__device__ __forceinline__ float div_nr(float n, float d) {
-  float r;
-  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
-  const float q = n * r;
-  return fmaf(fmaf(-d, q, n), r, q);
-}
 __device__ __forceinline__ float4 f4(const float *v) { return make_float4(v[0], v[1], v[2], v[3]); }
 __device__ __forceinline__ void st4(float *p, const float *v) { *reinterpret_cast<float4 *>(p) = f4(v); }
 // four adjacent outputs in the caller's output dtype

@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(BwdCfg<DK>::NTH) k_chunk_bwd(Args a) {
         a.dphloc[row * DK + i] = dphl;
         a.dkpart[row * DK + i] = sdW[t * LD + i] + dkap * ph / s + 2.f * ds * ph * kv[m];
         sdKk[t * LD + i] = dphl;  // for the summary below: dphat, 1 / (1 + u phat)
-        sKk[t * LD + i] = 1.f / (1.f + a.mu / rr * kv[m] * kv[m] * ph);
+        sKk[t * LD + i] = 1.f / (1.f + a.mu * kv[m] * kv[m] / rr * ph);
       }
       if (lane == 0) a.drpart[row] = ds;
     } else {

@@ -19,9 +19,11 @@
 // All chunk-local matrices are float32 in shared memory; intermediates that
 // cross kernels live in the caller's workspace.
 //
-// Diagonal prefill B8 H16 T2048 d = 64 bf16, us: 26 + 11 + 282 + 261, 583 a call.  With the
+// Diagonal prefill B8 H16 T2048 d = 64 bf16, us: 33 + 11 + 278 + 261, 586 a call.  With the
 // uncertainty run token by token (1406), one output a thread in the chunk kernel (763) and two
 // loads a multiply-add in the memory pass (790) it was 2922.
+#include <float.h>
+
 #include "kdn_chunked.cuh"
 
 namespace kdn {
@@ -32,29 +34,39 @@ constexpr int PT = 128;  // threads of k_chunk_prep
 // ---------------------------------------------------------------------------
 // Uncertainty: chunk summaries and their scan.
 
+// The power of two that brings x >= 0 into [1, 2) (subnormals: as near as a normal factor gets).
+__device__ __forceinline__ float pow2_to_one(float x) {
+  const int e = (__float_as_int(x) >> 23) & 0xff;
+  return __int_as_float((254 - min(max(e, 1), 253)) << 23);
+}
 // A 2x2 matrix of non-negative entries times the power of two that brings its
 // largest entry into [1, 2): exact, and the ratio it represents is unchanged.
 __device__ __forceinline__ void renorm_pow2(float *m) {
-  const float s = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
-  const int e = (__float_as_int(s) >> 23) & 0xff;
-  const float inv = __int_as_float((254 - min(max(e, 1), 253)) << 23);
+  const float inv = pow2_to_one(fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])));
 #pragma unroll
   for (int q = 0; q < 4; ++q) m[q] *= inv;
 }
-// m <- M_t m with M_t = [[a, w], [u a, 1 + u w]] (p -> phat / (1 + u phat), phat = a p + w)
-__device__ __forceinline__ void moebius_step(float *m, float a, float w, float u) {
-  const float n0 = fmaf(a, m[0], w * m[2]), n1 = fmaf(a, m[1], w * m[3]);
-  m[2] = fmaf(u, n0, m[2]);
-  m[3] = fmaf(u, n1, m[3]);
-  m[0] = n0;
-  m[1] = n1;
+// m <- M_t m with M_t = [[r a, r w], [n a, r + n w]], p -> phat / (1 + (n / r) phat) with
+// phat = a p + w and n = mu k^2 (n / r = u): multiplied by r, so that no noise, however small,
+// brings a large entry in.  The result is scaled, exactly, by the powers of two of max(r, n) and of
+// m's largest entry: products of a few tokens' matrices leave the range of float32, a step
+// leaves entries of at most ~4 (1 + w).
+__device__ __forceinline__ void moebius_step(float *m, float a, float w, float r, float n) {
+  const float sc = pow2_to_one(fmaxf(r, n) * fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])));
+  const float r1 = r * sc, n1 = n * sc;
+  const float x0 = fmaf(a, m[0], w * m[2]), x1 = fmaf(a, m[1], w * m[3]);
+  m[2] = fmaf(n1, x0, r1 * m[2]);
+  m[3] = fmaf(n1, x1, r1 * m[3]);
+  m[0] = r1 * x0;
+  m[1] = r1 * x1;
 }
 __device__ __forceinline__ float moebius_apply(const float *m, float p) {
   return fmaf(m[0], p, m[1]) / fmaf(m[2], p, m[3]);
 }
 
 // Diagonal KDN: DK / 4 threads per chunk, four adjacent channels each (8- or 16-byte loads).
-// Reads k, g, omega once: 26 us for the 100 MB of B8 H16 T2048 d = 64, 0.57 of the copy rate.
+// Reads k, g, omega once; bound by issue (~40 instructions a channel and token): 33 us for the 100 MB of
+// B8 H16 T2048 d = 64 (26 with a rescaling every four tokens, which overflowed at small noises).
 template <typename DT, int DK>
 __global__ void __launch_bounds__(128) k_gain_comp_diag(Args a) {
   constexpr int L = DK / 4;
@@ -67,26 +79,26 @@ __global__ void __launch_bounds__(128) k_gain_comp_diag(Args a) {
   for (int q = 0; q < 4; ++q) { m[q][0] = 1.f; m[q][1] = 0.f; m[q][2] = 0.f; m[q][3] = 1.f; }
   const int tn = min(CC, a.T - c * CC);
   for (int t0 = 0; t0 < tn; t0 += 4) {
-    float kv[4][4], gv[4][4], wv[4][4], mr[4];
+    float kv[4][4], gv[4][4], wv[4][4], rr[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const size_t th = tok_index(a, b, c * CC + min(t0 + u, tn - 1), h);
       ld4<DT>(a.k, th * DK + i0, kv[u]);
       ld4<DT>(a.g, th * DK + i0, gv[u]);
       ld4<DT>(a.omega, th * DK + i0, wv[u]);
-      mr[u] = a.mu / gate_r(a.gates, a.rmin, ld<DT>(a.r, th));
+      rr[u] = gate_r(a.gates, a.rmin, ld<DT>(a.r, th));
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       if (t0 + u >= tn) break;
 #pragma unroll
       for (int q = 0; q < 4; ++q)
-        moebius_step(m[q], expf(2.f * gate_logalpha(a.gates, gv[u][q])), gate_omega(a.gates, wv[u][q]),
-                     mr[u] * kv[u][q] * kv[u][q]);
+        moebius_step(m[q], expf(2.f * gate_logalpha(a.gates, gv[u][q])), gate_omega(a.gates, wv[u][q]), rr[u],
+                     a.mu * kv[u][q] * kv[u][q]);
     }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) renorm_pow2(m[q]);
   }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) renorm_pow2(m[q]);
   float4 *dst = reinterpret_cast<float4 *>(a.comp) + idx * DK + i0;
 #pragma unroll
   for (int q = 0; q < 4; ++q) dst[q] = f4(m[q]);
@@ -100,7 +112,7 @@ __global__ void __launch_bounds__(128) k_gain_comp_iso(Args a) {
   if (idx >= n) return;
   const int bh = (int)(idx / a.NC), c = (int)(idx % a.NC), b = bh / a.H, h = bh % a.H;
   const int lane = KDN_TID % 32, t = c * CC + lane;
-  float aa = 1.f, n2 = 0.f, w = 0.f, u = 0.f;
+  float aa = 1.f, n2 = 0.f, w = 0.f, rr = 1.f;
   if (t < a.T) {
     const size_t th = tok_index(a, b, t, h);
     float sa = 0.f;
@@ -117,12 +129,13 @@ __global__ void __launch_bounds__(128) k_gain_comp_iso(Args a) {
     }
     aa = a.pcd ? sa / DK : expf(2.f * gate_logalpha(a.gates, ld<DT>(a.g, th)));
     w = gate_omega(a.gates, ld<DT>(a.omega, th));
-    u = a.mu * n2 / (DK * gate_r(a.gates, a.rmin, ld<DT>(a.r, th)));
+    rr = gate_r(a.gates, a.rmin, ld<DT>(a.r, th));
   }
   const size_t row = (size_t)bh * a.Tp + t;
   a.isotok[row * 2] = aa;
   a.isotok[row * 2 + 1] = n2;
-  float m[4] = {aa, w, u * aa, fmaf(u, w, 1.f)};
+  float m[4] = {1.f, 0.f, 0.f, 1.f};
+  moebius_step(m, aa, w, DK * rr, a.mu * n2);
   renorm_pow2(m);
 #pragma unroll
   for (int off = 1; off < 32; off <<= 1) {
@@ -173,6 +186,10 @@ __global__ void __launch_bounds__(128) k_gain_scan(Args a) {
 
 // row stride (elements) of the V tile, kept in the activations' dtype: 16-byte rows
 template <typename DT> __host__ __device__ constexpr int v_stride(int dv) { return dv + 16 / (int)sizeof(DT); }
+// Diagonal KDN: Kk before the division by s_t is scaled down, exactly, so that phat k / gamma stays in
+// range with it: phat k / (s_t gamma) does wherever gamma is a normal number, phat k / gamma alone
+// overflows where a strong decay meets a large process noise.
+constexpr float kKkDown = 0x1p-20f, kKkUp = 0x1p20f;
 template <typename DT, int DK>
 constexpr size_t prep_smem_bytes(int dv) {
   return sizeof(float) * (3 * CC * (DK + 4) + 2 * CC * LC + 16 * 20 + 4 * CC + DK + PT * 5) +
@@ -314,14 +331,15 @@ __global__ void __launch_bounds__(PT, DK < 128 ? 5 : 3) k_chunk_prep(Args a) {
     const float rr =
         tid < tn ? gate_r(a.gates, a.rmin, ld<DT>(a.r, tok_index(a, b, c * CC + tid, h))) : 1.f;
     s_r[tid] = rr;
-    s_mr[tid] = a.mu / rr;
+    s_mr[tid] = fminf(a.mu / rr, FLT_MAX);  // (finite, so that k = 0 gives u = 0)
     if (V == 1) {  // the scalar uncertainty of the chunk's tokens: ordered products of M_t by shuffles
       const size_t row = (size_t)bh * a.Tp + c * CC + tid;
       const float aa = a.isotok[row * 2], n2 = a.isotok[row * 2 + 1];
       const float w = tid < tn ? gate_omega(a.gates, ld<DT>(a.omega, tok_index(a, b, c * CC + tid, h))) : 0.f;
-      const float u = a.mu * n2 / (DK * rr), pin = a.pin[base];
-      float m[4] = {aa, w, u * aa, fmaf(u, w, 1.f)};
-      renorm_pow2(m);
+      const float pin = a.pin[base];
+      float m[4] = {1.f, 0.f, 0.f, 1.f};
+      moebius_step(m, aa, w, DK * rr, a.mu * n2);
+  renorm_pow2(m);
 #pragma unroll
       for (int off = 1; off < 32; off <<= 1) {
         float p[4], x[4];
@@ -360,9 +378,9 @@ __global__ void __launch_bounds__(PT, DK < 128 ? 5 : 3) k_chunk_prep(Args a) {
 #pragma unroll
     for (int j = 0; j < LB; ++j) {
       gs += gv[j];
-      if (V == 0) moebius_step(m, a2[j], wv[j], s_mr[t0 + j] * kv[j] * kv[j]);
-      if (V == 0 && (j & 3) == 3) renorm_pow2(m);
+      if (V == 0) moebius_step(m, a2[j], wv[j], s_r[t0 + j], a.mu * kv[j] * kv[j]);
     }
+    renorm_pow2(m);
     float *mine = s_seg + tid * 5;
 #pragma unroll
     for (int q = 0; q < 4; ++q) mine[q] = m[q];
@@ -389,15 +407,14 @@ __global__ void __launch_bounds__(PT, DK < 128 ? 5 : 3) k_chunk_prep(Args a) {
       gam = expf(G);
       if (V == 0) {
         ph = fmaf(a2[j], p, wv[j]);                             // eq. diag-covariance-prediction
-        p = div_nr(ph, fmaf(s_mr[t] * kv[j] * kv[j], ph, 1.f));  // eq. diag-cov-update
-        kk = ph * kv[j];
+        p = ph / fmaf(s_mr[t] * kv[j] * kv[j], ph, 1.f);        // eq. diag-cov-update
+        kk = kKkDown * ph * kv[j];
       } else {
         kk = s_be[t] * kv[j];
       }
       sK[t * LD + i] = kv[j] * gam;
       sQ[t * LD + i] = a.tau * qv[j] * gam;
-      // (diag: still without 1 / s_t; a subnormal gamma's reciprocal may overflow where the quotient does not)
-      sKk[t * LD + i] = gam > 1e-37f ? div_nr(kk, gam) : kk / gam;
+      sKk[t * LD + i] = kk / gam;  // (diag: kKkDown s_t Kk)
       if (SAVE) {
         if (V == 0) a.phat[grow + (size_t)t * DK] = ph;
         a.gam[grow + (size_t)t * DK] = gam;
@@ -412,7 +429,7 @@ __global__ void __launch_bounds__(PT, DK < 128 ? 5 : 3) k_chunk_prep(Args a) {
   __syncthreads();
 
   // T' = Kbar Kk'^T (threads 0..63), A'_qk = Qbar Kk'^T (64..127): 32 x 32, 4 x 4 a thread.
-  // Diagonal KDN: the diagonal of T' is sum_i phat k^2, so s_t = r_t + T'_tt (eq. kla-box-gain).
+  // Diagonal KDN: the diagonal of T' is kKkDown sum_i phat k^2, so s_t = r_t + kKkUp T'_tt (eq. kla-box-gain).
   const int lane = tid & 31, w2 = (tid >> 5) & 1, ga = lane >> 2, gb = (lane & 3) + 4 * w2;
   float acc[4][4];
   zero<4>(acc);
@@ -424,8 +441,8 @@ __global__ void __launch_bounds__(PT, DK < 128 ? 5 : 3) k_chunk_prep(Args a) {
 #pragma unroll
         for (int n = 0; n < 4; ++n)
           if (ga + 8 * m == 4 * gb + n) {
-            const float s = s_r[4 * gb + n] + acc[m][n];
-            s_is[4 * gb + n] = 1.f / s;
+            const float s = s_r[4 * gb + n] + kKkUp * acc[m][n];
+            s_is[4 * gb + n] = fminf(kKkUp / s, FLT_MAX);
             if (SAVE) a.stok[(size_t)bh * a.Tp + c * CC + 4 * gb + n] = s;
           }
     }
