@@ -128,17 +128,27 @@ def _stream(stream):
     return stream.cuda_stream
 
 
+def _torch_stream(stream):
+    return stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(stream.cuda_stream)
+
+
 def _keep(stream, *made):
-    """Tensors made in this call for ``stream``: they come from the current stream's pool, which may
-    hand their memory on as soon as the last reference goes, also while ``stream`` still works there
-    (the workspace's goes with this call).  Recorded, they wait for it."""
+    """Results made in this call, which ``stream`` will write: they come from the current stream's pool,
+    which may hand their memory on as soon as the last reference goes, also while ``stream`` still
+    works there.  Recorded, they wait for it."""
+    if stream is not None:
+        for t in made:
+            if t is not None:
+                t.record_stream(_torch_stream(stream))
+
+
+def _scratch(desc, variant, backward, device, stream):
+    """The call's own workspace, which goes when the call returns: from the pool of the stream that
+    works in it, so that neither what ran there before nor what comes next overlaps that work."""
     if stream is None:
-        return
-    if not isinstance(stream, torch.cuda.Stream):
-        stream = torch.cuda.ExternalStream(stream.cuda_stream)
-    for t in made:
-        if t is not None:
-            t.record_stream(stream)
+        return alloc_workspace(desc, variant, backward, device)
+    with torch.cuda.stream(_torch_stream(stream)):
+        return alloc_workspace(desc, variant, backward, device)
 
 
 def _made(given, have):
@@ -272,7 +282,7 @@ def _fwd(name, variant, q, k, v, g, omega, r, S0, p0, *, chunk, mu, scale, o, ST
     ns, np_ = _state_sizes(variant, q, v)
     _arg(S0, "S0", torch.float32, ns, required=False)
     _arg(p0, "p0", torch.float32, np_, required=False)
-    given = (o, ST, pT, workspace)
+    given = (o, ST, pT)
     if o is None:
         o = torch.empty(B, T, H, dv, dtype=out_dtype, device=dev)
     if want_state and ST is None:
@@ -280,8 +290,8 @@ def _fwd(name, variant, q, k, v, g, omega, r, S0, p0, *, chunk, mu, scale, o, ST
     if want_state and pT is None:
         pT = torch.empty((B, H, dk) if variant == 0 else (B, H), dtype=torch.float32, device=dev)
     if workspace is None:
-        workspace = alloc_workspace(desc, variant, False, dev)
-    _keep(stream, *_made(given, (o, ST, pT, workspace)))
+        workspace = _scratch(desc, variant, False, dev, stream)
+    _keep(stream, *_made(given, (o, ST, pT)))
     _arg(o, "o", _torch_dtype(out_dtype), B * T * H * dv)
     _arg(ST, "ST", torch.float32, ns, required=False)
     _arg(pT, "pT", torch.float32, np_, required=False)
@@ -327,7 +337,7 @@ def _bwd(name, variant, q, k, v, g, omega, r, S0, p0, dO, dST, dpT, *, chunk, mu
     ns, np_ = _state_sizes(variant, q, v)
     for t, n, m in ((S0, "S0", ns), (p0, "p0", np_), (dST, "dST", ns), (dpT, "dpT", np_)):
         _arg(t, n, torch.float32, m, required=False)
-    given = (grads, workspace)
+    made = grads is None
     if grads is None:
         grads = {n: torch.empty(x.shape, dtype=out_dtype, device=dev) for n, x in
                  (("dq", q), ("dk", k), ("dv", v), ("dg", g), ("domega", omega), ("dr", r))}
@@ -337,8 +347,9 @@ def _bwd(name, variant, q, k, v, g, omega, r, S0, p0, dO, dST, dpT, *, chunk, mu
                                        dtype=torch.float32, device=dev)
             grads["dmu"] = torch.empty(B, H, dtype=torch.float32, device=dev)
     if workspace is None:
-        workspace = alloc_workspace(desc, variant, True, dev)
-    _keep(stream, *(grads.values() if given[0] is None else ()), *_made(given[1:], (workspace,)))
+        workspace = _scratch(desc, variant, True, dev, stream)
+    if made:
+        _keep(stream, *grads.values())
     G = grads
     _check_grads(G, q, k, v, g, omega, r, out_dtype, ns, np_)
     _arg(workspace, "workspace", torch.uint8)
@@ -393,7 +404,7 @@ def _fwd_save(name, variant, q, k, v, g, omega, r, S0, p0, *, mu, scale, o, ST, 
     ns, np_ = _state_sizes(variant, q, v)
     _arg(S0, "S0", torch.float32, ns, required=False)
     _arg(p0, "p0", torch.float32, np_, required=False)
-    given = (o, ST, pT, saved, workspace)
+    given = (o, ST, pT, saved)
     if o is None:
         o = torch.empty(B, T, H, dv, dtype=out_dtype, device=dev)
     if want_state and ST is None:
@@ -403,8 +414,8 @@ def _fwd_save(name, variant, q, k, v, g, omega, r, S0, p0, *, mu, scale, o, ST, 
     if saved is None:
         saved = torch.empty(max(saved_bytes(desc, variant), 256), dtype=torch.uint8, device=dev)
     if workspace is None:
-        workspace = alloc_workspace(desc, variant, False, dev)
-    _keep(stream, *_made(given, (o, ST, pT, saved, workspace)))
+        workspace = _scratch(desc, variant, False, dev, stream)
+    _keep(stream, *_made(given, (o, ST, pT, saved)))
     _arg(o, "o", _torch_dtype(out_dtype), B * T * H * dv)
     _arg(ST, "ST", torch.float32, ns, required=False)
     _arg(pT, "pT", torch.float32, np_, required=False)
@@ -454,7 +465,7 @@ def _bwd_saved(name, variant, q, k, v, g, omega, r, saved, dO, dST, dpT, *, mu, 
     _arg(saved, "saved", torch.uint8)
     _arg(dST, "dST", torch.float32, ns, required=False)
     _arg(dpT, "dpT", torch.float32, np_, required=False)
-    given = (grads, workspace)
+    made = grads is None
     if grads is None:
         grads = {n: torch.empty(x.shape, dtype=out_dtype, device=dev) for n, x in
                  (("dq", q), ("dk", k), ("dv", v), ("dg", g), ("domega", omega), ("dr", r))}
@@ -464,8 +475,9 @@ def _bwd_saved(name, variant, q, k, v, g, omega, r, saved, dO, dST, dpT, *, mu, 
                                        dtype=torch.float32, device=dev)
             grads["dmu"] = torch.empty(B, H, dtype=torch.float32, device=dev)
     if workspace is None:
-        workspace = alloc_workspace(desc, variant, False, dev)
-    _keep(stream, *(grads.values() if given[0] is None else ()), *_made(given[1:], (workspace,)))
+        workspace = _scratch(desc, variant, False, dev, stream)
+    if made:
+        _keep(stream, *grads.values())
     G = grads
     _check_grads(G, q, k, v, g, omega, r, out_dtype, ns, np_)
     _arg(workspace, "workspace", torch.uint8)

@@ -1,5 +1,7 @@
-"""``stream=`` other than the current one: what a call allocates is recorded on that stream, so that
-its memory is not handed on while the stream still works there."""
+"""``stream=`` other than the current one: results that a call makes are recorded on that stream, and
+the workspace it makes comes from that stream's own pool, so that their memory is not handed on
+while the stream still works there."""
+import contextlib
 import types
 
 import pytest
@@ -14,6 +16,17 @@ def test_everything_made_is_recorded(fake, monkeypatch, variant):  # noqa: F811
     seen = []
     monkeypatch.setattr(torch.Tensor, "record_stream", lambda t, s: seen.append((t, s)), raising=False)
     monkeypatch.setattr(torch.cuda, "ExternalStream", lambda handle: ("external", handle))
+    pool, scratch = [None], []
+
+    @contextlib.contextmanager
+    def under(stream):
+        pool[0], before = stream, pool[0]
+        yield
+        pool[0] = before
+
+    monkeypatch.setattr(torch.cuda, "stream", under)
+    alloc = kdn.alloc_workspace
+    monkeypatch.setattr(kdn, "alloc_workspace", lambda *a, **kw: scratch.append(pool[0]) or alloc(*a, **kw))
     st = types.SimpleNamespace(cuda_stream=7)
     fwd, bwd, fsave, bsaved, beff, dec = FNS[variant]
     B, T, H, d = 2, 150, 3, 128
@@ -22,24 +35,27 @@ def test_everything_made_is_recorded(fake, monkeypatch, variant):  # noqa: F811
     dO = torch.empty(B, T, H, d, dtype=BF, device="cuda")
     ws = torch.empty(256, dtype=torch.uint8, device="cuda")
 
-    def made(n, fn, *a, **kw):  # n tensors of the call's own
+    def made(n, w, fn, *a, **kw):  # n results and w workspaces of the call's own
         seen.clear()
+        scratch.clear()
         out = fn(*a, **kw)
-        assert not seen  # the current stream: nothing to record
+        assert not seen and scratch == [None] * w  # the current stream: nothing to record
+        scratch.clear()
         fn(*a, stream=st, **kw)
         assert len(seen) == n and all(s == ("external", 7) for _, s in seen), fn
+        assert scratch == [("external", 7)] * w, fn
         return out
 
-    made(4, fwd, *x)
-    made(2, fwd, *x, want_state=False)
-    made(1, fwd, *x, want_state=False, workspace=ws)
-    saved = made(5, fsave, *x)[3]
-    made(7, bsaved, *x, saved, dO, want_state_grads=False)
-    made(9, bsaved, *x, saved, dO, workspace=ws)
-    grads = made(10, bwd, *x, S, p, dO)
-    made(1, bwd, *x, S, p, dO, grads=grads)
-    made(1, beff, x[1], x[2], x[3], x[5], saved)
-    made(1, dec, *[t[:, 0].contiguous() for t in x], S, p)
+    made(3, 1, fwd, *x)
+    made(1, 1, fwd, *x, want_state=False)
+    made(1, 0, fwd, *x, want_state=False, workspace=ws)
+    saved = made(4, 1, fsave, *x)[3]
+    made(6, 1, bsaved, *x, saved, dO, want_state_grads=False)
+    made(9, 0, bsaved, *x, saved, dO, workspace=ws)
+    grads = made(9, 1, bwd, *x, S, p, dO)
+    made(0, 1, bwd, *x, S, p, dO, grads=grads)
+    made(1, 0, beff, x[1], x[2], x[3], x[5], saved)
+    made(1, 0, dec, *[t[:, 0].contiguous() for t in x], S, p)
 
 
 @pytest.mark.gpu
@@ -64,12 +80,16 @@ def test_memory_is_not_handed_on_early(T):
                 torch.full((n,), 255, dtype=torch.uint8, device="cuda")
 
     for _ in range(3):
+        # (the side stream waits for the current one before each call: the results' memory comes from there)
         with torch.cuda.stream(side):
             torch.cuda._sleep(20_000_000)
+        side.wait_stream(torch.cuda.current_stream())
         got = [kdn.kdn_diag_fwd(*x, stream=side, **kw)]
         over()
+        side.wait_stream(torch.cuda.current_stream())
         got.append(kdn.kdn_diag_fwd_save(*x, stream=side, **kw))
         over()
+        side.wait_stream(torch.cuda.current_stream())
         g2 = kdn.kdn_diag_bwd_saved(*x, got[1][3], d["dO"], want_state_grads=False, stream=side, **kw)
         over()
         torch.cuda.synchronize()
