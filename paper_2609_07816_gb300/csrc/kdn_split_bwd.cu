@@ -567,8 +567,8 @@ __global__ void __launch_bounds__(BT, 1)
   // takes the next ticket and leaves (job, b, h, c) in shared memory.
   struct Job { int j, b, h, c; const unsigned char *rec; size_t rc; };
   auto take = [&]() {
-    const int j = (int)atomicAdd(P.ticket, 1u);
-    const int jj = j < njobs ? j : 0, bh = jj % BH;
+    const unsigned u = atomicAdd(P.ticket, 1u);  // (unsigned: no job from whatever else the word may hold)
+    const int j = u < (unsigned)njobs ? (int)u : njobs, jj = j < njobs ? j : 0, bh = jj % BH;
     s_next[0] = j;
     s_next[1] = bh / a.H;
     s_next[2] = bh % a.H;

@@ -1803,6 +1803,11 @@ __global__ void __launch_bounds__(WT, 1)
   if (threadIdx.x == 0) s_place = (int)atomicAdd(P.ticket, 1u);
   __syncthreads();
   const int BH = P.a.B * P.a.H, block = s_place, workers = (int)gridDim.x - 2 * BH;
+  // (a workspace that something else writes to meanwhile: no place, no access; the others' waits end)
+  if ((unsigned)block >= gridDim.x) {
+    if (threadIdx.x == 0) atomicExch(P.a.status, (unsigned)KDN_ERR_TIMEOUT);
+    return;
+  }
   if (block < BH) wy_gain<SV, LG>(mk, mg, mw, P.a, P.pin, block);
   else if (block < BH + workers) wy_body<SV, LG, 1>(mk, mg, mw, mv, mq, P, block - BH, workers);
   else wy_state<SV>(mv, P, block - BH - workers);
