@@ -191,9 +191,7 @@ kdn_status_t kdn_iso_bwd(const kdn_desc_t *desc, const void *q, const void *k,
    chunk the memory S entering it, its R = U - W S_in, -W, A_qk,
    A = (I + T)^-1 and (Diagonal KDN) Y = V - Kbar S_in as fp16 tiles (96 KB),
    the pre-write variance phat and the cumulative decay gamma of every
-   (token, channel) in float32 (64 KB), per-token scalars (2 KB), for most
-   diagonal problems of 96 chunks and more also [-Kbar; Qbar] and
-   K'^T (48 KB), and the
+   (token, channel) in float32 (64 KB), per-token scalars (2 KB), and the
    float32 uncertainty p entering it.  kdn_diag_bwd_saved is kdn_diag_bwd that starts from that
    context instead of recomputing the forward (same gradients).  The diagonal
    backward may use dq, dk, dv, dg and domega as scratch before it writes them,

@@ -113,7 +113,6 @@ static_assert(O_AQ + 8 * KB <= O_WN && O_XT + 8 * KB <= O_RH, "map");
 
 struct BwdParams {
   Args a;
-  size_t rec;  // bytes of a context record
 };
 
 // G: the gate inputs are logits (KDN_GATES_LOGITS), a compile-time choice so
@@ -214,7 +213,7 @@ __global__ void __launch_bounds__(BT, 1)
   // bytes: one thread issuing them all holds the whole CTA up.
   float *n_tok = reinterpret_cast<float *>(sm + OFF_NX), *n_gm = n_tok + 5 * CM;
   auto issue_a_ctx = [&](int c) {
-    const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * P.rec;
+    const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * kCtxBytes;
     switch (lane == 0 ? warp : -1) {
       case 0: mbar_expect_tx(bar_a, 32768); bulk_g2s(sin, rec + kCtxS, 32768, bar_a); break;
       case 1:
@@ -260,7 +259,7 @@ __global__ void __launch_bounds__(BT, 1)
     }
   };
   auto issue_g = [&](int c) {
-    const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * P.rec;
+    const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * kCtxBytes;
     switch (lane == 0 ? warp : -1) {
       case 2: mbar_expect_tx(bar_g, 32768); bulk_g2s(sm + O_PHB, rec + kCtxPh, 32768, bar_g); break;
       case 3: mbar_expect_tx(bar_g, 16384); bulk_g2s(sm + O_GA0, rec + kCtxGa, 16384, bar_g); break;
@@ -412,7 +411,7 @@ __global__ void __launch_bounds__(BT, 1)
       s_fr[tid] = live ? dgate_sig(G, z) : 1.f;
       s_fw[tid] = V == 1 && G && live ? sigmoid_f(__bfloat162float(ny)) : 1.f;
     }
-    const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * P.rec;
+    const unsigned char *rec = a.fSin + ((size_t)bh * NC + c) * kCtxBytes;
     float e16[16], ph16[16];
     if (V != 0 && !SD) {  // gamma [64][128] of the isotropic KDN with per-channel decay
       const float *cga = reinterpret_cast<const float *>(rec + kCtxGa) + t0 * D + ci;
@@ -1022,7 +1021,7 @@ __global__ void __launch_bounds__(BT, 1)
     if (c > 0) {
       issue_a_ctx(c - 1);  // the context buffers are free
       // phat and gamma of chunk c - 1, which are read later, into L2 now
-      if (tid == 480) bulk_prefetch_l2(rec - P.rec + kCtxPh, SD ? 256 : 65536);
+      if (tid == 480) bulk_prefetch_l2(rec - kCtxBytes + kCtxPh, SD ? 256 : 65536);
     }
     // ---- [18] per channel (lane ci, tokens t0..t0+15): back through Gamma and the
     //           gain emission, then the uncertainty recursion backwards in time.
@@ -1421,16 +1420,15 @@ bool fused_bwd_supported(const Args &a) { return a.chunk != 32 && fused_fwd_supp
 size_t fused_saved_bytes(const Args &a) {
   if (!fused_bwd_supported(a)) return 0;
   const size_t nc = (a.T + CM - 1) / CM;
-  return (size_t)a.B * a.H * nc * (fused_ctx_record_bytes(a) + D * sizeof(float));
+  return (size_t)a.B * a.H * nc * (kCtxBytes + D * sizeof(float));
 }
 
-size_t fused_ctx_record_bytes(const Args &a) { return split_bwd_context(a) ? kCtxSplitBytes : kCtxBytes; }
+size_t fused_ctx_record_bytes() { return kCtxBytes; }
 
 kdn_status_t launch_fused_bwd_sweep(const Args &a, cudaStream_t s) {
   if (split_bwd_supported(a)) return launch_split_bwd(a, a.T % CM == 0 ? nullptr : a.split_ws, s);
   BwdParams P;
   P.a = a;
-  P.rec = fused_ctx_record_bytes(a);
   CUtensorMap mq, mk, mv, mdo;
   if (!make_map(&mq, a.q, a) || !make_map(&mk, a.k, a) || !make_map(&mv, a.v, a) ||
       !make_map(&mdo, a.dO, a))

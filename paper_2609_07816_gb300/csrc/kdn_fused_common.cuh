@@ -89,12 +89,6 @@ __device__ __forceinline__ void unpack_h8(uint4 u, float *v) {
 constexpr int kCtxS = 0, kCtxR = 32768, kCtxW = 49152, kCtxAqk = 65536, kCtxA = 73728;
 constexpr int kCtxPh = 81920, kCtxGa = 114688, kCtxTok = 147456, kCtxY = 149504;
 constexpr int kCtxBytes = 165888;
-// Records that feed the two-kernel backward (kdn_split_bwd.cu) go on with two operand
-// tiles of its serial part:
-//   [-Kbar; Qbar] fp16 [128][128 i], two slabs of 128 rows (rows 64..127: Qbar)  32 KB
-//   K'^T  fp16 [128 i][64 s]  (K_tail = diag(1/s) K')                            16 KB
-// and hold r_t and its input z_t after s_t among the per-token values.
-constexpr int kCtxKQ = kCtxBytes, kCtxKt = kCtxKQ + 32768, kCtxSplitBytes = kCtxKt + 16384;
 
 // Smallest cumulative decay gamma_C = exp(G_C) of a chunk the fused kernels
 // accept: they divide by gamma (Kk = kappa / gamma), which must stay a normal

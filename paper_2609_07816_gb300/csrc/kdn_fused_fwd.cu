@@ -935,11 +935,11 @@ __global__ void __launch_bounds__(FT, 1)
 // kappa = phat k / s_t, so k^T kappa = (s_t - r_t) / s_t = 1 - r_t / s_t;
 // Isotropic KDN kappa = beta_t k, so k^T kappa = beta_t |k_t|^2.  One thread per
 // token, one CTA per (chunk, batch * head).
-__global__ void __launch_bounds__(CM) k_beta_eff(const Args a, size_t rec, const unsigned char *saved, float *out) {
+__global__ void __launch_bounds__(CM) k_beta_eff(const Args a, const unsigned char *saved, float *out) {
   const int c = blockIdx.x, bh = blockIdx.y, t = threadIdx.x;
   const int b = bh / a.H, h = bh % a.H, NC = (a.T + CM - 1) / CM, tt = c * CM + t;
   if (tt >= a.T) return;
-  const float *tok = reinterpret_cast<const float *>(saved + ((size_t)bh * NC + c) * rec + kCtxTok);
+  const float *tok = reinterpret_cast<const float *>(saved + ((size_t)bh * NC + c) * kCtxBytes + kCtxTok);
   const size_t th = tok_index(a, b, tt, h);
   if (a.variant == 0) {
     const float rr = gate_r(a.gates, a.rmin, ld<__nv_bfloat16>(a.r, th));
@@ -977,7 +977,7 @@ kdn_status_t launch_wait_selftest(unsigned *status, cudaStream_t s) {
 kdn_status_t launch_beta_eff(const Args &a, const void *saved, float *out, cudaStream_t s) {
   const int NC = (a.T + CM - 1) / CM;
   k_beta_eff<<<dim3((unsigned)NC, (unsigned)(a.B * a.H)), CM, 0, s>>>(
-      a, fused_ctx_record_bytes(a), static_cast<const unsigned char *>(saved), out);
+      a, static_cast<const unsigned char *>(saved), out);
   return cudaGetLastError() == cudaSuccess ? KDN_OK : KDN_ERR_CUDA;
 }
 

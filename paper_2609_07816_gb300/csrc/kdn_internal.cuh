@@ -165,9 +165,8 @@ bool wy_fwd_supported(const Args &a, bool save);  // save: the context-saving in
 kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S = nullptr,
                            float *save_p = nullptr, char *ws = nullptr);
 // The same with the gain, the chunks and the memory on CTAs of their own where these sizes gain from it:
-// with the extended context, or with this much scratch in the workspace.
+// in the context's own records, or with this much scratch in the workspace.
 bool wy_split_sizes(const Args &a);
-bool wy_split_save(const Args &a);  // the context-saving forward
 size_t wy_split_workspace_bytes(const Args &a);
 // beta_eff [B,T,H] (float32) from the per-token gain scalars of a context saved by
 // the fused training forward (one launch).
@@ -184,11 +183,11 @@ kdn_status_t launch_fused_bwd_sweep(const Args &a, cudaStream_t s);
 // (batch, head) and 64-token chunk one record of fused_ctx_record_bytes(), then
 // per chunk the 128 float32 uncertainties entering it.
 size_t fused_saved_bytes(const Args &a);
-size_t fused_ctx_record_bytes(const Args &a);
-// Two-kernel backward of the Diagonal KDN (kdn_split_bwd.cu): whether the context of these
-// sizes feeds it, whether it serves this call, the scratch it needs in the workspace (ragged
+size_t fused_ctx_record_bytes();
+// Two-kernel backward of the Diagonal KDN (kdn_split_bwd.cu): whether these sizes gain from
+// it, whether it serves this call, the scratch it needs in the workspace (ragged
 // lengths; otherwise its scratch lies in the gradient buffers) and its launcher.
-bool split_bwd_context(const Args &a);
+bool split_bwd_sizes(const Args &a);
 bool split_bwd_supported(const Args &a);
 size_t split_bwd_workspace_bytes(const Args &a);
 kdn_status_t launch_split_bwd(const Args &a, char *ws, cudaStream_t s);

@@ -112,7 +112,6 @@ __device__ __forceinline__ void cp_wait() {
 struct SplitParams {
   Args a;
   Scratch s;
-  size_t rec;        // bytes of a context record
   unsigned *ticket;  // zeroed before k_bwd_chunk
 };
 
@@ -135,7 +134,7 @@ __global__ void __launch_bounds__(TT, 4)
   const int tid = threadIdx.x, half = (int)(blockIdx.x & 1u), r0 = 2 * (tid & 31), ci = 64 * half + r0;
   const int t0 = 8 * (tid >> 5), job = (int)(blockIdx.x >> 1);
   const int NC = (a.T + CM - 1) / CM, c = job % NC, bh = job / NC, b = bh / a.H, h = bh % a.H;
-  const unsigned char *rec = a.fSin + (size_t)job * P.rec;
+  const unsigned char *rec = a.fSin + (size_t)job * kCtxBytes;
   const float *cph = reinterpret_cast<const float *>(rec + kCtxPh) + t0 * D + ci;
   const float *cga = reinterpret_cast<const float *>(rec + kCtxGa) + ci;
   float2 ph[8], ga[8];
@@ -234,7 +233,7 @@ __global__ void __launch_bounds__(BT, 1)
   tc_fence_after();
   const uint32_t TS = *s_tbase, TX = TS + 128;
   const uint32_t lane_base = (uint32_t)(32 * wq) << 16;
-  auto record = [&](int c) { return a.fSin + ((size_t)bh * NC + c) * P.rec; };
+  auto record = [&](int c) { return a.fSin + ((size_t)bh * NC + c) * kCtxBytes; };
   // The copies are issued one per warp (lane 0): a single thread's run of them would hold
   // up the chain of products.  Warps 1..7 load, 8..11 store dS, 12..15 store dR.
   auto issue = [&](int c, int buf) {  // A_qk, K_tail, dO, gamma_C
@@ -270,8 +269,8 @@ __global__ void __launch_bounds__(BT, 1)
       case 7: mbar_expect_tx(bar_w, 16384); bulk_g2s(sm + SO_WN, rec + kCtxW, 16384, bar_w); break;
       case 8:  // the next chunk's, into L2
         if (c > 0) {
-          bulk_prefetch_l2(rec - P.rec + kCtxS, 32768);
-          bulk_prefetch_l2(rec - P.rec + kCtxW, 16384);
+          bulk_prefetch_l2(rec - kCtxBytes + kCtxS, 32768);
+          bulk_prefetch_l2(rec - kCtxBytes + kCtxW, 16384);
           for (int s = 0; s < 2; ++s) {
             tma_prefetch_4d(&m2, 64 * s, h, (c - 1) * CM, b);
             tma_prefetch_4d(&m3, 64 * s, h, (c - 1) * CM, b);
@@ -581,7 +580,7 @@ __global__ void __launch_bounds__(BT, 1)
     o.h = s_next[2];
     o.c = s_next[3];
     o.rc = (size_t)(o.b * a.H + o.h) * NC + o.c;
-    o.rec = a.fSin + o.rc * P.rec;
+    o.rec = a.fSin + o.rc * kCtxBytes;
     return o;
   };
   // The copies of a chunk's tiles, spread over lane 0 of the warps: one thread issuing them
@@ -1175,9 +1174,8 @@ __global__ void __launch_bounds__(BT, 1)
 // tiles 12.  B8 H16 T4096: 2.1 M cycles against 2.5 M (1120 us, 1326 us); B2 H16 T1999 with
 // logit gates: 0.49 M against 1.28 M (255 us, 668 us); with as many sequences as SMs and one
 // or two chunks each the sweep is ahead.  Fewer than 96 chunks in all are left to the sweep (a
-// few tens of us either way).  The rule reads sizes only: a context is saved before it is
-// known which gradients will be asked for.
-bool split_bwd_context(const Args &a) {
+// few tens of us either way).
+bool split_bwd_sizes(const Args &a) {
   if (a.variant != 0 || a.chunk == 32 || !fused_fwd_supported(a)) return false;
   const long long bh = (long long)a.B * a.H, nc = (a.T + CM - 1) / CM, waves = (bh + kSms - 1) / kSms;
   if (bh * nc < 96) return false;
@@ -1204,12 +1202,12 @@ static bool scratch_is_apart(const Args &a) {
 // The calls served: bf16 gradients and none of the initial state or mu, which the two kernels
 // do not form.
 bool split_bwd_supported(const Args &a) {
-  return split_bwd_context(a) && a.odt == KDN_BF16 && !a.dS0 && !a.dp0 && !a.dmu && (a.T % CM == 0 || a.split_ws) &&
+  return split_bwd_sizes(a) && a.odt == KDN_BF16 && !a.dS0 && !a.dp0 && !a.dmu && (a.T % CM == 0 || a.split_ws) &&
          scratch_is_apart(a);
 }
 
 size_t split_bwd_workspace_bytes(const Args &a) {
-  if (!split_bwd_context(a) || a.odt != KDN_BF16 || a.T % CM == 0) return 0;
+  if (!split_bwd_sizes(a) || a.odt != KDN_BF16 || a.T % CM == 0) return 0;
   const size_t n = (size_t)a.B * a.H * ((a.T + CM - 1) / CM);
   return n * 5 * 16384;
 }
@@ -1217,7 +1215,6 @@ size_t split_bwd_workspace_bytes(const Args &a) {
 kdn_status_t launch_split_bwd(const Args &a, char *ws, cudaStream_t s) {
   SplitParams P;
   P.a = a;
-  P.rec = fused_ctx_record_bytes(a);
   P.ticket = a.status + 1;
   const int NC = (a.T + CM - 1) / CM;
   void *buf[4] = {a.dq, a.dk_, a.dv_, a.dg};

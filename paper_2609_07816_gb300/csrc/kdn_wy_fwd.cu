@@ -455,9 +455,8 @@ __device__ __noinline__ void direct_products(int tid, const unsigned char *rk, c
 struct WyParams {
   Args a;
   unsigned char *save_S;  // SV: [BH][NC] context records of the backward
-  size_t rec;             // SV: bytes of a record; beyond kCtxBytes it also takes Qbar and K'^T
   float *save_p;          // SV: [BH][NC][128] uncertainty carry entering each chunk
-  // CH: records of the per-chunk operands (SV: the context records), what enters every chunk
+  // CH: records of the per-chunk operands (SV: in the context records), what enters every chunk
   unsigned char *pre;
   size_t prec;
   float *pin;             // [BH][NC][128], preset to kUnset
@@ -505,13 +504,14 @@ __device__ __forceinline__ bool flow_wait(const unsigned *flag) {
   return false;
 }
 
-// Per-chunk operands that k_wy_flow's chunk part leaves for its memory part, in a context record (SV) or in a record of
-// their own: [-Kbar; Qbar] fp16 32 KB, K'^T fp16 [128 i][64 s] 16 KB, A fp16 8 KB, A'_qk fp16
-// 8 KB (context: in R's place until R is there), gamma_C [128], s_t [64].
+// Per-chunk operands that k_wy_flow's chunk part leaves for its memory part, in a record of their
+// own or (SV) in the context record: [-Kbar; Qbar] fp16 32 KB, K'^T fp16 [128 i][64 s] 16 KB, A
+// fp16 8 KB, A'_qk fp16 8 KB, gamma_C [128], s_t [64].  In the context the first two and A'_qk lie where
+// S_in, Y and R go, which the memory part writes once it has read them.
 constexpr size_t kPreBytes = 66560;
 template <int SV>
 struct Pre {
-  static constexpr int KQ = SV ? kCtxKQ : 0, Kt = SV ? kCtxKt : 32768, A = SV ? kCtxA : 49152;
+  static constexpr int KQ = SV ? kCtxS : 0, Kt = SV ? kCtxY : 32768, A = SV ? kCtxA : 49152;
   static constexpr int Aq = SV ? kCtxR : 57344, gC = SV ? kCtxGa + 63 * D * 4 : 65536, s = SV ? kCtxTok : 66048;
 };
 
@@ -568,7 +568,6 @@ __device__ __forceinline__ void wy_body(const CUtensorMap &mk, const CUtensorMap
   };
   const bool issuer = tid == 128;  // copies; the MMAs: its whole warp with an elected lane
   const int warp_u = __shfl_sync(0xffffffffu, warp, 0);
-  const bool ext = SV && P.rec > (size_t)kCtxBytes;
   const uint32_t lane_base = (uint32_t)(32 * wq) << 16;
 
   if (issuer) {
@@ -701,11 +700,6 @@ __device__ __forceinline__ void wy_body(const CUtensorMap &mk, const CUtensorMap
       const float r = !live ? 1.f : LG ? a.rmin + softplus_w(z) : z;  // r = r_min + softplus(z) (Sec. 5)
       sr[tid] = r;
       smur[tid] = a.mu / r;
-      if (ext) {  // r_t and z_t for the backward (tokens past T: 1 and 0)
-        float *tok = reinterpret_cast<float *>(P.save_S + o.rc * P.rec + kCtxTok);
-        tok[CM + tid] = r;
-        tok[2 * CM + tid] = z;
-      }
     }
     load_r(c + 1);
     bar_sync(kBarGain, 128);
@@ -779,7 +773,7 @@ __device__ __forceinline__ void wy_body(const CUtensorMap &mk, const CUtensorMap
     const bool oor = !SV && bar_or(kBarGain, 128, cref < kMinHalfG);
     if (tid == 0) s_oor[sb] = oor ? 1 : 0;
     float Gt = 0.f;  // G_t of this channel (range mode)
-    unsigned char *gctx = SV ? P.save_S + o.rc * P.rec : nullptr;
+    unsigned char *gctx = SV ? P.save_S + o.rc * kCtxBytes : nullptr;
     unsigned char *gpre = CH ? P.pre + o.rc * P.prec : gctx;
     if (SV && !CH) P.save_p[o.rc * D + i] = p;
     float *cph = SV ? reinterpret_cast<float *>(gctx + kCtxPh) + i : nullptr;
@@ -861,7 +855,7 @@ __device__ __forceinline__ void wy_body(const CUtensorMap &mk, const CUtensorMap
           else kt[j >> 1] |= hb << 16;
         }
         if (!CH) tmem_st4u(tkt + lane_base + (uint32_t)(4 * blk), kt);
-        if (CH || ext)
+        if (CH)
           *reinterpret_cast<uint4 *>(gpre + Pre<SV>::Kt + chunk_off(i, blk)) = make_uint4(kt[0], kt[1], kt[2], kt[3]);
         if (blk < 7) {
 #pragma unroll
@@ -887,7 +881,7 @@ __device__ __forceinline__ void wy_body(const CUtensorMap &mk, const CUtensorMap
   for (int c = 0; c < NC; ++c) {
     const uint32_t tkt = TKT + (uint32_t)((c & 1) * 32);
     const Job o = job(c);
-    unsigned char *ctx = SV ? P.save_S + o.rc * P.rec : nullptr;
+    unsigned char *ctx = SV ? P.save_S + o.rc * kCtxBytes : nullptr;
     unsigned char *pre = CH ? P.pre + o.rc * P.prec : ctx;
     if ((SV || CH) && lane == 0) bulk_wait_read();  // the previous chunk's context tiles have left shared memory
     // ---- [0] the previous chunk's MMA-O / MMA-S2 must be done before V is brought
@@ -1141,8 +1135,6 @@ __device__ __forceinline__ void wy_body(const CUtensorMap &mk, const CUtensorMap
       bulk_commit();
     } else if (!CH && SV && lane == 0) {
       if (warp == 10) bulk_s2g(ctx + kCtxS, s16, 32768);
-      else if (ext && (warp == 11 || warp == 14))
-        bulk_s2g(ctx + kCtxKQ + (warp == 14) * 16384 + 8192, as1 + (warp == 14) * 16384 + 8192, 8192);
       bulk_commit();
     }
 
@@ -1634,7 +1626,7 @@ __device__ __forceinline__ void wy_state(const CUtensorMap &mv, const WyParams &
   const uint32_t id_16 = idesc_f16(128, 128, 0, 1);  // A K-major, B MN-major
   for (int c = 0; c < NC; ++c) {
     unsigned char *d = sm + (c & 1) * SB_BUF, *vr = d + SB_V;
-    unsigned char *ctx = SV ? P.save_S + ((size_t)bh * NC + c) * P.rec : nullptr;
+    unsigned char *ctx = SV ? P.save_S + ((size_t)bh * NC + c) * kCtxBytes : nullptr;
     const float *sc = reinterpret_cast<const float *>(d + SB_SC);
     const uint32_t TU = TUb + (c & 1) * 128;
     // ---- [1] S -> fp16; diag(gamma_C) S back
@@ -1837,10 +1829,6 @@ bool wy_split_sizes(const Args &a) {
   return std::max(nc * 7, (bh * nc + workers - 1) / workers * 19) + 45 < nc * 17;
 }
 
-bool wy_split_save(const Args &a) {
-  return wy_split_sizes(a) && fused_ctx_record_bytes(a) > (size_t)kCtxBytes;
-}
-
 size_t wy_split_workspace_bytes(const Args &a) {
   if (!wy_split_sizes(a)) return 0;
   return (size_t)a.B * a.H * ((a.T + CM - 1) / CM) * (kPreBytes + D * sizeof(float) + sizeof(unsigned));
@@ -1864,7 +1852,7 @@ kdn_status_t launch_wy(const WyParams &W, bool split, cudaStream_t s) {
   }
   if (cudaFuncSetAttribute(k_wy_flow<SV, LG>, attr, FLOW_SMEM) != cudaSuccess ||
       cudaMemsetAsync(W.pin, 0xff, n * D * sizeof(float), s) != cudaSuccess ||
-      (SV ? cudaMemset2DAsync(W.flag, W.rec, 0, sizeof(unsigned), n, s)
+      (SV ? cudaMemset2DAsync(W.flag, kCtxBytes, 0, sizeof(unsigned), n, s)
           : cudaMemsetAsync(W.flag, 0, n * sizeof(unsigned), s)) != cudaSuccess)
     return KDN_ERR_CUDA;
   k_wy_flow<SV, LG><<<kSms, WT, FLOW_SMEM, s>>>(mk, mg, mw, mv, mq, W);
@@ -1878,7 +1866,6 @@ kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S,
   WyParams P;
   P.a = a;
   P.save_S = save_S;
-  P.rec = fused_ctx_record_bytes(a);
   P.save_p = save_p;
   P.pre = nullptr;
   P.prec = 0;
@@ -1886,13 +1873,13 @@ kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S,
   P.flag = nullptr;
   P.fstride = 0;
   P.ticket = a.status + 2;
-  const bool split = save_S ? wy_split_save(a) : wy_split_sizes(a) && ws;
+  const bool split = wy_split_sizes(a) && (save_S || ws);
   if (split && save_S) {
     P.pre = save_S;
-    P.prec = P.rec;
+    P.prec = kCtxBytes;
     P.pin = save_p;
     P.flag = reinterpret_cast<unsigned *>(save_S + kCtxTok + 3 * CM * sizeof(float));  // (no value there)
-    P.fstride = P.rec / sizeof(unsigned);
+    P.fstride = kCtxBytes / sizeof(unsigned);
   } else if (split) {
     const size_t n = (size_t)a.B * a.H * ((a.T + CM - 1) / CM);
     P.pre = reinterpret_cast<unsigned char *>(ws);
