@@ -138,8 +138,7 @@ const char *kdn_status_string(kdn_status_t status);
    2 bytes per element of o, 6 when out_dtype is KDN_BF16).
    For sequences too few to fill the GPU but not served so, the diagonal
    forward uses 65.5 KB per (batch, head, chunk) to run all chunks' work that
-   needs no memory in parallel (same results), and the backward of the training
-   pair with bfloat16 gradients 80 KB per chunk when T is no multiple of 64.
+   needs no memory in parallel (same results).
    A smaller workspace that still holds the single-pass layout (256 bytes)
    runs the single pass. */
 size_t kdn_fwd_workspace_bytes(const kdn_desc_t *desc, int variant);
@@ -204,9 +203,13 @@ kdn_status_t kdn_iso_bwd(const kdn_desc_t *desc, const void *q, const void *k,
    aligned (a smaller or misaligned one -> KDN_ERR_WORKSPACE).  It is written
    by kdn_diag_fwd_save and read by kdn_diag_bwd_saved, which must see the same
    descriptor and the same q, k, v, g, omega, r (and the forward's S0, p0).
-   workspace: kdn_fwd_workspace_bytes(desc, variant) bytes for both calls.  The
-   other arguments are those of kdn_*_fwd / kdn_*_bwd. */
+   workspace: kdn_fwd_workspace_bytes(desc, variant) bytes serve both calls.  With
+   kdn_bwd_saved_workspace_bytes(desc, variant), which adds 80 KB per (batch, head)
+   where T is no multiple of 64, every diagonal backward with bfloat16 gradients
+   and no state gradients may run in parallel over the chunks (same gradients).
+   The other arguments are those of kdn_*_fwd / kdn_*_bwd. */
 size_t kdn_saved_bytes(const kdn_desc_t *desc, int variant);
+size_t kdn_bwd_saved_workspace_bytes(const kdn_desc_t *desc, int variant);
 
 kdn_status_t kdn_diag_fwd_save(const kdn_desc_t *desc, const void *q,
                                const void *k, const void *v, const void *g,

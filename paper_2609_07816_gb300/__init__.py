@@ -66,6 +66,7 @@ _SIG = {
     "kdn_diag_decode_step": ([ctypes.POINTER(kdn_desc_t)] + [_P] * 10, ctypes.c_int),
     "kdn_iso_decode_step": ([ctypes.POINTER(kdn_desc_t)] + [_P] * 10, ctypes.c_int),
     "kdn_diag_fwd_noalloc": ([ctypes.POINTER(kdn_desc_t)] + [_P] * 12, ctypes.c_int),
+    "kdn_bwd_saved_workspace_bytes": ([ctypes.POINTER(kdn_desc_t), ctypes.c_int], ctypes.c_size_t),
     "kdn_saved_bytes": ([ctypes.POINTER(kdn_desc_t), ctypes.c_int], ctypes.c_size_t),
     "kdn_diag_fwd_save": ([ctypes.POINTER(kdn_desc_t)] + [_P] * 12 + [ctypes.c_size_t, _P,
                                                                    ctypes.c_size_t, _P], ctypes.c_int),
@@ -260,8 +261,12 @@ def _desc_from(variant, q, v, g, *, chunk, mu, scale, out_dtype, gates=KDN_GATES
                  _code(out_dtype), int(gates), float(r_min))
 
 
-def workspace_bytes(desc: kdn_desc_t, variant: int, backward: bool = False) -> int:
-    fn = lib().kdn_bwd_workspace_bytes if backward else lib().kdn_fwd_workspace_bytes
+def workspace_bytes(desc: kdn_desc_t, variant: int, backward=False) -> int:
+    """``backward``: False for kdn_*_fwd and kdn_*_fwd_save, True for kdn_*_bwd, "saved" for
+    kdn_*_bwd_saved (which also takes the forward's, see kdn.h)."""
+    L = lib()
+    fn = (L.kdn_bwd_saved_workspace_bytes if backward == "saved" else
+          L.kdn_bwd_workspace_bytes if backward else L.kdn_fwd_workspace_bytes)
     return int(fn(ctypes.byref(desc), int(variant)))
 
 
@@ -475,7 +480,7 @@ def _bwd_saved(name, variant, q, k, v, g, omega, r, saved, dO, dST, dpT, *, mu, 
                                        dtype=torch.float32, device=dev)
             grads["dmu"] = torch.empty(B, H, dtype=torch.float32, device=dev)
     if workspace is None:
-        workspace = _scratch(desc, variant, False, dev, stream)
+        workspace = _scratch(desc, variant, "saved", dev, stream)
     if made:
         _keep(stream, *grads.values())
     G = grads

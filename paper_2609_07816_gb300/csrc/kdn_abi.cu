@@ -4,8 +4,6 @@
 #include <math.h>
 #include <stdint.h>
 
-#include <algorithm>
-
 #include "kdn_internal.cuh"
 
 namespace kdn {
@@ -371,10 +369,14 @@ size_t kdn_fwd_workspace_bytes(const kdn_desc_t *desc, int variant) {
   Args a;
   if (fill_sizes(desc, variant, false, &a) != KDN_OK) return 0;
   const int nseg = seg_count(a);
-  // (the training backward of ragged lengths takes its scratch from the same workspace)
   return workspace_layout(&a, nullptr, false) +
-         (nseg > 1 ? seg_workspace_bytes(a, nseg)
-                   : std::max(split_bwd_workspace_bytes(a), wy_split_workspace_bytes(a)));
+         (nseg > 1 ? seg_workspace_bytes(a, nseg) : wy_split_workspace_bytes(a));
+}
+
+size_t kdn_bwd_saved_workspace_bytes(const kdn_desc_t *desc, int variant) {
+  Args a;
+  if (fill_sizes(desc, variant, false, &a) != KDN_OK) return 0;
+  return workspace_layout(&a, nullptr, false) + split_bwd_workspace_bytes(a);
 }
 
 size_t kdn_bwd_workspace_bytes(const kdn_desc_t *desc, int variant) {

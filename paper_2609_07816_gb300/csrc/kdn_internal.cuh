@@ -185,8 +185,8 @@ kdn_status_t launch_fused_bwd_sweep(const Args &a, cudaStream_t s);
 size_t fused_saved_bytes(const Args &a);
 size_t fused_ctx_record_bytes();
 // Two-kernel backward of the Diagonal KDN (kdn_split_bwd.cu): whether these sizes gain from
-// it, whether it serves this call, the scratch it needs in the workspace (ragged
-// lengths; otherwise its scratch lies in the gradient buffers) and its launcher.
+// it, whether it serves this call, the scratch it needs in the workspace (the partial
+// last chunk of a ragged length; the rest lies in the gradient buffers) and its launcher.
 bool split_bwd_sizes(const Args &a);
 bool split_bwd_supported(const Args &a);
 size_t split_bwd_workspace_bytes(const Args &a);

@@ -16,11 +16,11 @@
 // busy on 152 SMs, 32 at B2 H16.  Here the serial part is ~6 K cycles a chunk.
 //
 // Scratch per chunk and head: dS fp16 (32 KB), dR as an fp16 pair (32 KB; K_tail and Qbar
-// before), and ~4 KB of small values.  With whole chunks (T a multiple of 64) it lies in the
-// gradient buffers themselves: a chunk's rows of dq, dk, dv, dg hold its tiles and its rows of
+// before), and ~4 KB of small values.  It lies in the gradient buffers
+// themselves: a chunk's rows of dq, dk, dv, dg hold its tiles and its rows of
 // domega the small values until k_bwd_chunk, which is the only one to read them, writes the
-// chunk's gradients there.  Ragged lengths use the workspace (a tile's rows are not
-// tokens, and rows past T do not exist in the gradients).
+// chunk's gradients there.  The partial last chunk of a ragged length has too few rows there: its
+// 80 KB lie in the workspace.
 //
 // It serves bf16 gradients without state gradients (see split_bwd_supported).  The gradients are
 // those of the one-kernel sweep bit for bit: the same operand tiles (fp16 tiles, hi/lo
@@ -47,12 +47,28 @@ constexpr int kSms = 152;
 // Where a chunk's small values lie: rows of 256 bytes, one per token of the chunk.
 // Rows 0..7: dgamma_C's dS part [4][128]; 8..11: dp [128] as (value, tag) pairs; 12: lambda;
 // 13: the r inputs z_t [64].
+// The partial last chunk of a ragged length (its tiles' rows are not tokens) has rows of its own.
 struct Scratch {
-  unsigned char *small;
-  int T;       // tokens of the scratch layout (a multiple of 64)
+  unsigned char *small;  // domega
+  unsigned char *tail;   // [5][B][64][H][128] 16-bit: the last chunk's tiles and small values (null: none)
+  int last;              // chunk that lies there
 };
 __device__ __forceinline__ unsigned char *small_row(const Scratch &s, const Args &a, int b, int h, int c, int n) {
-  return s.small + (((size_t)b * s.T + c * CM + n) * a.H + h) * (2 * D);
+  const bool tl = s.tail && c == s.last;
+  return (tl ? s.tail : s.small) +
+         ((tl ? ((size_t)4 * a.B + b) * CM + n : (size_t)b * a.T + c * CM + n) * a.H + h) * (2 * D);
+}
+// Box of scratch tile k (0, 1: dS, 2, 3: dR; m: the gradient buffer of whole chunks) of a chunk.
+struct Box { const CUtensorMap *m; int t, b; };
+__device__ __forceinline__ Box box_at(const Scratch &s, const Args &a, const CUtensorMap &m, const CUtensorMap &mt,
+                                      int k, int b, int c) {
+  return s.tail && c == s.last ? Box{&mt, 0, k * a.B + b} : Box{&m, c * CM, b};
+}
+__device__ __forceinline__ void box_load(void *dst, const Box &x, uint64_t *bar, int col, int h) {
+  tma_load_4d(dst, x.m, bar, col, h, x.t, x.b);
+}
+__device__ __forceinline__ void box_store(const Box &x, const void *src, int col, int h) {
+  tma_store_4d(x.m, src, col, h, x.t, x.b);
 }
 __device__ __forceinline__ float *small_dgc(const Scratch &s, const Args &a, int b, int h, int c, int i) {
   return reinterpret_cast<float *>(small_row(s, a, b, h, c, i >> 6)) + (i & 63);
@@ -125,7 +141,7 @@ constexpr int TT = 256, TILE_SMEM = 16 * KB + 1024;
 
 __global__ void __launch_bounds__(TT, 4)
     k_bwd_tiles(const __grid_constant__ CUtensorMap m2, const __grid_constant__ CUtensorMap m3,
-                const SplitParams P) {
+                const __grid_constant__ CUtensorMap mt, const SplitParams P) {
   const Args &a = P.a;
   extern __shared__ unsigned char smraw[];
   __shared__ float s_si[CM];
@@ -177,7 +193,8 @@ __global__ void __launch_bounds__(TT, 4)
   fence_proxy_async();
   __syncthreads();
   if (tid == 0 || tid == 32) {  // 64 rows of each: one box, at channel 64 half of the scratch tile
-    tma_store_4d(tid == 0 ? &m2 : &m3, sm + (tid >> 5) * 8 * KB, 64 * half, h, c * CM, b);
+    box_store(tid == 0 ? box_at(P.s, a, m2, mt, 2, b, c) : box_at(P.s, a, m3, mt, 3, b, c), sm + (tid >> 5) * 8 * KB,
+              64 * half, h);
     bulk_commit();
     bulk_wait_all();
   }
@@ -200,7 +217,8 @@ static_assert(STATE_SMEM <= 232448, "shared memory");
 __global__ void __launch_bounds__(BT, 1)
     k_bwd_state(const __grid_constant__ CUtensorMap mdo, const __grid_constant__ CUtensorMap m0,
                 const __grid_constant__ CUtensorMap m1, const __grid_constant__ CUtensorMap m2,
-                const __grid_constant__ CUtensorMap m3, const SplitParams P) {
+                const __grid_constant__ CUtensorMap m3, const __grid_constant__ CUtensorMap mt,
+                const SplitParams P) {
   const Args &a = P.a;
   extern __shared__ unsigned char smraw[];
   unsigned char *sm =
@@ -244,8 +262,7 @@ __global__ void __launch_bounds__(BT, 1)
       case 1: mbar_expect_tx(bar, 8192); bulk_g2s(d + SB_AQ, rec + kCtxAqk, 8192, bar); break;
       case 2:
         mbar_expect_tx(bar, 16384);
-        tma_load_4d(d + SB_KT, &m2, bar, 0, h, c * CM, b);
-        tma_load_4d(d + SB_KT + 8192, &m2, bar, 64, h, c * CM, b);
+        for (int s = 0; s < 2; ++s) box_load(d + SB_KT + s * 8192, box_at(P.s, a, m2, mt, 2, b, c), bar, 64 * s, h);
         break;
       case 3: mbar_expect_tx(bar, 8192); tma_load_4d(d + SB_DO, &mdo, bar, 0, h, c * CM, b); break;
       case 4: mbar_expect_tx(bar, 8192); tma_load_4d(d + SB_DO + 8192, &mdo, bar, 64, h, c * CM, b); break;
@@ -263,8 +280,7 @@ __global__ void __launch_bounds__(BT, 1)
     switch (lane == 0 ? warp : -1) {
       case 6:
         mbar_expect_tx(bar_w, 16384);
-        tma_load_4d(sm + SO_QB, &m3, bar_w, 0, h, c * CM, b);
-        tma_load_4d(sm + SO_QB + 8192, &m3, bar_w, 64, h, c * CM, b);
+        for (int s = 0; s < 2; ++s) box_load(sm + SO_QB + s * 8192, box_at(P.s, a, m3, mt, 3, b, c), bar_w, 64 * s, h);
         break;
       case 7: mbar_expect_tx(bar_w, 16384); bulk_g2s(sm + SO_WN, rec + kCtxW, 16384, bar_w); break;
       case 8:  // the next chunk's, into L2
@@ -405,8 +421,8 @@ __global__ void __launch_bounds__(BT, 1)
     }
     if (lane == 0 && warp >= 8 && warp < 12) {  // dS: rows i 0..63 in m0's tiles, 64..127 in m1's
       const int s = warp & 1;
-      if (warp < 10) tma_store_4d(&m0, dsh + s * 16384, 64 * s, h, c * CM, b);
-      else tma_store_4d(&m1, dsh + s * 16384 + 8192, 64 * s, h, c * CM, b);
+      if (warp < 10) box_store(box_at(P.s, a, m0, mt, 0, b, c), dsh + s * 16384, 64 * s, h);
+      else box_store(box_at(P.s, a, m1, mt, 1, b, c), dsh + s * 16384 + 8192, 64 * s, h);
       bulk_commit();
     }
     if (warp >= 4 && warp < 8) {  // the small values of this chunk
@@ -448,8 +464,8 @@ __global__ void __launch_bounds__(BT, 1)
     if (lane == 0 && warp >= 12) {  // dR^T rows j 0..63, 64..127, over K_tail and Qbar, which have been read
       const int s = warp & 1;
       ok = mbar_wait(bar_w, it & 1, kWaitIters) && ok;
-      if (warp < 14) tma_store_4d(&m2, drh + s * 8192, 64 * s, h, c * CM, b);
-      else tma_store_4d(&m3, drl + s * 8192, 64 * s, h, c * CM, b);
+      if (warp < 14) box_store(box_at(P.s, a, m2, mt, 2, b, c), drh + s * 8192, 64 * s, h);
+      else box_store(box_at(P.s, a, m3, mt, 3, b, c), drl + s * 8192, 64 * s, h);
       bulk_commit();
     }
   }
@@ -503,9 +519,10 @@ template <int G>  // G: logit gates
 __global__ void __launch_bounds__(BT, 1)
     k_bwd_chunk(const __grid_constant__ CUtensorMap mq, const __grid_constant__ CUtensorMap mk,
                 const __grid_constant__ CUtensorMap mdo, const __grid_constant__ CUtensorMap mw,
-                const __grid_constant__ CUtensorMap mdv, const __grid_constant__ CUtensorMap m0,
-                const __grid_constant__ CUtensorMap m1, const __grid_constant__ CUtensorMap m2,
-                const __grid_constant__ CUtensorMap m3, const SplitParams P) {
+                const __grid_constant__ CUtensorMap m0, const __grid_constant__ CUtensorMap m1,
+                const __grid_constant__ CUtensorMap m2, const __grid_constant__ CUtensorMap m3,
+                const __grid_constant__ CUtensorMap mt,
+                const SplitParams P) {
   const Args &a = P.a;
   extern __shared__ unsigned char smraw[];
   unsigned char *sm =
@@ -599,10 +616,10 @@ __global__ void __launch_bounds__(BT, 1)
       case 0: mbar_expect_tx(bar_a, 32768); bulk_g2s(sin, o.rec + kCtxS, 32768, bar_a); break;
       case 1: mbar_expect_tx(bar_a, 16384); bulk_g2s(sm + O_RV, o.rec + kCtxY, 16384, bar_a); break;
       case 2: mbar_expect_tx(bar_a, 8192); bulk_g2s(sm + O_AH, o.rec + kCtxA, 8192, bar_a); break;
-      case 3: mbar_expect_tx(bar_a, 8192); tma_load_4d(sm + O_WN, &m2, bar_a, 0, o.h, t, o.b); break;
-      case 4: mbar_expect_tx(bar_a, 8192); tma_load_4d(sm + O_WN + 8192, &m2, bar_a, 64, o.h, t, o.b); break;
-      case 5: mbar_expect_tx(bar_a, 8192); tma_load_4d(sm + O_KT, &m3, bar_a, 0, o.h, t, o.b); break;
-      case 6: mbar_expect_tx(bar_a, 8192); tma_load_4d(sm + O_KT + 8192, &m3, bar_a, 64, o.h, t, o.b); break;
+      case 3: mbar_expect_tx(bar_a, 8192); box_load(sm + O_WN, box_at(P.s, a, m2, mt, 2, o.b, o.c), bar_a, 0, o.h); break;
+      case 4: mbar_expect_tx(bar_a, 8192); box_load(sm + O_WN + 8192, box_at(P.s, a, m2, mt, 2, o.b, o.c), bar_a, 64, o.h); break;
+      case 5: mbar_expect_tx(bar_a, 8192); box_load(sm + O_KT, box_at(P.s, a, m3, mt, 3, o.b, o.c), bar_a, 0, o.h); break;
+      case 6: mbar_expect_tx(bar_a, 8192); box_load(sm + O_KT + 8192, box_at(P.s, a, m3, mt, 3, o.b, o.c), bar_a, 64, o.h); break;
       case 7:
         bulk_wait_read();  // the dv tile has left the R buffer
         mbar_expect_tx(bar_a, 16384);
@@ -613,8 +630,12 @@ __global__ void __launch_bounds__(BT, 1)
       case 10: mbar_expect_tx(bar_g, 32768); bulk_g2s(sm + O_G, o.rec + kCtxPh, 32768, bar_g); break;
       case 11: mbar_expect_tx(bar_g, 8192); bulk_g2s(sm + O_DT, o.rec + kCtxGa + 8192, 8192, bar_g); break;
       case 12: mbar_expect_tx(bar_g, 8192); bulk_g2s(sm + O_GA3, o.rec + kCtxGa + 24576, 8192, bar_g); break;
-      case 13: tma_prefetch_4d(&m0, 0, o.h, t, o.b); tma_prefetch_4d(&m0, 64, o.h, t, o.b); break;  // dS
-      case 14: tma_prefetch_4d(&m1, 0, o.h, t, o.b); tma_prefetch_4d(&m1, 64, o.h, t, o.b); break;
+      case 13:  // dS
+      case 14: {
+        const Box x = warp == 13 ? box_at(P.s, a, m0, mt, 0, o.b, o.c) : box_at(P.s, a, m1, mt, 1, o.b, o.c);
+        for (int s = 0; s < 2; ++s) tma_prefetch_4d(x.m, 64 * s, o.h, x.t, x.b);
+        break;
+      }
       case 15:
         if (G) bulk_prefetch_l2(o.rec + kCtxGa, 24576);
         break;
@@ -705,8 +726,8 @@ __global__ void __launch_bounds__(BT, 1)
     if (lane == 0 && warp >= 12) {  // dS over phat
       const int s = (warp >> 1) & 1;
       mbar_expect_tx(bar_d, 8192);
-      if (warp & 1) tma_load_4d(sm + O_G + s * 16384 + 8192, &m1, bar_d, 64 * s, h, c * CM, b);
-      else tma_load_4d(sm + O_G + s * 16384, &m0, bar_d, 64 * s, h, c * CM, b);
+      if (warp & 1) box_load(sm + O_G + s * 16384 + 8192, box_at(P.s, a, m1, mt, 1, b, c), bar_d, 64 * s, h);
+      else box_load(sm + O_G + s * 16384, box_at(P.s, a, m0, mt, 0, b, c), bar_d, 64 * s, h);
     }
     // ---- [3] A -> bf16; lambda dO -> fp16 in place
     {
@@ -869,8 +890,8 @@ __global__ void __launch_bounds__(BT, 1)
       }
       commit_if(lead, bar_mma);
     } else if (tid == 224) {
-      tma_store_4d(&mdv, sm + O_RH, 0, h, c * CM, b);
-      tma_store_4d(&mdv, sm + O_RH + 8192, 64, h, c * CM, b);
+      tma_store_4d(&m2, sm + O_RH, 0, h, c * CM, b);  // (m2: dv itself)
+      tma_store_4d(&m2, sm + O_RH + 8192, 64, h, c * CM, b);
       bulk_commit();
     }
     mm_ok = mma_poll();
@@ -1208,8 +1229,7 @@ bool split_bwd_supported(const Args &a) {
 
 size_t split_bwd_workspace_bytes(const Args &a) {
   if (!split_bwd_sizes(a) || a.odt != KDN_BF16 || a.T % CM == 0) return 0;
-  const size_t n = (size_t)a.B * a.H * ((a.T + CM - 1) / CM);
-  return n * 5 * 16384;
+  return (size_t)a.B * a.H * 5 * 16384;
 }
 
 kdn_status_t launch_split_bwd(const Args &a, char *ws, cudaStream_t s) {
@@ -1217,35 +1237,35 @@ kdn_status_t launch_split_bwd(const Args &a, char *ws, cudaStream_t s) {
   P.a = a;
   P.ticket = a.status + 1;
   const int NC = (a.T + CM - 1) / CM;
-  void *buf[4] = {a.dq, a.dk_, a.dv_, a.dg};
-  P.s.T = NC * CM;
   P.s.small = static_cast<unsigned char *>(a.domega);
-  if (ws) {
-    const size_t n = (size_t)a.B * a.H * NC * 16384;
-    for (int k = 0; k < 4; ++k) buf[k] = ws + k * n;
-    P.s.small = reinterpret_cast<unsigned char *>(ws + 4 * n);
-  }
-  Args t = a;  // the scratch tiles: bf16 tensors of whole chunks
-  t.T = P.s.T;
-  CUtensorMap m[4], mq, mk, mdo, mdv;
+  P.s.tail = a.T % CM ? reinterpret_cast<unsigned char *>(ws) : nullptr;
+  P.s.last = NC - 1;
+  const void *buf[4] = {a.dq, a.dk_, a.dv_, a.dg};
+  CUtensorMap m[4], mq, mk, mdo;
   for (int k = 0; k < 4; ++k)
-    if (!make_map(&m[k], buf[k], t)) return KDN_ERR_CUDA;
-  if (!make_map(&mq, a.q, a) || !make_map(&mk, a.k, a) || !make_map(&mdo, a.dO, a) || !make_map(&mdv, a.dv_, a))
-    return KDN_ERR_CUDA;
+    if (!make_map(&m[k], buf[k], a)) return KDN_ERR_CUDA;
+  CUtensorMap mt = m[0];
+  if (P.s.tail) {  // [5 B, 64, H, 128]
+    Args t = a;
+    t.B = 5 * a.B;
+    t.T = CM;
+    if (!make_map(&mt, P.s.tail, t)) return KDN_ERR_CUDA;
+  }
+  if (!make_map(&mq, a.q, a) || !make_map(&mk, a.k, a) || !make_map(&mdo, a.dO, a)) return KDN_ERR_CUDA;
   CUtensorMap mw = mq;  // the omega logits
   if (a.gates && !make_map(&mw, a.omega, a)) return KDN_ERR_CUDA;
   const long long njobs = (long long)a.B * a.H * NC;
-  k_bwd_tiles<<<(unsigned)(2 * njobs), TT, TILE_SMEM, s>>>(m[2], m[3], P);
+  k_bwd_tiles<<<(unsigned)(2 * njobs), TT, TILE_SMEM, s>>>(m[2], m[3], mt, P);
   if (cudaGetLastError() != cudaSuccess) return KDN_ERR_CUDA;
   if (cudaFuncSetAttribute(k_bwd_state, cudaFuncAttributeMaxDynamicSharedMemorySize, STATE_SMEM) != cudaSuccess)
     return KDN_ERR_CUDA;
-  k_bwd_state<<<a.B * a.H, BT, STATE_SMEM, s>>>(mdo, m[0], m[1], m[2], m[3], P);
+  k_bwd_state<<<a.B * a.H, BT, STATE_SMEM, s>>>(mdo, m[0], m[1], m[2], m[3], mt, P);
   if (cudaGetLastError() != cudaSuccess) return KDN_ERR_CUDA;
   const auto kern = a.gates ? k_bwd_chunk<1> : k_bwd_chunk<0>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, CHUNK_SMEM) != cudaSuccess)
     return KDN_ERR_CUDA;
-  kern<<<(unsigned)(njobs < kSms ? njobs : kSms), BT, CHUNK_SMEM, s>>>(mq, mk, mdo, mw, mdv, m[0], m[1], m[2],
-                                                                       m[3], P);
+  kern<<<(unsigned)(njobs < kSms ? njobs : kSms), BT, CHUNK_SMEM, s>>>(mq, mk, mdo, mw, m[0], m[1], m[2], m[3],
+                                                                       mt, P);
   return cudaGetLastError() == cudaSuccess ? KDN_OK : KDN_ERR_CUDA;
 }
 

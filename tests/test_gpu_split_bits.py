@@ -37,7 +37,7 @@ def test_two_kernels_equal_the_sweep(B, T, H, gates, slow, low):
     x = [d[n] for n in NAMES]
     G = kdn.KDN_GATES_LOGITS if gates == "logits" else kdn.KDN_GATES_POST
     desc = kdn.make_desc(B, T, H, 128, 128, torch.bfloat16, out_dtype=torch.bfloat16, gates=G, r_min=0.0)
-    kw = dict(out_dtype=torch.bfloat16, gates=G, r_min=0.0, workspace=kdn.alloc_workspace(desc, 0))
+    kw = dict(out_dtype=torch.bfloat16, gates=G, r_min=0.0, workspace=kdn.alloc_workspace(desc, 0, "saved"))
     cu = lambda y: torch.tensor(y, dtype=torch.float32, device="cuda")
     _, _, _, saved = kdn.kdn_diag_fwd_save(*x, d["S0"], d["p0"], **kw)
     for end in ((cu(dST), cu(dpT)), (None, None)):

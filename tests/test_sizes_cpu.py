@@ -21,3 +21,14 @@ def test_saved_context_is_one_record_a_chunk(B, T, H, out):
     """162 KB and 128 floats per 64-token chunk at every size: no kernel choice adds to it."""
     for variant in (0, 1):
         assert kdn.saved_bytes(_desc(B, T, H, out), variant) == B * H * ((T + 63) // 64) * (165888 + 512)
+
+
+@pytest.mark.parametrize("B,T,H", [(8, 4095, 16), (64, 1000, 32), (33, 191, 2), (8, 4096, 16)])
+def test_a_forward_pays_for_no_backward(B, T, H):
+    """More sequences than the parallel forward takes: a status word, at any length; the ragged
+    training backward asks for its partial last chunk (80 KB a sequence) by itself."""
+    d = _desc(B, T, H)
+    assert kdn.workspace_bytes(d, 0) == 256
+    assert kdn.workspace_bytes(d, 0, "saved") == 256 + (B * H * 81920 if T % 64 else 0)
+    assert kdn.workspace_bytes(_desc(B, T, H, kdn.KDN_F32), 0, "saved") == 256
+    assert kdn.workspace_bytes(d, 1, "saved") == 256
