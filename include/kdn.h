@@ -137,8 +137,8 @@ const char *kdn_status_string(kdn_status_t status);
    (160 KB per (batch, head, segment), 2 KB per (batch, head, chunk), and
    2 bytes per element of o, 6 when out_dtype is KDN_BF16).
    For sequences too few to fill the GPU but not served so, the diagonal
-   forward uses 65.5 KB per (batch, head, chunk) to run all chunks' work that
-   needs no memory in parallel (same results).
+   forward uses 65.5 KB per (batch, head, chunk), 140 MB at most, to run all chunks'
+   work that needs no memory in parallel (same results).
    A smaller workspace that still holds the single-pass layout (256 bytes)
    runs the single pass. */
 size_t kdn_fwd_workspace_bytes(const kdn_desc_t *desc, int variant);

@@ -463,6 +463,11 @@ struct WyParams {
   unsigned *flag;         // per chunk, fstride apart, zeroed: warps that have written their part of its record
   size_t fstride;
   unsigned *ticket;       // zeroed: CTAs of k_wy_flow that have started
+  // k_wy_flow: the chunks c0 .. c0 + nc - 1 of every sequence, and the states around them (null: the
+  // zero memory, the unit uncertainty; not written)
+  int c0, nc;
+  const float *S_in, *p_in;
+  float *S_out, *p_out;
 };
 
 // The uncertainty entering a chunk is handed over as the 4-byte value itself, in place of a
@@ -553,7 +558,7 @@ __device__ __forceinline__ void wy_body(const CUtensorMap &mk, const CUtensorMap
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int wq = warp & 3, wg = warp >> 2;  // TMEM lane quarter, column group
   const int bh = block;  // (not CH)
-  const int NCs = (a.T + CM - 1) / CM, BH = a.B * a.H;
+  const int NCs = CH ? P.nc : (a.T + CM - 1) / CM, BH = a.B * a.H;
   // chunks of this CTA, counted by `c` below; ct, b, h: a chunk's place in its sequence
   const int NC = CH ? (NCs * BH - block + nblocks - 1) / nblocks : NCs;
   struct Job { int ct, b, h; size_t rc; };
@@ -564,6 +569,7 @@ __device__ __forceinline__ void wy_body(const CUtensorMap &mk, const CUtensorMap
     o.b = q / a.H;
     o.h = q % a.H;
     o.rc = (size_t)q * NCs + o.ct;
+    if (CH) o.ct += P.c0;
     return o;
   };
   const bool issuer = tid == 128;  // copies; the MMAs: its whole warp with an elected lane
@@ -1380,14 +1386,15 @@ static_assert(SG_SMEM <= 232448, "shared memory");
 
 template <int SV, int LG>
 __device__ __forceinline__ void wy_gain(const CUtensorMap &mk, const CUtensorMap &mg, const CUtensorMap &mw,
-                                        const Args &a, float *pin, const int bh) {
+                                        const WyParams &P, const int bh) {
+  const Args &a = P.a;
   extern __shared__ unsigned char smraw[];
   unsigned char *sm =
       reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   float *s_ss = reinterpret_cast<float *>(sm + SG_SS), *s_mr = reinterpret_cast<float *>(sm + SG_MR);
   uint64_t *bars = reinterpret_cast<uint64_t *>(sm + SG_BAR);
   int *s_oor = reinterpret_cast<int *>(bars + 2);
-  const int tid = threadIdx.x, b = bh / a.H, h = bh % a.H, NC = (a.T + CM - 1) / CM;
+  const int tid = threadIdx.x, b = bh / a.H, h = bh % a.H, NC = P.nc;
   auto alpha = [&](int half) { return reinterpret_cast<float *>(sm + SG_X + half * SG_HALF); };  // then omega, u
   if (tid == 0) {
     mbar_init(bars, 1);
@@ -1396,9 +1403,9 @@ __device__ __forceinline__ void wy_gain(const CUtensorMap &mk, const CUtensorMap
   }
   __syncthreads();
   if (tid < D) {  // ---- the chain
-    float p = a.p0 ? a.p0[(size_t)bh * D + tid] : 1.f;
+    float p = P.p_in ? P.p_in[(size_t)bh * D + tid] : 1.f;
     for (int c = 0; c < NC; ++c) {
-      pin_put(pin + ((size_t)bh * NC + c) * D + tid, p);
+      pin_put(P.pin + ((size_t)bh * NC + c) * D + tid, p);
 #pragma unroll 1
       for (int half = 0; half < 2; ++half) {
         bar_sync(kBarFull + half, WT);
@@ -1420,22 +1427,23 @@ __device__ __forceinline__ void wy_gain(const CUtensorMap &mk, const CUtensorMap
         if (c + 1 < NC) bar_arrive(kBarEmpty + half, WT);
       }
     }
-    if (a.pT) a.pT[(size_t)bh * D + tid] = p;
+    if (P.p_out) P.p_out[(size_t)bh * D + tid] = p;
   } else {  // ---- its inputs
     const int pt = tid - D;
     auto issue = [&](int c) {
       unsigned char *d = sm + (c & 1) * SG_RAW;
       mbar_expect_tx(bars + (c & 1), SG_RAW);
+      const int t = (P.c0 + c) * CM;
       for (int s = 0; s < 2; ++s) {
-        tma_load_4d(d + s * 8192, &mk, bars + (c & 1), 64 * s, h, c * CM, b);
-        tma_load_4d(d + 16384 + s * 8192, &mg, bars + (c & 1), 64 * s, h, c * CM, b);
-        tma_load_4d(d + 32768 + s * 8192, &mw, bars + (c & 1), 64 * s, h, c * CM, b);
+        tma_load_4d(d + s * 8192, &mk, bars + (c & 1), 64 * s, h, t, b);
+        tma_load_4d(d + 16384 + s * 8192, &mg, bars + (c & 1), 64 * s, h, t, b);
+        tma_load_4d(d + 32768 + s * 8192, &mw, bars + (c & 1), 64 * s, h, t, b);
       }
     };
     __nv_bfloat16 znext = __float2bfloat16_rn(0.f);
     auto load_r = [&](int c) {
       if (pt < CM && c < NC)
-        znext = static_cast<const __nv_bfloat16 *>(a.r)[tok_index(a, b, min(c * CM + pt, a.T - 1), h)];
+        znext = static_cast<const __nv_bfloat16 *>(a.r)[tok_index(a, b, min((P.c0 + c) * CM + pt, a.T - 1), h)];
     };
     auto lga = [&](float x) { return LG ? -softplus_w(-x) : x; };
     if (pt == 0) {
@@ -1445,7 +1453,7 @@ __device__ __forceinline__ void wy_gain(const CUtensorMap &mk, const CUtensorMap
     load_r(0);
     bool ok = true;
     for (int c = 0; c < NC; ++c) {
-      const int left = a.T - c * CM;  // tokens past T: alpha 1, omega 0, u 0
+      const int left = a.T - (P.c0 + c) * CM;  // tokens past T: alpha 1, omega 0, u 0
       float *mr = s_mr + (c & 1) * CM;
       if (pt < CM) {
         const float z = __bfloat162float(znext), r = LG ? a.rmin + softplus_w(z) : z;
@@ -1535,7 +1543,7 @@ __device__ __forceinline__ void wy_state(const CUtensorMap &mv, const WyParams &
   uint64_t *bar_ld = bars, *bar_mma = bars + 2, *bar_o = bars + 3;
   uint32_t *s_tbase = reinterpret_cast<uint32_t *>(bars + 4);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, wq = warp & 3, wg = warp >> 2;
-  const int b = bh / a.H, h = bh % a.H, NC = (a.T + CM - 1) / CM;
+  const int b = bh / a.H, h = bh % a.H, NC = P.nc;
   const int warp_u = __shfl_sync(0xffffffffu, warp, 0);
   const uint32_t lane_base = (uint32_t)(32 * wq) << 16;
   bool ok = true;
@@ -1570,8 +1578,8 @@ __device__ __forceinline__ void wy_state(const CUtensorMap &mv, const WyParams &
       case 10: mbar_expect_tx(bar, 16384); bulk_g2s(d + SB_KT, rec + R::Kt, 16384, bar); break;
       case 11: mbar_expect_tx(bar, 8192); bulk_g2s(d + SB_AA, rec + R::A, 8192, bar); break;
       case 12: mbar_expect_tx(bar, 8192); bulk_g2s(d + SB_AA + 8192, rec + R::Aq, 8192, bar); break;
-      case 13: mbar_expect_tx(bar, 8192); tma_load_4d(d + SB_V, &mv, bar, 0, h, c * CM, b); break;
-      case 14: mbar_expect_tx(bar, 8192); tma_load_4d(d + SB_V + 8192, &mv, bar, 64, h, c * CM, b); break;
+      case 13: mbar_expect_tx(bar, 8192); tma_load_4d(d + SB_V, &mv, bar, 0, h, (P.c0 + c) * CM, b); break;
+      case 14: mbar_expect_tx(bar, 8192); tma_load_4d(d + SB_V + 8192, &mv, bar, 64, h, (P.c0 + c) * CM, b); break;
       case 15:
         mbar_expect_tx(bar, 768);
         bulk_g2s(d + SB_SC, rec + R::gC, 512, bar);
@@ -1583,8 +1591,8 @@ __device__ __forceinline__ void wy_state(const CUtensorMap &mv, const WyParams &
   const int i = 32 * wq + lane, j0 = 32 * wg;  // this thread's row and first column of S
   for (int c0 = 0; c0 < 32; c0 += 16) {
     float v[16];
-    if (a.S0) {
-      const float4 *src = reinterpret_cast<const float4 *>(a.S0 + ((size_t)bh * D + i) * D + j0 + c0);
+    if (P.S_in) {
+      const float4 *src = reinterpret_cast<const float4 *>(P.S_in + ((size_t)bh * D + i) * D + j0 + c0);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const float4 x = src[u];
@@ -1598,7 +1606,7 @@ __device__ __forceinline__ void wy_state(const CUtensorMap &mv, const WyParams &
   }
   tmem_st_wait();
   auto store_o = [&](int c) {  // O of chunk c: rows 64..127 of its TU, 32 columns a thread
-    const int t = 32 * (wq - 2) + lane, tt = c * CM + t;
+    const int t = 32 * (wq - 2) + lane, tt = (P.c0 + c) * CM + t;
     for (int c0 = 0; c0 < 32; c0 += 16) {
       float v[16];
       tmem_ld16(TUb + (c & 1) * 128 + lane_base + j0 + c0, v);
@@ -1754,11 +1762,11 @@ __device__ __forceinline__ void wy_state(const CUtensorMap &mv, const WyParams &
   if (__syncthreads_and(ok)) {
     tc_fence_after();
     if (wq >= 2 && a.o) store_o(NC - 1);
-    if (a.ST) {
+    if (P.S_out) {
       for (int c0 = 0; c0 < 32; c0 += 16) {
         float v[16];
         tmem_ld16(TS + lane_base + j0 + c0, v);
-        float4 *dst = reinterpret_cast<float4 *>(a.ST + ((size_t)bh * D + i) * D + j0 + c0);
+        float4 *dst = reinterpret_cast<float4 *>(P.S_out + ((size_t)bh * D + i) * D + j0 + c0);
 #pragma unroll
         for (int u = 0; u < 4; ++u) dst[u] = make_float4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
       }
@@ -1800,7 +1808,7 @@ __global__ void __launch_bounds__(WT, 1)
     if (threadIdx.x == 0) atomicExch(P.a.status, (unsigned)KDN_ERR_TIMEOUT);
     return;
   }
-  if (block < BH) wy_gain<SV, LG>(mk, mg, mw, P.a, P.pin, block);
+  if (block < BH) wy_gain<SV, LG>(mk, mg, mw, P, block);
   else if (block < BH + workers) wy_body<SV, LG, 1>(mk, mg, mw, mv, mq, P, block - BH, workers);
   else wy_state<SV>(mv, P, block - BH - workers);
 }
@@ -1821,57 +1829,88 @@ bool wy_fwd_supported(const Args &a, bool save) {
 // logit gates: 95 and 158, 182 and 347, 503 and 1353, 201 and 359, 66 and 80.  With 48 sequences
 // the one is ahead (B3 H16 T1300 216 and 198, T2047 301 and 298); more sequences than 56 leave too few workers.  Fewer than 96
 // chunks in all are left to the one kernel (tens of us either way).
+// A workspace holds the records of kSlice chunks of all sequences (136 MB); longer sequences take
+// several launches, which hand the state on in float32 (the same results), each with its 45.
+constexpr long long kSlice = 2048;
+static int wy_slices(const Args &a) {
+  const long long bh = (long long)a.B * a.H, nc = (a.T + CM - 1) / CM, per = kSlice / bh;
+  return (int)((nc + per - 1) / per);
+}
+static long long wy_slice_chunks(const Args &a) {
+  const long long nc = (a.T + CM - 1) / CM, ns = wy_slices(a);
+  return (nc + ns - 1) / ns;
+}
 bool wy_split_sizes(const Args &a) {
   if (!wy_fwd_supported(a, false)) return false;
   const long long bh = (long long)a.B * a.H, nc = (a.T + CM - 1) / CM;
   if (bh * nc < 96 || bh > 56) return false;
-  const long long workers = kSms - 2 * bh;
-  return std::max(nc * 7, (bh * nc + workers - 1) / workers * 19) + 45 < nc * 17;
+  const long long workers = kSms - 2 * bh, sc = wy_slice_chunks(a);
+  return wy_slices(a) * (std::max(sc * 7, (bh * sc + workers - 1) / workers * 19) + 45) < nc * 17;
 }
 
 size_t wy_split_workspace_bytes(const Args &a) {
   if (!wy_split_sizes(a)) return 0;
-  return (size_t)a.B * a.H * ((a.T + CM - 1) / CM) * (kPreBytes + D * sizeof(float) + sizeof(unsigned));
+  const size_t bh = (size_t)a.B * a.H;
+  return bh * wy_slice_chunks(a) * (kPreBytes + D * sizeof(float) + sizeof(unsigned)) +
+         (wy_slices(a) > 1 ? bh * (D * D + D) * sizeof(float) + 256 : 0);
 }
 
 namespace {
 template <int SV, int LG>
-kdn_status_t launch_wy(const WyParams &W, bool split, cudaStream_t s) {
+kdn_status_t launch_wy(WyParams &W, bool split, char *ws, cudaStream_t s) {
   const Args &a = W.a;
   CUtensorMap mk, mg, mw, mv, mq;
   if (!make_map(&mk, a.k, a) || !make_map(&mg, a.g, a) || !make_map(&mw, a.omega, a) ||
       !make_map(&mv, a.v, a) || !make_map(&mq, a.q, a))
     return KDN_ERR_CUDA;
-  const int bh = a.B * a.H;
-  const size_t n = (size_t)bh * ((a.T + CM - 1) / CM);
+  const int bh = a.B * a.H, NC = (a.T + CM - 1) / CM;
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
   if (!split) {
     if (cudaFuncSetAttribute(k_wy_fwd<SV, LG>, attr, SMEM_BYTES) != cudaSuccess) return KDN_ERR_CUDA;
     k_wy_fwd<SV, LG><<<bh, WT, SMEM_BYTES, s>>>(mk, mg, mw, mv, mq, W);
     return cudaGetLastError() == cudaSuccess ? KDN_OK : KDN_ERR_CUDA;
   }
-  if (cudaFuncSetAttribute(k_wy_flow<SV, LG>, attr, FLOW_SMEM) != cudaSuccess ||
-      cudaMemsetAsync(W.pin, 0xff, n * D * sizeof(float), s) != cudaSuccess ||
-      (SV ? cudaMemset2DAsync(W.flag, kCtxBytes, 0, sizeof(unsigned), n, s)
-          : cudaMemsetAsync(W.flag, 0, n * sizeof(unsigned), s)) != cudaSuccess)
-    return KDN_ERR_CUDA;
-  k_wy_flow<SV, LG><<<kSms, WT, FLOW_SMEM, s>>>(mk, mg, mw, mv, mq, W);
-  return cudaGetLastError() == cudaSuccess ? KDN_OK : KDN_ERR_CUDA;
+  if (cudaFuncSetAttribute(k_wy_flow<SV, LG>, attr, FLOW_SMEM) != cudaSuccess) return KDN_ERR_CUDA;
+  const int per = SV ? NC : (int)wy_slice_chunks(a);  // (the context has room for every chunk)
+  float *Sc = nullptr, *pc = nullptr;                 // the state between two slices
+  if (!SV) {
+    const size_t n = (size_t)bh * per;
+    W.pre = reinterpret_cast<unsigned char *>(ws);
+    W.prec = kPreBytes;
+    W.pin = reinterpret_cast<float *>(ws + n * kPreBytes);
+    W.flag = reinterpret_cast<unsigned *>(W.pin + n * D);
+    W.fstride = 1;
+    const uintptr_t end = reinterpret_cast<uintptr_t>(W.flag + n);
+    Sc = reinterpret_cast<float *>((end + 255) & ~uintptr_t(255));
+    pc = Sc + (size_t)bh * D * D;
+  }
+  for (W.c0 = 0; W.c0 < NC; W.c0 += per) {
+    const bool first = W.c0 == 0, last = W.c0 + per >= NC;
+    W.nc = last ? NC - W.c0 : per;
+    W.S_in = first ? a.S0 : Sc;
+    W.p_in = first ? a.p0 : pc;
+    W.S_out = last ? a.ST : Sc;
+    W.p_out = last ? a.pT : pc;
+    const size_t n = (size_t)bh * W.nc;
+    if (cudaMemsetAsync(W.pin, 0xff, n * D * sizeof(float), s) != cudaSuccess ||
+        (SV ? cudaMemset2DAsync(W.flag, kCtxBytes, 0, sizeof(unsigned), n, s)
+            : cudaMemsetAsync(W.flag, 0, n * sizeof(unsigned), s)) != cudaSuccess ||
+        (!first && cudaMemsetAsync(W.ticket, 0, sizeof(unsigned), s) != cudaSuccess))
+      return KDN_ERR_CUDA;
+    k_wy_flow<SV, LG><<<kSms, WT, FLOW_SMEM, s>>>(mk, mg, mw, mv, mq, W);
+    if (cudaGetLastError() != cudaSuccess) return KDN_ERR_CUDA;
+  }
+  return KDN_OK;
 }
 }  // namespace
 
 // ws: room for wy_split_workspace_bytes() (null: the one kernel, unless the context has the room)
 kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S, float *save_p, char *ws) {
   if (!wy_fwd_supported(a, save_S != nullptr) || (!save_S) != (!save_p)) return KDN_ERR_UNSUPPORTED;
-  WyParams P;
+  WyParams P{};
   P.a = a;
   P.save_S = save_S;
   P.save_p = save_p;
-  P.pre = nullptr;
-  P.prec = 0;
-  P.pin = nullptr;
-  P.flag = nullptr;
-  P.fstride = 0;
   P.ticket = a.status + 2;
   const bool split = wy_split_sizes(a) && (save_S || ws);
   if (split && save_S) {
@@ -1880,16 +1919,10 @@ kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S,
     P.pin = save_p;
     P.flag = reinterpret_cast<unsigned *>(save_S + kCtxTok + 3 * CM * sizeof(float));  // (no value there)
     P.fstride = kCtxBytes / sizeof(unsigned);
-  } else if (split) {
-    const size_t n = (size_t)a.B * a.H * ((a.T + CM - 1) / CM);
-    P.pre = reinterpret_cast<unsigned char *>(ws);
-    P.prec = kPreBytes;
-    P.pin = reinterpret_cast<float *>(ws + n * kPreBytes);
-    P.flag = reinterpret_cast<unsigned *>(P.pin + n * D);
-    P.fstride = 1;
   }
-  if (a.gates == KDN_GATES_LOGITS) return save_S ? launch_wy<1, 1>(P, split, s) : launch_wy<0, 1>(P, split, s);
-  return save_S ? launch_wy<1, 0>(P, split, s) : launch_wy<0, 0>(P, split, s);
+  if (a.gates == KDN_GATES_LOGITS)
+    return save_S ? launch_wy<1, 1>(P, split, ws, s) : launch_wy<0, 1>(P, split, ws, s);
+  return save_S ? launch_wy<1, 0>(P, split, ws, s) : launch_wy<0, 0>(P, split, ws, s);
 }
 
 }  // namespace kdn

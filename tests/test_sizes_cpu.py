@@ -32,3 +32,11 @@ def test_a_forward_pays_for_no_backward(B, T, H):
     assert kdn.workspace_bytes(d, 0, "saved") == 256 + (B * H * 81920 if T % 64 else 0)
     assert kdn.workspace_bytes(_desc(B, T, H, kdn.KDN_F32), 0, "saved") == 256
     assert kdn.workspace_bytes(d, 1, "saved") == 256
+
+
+@pytest.mark.parametrize("B,T,H", [(1, 65472, 16), (1, 131008, 16), (2, 40001, 16), (1, 1 << 20, 1), (7, 20001, 8)])
+def test_the_parallel_forward_is_bounded(B, T, H):
+    """Few sequences of any length: the records of at most 2048 chunks and a state per sequence."""
+    n = kdn.workspace_bytes(_desc(B, T, H), 0)
+    if T != 1 << 20:  # (that one is cut into segments)
+        assert n <= 256 + 2048 * (66560 + 516) + 512 + B * H * (128 * 129 * 4)
