@@ -321,10 +321,12 @@ kdn_status_t kdn_noalloc_device_status(void *stream);
 
 /* Number of CUDA kernels one call of an entry point launches for this
    descriptor when T > 0 (op 0 = kdn_*_fwd, 1 = kdn_*_bwd, 2 = kdn_*_decode_step,
-   3 = kdn_*_fwd_save, 4 = kdn_*_bwd_saved, 5 = kdn_*_beta_eff; variant 0 = diagonal,
+   3 = kdn_*_fwd_save, 4 = kdn_*_bwd_saved, 5 = kdn_*_beta_eff, 6 = kdn_*_bwd_saved without
+   dS0, dp0 and dmu; variant 0 = diagonal,
    1 = isotropic).  -1 for an invalid descriptor or op, or an op the descriptor
-   does not serve.  A backward is counted with every gradient asked for; the diagonal
-   backward with bf16 gradients and no state gradients may take one launch more.
+   does not serve.  Ops 1 and 4 count a backward with every gradient asked for; kdn_*_bwd
+   without dS0, dp0 and dmu takes the launches of ops 3 and 6 where the descriptor serves them.
+   Counted with the workspaces that the size queries name and buffers that do not overlap.
    Calls with T = 0 launch at most one small fill kernel. */
 int kdn_kernel_launches(const kdn_desc_t *desc, int variant, int op);
 

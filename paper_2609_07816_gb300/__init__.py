@@ -614,7 +614,8 @@ def kdn_diag_fwd_noalloc(q, k, v, g, omega, r, S0=None, p0=None, *, o, ST=None, 
 
 
 def kdn_kernel_launches(desc: kdn_desc_t, variant: int, op: int) -> int:
-    """Kernels one call launches (op 0 fwd, 1 bwd, 2 decode step)."""
+    """Kernels one call launches (op 0 fwd, 1 bwd, 2 decode step, 3 fwd_save, 4 bwd_saved,
+    5 beta_eff, 6 bwd_saved without state gradients)."""
     return int(lib().kdn_kernel_launches(ctypes.byref(desc), int(variant), int(op)))
 
 

@@ -483,12 +483,13 @@ int kdn_kernel_launches(const kdn_desc_t *desc, int variant, int op) {
   Args a;
   if (fill_sizes(desc, variant, op == 2, &a) != KDN_OK) return -1;
   switch (op) {
-    case 0: return seg_count(a) > 1 ? 5 : use_fused(a) ? 1 : chunked_fwd_launches(a);
+    case 0: return seg_count(a) > 1 ? 5 : wy_split_sizes(a) ? wy_slices(a) : use_fused(a) ? 1 : chunked_fwd_launches(a);
     case 1: return (a.T > 0 && use_fused_bwd(a)) ? 2 : chunked_bwd_launches(a);
     case 2: return 1;
     case 3:
     case 4:
     case 5: return fused_saved_bytes(a) > 0 ? 1 : -1;
+    case 6: return fused_saved_bytes(a) == 0 ? -1 : split_bwd_sizes(a) && a.odt == KDN_BF16 ? 3 : 1;
   }
   return -1;
 }

@@ -167,6 +167,7 @@ kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S 
 // The same with the gain, the chunks and the memory on CTAs of their own where these sizes gain from it:
 // in the context's own records, or with this much scratch in the workspace.
 bool wy_split_sizes(const Args &a);
+int wy_slices(const Args &a);  // its launches without the context
 size_t wy_split_workspace_bytes(const Args &a);
 // beta_eff [B,T,H] (float32) from the per-token gain scalars of a context saved by
 // the fused training forward (one launch).

@@ -1832,7 +1832,7 @@ bool wy_fwd_supported(const Args &a, bool save) {
 // A workspace holds the records of kSlice chunks of all sequences (136 MB); longer sequences take
 // several launches, which hand the state on in float32 (the same results), each with its 45.
 constexpr long long kSlice = 2048;
-static int wy_slices(const Args &a) {
+int wy_slices(const Args &a) {
   const long long bh = (long long)a.B * a.H, nc = (a.T + CM - 1) / CM, per = kSlice / bh;
   return (int)((nc + per - 1) / per);
 }

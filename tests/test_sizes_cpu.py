@@ -40,3 +40,15 @@ def test_the_parallel_forward_is_bounded(B, T, H):
     n = kdn.workspace_bytes(_desc(B, T, H), 0)
     if T != 1 << 20:  # (that one is cut into segments)
         assert n <= 256 + 2048 * (66560 + 516) + 512 + B * H * (128 * 129 * 4)
+
+
+def test_launch_counts():
+    n = kdn.kdn_kernel_launches
+    for d, bf in ((_desc(8, 4096, 16), True), (_desc(8, 4096, 16, kdn.KDN_F32), False), (_desc(2, 1999, 16), True)):
+        assert [n(d, 0, op) for op in (1, 3, 4)] == [2, 1, 1]
+        assert n(d, 0, 6) == (3 if bf else 1)  # tiles, memory, chunks; or the sweep
+        assert n(d, 1, 6) == 1
+    assert n(_desc(2, 130, 3), 0, 6) == 1  # too few chunks for the two-kernel backward
+    assert n(_desc(2, 130, 3, chunk=32), 0, 6) == -1
+    # the parallel forward of few sequences: one launch a slice (2048 chunks of all sequences)
+    assert n(_desc(2, 1999, 16), 0, 0) == 1 and n(_desc(2, 5000, 16), 0, 0) == 2 and n(_desc(1, 65472, 16), 0, 0) == 8
