@@ -19,6 +19,7 @@ from __future__ import annotations
 import ctypes
 import functools
 import math
+import operator
 import os
 import threading
 
@@ -257,7 +258,7 @@ def _desc_from(variant, q, v, g, *, chunk, mu, scale, out_dtype, gates=KDN_GATES
     B, T, H, dk = q.shape
     dv = v.shape[-1]
     pcd = 1 if variant == 0 else int(g.dim() == 4)
-    return _desc(B, T, H, dk, dv, q.dtype, int(chunk), _number(mu), _number(scale), pcd,
+    return _desc(B, T, H, dk, dv, q.dtype, operator.index(chunk), _number(mu), _number(scale), pcd,
                  _code(out_dtype), int(gates), float(r_min))
 
 
