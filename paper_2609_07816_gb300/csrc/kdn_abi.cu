@@ -179,9 +179,6 @@ kdn_status_t bwd_entry(int variant, const kdn_desc_t *d, const void *q, const vo
   if ((size_t)a.B * a.H == 0) return KDN_OK;
   if (a.T == 0) return empty_bwd(a, s);
   if (use_fused_bwd(a)) return launch_fused_bwd(a, s);
-  // the general kernels accumulate dmu with atomics
-  if (a.dmu && cudaMemsetAsync(a.dmu, 0, (size_t)a.B * a.H * sizeof(float), s) != cudaSuccess)
-    return KDN_ERR_CUDA;
   return launch_chunked_bwd(a, s);
 }
 

@@ -7,7 +7,8 @@
 //                  chunk's summary of the uncertainty adjoint (dp_in = A dp_out + B);
 //   k_dp_scan      chains the summaries backwards;
 //   k_gain_bwd_*   runs the adjoint of the uncertainty recursion inside every chunk,
-//                  in parallel over chunks, and writes the gradients that need it.
+//                  in parallel over chunks, and writes the gradients that need it;
+//   k_dmu_sum      adds up the chunks' parts of dmu, where that is asked for.
 #include "kdn_chunked.cuh"
 
 namespace kdn {
@@ -469,6 +470,18 @@ __global__ void __launch_bounds__(128) k_dp_scan(Args a) {
   if (a.dp0) a.dp0[e] = dp;
 }
 
+// A chunk's part of dmu, in its summary's place (which k_dp_scan has read).
+__device__ __forceinline__ float *dmu_part(const Args &a, size_t chunk) { return a.aff + chunk * a.P * 2; }
+
+// One warp per sequence: dmu, its chunks' parts in an order of their own, so that it repeats exactly.
+__global__ void __launch_bounds__(32) k_dmu_sum(Args a) {
+  const size_t base = (size_t)blockIdx.x * a.NC;
+  float s = 0.f;
+  for (int c = KDN_TID; c < a.NC; c += 32) s += *dmu_part(a, base + c);
+  s = warp_sum(s);
+  if (KDN_TID == 0) a.dmu[blockIdx.x] = s;
+}
+
 // One CTA per chunk, one thread per channel, eight tokens loaded at a time.
 template <typename DT, int DK>
 __global__ void __launch_bounds__(DK) k_gain_bwd_diag(Args a) {
@@ -545,7 +558,7 @@ __global__ void __launch_bounds__(DK) k_gain_bwd_diag(Args a) {
     float tot = 0.f;
 #pragma unroll
     for (int w = 0; w < DK / 32; ++w) tot += s_mu[w];
-    atomicAdd(a.dmu + bh, tot);
+    *dmu_part(a, base) = tot;
   }
 }
 
@@ -591,7 +604,7 @@ __global__ void __launch_bounds__(128) k_gain_bwd_iso(Args a) {
     }
     if (a.dmu) {
       const float dmu = warp_sum(lane < tn ? du * n2 / (DK * rr) : 0.f);  // u = mu |k|^2 / (dk r)
-      if (lane == 0) atomicAdd(a.dmu + bh, dmu);
+      if (lane == 0) *dmu_part(a, base) = dmu;
     }
   }
   __syncthreads();
@@ -663,6 +676,7 @@ kdn_status_t bwd_impl(const Args &a0, cudaStream_t s) {
   ok = ok && launch(k_dp_scan, (BH * a.P + 127) / 128, 128, 0, s, a);
   if (V == 0) ok = ok && launch(k_gain_bwd_diag<DT, DK>, n, DK, 0, s, a);
   else ok = ok && launch(k_gain_bwd_iso<DT, DK>, n, 128, 0, s, a);
+  if (a.dmu) ok = ok && launch(k_dmu_sum, BH, 32, 0, s, a);
   return ok ? KDN_OK : KDN_ERR_CUDA;
 }
 
@@ -678,7 +692,7 @@ kdn_status_t bwd_dk(const Args &a, cudaStream_t s) {
 
 }  // namespace
 
-int chunked_bwd_launches(const Args &a) { return chunked_fwd_launches(a) + 4; }
+int chunked_bwd_launches(const Args &a) { return chunked_fwd_launches(a) + 5; }
 
 kdn_status_t launch_chunked_bwd(const Args &a, cudaStream_t s) {
   if (a.variant == 0)
