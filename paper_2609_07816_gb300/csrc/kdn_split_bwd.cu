@@ -29,6 +29,8 @@
 // power of two.
 //
 // Every wait is bounded; on timeout KDN_ERR_TIMEOUT goes to the status word.
+#include <algorithm>
+
 #include "kdn_internal.cuh"
 #include "kdn_sm103.cuh"
 #include "kdn_bwd_common.cuh"
@@ -1189,18 +1191,22 @@ __global__ void __launch_bounds__(BT, 1)
 
 }  // namespace
 
-// Where the two kernels finish sooner than the one-kernel sweep, in thousands of cycles as
-// measured: the sweep takes 40 a chunk with one CTA per sequence; k_bwd_state 6 a chunk with
-// one CTA per sequence, k_bwd_chunk 32 a chunk on any SM, and the second launch with its first
-// tiles 12.  B8 H16 T4096: 2.1 M cycles against 2.5 M (1120 us, 1326 us); B2 H16 T1999 with
-// logit gates: 0.49 M against 1.28 M (255 us, 668 us); with as many sequences as SMs and one
-// or two chunks each the sweep is ahead.  Fewer than 96 chunks in all are left to the sweep (a
-// few tens of us either way).
+// Where the two kernels (with k_bwd_tiles) finish sooner than the one-kernel sweep, in tenths of a
+// microsecond as measured.  The sweep: 208 a chunk of each wave of sequences.  Here: k_bwd_tiles 0.19 a
+// job, k_bwd_state 31 a chunk of a sequence or 0.3 a job (HBM), k_bwd_chunk 162 a round of 152
+// jobs, but with few sequences 17 a chunk (the chain of dp), and 280 until its rounds run evenly.
+// Two kernels against the sweep, us: B8 H16 T4096 1295 and 1317; B2 H16 T1984 280 and 600, B1 H16 T4096 382 and
+// 1213, B64 H1 T512 139 and 171, B40 H5 T512 322 and 353; on the other side B8 H16 T1024 380 and 347, B19 H8 T2048
+// 793 and 684, B100 H1 T512 186 and 177, B16 H16 T2048 1345 and 1308.  Fewer than 96 chunks in all are left to the
+// sweep (a few tens of us either way).
 bool split_bwd_sizes(const Args &a) {
   if (a.variant != 0 || a.chunk == 32 || !fused_fwd_supported(a)) return false;
-  const long long bh = (long long)a.B * a.H, nc = (a.T + CM - 1) / CM, waves = (bh + kSms - 1) / kSms;
-  if (bh * nc < 96) return false;
-  return waves * nc * 6 + (bh * nc + kSms - 1) / kSms * 32 + 12 < waves * nc * 40;
+  const long long bh = (long long)a.B * a.H, nc = (a.T + CM - 1) / CM, jobs = bh * nc;
+  if (jobs < 96) return false;
+  const long long waves = (bh + kSms - 1) / kSms, rounds = (jobs + kSms - 1) / kSms;
+  const long long state = waves * std::max(31 * nc, 3 * std::min<long long>(bh, kSms) * nc / 10);
+  const long long chunk = std::max(162 * rounds, 17 * nc + 160) + (rounds > 1 ? 280 : 0);
+  return 140 + jobs * 19 / 100 + state + chunk < waves * (208 * nc + 60);
 }
 
 // The gradient buffers serve as scratch only where they overlap neither each other nor anything the

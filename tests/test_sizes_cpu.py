@@ -29,7 +29,9 @@ def test_a_forward_pays_for_no_backward(B, T, H):
     training backward asks for its partial last chunk (80 KB a sequence) by itself."""
     d = _desc(B, T, H)
     assert kdn.workspace_bytes(d, 0) == 256
-    assert kdn.workspace_bytes(d, 0, "saved") == 256 + (B * H * 81920 if T % 64 else 0)
+    two = kdn.kdn_kernel_launches(d, 0, 6) > 1
+    assert two or (B, H) != (8, 16)
+    assert kdn.workspace_bytes(d, 0, "saved") == 256 + (B * H * 81920 if T % 64 and two else 0)
     assert kdn.workspace_bytes(_desc(B, T, H, kdn.KDN_F32), 0, "saved") == 256
     assert kdn.workspace_bytes(d, 1, "saved") == 256
 
