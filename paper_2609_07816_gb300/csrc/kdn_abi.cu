@@ -144,7 +144,7 @@ kdn_status_t fwd_entry(int variant, const kdn_desc_t *d, const void *q, const vo
   if ((size_t)a.B * a.H == 0) return KDN_OK;
   if (a.T == 0) return empty_fwd(a, s);
   if (nseg > 1) return launch_seg_fwd(a, nseg, static_cast<char *>(ws) + base, s);
-  if (use_fused(a) && wy_fwd_supported(a, false)) {
+  if (use_fused(a) && wy_fwd_supported(a)) {
     const size_t split = wy_split_workspace_bytes(a);
     return launch_wy_fwd(a, s, nullptr, nullptr,
                          split && ws_bytes >= base + split ? static_cast<char *>(ws) + base : nullptr);
@@ -194,7 +194,7 @@ kdn_status_t fwd_save_entry(int variant, const kdn_desc_t *d, const void *q, con
   const bool work = (size_t)a.B * a.H * a.T > 0;
   if (work && !use_fused_bwd(a)) return KDN_ERR_UNSUPPORTED;
   // (the diagonal backward reads Y = V - Kbar S_in from the context, which the WY forward writes)
-  if (work && variant == 0 && !wy_fwd_supported(a, true)) return KDN_ERR_UNSUPPORTED;
+  if (work && variant == 0 && !wy_fwd_supported(a)) return KDN_ERR_UNSUPPORTED;
   if (work && !ptrs_ok({q, k, v, g, omega, r, o, saved}, {S0, p0, ST, pT})) return KDN_ERR_INVALID_ARG;
   if (!work && !ptrs_ok({}, {S0, p0, ST, pT})) return KDN_ERR_INVALID_ARG;
   if (work && (saved_bytes < fused_saved_bytes(a) || ((uintptr_t)saved % kAlign)))
@@ -209,7 +209,7 @@ kdn_status_t fwd_save_entry(int variant, const kdn_desc_t *d, const void *q, con
   if ((size_t)a.B * a.H == 0) return KDN_OK;
   if (a.T == 0) return empty_fwd(a, s);
   const size_t nsv = (size_t)a.B * a.H * ((a.T + 63) / 64) * fused_ctx_record_bytes();
-  if (wy_fwd_supported(a, true))
+  if (wy_fwd_supported(a))
     return launch_wy_fwd(a, s, static_cast<unsigned char *>(saved),
                          reinterpret_cast<float *>(static_cast<char *>(saved) + nsv));
   return launch_fused_fwd(a, s, static_cast<unsigned char *>(saved),

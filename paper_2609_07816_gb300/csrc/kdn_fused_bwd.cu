@@ -1464,8 +1464,8 @@ kdn_status_t launch_fused_bwd(const Args &a, cudaStream_t s) {
   f.ST = nullptr;
   f.pT = nullptr;
   // (the diagonal sweep reads Y = V - Kbar S_in from the context, which the WY forward writes)
-  if (a.variant == 0 && !wy_fwd_supported(f, true)) return KDN_ERR_UNSUPPORTED;
-  kdn_status_t st = wy_fwd_supported(f, true) ? launch_wy_fwd(f, s, a.fSin, a.fpin)
+  if (a.variant == 0 && !wy_fwd_supported(f)) return KDN_ERR_UNSUPPORTED;
+  kdn_status_t st = wy_fwd_supported(f) ? launch_wy_fwd(f, s, a.fSin, a.fpin)
                                          : launch_fused_fwd(f, s, a.fSin, a.fpin, false);
   if (st != KDN_OK) return st;
   return launch_fused_bwd_sweep(a, s);

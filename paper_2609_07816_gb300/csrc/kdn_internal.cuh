@@ -11,6 +11,8 @@
 
 namespace kdn {
 
+constexpr int kSms = 152;  // SMs of a GB300
+
 // ---------------------------------------------------------------------------
 // dtype helpers: activations are float32 or bfloat16, arithmetic is float32.
 
@@ -161,7 +163,7 @@ kdn_status_t launch_fused_fwd(const Args &a, cudaStream_t s, unsigned char *save
 // 128, 64-token chunks; writes o, S_T, p_T where their pointers are non-null,
 // and with save_S / save_p the fused backward's context (the layout of
 // launch_fused_fwd's saving mode).
-bool wy_fwd_supported(const Args &a, bool save);  // save: the context-saving instantiation
+bool wy_fwd_supported(const Args &a);
 kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S = nullptr,
                            float *save_p = nullptr, char *ws = nullptr);
 // The same with the gain, the chunks and the memory on CTAs of their own where these sizes gain from it:

@@ -35,7 +35,6 @@ namespace {
 
 constexpr int D = 128;       // d_k = d_v served by the fused kernels
 constexpr int CM = 64;       // their chunk length
-constexpr int kSegCtas = 152;  // one CTA per SM of a GB300 (152 SMs)
 constexpr int kMinSegChunks = 8;
 
 using bf16 = __nv_bfloat16;
@@ -442,7 +441,7 @@ int seg_count(const Args &a) {
   const long long bh = (long long)a.B * a.H;
   int best = 1;
   for (int p = 4; p * kMinSegChunks <= nc; ++p)
-    if (nc % p == 0 && bh * p <= kSegCtas) best = p;
+    if (nc % p == 0 && bh * p <= kSms) best = p;
   return best;
 }
 

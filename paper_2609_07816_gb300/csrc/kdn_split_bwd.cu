@@ -44,7 +44,6 @@ using namespace fused;
 constexpr int BT = 512, CM = 64, D = 128, KB = 1024;
 constexpr uint32_t kWaitIters = 1u << 25;
 constexpr uint32_t kDpWait = 1u << 22;  // polls for the uncertainty cotangent of the next chunk
-constexpr int kSms = 152;
 
 // Where a chunk's small values lie: rows of 256 bytes, one per token of the chunk.
 // Rows 0..7: dgamma_C's dS part [4][128]; 8..11: dp [128] as (value, tag) pairs; 12: lambda;

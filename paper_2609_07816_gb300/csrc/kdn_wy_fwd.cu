@@ -87,7 +87,6 @@ constexpr int WT = 512;  // threads
 constexpr int CM = 64;   // chunk length
 constexpr int D = 128;   // d_k = d_v
 constexpr uint32_t kWait = 1u << 25;
-constexpr int kSms = 152;
 constexpr uint32_t kDrain = 1u << 14;  // bounded waits of the failure path
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
@@ -755,20 +754,20 @@ __device__ __forceinline__ void wy_body(const CUtensorMap &mk, const CUtensorMap
       }
     } else {
 #pragma unroll
-    for (int s2 = 0; s2 < 4; ++s2) {
-      float x[16];
+      for (int s2 = 0; s2 < 4; ++s2) {
+        float x[16];
 #pragma unroll
-      for (int j = 0; j < 16; ++j) x[j] = lga(raw(pg, 16 * s2 + j));
+        for (int j = 0; j < 16; ++j) x[j] = lga(raw(pg, 16 * s2 + j));
 #pragma unroll
-      for (int h2 = 0; h2 < 2; ++h2) {
-        const float *y = x + 8 * h2;
-        const float ss = ((y[0] + y[1]) + (y[2] + y[3])) + ((y[4] + y[5]) + (y[6] + y[7]));
-        s_part[(2 * s2 + h2) * D + i] = ss;
-        GC += ss;
+        for (int h2 = 0; h2 < 2; ++h2) {
+          const float *y = x + 8 * h2;
+          const float ss = ((y[0] + y[1]) + (y[2] + y[3])) + ((y[4] + y[5]) + (y[6] + y[7]));
+          s_part[(2 * s2 + h2) * D + i] = ss;
+          GC += ss;
+        }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) *reinterpret_cast<float *>(pb + sw32_off(16 * s2 + j, cb)) = x[j];
       }
-#pragma unroll
-      for (int j = 0; j < 16; ++j) *reinterpret_cast<float *>(pb + sw32_off(16 * s2 + j, cb)) = x[j];
-    }
     }
     const float cref = 0.5f * GC;
     s_c[i] = cref;
@@ -1310,9 +1309,7 @@ __device__ __forceinline__ void wy_body(const CUtensorMap &mk, const CUtensorMap
     failed = !__syncthreads_and(mine);
     tc_fence_after();
   }
-  if (CH && !failed) {
-    // (nothing is in flight but the copies of the records, awaited below)
-  } else if (!failed) {
+  if (!CH && !failed) {
     const Job o = job(NC - 1);
     if (!gain && wq >= 2 && NC > 0 && a.o) {  // O of the last chunk
       const int t = 32 * (wq - 2) + lane, tt = (NC - 1) * CM + t;
@@ -1346,7 +1343,7 @@ __device__ __forceinline__ void wy_body(const CUtensorMap &mk, const CUtensorMap
       }
     }
     if (a.pT && gain) a.pT[(size_t)bh * D + tid] = p;
-  } else {
+  } else if (failed) {
     if (tid == 0) atomicExch(a.status, (unsigned)KDN_ERR_TIMEOUT);
     // copies and MMAs in flight land before the CTA's memory goes away
     // (short bounds: a copy or MMA that was issued lands within microseconds,
@@ -1815,8 +1812,7 @@ __global__ void __launch_bounds__(WT, 1)
 
 }  // namespace
 
-bool wy_fwd_supported(const Args &a, bool save) {
-  (void)save;
+bool wy_fwd_supported(const Args &a) {
   return a.variant == 0 && (a.gates == KDN_GATES_POST || a.gates == KDN_GATES_LOGITS) &&
          a.dtype == KDN_BF16 && a.dk == D && a.dv == D && a.T > 0 && a.chunk != 32;
 }
@@ -1841,7 +1837,7 @@ static long long wy_slice_chunks(const Args &a) {
   return (nc + ns - 1) / ns;
 }
 bool wy_split_sizes(const Args &a) {
-  if (!wy_fwd_supported(a, false)) return false;
+  if (!wy_fwd_supported(a)) return false;
   const long long bh = (long long)a.B * a.H, nc = (a.T + CM - 1) / CM;
   if (bh * nc < 96 || bh > 56) return false;
   const long long workers = kSms - 2 * bh, sc = wy_slice_chunks(a);
@@ -1906,7 +1902,7 @@ kdn_status_t launch_wy(WyParams &W, bool split, char *ws, cudaStream_t s) {
 
 // ws: room for wy_split_workspace_bytes() (null: the one kernel, unless the context has the room)
 kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S, float *save_p, char *ws) {
-  if (!wy_fwd_supported(a, save_S != nullptr) || (!save_S) != (!save_p)) return KDN_ERR_UNSUPPORTED;
+  if (!wy_fwd_supported(a) || (!save_S) != (!save_p)) return KDN_ERR_UNSUPPORTED;
   WyParams P{};
   P.a = a;
   P.save_S = save_S;
