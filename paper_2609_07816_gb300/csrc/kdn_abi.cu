@@ -13,8 +13,8 @@ int chunked_chunk_len();
 namespace {
 
 constexpr size_t kAlign = 256;
-// the status word and the tickets of the two-kernel backward and of k_wy_flow
-constexpr size_t kStatusBytes = 3 * sizeof(unsigned);
+// the status word and the ticket of the two-kernel backward
+constexpr size_t kStatusBytes = 2 * sizeof(unsigned);
 
 size_t round_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 

@@ -461,7 +461,6 @@ struct WyParams {
   float *pin;             // [BH][NC][128], preset to kUnset
   unsigned *flag;         // per chunk, fstride apart, zeroed: warps that have written their part of its record
   size_t fstride;
-  unsigned *ticket;       // zeroed: CTAs of k_wy_flow that have started
   // k_wy_flow: the chunks c0 .. c0 + nc - 1 of every sequence, and the states around them (null: the
   // zero memory, the unit uncertainty; not written)
   int c0, nc;
@@ -1784,11 +1783,12 @@ __device__ __forceinline__ void wy_state(const CUtensorMap &mv, const WyParams &
 
 // ---------------------------------------------------------------------------
 // k_wy_flow: the three parts at once, one CTA per SM: first the gain's CTAs (one per sequence),
-// then the chunk part's, then the memory's (one per sequence).  A CTA takes its place by the order
-// in which the CTAs start, and a part waits only for earlier places (bounded), so whatever of
-// the grid is resident makes progress.  B1 H16 T777 with
+// then the chunk part's, then the memory's (one per sequence).  The parts wait for one another
+// (bounded), so the launch is cooperative: it starts once all its CTAs can be resident.  (Places by
+// the order of start would do as well, but mix the parts on the two SMs of a TPC, which fetch
+// instructions together: B2 H16 T1999 with logit gates 230 us, not 207.)  B1 H16 T777 with
 // logit gates 119 us as three launches, 78 us as one (one CTA per sequence: 143 us); training
-// forward B2 H16 T1999 302 and ~200 us (430).
+// forward B2 H16 T1999 302 and 207 us (430).
 constexpr int FLOW_SMEM = SMEM_BYTES > SG_SMEM ? (SMEM_BYTES > ST_SMEM ? SMEM_BYTES : ST_SMEM)
                                                : (SG_SMEM > ST_SMEM ? SG_SMEM : ST_SMEM);
 template <int SV, int LG>
@@ -1796,15 +1796,7 @@ __global__ void __launch_bounds__(WT, 1)
     k_wy_flow(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mg,
               const __grid_constant__ CUtensorMap mw, const __grid_constant__ CUtensorMap mv,
               const __grid_constant__ CUtensorMap mq, const WyParams P) {
-  __shared__ int s_place;
-  if (threadIdx.x == 0) s_place = (int)atomicAdd(P.ticket, 1u);
-  __syncthreads();
-  const int BH = P.a.B * P.a.H, block = s_place, workers = (int)gridDim.x - 2 * BH;
-  // (a workspace that something else writes to meanwhile: no place, no access; the others' waits end)
-  if ((unsigned)block >= gridDim.x) {
-    if (threadIdx.x == 0) atomicExch(P.a.status, (unsigned)KDN_ERR_TIMEOUT);
-    return;
-  }
+  const int BH = P.a.B * P.a.H, block = (int)blockIdx.x, workers = (int)gridDim.x - 2 * BH;
   if (block < BH) wy_gain<SV, LG>(mk, mg, mw, P, block);
   else if (block < BH + workers) wy_body<SV, LG, 1>(mk, mg, mw, mv, mq, P, block - BH, workers);
   else wy_state<SV>(mv, P, block - BH - workers);
@@ -1861,11 +1853,12 @@ kdn_status_t launch_wy(WyParams &W, bool split, char *ws, cudaStream_t s) {
     return KDN_ERR_CUDA;
   const int bh = a.B * a.H, NC = (a.T + CM - 1) / CM;
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  if (!split) {
+  auto one = [&]() {
     if (cudaFuncSetAttribute(k_wy_fwd<SV, LG>, attr, SMEM_BYTES) != cudaSuccess) return KDN_ERR_CUDA;
     k_wy_fwd<SV, LG><<<bh, WT, SMEM_BYTES, s>>>(mk, mg, mw, mv, mq, W);
     return cudaGetLastError() == cudaSuccess ? KDN_OK : KDN_ERR_CUDA;
-  }
+  };
+  if (!split) return one();
   if (cudaFuncSetAttribute(k_wy_flow<SV, LG>, attr, FLOW_SMEM) != cudaSuccess) return KDN_ERR_CUDA;
   const int per = SV ? NC : (int)wy_slice_chunks(a);  // (the context has room for every chunk)
   float *Sc = nullptr, *pc = nullptr;                 // the state between two slices
@@ -1890,11 +1883,25 @@ kdn_status_t launch_wy(WyParams &W, bool split, char *ws, cudaStream_t s) {
     const size_t n = (size_t)bh * W.nc;
     if (cudaMemsetAsync(W.pin, 0xff, n * D * sizeof(float), s) != cudaSuccess ||
         (SV ? cudaMemset2DAsync(W.flag, kCtxBytes, 0, sizeof(unsigned), n, s)
-            : cudaMemsetAsync(W.flag, 0, n * sizeof(unsigned), s)) != cudaSuccess ||
-        (!first && cudaMemsetAsync(W.ticket, 0, sizeof(unsigned), s) != cudaSuccess))
+            : cudaMemsetAsync(W.flag, 0, n * sizeof(unsigned), s)) != cudaSuccess)
       return KDN_ERR_CUDA;
-    k_wy_flow<SV, LG><<<kSms, WT, FLOW_SMEM, s>>>(mk, mg, mw, mv, mq, W);
-    if (cudaGetLastError() != cudaSuccess) return KDN_ERR_CUDA;
+    cudaLaunchAttribute coop;
+    coop.id = cudaLaunchAttributeCooperative;
+    coop.val.cooperative = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = kSms;
+    cfg.blockDim = WT;
+    cfg.dynamicSmemBytes = FLOW_SMEM;
+    cfg.stream = s;
+    cfg.attrs = &coop;
+    cfg.numAttrs = 1;
+    const cudaError_t e =
+        cudaLaunchKernelEx(&cfg, k_wy_flow<SV, LG>, mk, mg, mw, mv, mq, static_cast<const WyParams>(W));
+    if (e == cudaErrorCooperativeLaunchTooLarge && first) {  // (fewer SMs than a whole GPU's are ours)
+      cudaGetLastError();
+      return one();
+    }
+    if (e != cudaSuccess) return KDN_ERR_CUDA;
   }
   return KDN_OK;
 }
@@ -1907,7 +1914,6 @@ kdn_status_t launch_wy_fwd(const Args &a, cudaStream_t s, unsigned char *save_S,
   P.a = a;
   P.save_S = save_S;
   P.save_p = save_p;
-  P.ticket = a.status + 2;
   const bool split = wy_split_sizes(a) && (save_S || ws);
   if (split && save_S) {
     P.pre = save_S;
