@@ -19,7 +19,7 @@
 // All chunk-local matrices are float32 in shared memory; intermediates that
 // cross kernels live in the caller's workspace.
 //
-// Diagonal prefill B8 H16 T2048 d = 64 bf16, us: 33 + 11 + 278 + 261, 586 a call.  With the
+// Diagonal prefill B8 H16 T2048 d = 64 bf16, us: 33 + 11 + 279 + 261, 589 a call.  With the
 // uncertainty run token by token (1406), one output a thread in the chunk kernel (763) and two
 // loads a multiply-add in the memory pass (790) it was 2922.
 #include <float.h>
@@ -268,7 +268,7 @@ __device__ __forceinline__ void inverse32(const float *sT, float *sA, float *sX)
 // One CTA of 128 threads per chunk; five of them on an SM cover each other's load and barrier
 // latencies.  Bound by shared-memory loads and issue (ncu, B8 H16 T2048 d = 64: 58 % of the
 // shared-memory cycles, 51 % of the issue slots, the rest waits for the first loads); register
-// tiles of 4 x 4 outputs, since a 16-byte load costs four cycles of the SM.  282 us (763 with
+// tiles of 4 x 4 outputs, since a 16-byte load costs four cycles of the SM.  279 us (763 with
 // one output a thread).
 template <int V, typename DT, int DK, int SAVE>
 __global__ void __launch_bounds__(PT, DK < 128 ? 5 : 3) k_chunk_prep(Args a) {

@@ -53,7 +53,7 @@
 // Bound by the chain of a chunk's stages on one SM (~40 K cycles diagonal, ~33 K isotropic;
 // ~45 % of the issue slots).  Copies are issued one per warp and the per-token inputs arrive by
 // bulk copies: one thread's run of TMA operations and loads held at a barrier cost 2-3 K
-// cycles a chunk (isotropic B8 H12 T2048: 561 -> 524 us; diagonal B8 H16 T4096: 1326 us).
+// cycles a chunk (isotropic B8 H12 T2048: 561 -> 524 us; diagonal B8 H16 T4096: 1317 us).
 //
 // Every wait on an mbarrier is bounded; on timeout the kernel records
 // KDN_ERR_TIMEOUT in the workspace status word and returns.

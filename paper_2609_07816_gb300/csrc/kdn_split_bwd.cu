@@ -137,7 +137,8 @@ struct SplitParams {
 // the context's phat, gamma and s_t, in the operations of the one-kernel sweep (the context does not
 // hold them: K_tail needs s_t, which the forward knows only after the gain has moved on).  Left where
 // the chunk's dR goes, which k_bwd_state writes once it has read them.  Bound by HBM: 96 KB read and
-// 32 KB written per chunk.  A thread takes two channels of eight tokens, all loads ahead.
+// 32 KB written per chunk, 154 us at B8 H16 T4096 (6.9 TB/s).  A thread takes two channels of eight
+// tokens, all loads ahead; with one CTA of 512 threads a chunk, 16 tokens a thread, it took 218.
 constexpr int TT = 256, TILE_SMEM = 16 * KB + 1024;
 
 __global__ void __launch_bounds__(TT, 4)
@@ -202,8 +203,8 @@ __global__ void __launch_bounds__(TT, 4)
 }
 
 // ---------------------------------------------------------------------------
-// k_bwd_state.  Bound by HBM: 104 KB read and 64 KB written per chunk, 255 us at B8 H16 T4096
-// (5.4 TB/s); with few sequences by its chain, ~6 K cycles a chunk (94 us at B2 H16 T1999).
+// k_bwd_state.  Bound by HBM: 104 KB read and 64 KB written per chunk, 247 us at B8 H16 T4096
+// (5.7 TB/s); with few sequences by its chain, ~6 K cycles a chunk (98 us at B2 H16 T1999).
 // 16 warps; warp w holds TMEM lanes 32 (w % 4) .. + 31 and value columns
 // 32 (w / 4) .. + 31 of dS.  Per chunk: dS -> fp16 tile; MMA dR; dR -> fp16 hi + lo;
 // MMA dS.  A_qk, K_tail and dO are double-buffered bulk copies; Qbar, W (needed
@@ -491,8 +492,8 @@ __global__ void __launch_bounds__(BT, 1)
 // k_bwd_chunk.  Bound by the chain of a chunk's stages (ncu, B2 H16 T4096: 40 % of the issue
 // slots, tensor pipe 8 %; the waits are on tensor-memory reads, barriers and instruction
 // fetches): ~32 K cycles a chunk, of which the four tensor-core rounds with their read-outs 13 K
-// and the per-channel passes 14 K.  865 us at B8 H16 T4096 (with k_bwd_state 1120; the one-kernel
-// sweep 1326), 161 us at B2 H16 T1999 logits (255; 668).
+// and the per-channel passes 14 K.  872 us at B8 H16 T4096 (with the tiles and k_bwd_state 1295; the
+// one-kernel sweep 1317), 165 us at B2 H16 T1999 logits (285; 668).
 // Shared-memory map (bytes from the 1024-aligned base), with the sequence
 // of tenants within a chunk; the next chunk's tiles arrive as their buffers fall free.
 constexpr int O_RKQ = 0;         // raw k | q, interleaved per 64-channel slab

@@ -42,7 +42,7 @@
 // one chunk ahead on its own warps) is as long as the rest: the kernel is bound by
 // that latency, not by HBM or shared-memory throughput.  B8 H16 T4096: 545 us (646 with the
 // solve's diagonal blocks and Y on the same warps, and MMAs issued under a divergent branch),
-// with the context 687 us (730; its copies go out one per warp, and A_qk is written
+// with the context 633 us (730; its copies go out one per warp, and A_qk is written
 // beside the -W product).  Few sequences: k_wy_flow (below).
 // Every per-element pass
 // still reads and writes 8 or 16 bytes per shared-memory instruction wherever the
@@ -1812,11 +1812,12 @@ bool wy_fwd_supported(const Args &a) {
 // Where k_wy_flow finishes sooner than k_wy_fwd, in thousands of cycles as measured: the one
 // takes 17 a chunk with one CTA per sequence; k_wy_flow 7 a chunk of a sequence (its memory part)
 // or 19 a chunk of all sequences over its workers, whichever is longer, and 45 until the first
-// records are there.  Post-activation gates, k_wy_flow and k_wy_fwd in us: B1 H16 T824 87 and
-// 131, T2047 161 and 282, T8191 488 and 1060, B2 H16 T2047 175 and 287, B24 H1 T257 59 and 66;
-// logit gates: 95 and 158, 182 and 347, 503 and 1353, 201 and 359, 66 and 80.  With 48 sequences
-// the one is ahead (B3 H16 T1300 216 and 198, T2047 301 and 298); more sequences than 56 leave too few workers.  Fewer than 96
-// chunks in all are left to the one kernel (tens of us either way).
+// records are there.  Post-activation gates, k_wy_flow and k_wy_fwd in us: B1 H16 T823 75 and
+// 118, T2047 141 and 269, T8191 483 and 1046, T65471 3869 and 8172, B2 H16 T2047 168 and 278, B1 H40 T4001 424
+// and 540, B24 H1 T257 48 and 55; logit gates: 82 and 146, 151 and 333, 497 and 1315, 3999 and 10284,
+// 224 and 353, 580 and 670, 55 and 68.  With 48 sequences
+// the one is ahead (B3 H16 T1300 216 and 198, T2047 301 and 298); more sequences than 56 leave too few workers.
+// Fewer than 96 chunks in all are left to the one kernel (tens of us either way).
 // A workspace holds the records of kSlice chunks of all sequences (136 MB); longer sequences take
 // several launches, which hand the state on in float32 (the same results), each with its 45.
 constexpr long long kSlice = 2048;
