@@ -93,6 +93,18 @@ __device__ __forceinline__ void tile_mm_t(float (*acc)[4], const float *A, int l
       for (int n = 0; n < 4; ++n) acc[m][n] = fmaf(a[m], b[n], acc[m][n]);
   }
 }
+// The same in two halves of k, each summed by itself (their partial sums round less): the inter-chunk
+// passes, whose sums go on through every chunk.
+template <int K, int TM>
+__device__ __forceinline__ void tile_mm2(float (*acc)[4], const float *A, int sa, const float *B, int ldb) {
+  float t[TM][4] = {};
+  tile_mm<K / 2, TM, false>(acc, A, sa, B, ldb);
+  tile_mm<K / 2, TM, false>(t, A + K / 2, sa, B + K / 2 * ldb, ldb);
+#pragma unroll
+  for (int m = 0; m < TM; ++m)
+#pragma unroll
+    for (int n = 0; n < 4; ++n) acc[m][n] += t[m][n];
+}
 template <int TM> __device__ __forceinline__ void zero(float (*acc)[4]) {
 #pragma unroll
   for (int m = 0; m < TM; ++m)

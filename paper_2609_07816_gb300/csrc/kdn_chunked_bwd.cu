@@ -60,33 +60,37 @@ __global__ void __launch_bounds__(StateCfg<DK, CW, TM>::NTH) k_state_bwd(Args a)
 #pragma unroll
         for (int n = 0; n < 4; ++n) acc[m][n] = fmaf(sAqk[s2 * LC + r0 + m], d[n], acc[m][n]);
     }
-    tile_mm<DK, TH, false>(acc, sKt + r0 * LD, LD, sS + col, LS);
+    tile_mm2<DK, TH>(acc, sKt + r0 * LD, LD, sS + col, LS);
 #pragma unroll
     for (int m = 0; m < TH; ++m) {
       st4(sdR + (r0 + m) * LS + col, acc[m]);
       st4(a.dR + (base * CC + r0 + m) * dv + j0 + col, acc[m]);
     }
     __syncthreads();
+    float inc[2][RS][4];  // the chunk's part first, in halves, so that S is rounded once
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      zero<RS>(inc[hf]);
+#pragma unroll 4
+      for (int r = hf * (CC / 2); r < (hf + 1) * (CC / 2); ++r) {
+        float d[4], e[4];
+        dO(r, d);
+        ld4<float>(sdR + r * LS, col, e);
+#pragma unroll
+        for (int m = 0; m < RS; ++m) {
+          const float qv = sQ[r * LD + i0 + m], wv = sW[r * LD + i0 + m];
+#pragma unroll
+          for (int n = 0; n < 4; ++n) inc[hf][m][n] = fmaf(qv, d[n], fmaf(-wv, e[n], inc[hf][m][n]));
+        }
+      }
+    }
 #pragma unroll
     for (int m = 0; m < RS; ++m) {
       const float g = sgC[i0 + m];
 #pragma unroll
-      for (int n = 0; n < 4; ++n) S[m][n] *= g;
+      for (int n = 0; n < 4; ++n) S[m][n] = fmaf(g, S[m][n], inc[0][m][n] + inc[1][m][n]);
+      st4(sS + (i0 + m) * LS + col, S[m]);
     }
-#pragma unroll 4
-    for (int r = 0; r < CC; ++r) {
-      float d[4], e[4];
-      dO(r, d);
-      ld4<float>(sdR + r * LS, col, e);
-#pragma unroll
-      for (int m = 0; m < RS; ++m) {
-        const float qv = sQ[r * LD + i0 + m], wv = sW[r * LD + i0 + m];
-#pragma unroll
-        for (int n = 0; n < 4; ++n) S[m][n] = fmaf(qv, d[n], fmaf(-wv, e[n], S[m][n]));
-      }
-    }
-#pragma unroll
-    for (int m = 0; m < RS; ++m) st4(sS + (i0 + m) * LS + col, S[m]);
   }
   if (a.dS0) {
 #pragma unroll

@@ -19,7 +19,7 @@
 // All chunk-local matrices are float32 in shared memory; intermediates that
 // cross kernels live in the caller's workspace.
 //
-// Diagonal prefill B8 H16 T2048 d = 64 bf16, us: 33 + 11 + 279 + 261, 589 a call.  With the
+// Diagonal prefill B8 H16 T2048 d = 64 bf16, us: 33 + 11 + 264 + 267, 578 a call.  With the
 // uncertainty run token by token (1406), one output a thread in the chunk kernel (763) and two
 // loads a multiply-add in the memory pass (790) it was 2922.
 #include <float.h>
@@ -192,7 +192,7 @@ template <typename DT> __host__ __device__ constexpr int v_stride(int dv) { retu
 constexpr float kKkDown = 0x1p-20f, kKkUp = 0x1p20f;
 template <typename DT, int DK>
 constexpr size_t prep_smem_bytes(int dv) {
-  return sizeof(float) * (3 * CC * (DK + 4) + 2 * CC * LC + 16 * 20 + 4 * CC + DK + PT * 5) +
+  return sizeof(float) * (3 * CC * (DK + 4) + 2 * CC * LC + 16 * 20 + 8 * CC + DK + PT * 5) +
          sizeof(DT) * CC * v_stride<DT>(dv);
 }
 
@@ -264,11 +264,32 @@ __device__ __forceinline__ void inverse32(const float *sT, float *sA, float *sX)
   __syncthreads();
 }
 
+// Reduce-scatter of N = 8 or 16 per-lane values over a warp: the warp-wide sum of v[lane / (32 / N)],
+// by pairs.
+template <int N>
+__device__ __forceinline__ float warp_sums(const float *v, int lane) {
+  float w[N];
+#pragma unroll
+  for (int j = 0; j < N; ++j) w[j] = v[j];
+  int o = 16;
+#pragma unroll
+  for (int n = N / 2; n > 0; n >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int j = 0; j < n; ++j) {
+      const float keep = up ? w[n + j] : w[j], send = up ? w[j] : w[n + j];
+      w[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  for (; o > 0; o >>= 1) w[0] += __shfl_xor_sync(0xffffffffu, w[0], o);
+  return w[0];
+}
+
 // SAVE: also keep phat, gamma, A and s_t (iso: beta_t) for the backward.
 // One CTA of 128 threads per chunk; five of them on an SM cover each other's load and barrier
 // latencies.  Bound by shared-memory loads and issue (ncu, B8 H16 T2048 d = 64: 58 % of the
 // shared-memory cycles, 51 % of the issue slots, the rest waits for the first loads); register
-// tiles of 4 x 4 outputs, since a 16-byte load costs four cycles of the SM.  279 us (763 with
+// tiles of 4 x 4 outputs, since a 16-byte load costs four cycles of the SM.  264 us (763 with
 // one output a thread).
 template <int V, typename DT, int DK, int SAVE>
 __global__ void __launch_bounds__(PT, DK < 128 ? 5 : 3) k_chunk_prep(Args a) {
@@ -277,7 +298,7 @@ __global__ void __launch_bounds__(PT, DK < 128 ? 5 : 3) k_chunk_prep(Args a) {
   const int dv = a.dv, lv = v_stride<DT>(dv);
   float *sK = sm, *sQ = sK + CC * LD, *sKk = sQ + CC * LD, *sT = sKk + CC * LD, *sA = sT + CC * LC;
   float *sX = sA + CC * LC, *s_r = sX + 16 * 20, *s_mr = s_r + CC;
-  float *s_is = s_mr + CC, *s_be = s_is + CC, *s_gC = s_be + CC, *s_seg = s_gC + DK;
+  float *s_is = s_mr + CC, *s_be = s_is + CC, *s_k2 = s_be + CC, *s_gC = s_k2 + 4 * CC, *s_seg = s_gC + DK;
   DT *sV = reinterpret_cast<DT *>(s_seg + PT * 5);
   const int tid = KDN_TID;
   const int bh = (int)(blockIdx.x / (unsigned)a.NC), c = (int)(blockIdx.x % (unsigned)a.NC);
@@ -355,10 +376,16 @@ __global__ void __launch_bounds__(PT, DK < 128 ? 5 : 3) k_chunk_prep(Args a) {
         }
         renorm_pow2(m);
       }
-      const float bt = moebius_apply(m, pin);  // b_t
-      float bp = __shfl_up_sync(0xffffffffu, bt, 1);
-      if (tid == 0) bp = pin;
-      const float bhat = fmaf(aa, bp, w);  // eq. iso-kla-box-cov-update
+      // b_t, then twice one step of the recursion from b_{t-1}, which damps the products' rounding
+      float bt = moebius_apply(m, pin), bhat;
+      const float u = fminf(a.mu * n2 / (DK * rr), FLT_MAX);
+#pragma unroll
+      for (int it = 0; it < 3; ++it) {
+        float bp = __shfl_up_sync(0xffffffffu, bt, 1);
+        if (tid == 0) bp = pin;
+        bhat = fmaf(aa, bp, w);  // eq. iso-kla-box-cov-update
+        if (it < 2) bt = bhat / fmaf(u, bhat, 1.f);
+      }
       const float beta = tid < tn ? bhat / (rr + bhat * n2) : 0.f;
       s_be[tid] = beta;
       if (SAVE) {
@@ -409,6 +436,7 @@ __global__ void __launch_bounds__(PT, DK < 128 ? 5 : 3) k_chunk_prep(Args a) {
         ph = fmaf(a2[j], p, wv[j]);                             // eq. diag-covariance-prediction
         p = ph / fmaf(s_mr[t] * kv[j] * kv[j], ph, 1.f);        // eq. diag-cov-update
         kk = kKkDown * ph * kv[j];
+        a2[j] = ph * kv[j] * kv[j];
       } else {
         kk = s_be[t] * kv[j];
       }
@@ -420,6 +448,10 @@ __global__ void __launch_bounds__(PT, DK < 128 ? 5 : 3) k_chunk_prep(Args a) {
         a.gam[grow + (size_t)t * DK] = gam;
       }
     }
+    if (V == 0) {  // sum_i phat k^2 over this warp's channels
+      const float s = warp_sums<LB>(a2, tid & 31);
+      if ((tid & (32 / LB - 1)) == 0) s_k2[(i >> 5) * CC + tb + (tid & 31) / (32 / LB)] = s;
+    }
   }
   if (t0 + SL == CC) {
     s_gC[i] = gam;
@@ -428,26 +460,20 @@ __global__ void __launch_bounds__(PT, DK < 128 ? 5 : 3) k_chunk_prep(Args a) {
   }
   __syncthreads();
 
+  if (V == 0 && tid < CC) {  // s_t = r_t + sum_i phat k^2 (eq. kla-box-gain)
+    float s = s_k2[tid];
+#pragma unroll
+    for (int w = 1; w < DK / 32; ++w) s += s_k2[w * CC + tid];
+    s += s_r[tid];
+    s_is[tid] = fminf(kKkUp / s, FLT_MAX);
+    if (SAVE) a.stok[(size_t)bh * a.Tp + c * CC + tid] = s;
+  }
   // T' = Kbar Kk'^T (threads 0..63), A'_qk = Qbar Kk'^T (64..127): 32 x 32, 4 x 4 a thread.
-  // Diagonal KDN: the diagonal of T' is kKkDown sum_i phat k^2, so s_t = r_t + kKkUp T'_tt (eq. kla-box-gain).
   const int lane = tid & 31, w2 = (tid >> 5) & 1, ga = lane >> 2, gb = (lane & 3) + 4 * w2;
   float acc[4][4];
   zero<4>(acc);
   tile_mm<DK, 4, true>(acc, (tid < 64 ? sK : sQ) + ga * LD, 8 * LD, sKk + 4 * gb * LD, LD);
-  if (V == 0) {
-    if (tid < 64) {
-#pragma unroll
-      for (int m = 0; m < 4; ++m)
-#pragma unroll
-        for (int n = 0; n < 4; ++n)
-          if (ga + 8 * m == 4 * gb + n) {
-            const float s = s_r[4 * gb + n] + kKkUp * acc[m][n];
-            s_is[4 * gb + n] = fminf(kKkUp / s, FLT_MAX);
-            if (SAVE) a.stok[(size_t)bh * a.Tp + c * CC + 4 * gb + n] = s;
-          }
-    }
-    __syncthreads();
-  }
+  if (V == 0) __syncthreads();  // s_is
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
     const int r = ga + 8 * m;
@@ -502,8 +528,9 @@ __global__ void __launch_bounds__(PT, DK < 128 ? 5 : 3) k_chunk_prep(Args a) {
 // The inter-chunk pass: a chain over the chunks, one CTA per (sequence, value columns), the next
 // chunk's factors in flight.  A thread keeps its rows of S in registers and forms 8 x 4 tiles of
 // [W; Qbar] S.  With one warp per scheduler it is bound by latency and shared-memory loads (ncu,
-// B8 H16 T2048 d = 64: 55 % of the issue slots, 52 % of the shared-memory cycles): 261 us for
-// 64 chunks, 790 before.
+// B8 H16 T2048 d = 64: 55 % of the issue slots, 52 % of the shared-memory cycles): 267 us for
+// 64 chunks, 790 before.  The sums are split in halves and a chunk's part is added to S at once, so that
+// they round no more than a token loop's would (261 us in one chain, S and dS off by up to 1.5 times as much).
 
 template <int DK, int CW, int TM, int SAVE>
 __global__ void __launch_bounds__(StateCfg<DK, CW, TM>::NTH) k_state_fwd(Args a) {
@@ -539,7 +566,7 @@ __global__ void __launch_bounds__(StateCfg<DK, CW, TM>::NTH) k_state_fwd(Args a)
     }
     float acc[TM][4];
     zero<TM>(acc);
-    tile_mm<DK, TM, false>(acc, buf + ga * LD, GA * LD, sS + col, LS);
+    tile_mm2<DK, TM>(acc, buf + ga * LD, GA * LD, sS + col, LS);
     // R = U - W S_in
 #pragma unroll
     for (int m = 0; m < TH; ++m) {
@@ -554,23 +581,31 @@ __global__ void __launch_bounds__(StateCfg<DK, CW, TM>::NTH) k_state_fwd(Args a)
     __syncthreads();
     // O = Qbar S_in + A_qk R
     if (a.o) {
-      tile_mm<CC, TH, false>(acc + TH, sAqk + ga * LC, GA * LC, sR + col, LS);
+      float t[TH][4];
+      zero<TH>(t);
+      tile_mm<CC, TH, false>(t, sAqk + ga * LC, GA * LC, sR + col, LS);
 #pragma unroll
       for (int m = 0; m < TH; ++m) {
         const int tt = c * CC + ga + GA * m;
-        if (tt < a.T) sto4(a.odt, a.o, tok_index(a, b, tt, h) * dv + j0 + col, acc[TH + m]);
+#pragma unroll
+        for (int n = 0; n < 4; ++n) t[m][n] += acc[TH + m][n];
+        if (tt < a.T) sto4(a.odt, a.o, tok_index(a, b, tt, h) * dv + j0 + col, t[m]);
       }
     }
-    // S_out = diag(gamma_C) S_in + K_tail^T R
+    // S_out = diag(gamma_C) S_in + K_tail^T R: the chunk's part first, so that S is rounded once
+    float inc[2][RS][4];
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      zero<RS>(inc[hf]);
+      tile_mm_t<CC / 2, RS>(inc[hf], sKt + hf * (CC / 2) * LD + i0, LD, sR + hf * (CC / 2) * LS + col, LS);
+    }
 #pragma unroll
     for (int m = 0; m < RS; ++m) {
       const float g = sgC[i0 + m];
 #pragma unroll
-      for (int n = 0; n < 4; ++n) S[m][n] *= g;
+      for (int n = 0; n < 4; ++n) S[m][n] = fmaf(g, S[m][n], inc[0][m][n] + inc[1][m][n]);
+      st4(sS + (i0 + m) * LS + col, S[m]);
     }
-    tile_mm_t<CC, RS>(S, sKt + i0, LD, sR + col, LS);
-#pragma unroll
-    for (int m = 0; m < RS; ++m) st4(sS + (i0 + m) * LS + col, S[m]);
   }
   if (a.ST) {
 #pragma unroll
